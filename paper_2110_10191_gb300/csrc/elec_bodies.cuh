@@ -125,9 +125,10 @@ __device__ __forceinline__ void elec_recon_body(const StepArgs &A, const double 
     const double *p = K + q * D.ntot + c;
     double lo, hi;
     if (A.recon == 1) {
-      weno5_pair(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st), __ldg(p + 2 * st), lo, hi);
+      weno5_wide_pair(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st), __ldg(p + 2 * st),
+                      lo, hi);
     } else {
-      const double x1 = __ldg(p), h = 0.5 * mc_slope(__ldg(p - st), x1, __ldg(p + st));
+      const double x1 = __ldg(p), h = mc_half_slope(x1 - __ldg(p - st), __ldg(p + st) - x1);
       lo = x1 - h;
       hi = x1 + h;
     }

@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "wide.cuh"
+
 namespace grmhd {
 
 constexpr int NV = 8;
@@ -273,122 +275,97 @@ __device__ __forceinline__ double mhd_cmax(const double P[NV], const FState &s, 
 // ---------------------------------------------------------------------------
 // Reconstruction
 // ---------------------------------------------------------------------------
-// MC limited slope of x1 with neighbours x0, x2.
-__device__ __forceinline__ double mc_slope(double x0, double x1, double x2) {
-  const double dm = x1 - x0, dp = x2 - x1;
-  if (!(dm * dp > 0.0)) return 0.0;
-  const double dc = 0.5 * (dm + dp);
-  const double m = fmin(fmin(fabs(2.0 * dm), fabs(dc)), fabs(2.0 * dp));
-  return (dc > 0.0) ? m : -m;
+// Half the MC limited slope of a zone from its first differences dm (low side)
+// and dp: 0 at an extremum, else the least magnitude of dm, dp and (dm + dp)/4,
+// the sign theirs.  Only the sum takes the FP64 pipe: magnitudes order like
+// their bit patterns, and /4 is an exponent step (a multiplication near the
+// subnormals).
+__device__ __forceinline__ double mc_half_slope(double dm, double dp) {
+  const u64 bm = w_bits(dm), bp = w_bits(dp), mag = ~0ull >> 1, inf = 0x7ffull << 52;
+  const u64 a = bm & mag, b = bp & mag;
+  if ((s64)(bm ^ bp) < 0 || a == 0 || b == 0 || a > inf || b > inf) return 0.0;
+  const double s = dm + dp;
+  const u64 c = w_bits(s) & mag;
+  u64 h = (a < b) ? a : b;
+  if ((u32)(c >> 52) - 3u < 0x7fcu) {  // s / 4 is normal
+    const u64 q = c - (2ull << 52);
+    h = (q < h) ? q : h;
+  } else {
+    const u64 q = w_bits(0.25 * s) & mag;
+    h = (q < h) ? q : h;
+  }
+  return w_double(h | (bm & ~mag));
 }
 
-// Jiang-Shu WENO5 value at the high face of the middle zone of a..e
-// (cell averages; epsilon 1e-26, weights d_k/(eps + beta_k)^2).
-__device__ __forceinline__ double weno5_hi(double a, double b, double c, double d, double e) {
-  const double eps = 1.0e-26;
-  const double t0 = a - 2.0 * b + c, t1 = b - 2.0 * c + d, t2 = c - 2.0 * d + e;
-  const double s0 = a - 4.0 * b + 3.0 * c, s1 = b - d, s2 = 3.0 * c - 4.0 * d + e;
-  const double b0 = (13.0 / 12.0) * t0 * t0 + 0.25 * s0 * s0;
-  const double b1 = (13.0 / 12.0) * t1 * t1 + 0.25 * s1 * s1;
-  const double b2 = (13.0 / 12.0) * t2 * t2 + 0.25 * s2 * s2;
-  const double e0 = eps + b0, e1 = eps + b1, e2 = eps + b2;
-  const double q0 = e0 * e0, q1 = e1 * e1, q2 = e2 * e2;
-  // alpha_k = d_k / q_k ; common denominator q0 q1 q2
-  const double a0 = 0.1 * (q1 * q2), a1 = 0.6 * (q0 * q2), a2 = 0.3 * (q0 * q1);
-  const double p0 = (2.0 * a - 7.0 * b + 11.0 * c) * (1.0 / 6.0);
-  const double p1 = (-b + 5.0 * c + 2.0 * d) * (1.0 / 6.0);
-  const double p2 = (2.0 * c + 5.0 * d - e) * (1.0 / 6.0);
-  return (a0 * p0 + a1 * p1 + a2 * p2) / (a0 + a1 + a2);
-}
+// Both face values of consecutive zones of one column: start() on the first
+// zone's stencil (xm2 .. xp2), faces() of the current zone, next() with the
+// value two zones above the next one.  Each zone after the first forms one new
+// first difference and one new pair; the values equal weno5_wide_pair's on each
+// zone's own stencil bit for bit.
+struct WenoWalk {
+  double x0, xp1, xp2;  // the current zone and the two above
+  WideDiff f;           // xp2 - xp1
+  WidePair p0, p1, p2;  // the current zone's substencils, lowest first
+  WideNum q0, q1, q2;   // their squared indicators in those roles
+  WideNum r1, r2, s2;   // p1's as the lowest, p2's as the middle and the lowest
 
-// Both WENO5 face values of the middle zone of a..e (zones c-2..c+2), written
-// in the stencil's first differences (dm2 = b-a, dm1 = c-b, dp1 = d-c,
-// dp2 = e-d), second differences (D0 = a-2b+c, D1 = b-2c+d, D2 = c-2d+e) and
-// s0 = D0 + 2 dm1, s1 = dm1 + dp1, s2 = D2 - 2 dp1:
-//   4 beta_k = (13/3) D_k^2 + s_k^2,
-// and, with q_k the candidate values at the high face,
-//   6 (q_0 - c) = A = 2 D0 + 3 dm1 = Cl + D0,   Cl = D0 + 3 dm1 = s0 + dm1,
-//   6 (q_1 - c) = B = dm1 + 2 dp1  = s1 + dp1,
-//   6 (q_2 - c) = C = 3 dp1 - D2   = dp1 - s2,
-// the low face's by mirroring: Al = 2 D2 - 3 dp1 = D2 - C, Bl = dp1 + 2 dm1
-// = s1 + dm1, Cl.  The weights d_k/(eps + beta_k)^2 are taken over the
-// common denominator q0 q1 q2 of the squared (4 eps + 4 beta_k) and scaled
-// by 10, which leaves their ratios unchanged, and one reciprocal serves
-// both faces, with the 1/6 of the candidate differences folded into it.
-// 4 eps + 4 beta_k = s_k^2 + T_k with T_k = (13/3) D_k^2 + 4 eps, a
-// function of the one second difference D_k: along a column the T_k of
-// one zone are T_{k+1}, T_{k+2} of its lower neighbours, so a walk forms one
-// new D and T per zone (weno5_walk).  The terms pair up under the mirror
-// a <-> e, b <-> d (A <-> Al, B <-> -Bl, C <-> -Cl, D0 <-> D2, s0 <-> -s2),
-// so a mirrored stencil gives the same two values swapped, bit for bit.
-__device__ __forceinline__ double weno5_T(double Dk) {
-  return fma((13.0 / 3.0) * Dk, Dk, 4.0e-26);
-}
-
-__device__ __forceinline__ void weno5_pair_dt(double c, double dm1, double dp1, double D0,
-                                              double D1, double D2, double T0, double T1,
-                                              double T2, double &lo, double &hi) {
-  const double s0 = fma(2.0, dm1, D0), s1 = dm1 + dp1, s2 = fma(-2.0, dp1, D2);
-  const double e0 = fma(s0, s0, T0), e1 = fma(s1, s1, T1), e2 = fma(s2, s2, T2);
-  const double q0 = e0 * e0, q1 = e1 * e1, q2 = e2 * e2;
-  // linear weights in the ratio 1 : 6 : 3 (only ratios enter)
-  const double q12 = q1 * q2, q02 = 6.0 * (q0 * q2), q01 = q0 * q1;
-  const double t01 = 3.0 * q01, t12 = 3.0 * q12;
-  const double Cl = s0 + dm1, A = Cl + D0, B = s1 + dp1, C = dp1 - s2;
-  const double Al = D2 - C, Bl = s1 + dm1;
-  // high face: weights q12, 6 q02, 3 q01
-  const double nh = fma(t01, C, fma(q02, B, q12 * A));
-  const double H = (q12 + q02) + t01;
-  // low face (mirrored stencil): weights q01, 6 q02, 3 q12
-  const double nl = fma(-t12, Cl, fma(-q02, Bl, q01 * Al));
-  const double L = (q01 + q02) + t12;
-  const double r = rcp_nr(H * L) * (1.0 / 6.0);
-  hi = fma(nh, L * r, c);
-  lo = fma(nl, H * r, c);
-}
-
-__device__ __forceinline__ void weno5_pair(double a, double b, double c, double d, double e,
-                                           double &lo, double &hi) {
-  const double dm2 = b - a, dm1 = c - b, dp1 = d - c, dp2 = e - d;
-  const double D0 = dm1 - dm2, D1 = dp1 - dm1, D2 = dp2 - dp1;
-  weno5_pair_dt(c, dm1, dp1, D0, D1, D2, weno5_T(D0), weno5_T(D1), weno5_T(D2), lo, hi);
-}
-
-// Both face values of n <= 16 consecutive zones of one column (stride st;
-// p, lf and rf point at the first zone): each zone after the first loads one
-// new value and forms one first difference, one second difference and one
-// T_k; the values equal weno5_pair's on each zone's stencil bit for bit.
-__device__ __forceinline__ void weno5_walk(const double *__restrict__ p, double *__restrict__ lf,
-                                           double *__restrict__ rf, long long st, int n) {
-  const double xm1 = __ldg(p - st);
-  double x0 = __ldg(p), xp1 = __ldg(p + st), xp2 = __ldg(p + 2 * st);
-  double dm1 = x0 - xm1, dp1 = xp1 - x0, dp2 = xp2 - xp1;
-  double D0 = dm1 - (xm1 - __ldg(p - 2 * st)), D1 = dp1 - dm1, D2 = dp2 - dp1;
-  double T0 = weno5_T(D0), T1 = weno5_T(D1), T2 = weno5_T(D2);
-  // unrolled over the longest segment (the segments' length is at most 16):
-  // a rolled loop of unknown trip count ran 12% slower
-#pragma unroll
-  for (int m = 0; m < 16; m++) {
-    // the next zone's new value, loaded before this zone's arithmetic
-    const double xn = (m + 1 < n) ? __ldg(p + (m + 3) * st) : 0.0;
-    double lo, hi;
-    weno5_pair_dt(x0, dm1, dp1, D0, D1, D2, T0, T1, T2, lo, hi);
-    lf[m * st] = lo;
-    rf[m * st] = hi;
-    if (m + 1 >= n) break;
-    const double dn = xn - xp2;
+  __device__ __forceinline__ void start(double xm2, double xm1, double x, double x1, double x2) {
+    x0 = x;
+    xp1 = x1;
+    xp2 = x2;
+    const WideDiff d0 = wide_diff(xm1 - xm2), d1 = wide_diff(x0 - xm1), d2 = wide_diff(x1 - x0);
+    f = wide_diff(x2 - x1);
+    p0 = wide_pair(d0, d1);
+    p1 = wide_pair(d1, d2);
+    p2 = wide_pair(d2, f);
+    const u64 D0 = wide_D13(p0), D1 = wide_D13(p1), D2 = wide_D13(p2);
+    q0 = wide_q_low(p0, D0);
+    q1 = wide_q_mid(p1, D1);
+    r1 = wide_q_low(p1, D1);
+    q2 = wide_q_high(p2, D2);
+    r2 = wide_q_mid(p2, D2);
+    s2 = wide_q_low(p2, D2);
+  }
+  __device__ __forceinline__ void faces(double &lo, double &hi) const {
+    weno5_wide(x0, p0, p1, p2, q0, q1, q2, lo, hi);
+  }
+  __device__ __forceinline__ void next(double xn) {
+    const WideDiff g = wide_diff(xn - xp2);
     x0 = xp1;
     xp1 = xp2;
     xp2 = xn;
-    dm1 = dp1;
-    dp1 = dp2;
-    D0 = D1;
-    D1 = D2;
-    D2 = dn - dp2;
-    dp2 = dn;
-    T0 = T1;
-    T1 = T2;
-    T2 = weno5_T(D2);
+    p0 = p1;
+    p1 = p2;
+    p2 = wide_pair(f, g);
+    f = g;
+    const u64 D = wide_D13(p2);
+    q0 = r1;
+    q1 = r2;
+    r1 = s2;
+    q2 = wide_q_high(p2, D);
+    r2 = wide_q_mid(p2, D);
+    s2 = wide_q_low(p2, D);
+  }
+};
+
+// Both face values of n consecutive zones of one column (stride st; p, lf and
+// rf point at the first zone).
+__device__ __forceinline__ void weno5_walk(const double *__restrict__ p, double *__restrict__ lf,
+                                           double *__restrict__ rf, long long st, int n) {
+  WenoWalk w;
+  w.start(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st), __ldg(p + 2 * st));
+#pragma unroll 1
+  for (int m = 0; m < n; m++) {
+    // the next zone's new value, loaded before this zone's arithmetic
+    const double xn = (m + 1 < n) ? __ldg(p + 3 * st) : 0.0;
+    double lo, hi;
+    w.faces(lo, hi);
+    *lf = lo;
+    *rf = hi;
+    p += st;
+    lf += st;
+    rf += st;
+    w.next(xn);
   }
 }
 

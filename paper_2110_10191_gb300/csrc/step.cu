@@ -46,13 +46,14 @@ __global__ void __launch_bounds__(BS) k_flux(StepArgs A, const double *__restric
       if (RECON == 1) {
         const double x0 = __ldg(p - 3 * st), x1 = __ldg(p - 2 * st), x2 = __ldg(p - st);
         const double x3 = __ldg(p), x4 = __ldg(p + st), x5 = __ldg(p + 2 * st);
-        PL[v] = weno5_hi(x0, x1, x2, x3, x4);
-        PR[v] = weno5_hi(x5, x4, x3, x2, x1);
+        double other;
+        weno5_wide_pair(x0, x1, x2, x3, x4, other, PL[v]);
+        weno5_wide_pair(x1, x2, x3, x4, x5, PR[v], other);
       } else {
         const double x1 = __ldg(p - 2 * st), x2 = __ldg(p - st);
         const double x3 = __ldg(p), x4 = __ldg(p + st);
-        PL[v] = x2 + 0.5 * mc_slope(x1, x2, x3);
-        PR[v] = x3 - 0.5 * mc_slope(x2, x3, x4);
+        PL[v] = x2 + mc_half_slope(x2 - x1, x3 - x2);
+        PR[v] = x3 - mc_half_slope(x3 - x2, x4 - x3);
       }
     }
     const int loc = (DIR == 0) ? LOC_FACE1 : (DIR == 1) ? LOC_FACE2 : LOC_CENT;

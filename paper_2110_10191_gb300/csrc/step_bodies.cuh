@@ -54,7 +54,6 @@ __host__ __device__ inline long long n_recon(const Dims &D, int flat3) {
 }
 // longest FP64 reconstruction walk (zones per thread)
 constexpr int RWALK = 16;
-static_assert(RWALK <= 16, "weno5_walk unrolls over at most 16 zones");
 // threads of the FP64 reconstruction along dir: one per column and segment
 // of rw zones along dir (rw >= 2), or one per zone (rw = 1)
 __host__ __device__ inline long long n_recon_walk(const Dims &D, int dir, int flat3, int rw) {
@@ -230,10 +229,10 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
       const double *p = P + v * D.ntot + c;
       double lo, hi;
       if (RECON == 1) {
-        weno5_pair(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st), __ldg(p + 2 * st),
-                   lo, hi);
+        weno5_wide_pair(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st),
+                        __ldg(p + 2 * st), lo, hi);
       } else {
-        const double x1 = __ldg(p), h = 0.5 * mc_slope(__ldg(p - st), x1, __ldg(p + st));
+        const double x1 = __ldg(p), h = mc_half_slope(x1 - __ldg(p - st), __ldg(p + st) - x1);
         lo = x1 - h;
         hi = x1 + h;
       }
@@ -263,11 +262,13 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
     if (RECON == 1) {
       weno5_walk(p, lf, rf, st, n);
     } else {
+      double x1 = __ldg(p), dm = x1 - __ldg(p - st);
       for (int m = 0; m < n; m++) {
-        const double *q = p + m * st;
-        const double x1 = __ldg(q), h = 0.5 * mc_slope(__ldg(q - st), x1, __ldg(q + st));
+        const double x2 = __ldg(p + (m + 1) * st), dp = x2 - x1, h = mc_half_slope(dm, dp);
         lf[m * st] = x1 - h;
         rf[m * st] = x1 + h;
+        x1 = x2;
+        dm = dp;
       }
     }
   }
@@ -324,33 +325,16 @@ __device__ __forceinline__ void recon_x1_staged(const StepArgs &A, const double 
       if (nq > 0 && xq < nq + 4) tin[q * X1_IN + xq] = __ldg(P + ov + rbase[q] - 2 + xq);
     }
     __syncwarp();
-    const double xm1 = x[1];
-    double x0 = x[2], xp1 = x[3], xp2 = x[4];
-    double dm1 = x0 - xm1, dp1 = xp1 - x0, dp2 = xp2 - xp1;
-    double D0 = dm1 - (xm1 - x[0]), D1 = dp1 - dm1, D2 = dp2 - dp1;
-    double T0 = weno5_T(D0), T1 = weno5_T(D1), T2 = weno5_T(D2);
-#pragma unroll
+    WenoWalk w;
+    w.start(x[0], x[1], x[2], x[3], x[4]);
+#pragma unroll 1
     for (int m = 0; m < RWALK; m++) {
       if (m < n) {
         double lo, hi;
-        weno5_pair_dt(x0, dm1, dp1, D0, D1, D2, T0, T1, T2, lo, hi);
+        w.faces(lo, hi);
         tout[lane * X1_OUT + (m & 7)] = lo;
         tout[X1_HI + lane * X1_OUT + (m & 7)] = hi;
-        if (m + 1 < n) {
-          const double dn = x[m + 5] - xp2;
-          x0 = xp1;
-          xp1 = xp2;
-          xp2 = x[m + 5];
-          dm1 = dp1;
-          dp1 = dp2;
-          D0 = D1;
-          D1 = D2;
-          D2 = dn - dp2;
-          dp2 = dn;
-          T0 = T1;
-          T1 = T2;
-          T2 = weno5_T(D2);
-        }
+        if (m + 1 < n) w.next(x[m + 5]);
       }
       if ((m & 7) == 7) {  // write zones m-7 .. m of every row: 4 rows x 8 zones per store
         __syncwarp();
