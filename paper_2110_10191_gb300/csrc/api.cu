@@ -727,6 +727,17 @@ extern "C" int grmhd_set_geometry(grmhd_sim *s, int loc, const double *in) {
     g[(size_t)(G_IGDET * n2d + q)] = 1.0 / in[32 * n2d + q];
     g[(size_t)(G_OMALPHA * n2d + q)] = (1.0 + 1.0 / in[(16 + 0) * n2d + q]) / (1.0 + al);
   }
+  // whether this location's metric couples X2 to the other coordinates
+  Clock c;
+  CK(cudaMemcpyAsync(&c, s->clk, sizeof(c), cudaMemcpyDeviceToHost, s->st));
+  CK(cudaStreamSynchronize(s->st));
+  c.coupled &= ~(1 << loc);
+  const int cross[] = {SY(0, 2), SY(1, 2), SY(2, 3)};
+  for (const int base : {G_GCOV, G_GCON})
+    for (const int k : cross)
+      for (long long q = 0; q < n2d; q++)
+        if (g[(size_t)((base + k) * n2d + q)] != 0.0) c.coupled |= 1 << loc;
+  CK(cudaMemcpyAsync(&s->clk->coupled, &c.coupled, sizeof(c.coupled), cudaMemcpyHostToDevice, s->st));
   CK(cudaMemcpyAsync(s->geom + (long long)loc * G_NCOMP * n2d, g.data(), sizeof(double) * g.size(),
                      cudaMemcpyHostToDevice, s->st));
   if (s->geomf)

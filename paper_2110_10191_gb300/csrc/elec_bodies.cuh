@@ -115,9 +115,8 @@ __device__ __forceinline__ void elec_recon_body(const StepArgs &A, const double 
   const Dims &D = A.D;
   const int e0 = D.n[0] + 2, e1 = D.n[1] + 2;
   if (t >= n_recon(D, A.flat3)) return;
-  const int i = NG - 1 + (int)(t % e0);
-  const int j = NG - 1 + (int)((t / e0) % e1);
-  const int k = (A.flat3 ? NG : NG - 1) + (int)(t / ((long long)e0 * e1));
+  const Idx3 q3 = unflatten(t, e0, e1);
+  const int i = NG - 1 + q3.i, j = NG - 1 + q3.j, k = (A.flat3 ? NG : NG - 1) + q3.k;
   const long long c = zid(D, i, j, k);
   const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
 #pragma unroll
@@ -151,9 +150,8 @@ __device__ __forceinline__ void elec_flux_body(const StepArgs &A, const double *
   int lo[3], ext[3];
   face_box(D, DIR, A.flat3, lo, ext);
   if (t >= (long long)ext[0] * ext[1] * ext[2]) return;
-  const int i = lo[0] + (int)(t % ext[0]);
-  const int j = lo[1] + (int)((t / ext[0]) % ext[1]);
-  const int k = lo[2] + (int)(t / ((long long)ext[0] * ext[1]));
+  const Idx3 q3 = unflatten(t, ext[0], ext[1]);
+  const int i = lo[0] + q3.i, j = lo[1] + q3.j, k = lo[2] + q3.k;
   const long long c = zid(D, i, j, k), N = D.ntot;
   const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
   const double wl = A.elec_w[(2 * DIR) * N + c], wr = A.elec_w[(2 * DIR + 1) * N + c];
@@ -187,9 +185,8 @@ __device__ __forceinline__ void elec_post_body(const StepArgs &A, const double *
   const bool active = t < n_zone(D);
   int ff = 0;
   if (active) {
-    const int i = NG + (int)(t % D.n[0]);
-    const int j = NG + (int)((t / D.n[0]) % D.n[1]);
-    const int k = NG + (int)(t / ((long long)D.n[0] * D.n[1]));
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
     Geo G;
@@ -256,9 +253,8 @@ __device__ __forceinline__ void elec_fix_body(const StepArgs &A, double *P, doub
   const bool active = t < n_zone(D);
   bool hit = false;
   if (active) {
-    const int i = NG + (int)(t % D.n[0]);
-    const int j = NG + (int)((t / D.n[0]) % D.n[1]);
-    const int k = NG + (int)(t / ((long long)D.n[0] * D.n[1]));
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     if (pflag[c] != 0) {
       double sum = 0.0;

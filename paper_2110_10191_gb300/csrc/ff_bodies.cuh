@@ -148,9 +148,8 @@ __device__ __forceinline__ void recon_ff_body(const StepArgs &A, const float *__
   const Dims &D = A.D;
   const int e0 = D.n[0] + 2, e1 = D.n[1] + 2;
   if (t >= n_recon(D, A.flat3)) return;
-  const int i = NG - 1 + (int)(t % e0);
-  const int j = NG - 1 + (int)((t / e0) % e1);
-  const int k = (A.flat3 ? NG : NG - 1) + (int)(t / ((long long)e0 * e1));
+  const Idx3 q3 = unflatten(t, e0, e1);
+  const int i = NG - 1 + q3.i, j = NG - 1 + q3.j, k = (A.flat3 ? NG : NG - 1) + q3.k;
   const long long c = zid(D, i, j, k);
   const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
   const long long half = (long long)NV * D.ntot;
@@ -309,9 +308,8 @@ __device__ __forceinline__ void face_ff_body(const StepArgs &A, const float *__r
   const bool active = t < nface;
   double ctop = 0.0;
   if (active) {
-    const int i = lo[0] + (int)(t % ext[0]);
-    const int j = lo[1] + (int)((t / ext[0]) % ext[1]);
-    const int k = lo[2] + (int)(t / ((long long)ext[0] * ext[1]));
+    const Idx3 q3 = unflatten(t, ext[0], ext[1]);
+    const int i = lo[0] + q3.i, j = lo[1] + q3.j, k = lo[2] + q3.k;
     const long long c = zid(D, i, j, k);
     const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
     const long long half = (long long)NV * D.ntot;
@@ -571,9 +569,8 @@ __device__ __forceinline__ void update_ff_body(const StepArgs &A, const double *
   const bool active = t < nz;
   int pf = 0, fl = 0;
   if (active) {
-    const int i = NG + (int)(t % D.n[0]);
-    const int j = NG + (int)((t / D.n[0]) % D.n[1]);
-    const int k = NG + (int)(t / ((long long)D.n[0] * D.n[1]));
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
     GeoFF G;

@@ -209,66 +209,29 @@ __device__ __forceinline__ void prim_flux(const double P[NV], const FState &s, c
   F[B3] = G.gdet * (s.bcon[3] * ud - bd * s.ucon[3]);
 }
 
-// acc (+)= F^dir + coef * U without the sqrt(-g) factor: the two rows
-// T^dir_nu and T^t_nu share (rho + u + p + b^2) u_nu and b_nu.  FIRST: acc
-// is set rather than added to (the first state of a face).  gm1 = gamma - 1.
-template <bool FIRST>
-__device__ __forceinline__ void flux_cons_acc(const double P[NV], const FState &s, double gm1,
-                                              int dir, double coef, double acc[NV]) {
-  const double pg = gm1 * P[UU];
-  const double w = P[RHO] + P[UU] + pg + s.bsq;
-  const double pt = pg + 0.5 * s.bsq;
-  const double ud = s.ucon[dir], ut = s.ucon[0];
-  const double bd = s.bcon[dir], bt = s.bcon[0];
-  // combined contravariant weights: F + coef U = (u^d + coef u^t) ... - (b^d + coef b^t) ...
-  const double uc = ud + coef * ut;
-  const double bc = bd + coef * bt;
-  const double wuc = w * uc;
-  double T[4];
-#pragma unroll
-  for (int nu = 0; nu < 4; nu++) T[nu] = wuc * s.ucov[nu] - bc * s.bcov[nu];
-  T[dir] += pt;
-  T[0] += coef * pt;
-  const double mf = P[RHO] * uc;
-  const double add[NV] = {mf,
-                          T[0] + mf,
-                          T[1],
-                          T[2],
-                          T[3],
-                          s.bcon[1] * uc - bc * s.ucon[1],
-                          s.bcon[2] * uc - bc * s.ucon[2],
-                          s.bcon[3] * uc - bc * s.ucon[3]};
-#pragma unroll
-  for (int v = 0; v < NV; v++) acc[v] = FIRST ? add[v] : acc[v] + add[v];
-}
-
 // Fast-magnetosonic coordinate speeds along dir: roots v of
 // (k.u)^2 = cms2 (k.k + (k.u)^2) for k_mu = delta^dir_mu - v delta^t_mu,
 // cms2 = cs2 + va2 - cs2 va2; a negative discriminant counts as zero.
 // With cs2 = gamma (gamma - 1) u / e_f, va2 = b^2 / (b^2 + e_f) and
 // e_f = rho + gamma u, the combination is exactly
 // cms2 = (gamma (gamma - 1) u + b^2) / (b^2 + e_f): one reciprocal, no
-// cancellation.  ggm1 = gamma (gamma - 1).  Returns the larger magnitude of
+// cancellation.  Returns the larger magnitude of
 // the two roots (hb +- disc)/qa, disc >= 0: (|hb| + disc)/|qa|, the same
 // rounded value as the larger rounded root's magnitude (the LLF flux and
 // the time step need only it).
-__device__ __forceinline__ double mhd_cmax(const double P[NV], const FState &s, const Geo &G,
-                                           double gam, double ggm1, int dir) {
-  const double ef = fma(gam, P[UU], P[RHO]);
-  const double ee = s.bsq + ef;
-  const double cms2 = fma(ggm1, P[UU], s.bsq) * rcp_nr(ee);
-  const double Asq = G.gcon[SY(dir, dir)];
-  const double Bsq = G.gcon[SY(0, 0)];
-  const double AB = G.gcon[SY(0, dir)];
-  const double Au = s.ucon[dir];
-  const double Bu = s.ucon[0];
+// num = gamma (gamma - 1) u + b^2, ee = e_f + b^2; Bu = u^t, Au = u^dir; Bsq, Asq,
+// AB: g^tt, g^dirdir, g^tdir.
+__device__ __forceinline__ double mhd_cmax(double num, double ee, double Bu, double Au, double Bsq,
+                                           double Asq, double AB) {
+  const double cms2 = num * rcp_nr(ee);
   const double AuBu = Au * Bu;
   // qa v^2 - 2 hb v + qc = 0: roots (hb +- sqrt(hb^2 - qa qc)) / qa
   const double qa = Bu * Bu - (Bsq + Bu * Bu) * cms2;
   const double hb = AuBu - (AB + AuBu) * cms2;
   const double qc = Au * Au - (Asq + Au * Au) * cms2;
   double disc = fma(hb, hb, -(qa * qc));
-  disc = (disc >= DBL_NORMAL_MIN) ? sqrt_nr(disc) : 0.0;  // a subnormal root is negligible
+  // (a subnormal root is negligible)
+  disc = ((s64)w_bits(disc) >= (s64)w_bits(DBL_NORMAL_MIN)) ? sqrt_nr(disc) : 0.0;
   return (fabs(hb) + disc) * fabs(rcp_nr(qa));
 }
 

@@ -27,6 +27,9 @@ struct Clock {
   long long steps;
   unsigned long long ctop_bits[3];  // max signal speed per direction (as bits, >= 0)
   unsigned long long counters[4];   // inversion failures, floor hits, unrecoverable, spare
+  // locations (bit LOC_*) whose loaded metric couples X2 to t, X1 or X3; none of
+  // the library's own does (wide_face.cuh, BLK)
+  int coupled;
 };
 
 // boundary code of a side shared with another block of a decomposed grid:

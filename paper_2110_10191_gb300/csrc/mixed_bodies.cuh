@@ -162,10 +162,11 @@ __device__ __forceinline__ void flux_f32_x1_body(const StepArgs &A, const float 
   int i = 0, j = 0, k = 0, ii = 0;
   long long c = 0;
   if (have) {
-    ii = (int)(q % e0);
+    const Idx3 q3 = unflatten(q, e0, ext[1]);
+    ii = q3.i;
     i = lo[0] - 1 + ii;
-    j = lo[1] + (int)((q / e0) % ext[1]);
-    k = lo[2] + (int)(q / ((long long)e0 * ext[1]));
+    j = lo[1] + q3.j;
+    k = lo[2] + q3.k;
     c = zid(D, i, j, k);
     recon_zone_f32<RECON>(D, P, c, 1, zl, zh);
   } else {
@@ -197,10 +198,8 @@ __device__ __forceinline__ void flux_f32_walk_body(const StepArgs &A,
   const int nseg = (ext[DIR] + WALK - 1) / WALK;
   double ctop = 0.0;
   if (t < ncol * nseg) {
-    const long long col = t % ncol;
-    const int seg = (int)(t / ncol);
-    const int i = lo[0] + (int)(col % ext[0]);
-    const int tb = lo[b] + (int)(col / ext[0]);
+    const Idx3 q3 = unflatten(t, ext[0], ext[b]);
+    const int seg = q3.k, i = lo[0] + q3.i, tb = lo[b] + q3.j;
     const int f0 = seg * WALK, f1 = min(f0 + WALK, ext[DIR]);
     const long long st = (DIR == 1) ? D.s[0] : D.n2d;
     const int j0 = (DIR == 1) ? lo[1] + f0 : tb, k0 = (DIR == 1) ? tb : lo[2] + f0;

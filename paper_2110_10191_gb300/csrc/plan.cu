@@ -56,23 +56,24 @@ __global__ void __launch_bounds__(BS_MAX) kp_recon(BView V, int in) {
   const long long t = block_tid(V, g);
   const double *Ps = arr(it, in);
   if (it.A.recon == 1) {
-    if (DIR == 0 && it.A.rwalk > 1) {  // launched with X1_WARP_BYTES of shared memory per warp
-      extern __shared__ __align__(16) unsigned char recon_sm[];
-      recon_x1_staged(it.A, Ps, it.Lf, it.Rf, t, recon_sm + (threadIdx.x >> 5) * X1_WARP_BYTES);
-    } else {
+    if (DIR == 0)
+      recon_x1_body<1>(it.A, Ps, it.Lf, it.Rf, t);
+    else
       recon_body<DIR, 1>(it.A, Ps, it.Lf, it.Rf, t);
-    }
   } else {
-    recon_body<DIR, 0>(it.A, Ps, it.Lf, it.Rf, t);
+    if (DIR == 0)
+      recon_x1_body<0>(it.A, Ps, it.Lf, it.Rf, t);
+    else
+      recon_body<DIR, 0>(it.A, Ps, it.Lf, it.Rf, t);
   }
 }
 
-// dynamic shared memory of a kp_recon<0> launch of bs threads
-inline unsigned recon_x1_smem(unsigned bs) { return (bs / 32) * X1_WARP_BYTES; }
-
 // ELEC: the grids of the launch evolve electron entropies (a class of their own)
+// at most 72 registers: 28 warps per SM, whose integer and FP64 work overlap,
+// against the spills (per cycle of a 128^3 grid: 168 registers 3.37 ms, 128 2.88,
+// 96 2.92, 80 2.80, 72 2.77, 64 2.83)
 template <int DIR, bool ELEC = false>
-__global__ void __launch_bounds__(BS_MAX) kp_face(BView V, int in) {
+__global__ void __maxnreg__(72) kp_face(BView V, int in) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   const long long t = block_tid(V, g);
@@ -322,8 +323,8 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_RECON1] = f64 ? n_recon_walk(D, 1, fl, rwalk) : 0;
   c[PC_RECON2] = (f64 && !fl) ? n_recon_walk(D, 2, 0, rwalk) : 0;
   for (int d = 0; d < 3; d++) {
-    c[PC_FACE0 + d] = (f64 && !elec) ? n_face(D, d, fl) : 0;
-    c[PC_FACE0E + d] = (f64 && elec) ? n_face(D, d, fl) : 0;
+    c[PC_FACE0 + d] = (f64 && !elec) ? n_face_threads(n_face(D, d, fl)) : 0;
+    c[PC_FACE0E + d] = (f64 && elec) ? n_face_threads(n_face(D, d, fl)) : 0;
     c[PC_FACE0F + d] = mx ? (d == 0 ? n_flux_f32_x1(D, fl) : n_flux_f32_walk(D, d, fl)) : 0;
     c[PC_FACE0X + d] = fx ? n_face(D, d, fl) : 0;
   }
@@ -353,9 +354,9 @@ long long plan_bytes(const Dims &D, int flat3, int prec, int drift, int elec) {
 
 int plan_rwalk(const StageItem *items, int n) {
   for (int rw = RWALK; rw >= 2; rw /= 2) {
-    long long least = -1;  // the FP64 reconstruction launch with the fewest threads
+    long long least = -1;  // the FP64 walk launch (X2 or X3) with the fewest threads
     bool any = false;
-    for (int d = 0; d < 3; d++) {
+    for (int d = 1; d < 3; d++) {
       long long tot = 0;
       for (int g = 0; g < n; g++) {
         const StepArgs &A = items[g].A;
@@ -402,14 +403,6 @@ int plan_build(Plan &p, const StageItem *items, int n) {
   }
   p.zones = zones;
   p.tab_cap = cap;
-  // kp_recon<0> takes more than the default 48 KiB of dynamic shared memory
-  // at the largest block (on the device current now, the plan's)
-  if (cudaFuncSetAttribute(kp_recon<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)recon_x1_smem(BS_MAX)) != cudaSuccess) {
-    cudaGetLastError();
-    plan_free(p);
-    return GRMHD_ERR_CUDA;
-  }
   if (cudaMalloc(&p.items, sizeof(StageItem) * n) != cudaSuccess ||
       cudaMalloc(&p.tab, sizeof(int) * (size_t)(cap > 0 ? cap : 1)) != cudaSuccess) {
     cudaGetLastError();
@@ -484,7 +477,7 @@ int plan_fluxes(const Plan &p, int in, cudaStream_t st, PlanHook *h) {
   int nl = plan_clock(p, 0, st, h);
   const int R = GRMHD_K_RECON, F = GRMHD_K_FLUX;
   // FP64 grids
-  nl += launch(p, PC_RECON0, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<0><<<nb, bs, recon_x1_smem(bs), st>>>(V, in); });
+  nl += launch(p, PC_RECON0, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<0><<<nb, bs, 0, st>>>(V, in); });
   nl += launch(p, PC_FACE0, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<0><<<nb, bs, 0, st>>>(V, in); });
   nl += launch(p, PC_FACE0E, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<0, true><<<nb, bs, 0, st>>>(V, in); });
   nl += launch(p, PC_RECON1, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<1><<<nb, bs, 0, st>>>(V, in); });
@@ -639,7 +632,7 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
     auto L = [&](int cls, auto &&body) { launch(p, cls, 0, nullptr, body); };
     switch (which) {
       case 0:
-        L(PC_RECON0, [&](unsigned nb, unsigned bs, BView V) { kp_recon<0><<<nb, bs, recon_x1_smem(bs), st>>>(V, 0); });
+        L(PC_RECON0, [&](unsigned nb, unsigned bs, BView V) { kp_recon<0><<<nb, bs, 0, st>>>(V, 0); });
         break;
       case 6:
         L(PC_RECON1, [&](unsigned nb, unsigned bs, BView V) { kp_recon<1><<<nb, bs, 0, st>>>(V, 0); });

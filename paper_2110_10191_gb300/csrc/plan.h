@@ -37,7 +37,7 @@ enum {
   PC_BX1,
   PC_BX2,
   PC_BX3,
-  PC_RECON0,  // FP64 reconstruction along X1 (column walks)
+  PC_RECON0,  // FP64 reconstruction along X1 (a lane per pair of differences)
   PC_RECON1,  // along X2
   PC_RECON2,  // along X3 (none for flat-X3 grids)
   PC_FACE0,
@@ -110,13 +110,11 @@ int plan_build(Plan &p, const StageItem *items, int n);
 // walk length)
 void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rwalk,
                  long long c[PC_N]);
-// The FP64 reconstruction's walk length for a plan of these grids: the
-// longest of 16, 8, 4, 2 zones per thread that still gives each of its
-// launches RWALK_MIN_THREADS threads, else 1 (one thread per zone).  About
-// 20 warps per SM keep the FP64 unit at its issue rate; with fewer, each
-// thread's longer chain of dependent work shows (64 small 2D grids with
-// 2-zone walks, 11 warps per SM: 115 us per launch against 84 us one
-// thread per zone).
+// The FP64 reconstruction's walk length along X2 and X3 for a plan of these
+// grids: the longest of 16, 8, 4, 2 zones per thread that still gives each of
+// those launches RWALK_MIN_THREADS threads, 20 warps per SM, else 1 (one thread
+// per zone, which forms each pair of differences three times and costs 6% more
+// where both fill the GPU: 301 against 283 us over 128x128x64 zones).
 constexpr long long RWALK_MIN_THREADS = 152 * 640;
 int plan_rwalk(const StageItem *items, int n);
 // Set the plan's reconstruction walk length (1, 2, 4, 8 or 16 zones per

@@ -23,64 +23,24 @@ template <int DIR, int RECON>
 __global__ void __launch_bounds__(BS) k_flux(StepArgs A, const double *__restrict__ P,
                                              double *__restrict__ F) {
   const Dims &D = A.D;
-  int lo[3], ext[3];
-#pragma unroll
-  for (int e = 0; e < 3; e++) {
-    lo[e] = (e == DIR) ? NG : NG - 1;
-    ext[e] = (e == DIR) ? D.n[e] + 1 : D.n[e] + 2;
-  }
-  const long long nface = (long long)ext[0] * ext[1] * ext[2];
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const bool active = t < nface;
-  double ctop = 0.0;
-  if (active) {
-    const int i = lo[0] + (int)(t % ext[0]);
-    const int j = lo[1] + (int)((t / ext[0]) % ext[1]);
-    const int k = lo[2] + (int)(t / ((long long)ext[0] * ext[1]));
-    const long long c = zid(D, i, j, k);
-    const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
-    double PL[NV], PR[NV];
-#pragma unroll
-    for (int v = 0; v < NV; v++) {
-      const double *p = P + v * D.ntot + c;
-      if (RECON == 1) {
-        const double x0 = __ldg(p - 3 * st), x1 = __ldg(p - 2 * st), x2 = __ldg(p - st);
-        const double x3 = __ldg(p), x4 = __ldg(p + st), x5 = __ldg(p + 2 * st);
-        double other;
-        weno5_wide_pair(x0, x1, x2, x3, x4, other, PL[v]);
-        weno5_wide_pair(x1, x2, x3, x4, x5, PR[v], other);
-      } else {
-        const double x1 = __ldg(p - 2 * st), x2 = __ldg(p - st);
-        const double x3 = __ldg(p), x4 = __ldg(p + st);
-        PL[v] = x2 + mc_half_slope(x2 - x1, x3 - x2);
-        PR[v] = x3 - mc_half_slope(x3 - x2, x4 - x3);
-      }
+  const FaceLane L = face_lane<DIR>(D, 0, gtid());
+  const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
+  // the lane's state: the high face of the zone below, or the low face of the
+  // zone above, whose mirrored stencil gives it as a high face
+  const long long up = L.right ? -st : st;
+  const double *p = P + (L.right ? L.c : L.c - st);
+  double S[NV];
+#pragma unroll 1
+  for (int v = 0; v < NV; v++, p += D.ntot) {
+    const double x = __ldg(p), xm = __ldg(p - up), xp = __ldg(p + up);
+    if (RECON == 1) {
+      double other;
+      weno5_wide_pair(__ldg(p - 2 * up), xm, x, xp, __ldg(p + 2 * up), other, S[v]);
+    } else {
+      S[v] = x + mc_half_slope(x - xm, xp - x);
     }
-    const int loc = (DIR == 0) ? LOC_FACE1 : (DIR == 1) ? LOC_FACE2 : LOC_CENT;
-    Geo G;
-    load_geo(A.geom + (long long)loc * G_NCOMP * D.n2d, D.n2d, (long long)j * D.s[0] + i, G);
-    FState sL, sR;
-    fluid_state(PL, G, sL);
-    fluid_state(PR, G, sR);
-    const double ct = fmax(mhd_cmax(PL, sL, G, A.gam, A.ggm1, DIR + 1),
-                           mhd_cmax(PR, sR, G, A.gam, A.ggm1, DIR + 1));
-    double FL[NV], FR[NV], UL[NV], UR[NV];
-    prim_flux(PL, sL, G, A.gam, DIR + 1, FL);
-    prim_flux(PR, sR, G, A.gam, DIR + 1, FR);
-    prim_flux(PL, sL, G, A.gam, 0, UL);
-    prim_flux(PR, sR, G, A.gam, 0, UR);
-#pragma unroll
-    for (int v = 0; v < NV; v++) F[v * D.ntot + c] = 0.5 * (FL[v] + FR[v] - ct * (UR[v] - UL[v]));
-    bool interior = true;
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      if (e == DIR) continue;
-      const int q = (e == 0) ? i : (e == 1) ? j : k;
-      interior = interior && (q >= NG) && (q < D.n[e] + NG);
-    }
-    if (interior) ctop = ct;
   }
-  warp_block_max(ctop, &A.clk->ctop_bits[DIR]);
+  face_flux<DIR, false>(A, L, S, F);
 }
 
 template <int DIR>
@@ -89,9 +49,9 @@ static void launch_flux_dir(const StepArgs &A, const double *P, double *F, cudaS
   long long nf = 1;
   for (int e = 0; e < 3; e++) nf *= (e == DIR) ? D.n[e] + 1 : D.n[e] + 2;
   if (A.recon == 1)
-    k_flux<DIR, 1><<<nblk(nf), BS, 0, st>>>(A, P, F);
+    k_flux<DIR, 1><<<nblk(n_face_threads(nf)), BS, 0, st>>>(A, P, F);
   else
-    k_flux<DIR, 0><<<nblk(nf), BS, 0, st>>>(A, P, F);
+    k_flux<DIR, 0><<<nblk(n_face_threads(nf)), BS, 0, st>>>(A, P, F);
 }
 
 void launch_fluxes(const StepArgs &A, const double *P, double *F[3], cudaStream_t st) {
@@ -100,7 +60,11 @@ void launch_fluxes(const StepArgs &A, const double *P, double *F[3], cudaStream_
   launch_flux_dir<2>(A, P, F[2], st);
 }
 
-__global__ void k_reset_ctop(Clock *clk) { reset_ctop_body(clk); }
+// (the entry point builds its own metric, which does not couple X2)
+__global__ void k_reset_ctop(Clock *clk) {
+  reset_ctop_body(clk);
+  clk->coupled = 0;
+}
 
 void launch_ctop_reset(const StepArgs &A, cudaStream_t st) { k_reset_ctop<<<1, 1, 0, st>>>(A.clk); }
 

@@ -26,6 +26,7 @@
 
 #include "grmhd_dev.cuh"
 #include "grmhd_impl.h"
+#include "wide_face.cuh"
 
 namespace grmhd {
 
@@ -36,6 +37,18 @@ __device__ __forceinline__ int wrap(int g, int n) {  // periodic image of ghost 
   int q = (g - NG) % n;
   if (q < 0) q += n;
   return NG + q;
+}
+
+// t as (i, j, k) of a range n0 x n1 x ..., i fastest.  Every range of a grid has
+// fewer than 2^32 entries (the library refuses grids of 2^31 zones, ghosts
+// included), so that two 32-bit divisions do, a fifth of the instructions of the
+// 64-bit ones.
+struct Idx3 {
+  int i, j, k;
+};
+__device__ __forceinline__ Idx3 unflatten(long long t, int n0, int n1) {
+  const u32 u = (u32)t, q = u / (u32)n0, k = q / (u32)n1;
+  return {(int)(u - q * n0), (int)(q - k * n1), (int)k};
 }
 
 // ---------------------------------------------------------------------------
@@ -54,10 +67,14 @@ __host__ __device__ inline long long n_recon(const Dims &D, int flat3) {
 }
 // longest FP64 reconstruction walk (zones per thread)
 constexpr int RWALK = 16;
-// threads of the FP64 reconstruction along dir: one per column and segment
-// of rw zones along dir (rw >= 2), or one per zone (rw = 1)
+// pairs that a warp of recon_x1_body finishes
+constexpr int X1_LANES = 30;
+// threads of the FP64 reconstruction along dir: along X1 a warp per X1_LANES
+// pairs (recon_x1_body); else one per column and segment of rw zones along dir
+// (rw >= 2), or one per zone (rw = 1)
 __host__ __device__ inline long long n_recon_walk(const Dims &D, int dir, int flat3, int rw) {
   const long long e[3] = {D.n[0] + 2, D.n[1] + 2, flat3 ? 1 : D.n[2] + 2};
+  if (dir == 0) return 32 * (((e[0] + 2) * e[1] * e[2] - 2 + X1_LANES - 1) / X1_LANES);
   if (rw <= 1) return e[0] * e[1] * e[2];
   return e[0] * e[1] * e[2] / e[dir] * ((e[dir] + rw - 1) / rw);
 }
@@ -108,11 +125,8 @@ __device__ __forceinline__ void bounds_x1_body(const StepArgs &A, double *P, dou
                                                long long t) {
   const Dims &D = A.D;
   if (t >= n_bounds_x1(D)) return;
-  const int g = (int)(t % NG);
-  const int side = (int)((t / NG) % 2);
-  const long long r = t / (2 * NG);
-  const int j = NG + (int)(r % D.n[1]);
-  const int k = NG + (int)(r / D.n[1]);
+  const Idx3 q3 = unflatten(t, 2 * NG, D.n[1]);
+  const int g = q3.i % NG, side = q3.i / NG, j = NG + q3.j, k = NG + q3.k;
   const int bc = A.bc[0][side];
   const int ig = side ? D.n[0] + NG + g : g;
   const long long d = zid(D, ig, j, k);
@@ -136,11 +150,8 @@ __device__ __forceinline__ void bounds_x2_body(const StepArgs &A, double *P, dou
                                                long long t) {
   const Dims &D = A.D;
   if (t >= n_bounds_x2(D)) return;
-  const int i = (int)(t % D.s[0]);
-  const long long r = t / D.s[0];
-  const int g = (int)(r % NG);
-  const int side = (int)((r / NG) % 2);
-  const int k = NG + (int)(r / (2 * NG));
+  const Idx3 q3 = unflatten(t, D.s[0], 2 * NG);
+  const int i = q3.i, g = q3.j % NG, side = q3.j / NG, k = NG + q3.k;
   const int bc = A.bc[1][side];
   const int jg = side ? D.n[1] + NG + g : NG - 1 - g;
   const long long d = zid(D, i, jg, k);
@@ -160,12 +171,10 @@ __device__ __forceinline__ void bounds_x2_body(const StepArgs &A, double *P, dou
 __device__ __forceinline__ void bounds_x3_body(const StepArgs &A, double *P, double *K,
                                                long long t) {
   const Dims &D = A.D;
-  const long long nrow = D.n2d;
   if (t >= n_bounds_x3(D)) return;
-  const long long ij = t % nrow;
-  const long long r = t / nrow;
-  const int g = (int)(r % NG);
-  const int side = (int)(r / NG);
+  const Idx3 q3 = unflatten(t, (int)D.n2d, NG);
+  const long long ij = q3.i;
+  const int g = q3.j, side = q3.k;
   const int bc = A.bc[2][side];
   const int kg = side ? D.n[2] + NG + g : NG - 1 - g;
   const long long d = (long long)kg * D.n2d + ij;
@@ -182,16 +191,14 @@ __device__ __forceinline__ void bounds_x3_body(const StepArgs &A, double *P, dou
 // Block maximum of v >= 0 (any block size that is a multiple of 32, up to
 // 1024), one atomicMax per block; every thread of the block must call it.
 __device__ __forceinline__ void warp_block_max(double v, unsigned long long *dst) {
-  // v >= 0: its bit pattern orders like the value
-  unsigned long long b = __double_as_longlong(v);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long x = __shfl_xor_sync(0xffffffffu, b, o);
-    b = (x > b) ? x : b;
-  }
+  // v >= 0: its bit pattern orders like the value; high words first, then the
+  // low words of the lanes that have the highest
+  const u64 b = w_bits(v);
+  const u32 hi = __reduce_max_sync(0xffffffffu, w_hi(b));
+  const u32 lo = __reduce_max_sync(0xffffffffu, (w_hi(b) == hi) ? w_lo(b) : 0u);
   __shared__ unsigned long long sm[32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sm[w] = b;
+  if (lane == 0) sm[w] = (u64)hi << 32 | lo;
   __syncthreads();
   if (threadIdx.x == 0) {
     const int nw = blockDim.x >> 5;
@@ -201,16 +208,14 @@ __device__ __forceinline__ void warp_block_max(double v, unsigned long long *dst
   }
 }
 
-// Zone-centric reconstruction: both face values of each zone's 8 primitives
-// along DIR (zones NG-1 .. n+NG along DIR and the extended transverse
-// range), each zone's WENO smoothness indicators formed once.  With
-// A.rwalk >= 2 one thread walks a segment of A.rwalk zones of one column
-// along DIR, so consecutive zones share their differences (weno5_walk);
-// consecutive threads take neighbouring columns (along X2 for DIR = 0, along
-// X1 otherwise).  With A.rwalk = 1 (grids too small to fill the GPU with
-// walks) one thread takes one zone, consecutive threads along X1.  Same
-// values either way.  Lf = value at the zone's low face, Rf = at its high
-// face.
+// Zone-centric reconstruction along X2 or X3: both face values of each zone's
+// 8 primitives (zones NG-1 .. n+NG along DIR and the extended transverse range),
+// each zone's WENO smoothness indicators formed once.  With A.rwalk >= 2 one
+// thread walks a segment of A.rwalk zones of one column along DIR, so that
+// consecutive zones share their differences and indicators (WenoWalk);
+// consecutive threads take neighbouring columns along X1.  With A.rwalk = 1
+// (grids too small to fill the GPU with walks) one thread takes one zone.  Same
+// values either way.  Lf = value at the zone's low face, Rf = at its high face.
 template <int DIR, int RECON>
 __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__restrict__ P,
                                            double *__restrict__ Lf, double *__restrict__ Rf,
@@ -218,12 +223,12 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
   const Dims &D = A.D;
   const int e0 = D.n[0] + 2, e1 = D.n[1] + 2, e2 = A.flat3 ? 1 : D.n[2] + 2;
   const int kb = A.flat3 ? NG : NG - 1;
-  const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
+  const long long st = (DIR == 1) ? D.s[0] : D.n2d;
   const int rw = A.rwalk;
   if (rw <= 1) {
     if (t >= (long long)e0 * e1 * e2) return;
-    const long long c = zid(D, NG - 1 + (int)(t % e0), NG - 1 + (int)((t / e0) % e1),
-                            kb + (int)(t / ((long long)e0 * e1)));
+    const Idx3 q3 = unflatten(t, e0, e1);
+    const long long c = zid(D, NG - 1 + q3.i, NG - 1 + q3.j, kb + q3.k);
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       const double *p = P + v * D.ntot + c;
@@ -241,17 +246,13 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
     }
     return;
   }
-  const int ed = (DIR == 0) ? e0 : (DIR == 1) ? e1 : e2;
-  const int ea = (DIR == 0) ? e1 : e0;  // the column index that varies fastest
+  const int ed = (DIR == 1) ? e1 : e2;
   const int eb = (DIR == 2) ? e1 : e2;
   const int nseg = (ed + rw - 1) / rw;
-  if (t >= (long long)ea * eb * nseg) return;
-  const int ca = (int)(t % ea);
-  const long long r = t / ea;
-  const int cb = (int)(r % eb);
-  const int m0 = (int)(r / eb) * rw;
-  const int i = NG - 1 + ((DIR == 0) ? m0 : ca);
-  const int j = NG - 1 + ((DIR == 1) ? m0 : (DIR == 0) ? ca : cb);
+  if (t >= (long long)e0 * eb * nseg) return;
+  const Idx3 q3 = unflatten(t, e0, eb);
+  const int i = NG - 1 + q3.i, cb = q3.j, m0 = q3.k * rw;
+  const int j = NG - 1 + ((DIR == 1) ? m0 : cb);
   const int k = (DIR == 2) ? NG - 1 + m0 : kb + cb;
   const int n = min(rw, ed - m0);
   const long long c = zid(D, i, j, k);
@@ -274,142 +275,161 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
   }
 }
 
-// The WENO5 reconstruction along X1 with each warp's rows staged in shared
-// memory.  The lanes of a warp walk 32 different rows (neighbouring j), so
-// their direct loads and stores touch 32 rows' sectors per instruction; here
-// the warp loads its rows' stencil values together (consecutive addresses),
-// walks them in shared memory, collects the face values of 8 zones per row
-// and writes them back row by row.  Same arithmetic and results as
-// recon_body<0, 1>, for A.rwalk >= 2.  Every thread of the block must call it
-// (warp synchronisation); wsm: the warp's X1_WARP_BYTES of shared memory.
-constexpr int X1_IN = RWALK + 5;  // a row's values at zones -2 .. RWALK+1, odd stride
-constexpr int X1_OUT = 9;         // 8 face values per row and chunk, odd stride
-constexpr int X1_HI = 32 * X1_OUT + 8;  // offset of the high-face chunk (another bank half)
-constexpr int X1_WARP_BYTES = (32 * X1_IN + 2 * X1_HI) * 8 + 32 * 8 + 32 * 4;
-
-__device__ __forceinline__ void recon_x1_staged(const StepArgs &A, const double *__restrict__ P,
-                                                double *__restrict__ Lf, double *__restrict__ Rf,
-                                                long long t, unsigned char *wsm) {
+// The reconstruction along X1, for every A.rwalk.  A lane takes one pair of
+// neighbouring first differences of a row, (x1 - x0, x2 - x1) from zone x0 on,
+// forms the substencil's indicators in its three roles and gets the two
+// substencils below from the two lanes below by warp shuffles, so that each
+// pair is formed once, as along a walk, and loads and stores stay coalesced.  The
+// pairs of all rows (n1 + 4 per row) are numbered through; a warp takes 32
+// consecutive ones, 30 of them its own (lanes 0 and 1 only serve the lanes
+// above).  Against walks of 32 rows per warp staged in shared memory, whose 152
+// registers and tile left 10 warps per SM waiting for loads, a 128x128x64 grid's
+// launch went from 446 to 220 us.  Same values as recon_body's.  Every thread of the warp must call it.
+template <int RECON>
+__device__ __forceinline__ void recon_x1_body(const StepArgs &A, const double *__restrict__ P,
+                                              double *__restrict__ Lf, double *__restrict__ Rf,
+                                              long long t) {
   const Dims &D = A.D;
-  const int e0 = D.n[0] + 2, e1 = D.n[1] + 2, e2 = A.flat3 ? 1 : D.n[2] + 2;
-  const int rw = A.rwalk;  // 2 .. RWALK
-  const int nseg = (e0 + rw - 1) / rw;
-  const int lane = threadIdx.x & 31;
-  double *tin = reinterpret_cast<double *>(wsm);
-  double *tout = tin + 32 * X1_IN;
-  long long *rbase = reinterpret_cast<long long *>(tout + 2 * X1_HI);
-  int *rn = reinterpret_cast<int *>(rbase + 32);
-  int n = 0;  // this lane's zones (0: past the end of the grid's threads)
-  long long c = 0;
-  if (t < (long long)e1 * e2 * nseg) {
-    const int ca = (int)(t % e1);
-    const long long r = t / e1;
-    const int cb = (int)(r % e2);
-    const int m0 = (int)(r / e2) * rw;
-    c = zid(D, NG - 1 + m0, NG - 1 + ca, (A.flat3 ? NG : NG - 1) + cb);
-    n = min(rw, e0 - m0);
-  }
-  rbase[lane] = c;
-  rn[lane] = n;
-  if (n == 0)  // a row past the end is never loaded: its walk reads zeros, stores nothing
-    for (int q = 0; q < X1_IN; q++) tin[lane * X1_IN + q] = 0.0;
-  __syncwarp();
-  const double *x = tin + lane * X1_IN;  // x[q]: this row's value at zone q - 2
+  const int e1 = D.n[1] + 2, e2 = A.flat3 ? 1 : D.n[2] + 2, row = D.n[0] + 4;
+  const int lane = (int)(t & 31);
+  const long long npair = (long long)row * e1 * e2;
+  const long long g = (t >> 5) * X1_LANES + lane;
+  const long long h = (g < npair) ? g : npair - 1;
+  const Idx3 q3 = unflatten(h, row, e1);
+  const int q = q3.i;  // zone NG - 3 + q: the row's first two lie below the range
+  const long long c = zid(D, NG - 3 + q, NG - 1 + q3.j, (A.flat3 ? NG : NG - 1) + q3.k);
+  const bool own = g < npair && lane >= 2 && q >= 2;
 #pragma unroll 1
   for (int v = 0; v < NV; v++) {
-    const long long ov = v * D.ntot;
-#pragma unroll 4
-    for (int e = lane; e < 32 * (RWALK + 4); e += 32) {
-      const int q = e / (RWALK + 4), xq = e - q * (RWALK + 4);
-      const int nq = rn[q];  // rows past the end (nq = 0) load nothing
-      if (nq > 0 && xq < nq + 4) tin[q * X1_IN + xq] = __ldg(P + ov + rbase[q] - 2 + xq);
+    const double *p = P + v * D.ntot + c;
+    const double x0 = __ldg(p), x1 = __ldg(p + 1);
+    double lo, hi;
+    if (RECON == 1) {
+      const WidePair p2 = wide_pair(wide_diff(x1 - x0), wide_diff(__ldg(p + 2) - x1));
+      const u64 D13 = wide_D13(p2);
+      const WideNum low = wide_q_low(p2, D13), mid = wide_q_mid(p2, D13);
+      const unsigned all = 0xffffffffu;
+      WidePair p0, p1;
+      WideNum q0, q1;
+      p1.a = __shfl_up_sync(all, p2.a, 1);
+      p1.b = __shfl_up_sync(all, p2.b, 1);
+      p1.x = __shfl_up_sync(all, p2.x, 1);
+      q1.m = __shfl_up_sync(all, mid.m, 1);
+      q1.x = __shfl_up_sync(all, mid.x, 1);
+      p0.a = __shfl_up_sync(all, p2.a, 2);
+      p0.b = __shfl_up_sync(all, p2.b, 2);
+      p0.x = __shfl_up_sync(all, p2.x, 2);
+      q0.m = __shfl_up_sync(all, low.m, 2);
+      q0.x = __shfl_up_sync(all, low.x, 2);
+      if (own) weno5_wide(x0, p0, p1, p2, q0, q1, wide_q_high(p2, D13), lo, hi);
+    } else if (own) {
+      const double d = mc_half_slope(x0 - __ldg(p - 1), x1 - x0);
+      lo = x0 - d;
+      hi = x0 + d;
     }
-    __syncwarp();
-    WenoWalk w;
-    w.start(x[0], x[1], x[2], x[3], x[4]);
-#pragma unroll 1
-    for (int m = 0; m < RWALK; m++) {
-      if (m < n) {
-        double lo, hi;
-        w.faces(lo, hi);
-        tout[lane * X1_OUT + (m & 7)] = lo;
-        tout[X1_HI + lane * X1_OUT + (m & 7)] = hi;
-        if (m + 1 < n) w.next(x[m + 5]);
-      }
-      if ((m & 7) == 7) {  // write zones m-7 .. m of every row: 4 rows x 8 zones per store
-        __syncwarp();
-#pragma unroll
-        for (int it = 0; it < 16; it++) {
-          const int e = it * 32 + lane;
-          const int q = (e >> 3) & 31, col = e & 7, z = (m & ~7) + col;
-          if (z < rn[q]) {
-            double *dst = (it < 8) ? Lf : Rf;
-            dst[ov + rbase[q] + z] = tout[((it < 8) ? 0 : X1_HI) + q * X1_OUT + col];
-          }
-        }
-        __syncwarp();
-      }
+    if (own) {
+      Lf[v * D.ntot + c] = lo;
+      Rf[v * D.ntot + c] = hi;
     }
   }
 }
 
-// One thread per face combines Rf of zone c-1 (left state) and Lf of zone c
-// (right state) into the LLF flux; every thread of the block must call it.
+// The two threads of a face: lanes 0..15 of a warp take the left states of 16
+// consecutive faces, lanes 16..31 their right states.
+__host__ __device__ inline long long n_face_threads(long long nface) { return 32 * ((nface + 15) / 16); }
+struct FaceLane {
+  bool active, right;
+  int i, j, k;
+  long long c;  // zone above the face (inactive lanes: of the last face)
+};
+template <int DIR>
+__device__ __forceinline__ FaceLane face_lane(const Dims &D, int flat3, long long t) {
+  int lo[3], ext[3];
+  face_box(D, DIR, flat3, lo, ext);
+  const long long nface = (long long)ext[0] * ext[1] * ext[2];
+  long long f = (t >> 5) * 16 + (t & 15);
+  FaceLane L;
+  L.active = f < nface;
+  L.right = (t & 16) != 0;
+  if (!L.active) f = nface - 1;
+  const Idx3 q = unflatten(f, ext[0], ext[1]);
+  L.i = lo[0] + q.i;
+  L.j = lo[1] + q.j;
+  L.k = lo[2] + q.k;
+  L.c = zid(D, L.i, L.j, L.k);
+  return L;
+}
+
+// The larger of two signal speeds; one that is not a number loses, as in fmax.
+__device__ __forceinline__ double speed_max(double a, double b) {
+  const s64 x = (s64)w_bits(a), y = (s64)w_bits(b), inf = 0x7ffll << 52;
+  return (x > inf || x < 0) ? b : (y > inf || y < 0 || x > y) ? a : b;
+}
+
+// LLF flux of a face from its two states P, one per lane (face_lane): each lane
+// forms its state and signal speed, takes the pair's larger speed ct, forms
+// 1/2 sqrt(-g) (F +- ct U) and adds the other lane's for half of the variables.
+// The states' and fluxes' dot products run in Wide numbers on the integer pipes
+// (wide_face.cuh), the signal speeds (about 30 instructions) beside them on the
+// FP64 unit, whose 241 instructions a face bound the former all-FP64 form (0.937 ms
+// per launch on a 128^3 grid; 0.462 ms so).  Two lanes a face, so that a thread
+// keeps one state's values and the warps are many; the FP64 unit and the ALU are
+// each busy about 60% of the time.
 // ELEC: the grid evolves electron entropies, whose flux weights it stores.
+// Every thread of the block must call it.
+template <int DIR, bool ELEC>
+__device__ __forceinline__ void face_flux(const StepArgs &A, const FaceLane &L, const double P[NV],
+                                          double *__restrict__ F) {
+  const Dims &D = A.D;
+  const int loc = (DIR == 0) ? LOC_FACE1 : (DIR == 1) ? LOC_FACE2 : LOC_CENT;
+  const double *g = A.geom + (long long)loc * G_NCOMP * D.n2d + (long long)L.j * D.s[0] + L.i;
+  const auto geo = [g, &D](int comp) { return __ldg(g + comp * D.n2d); };
+  WideState s;
+  if (A.clk->coupled)
+    wide_state<false>(P, geo, s);
+  else
+    wide_state<true>(P, geo, s);
+  const double bsq = w_to_double(s.bsq), ee = bsq + fma(A.gam, P[UU], P[RHO]);
+  const double ut = w_to_double(s.ucon[0]), ud = w_to_double(s.ucon[DIR + 1]);
+  const double own = mhd_cmax(fma(A.ggm1, P[UU], bsq), ee, ut, ud, geo(G_GCON + SY(0, 0)),
+                              geo(G_GCON + SY(DIR + 1, DIR + 1)), geo(G_GCON + SY(0, DIR + 1)));
+  // c_top = max(0, vmax_L, vmax_R, -vmin_L, -vmin_R): the larger root
+  // magnitude of either side
+  const double ct = speed_max(own, __shfl_xor_sync(0xffffffffu, own, 16));
+  double out[NV];
+  wide_flux(P, s, ee, A.gm1, DIR + 1, L.right ? -ct : ct, 0.5 * geo(G_GDET), out);
+  // the electron entropies' flux weights (LLF of rho u^d K, rho u^t K)
+  if (ELEC && L.active) A.elec_w[(2 * DIR + (L.right ? 1 : 0)) * D.ntot + L.c] = out[RHO];
+#pragma unroll
+  for (int q = 0; q < NV / 2; q++) {
+    const double keep = L.right ? out[q + NV / 2] : out[q];
+    const double got = __shfl_xor_sync(0xffffffffu, L.right ? out[q] : out[q + NV / 2], 16);
+    if (L.active) F[(q + (L.right ? NV / 2 : 0)) * D.ntot + L.c] = keep + got;
+  }
+  bool interior = L.active;
+#pragma unroll
+  for (int e = 0; e < 3; e++) {
+    if (e == DIR) continue;
+    const int q = (e == 0) ? L.i : (e == 1) ? L.j : L.k;
+    interior = interior && (q >= NG) && (q < D.n[e] + NG);
+  }
+  warp_block_max(interior ? ct : 0.0, &A.clk->ctop_bits[DIR]);
+}
+
+// The face's left state is Rf of zone c-1, the right state Lf of zone c; every
+// thread of the block must call it.
 template <int DIR, bool ELEC = false>
 __device__ __forceinline__ void face_body(const StepArgs &A, const double *__restrict__ Lf,
                                           const double *__restrict__ Rf, double *__restrict__ F,
                                           long long t) {
   const Dims &D = A.D;
-  int lo[3], ext[3];
-  face_box(D, DIR, A.flat3, lo, ext);
-  const long long nface = (long long)ext[0] * ext[1] * ext[2];
-  const bool active = t < nface;
-  double ctop = 0.0;
-  if (active) {
-    const int i = lo[0] + (int)(t % ext[0]);
-    const int j = lo[1] + (int)((t / ext[0]) % ext[1]);
-    const int k = lo[2] + (int)(t / ((long long)ext[0] * ext[1]));
-    const long long c = zid(D, i, j, k);
-    const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
-    double PL[NV], PR[NV];
+  const FaceLane L = face_lane<DIR>(D, A.flat3, t);
+  const long long st = (DIR == 0) ? 1 : (DIR == 1) ? D.s[0] : D.n2d;
+  const double *p = L.right ? Lf + L.c : Rf + L.c - st;
+  double P[NV];
 #pragma unroll
-    for (int v = 0; v < NV; v++) {
-      PL[v] = __ldg(Rf + v * D.ntot + c - st);
-      PR[v] = __ldg(Lf + v * D.ntot + c);
-    }
-    const int loc = (DIR == 0) ? LOC_FACE1 : (DIR == 1) ? LOC_FACE2 : LOC_CENT;
-    Geo G;
-    load_geo(A.geom + (long long)loc * G_NCOMP * D.n2d, D.n2d, (long long)j * D.s[0] + i, G);
-    FState sL, sR;
-    fluid_state(PL, G, sL);
-    fluid_state(PR, G, sR);
-    // c_top = max(0, vmax_L, vmax_R, -vmin_L, -vmin_R): the larger root
-    // magnitude of either side
-    const double ct = fmax(mhd_cmax(PL, sL, G, A.gam, A.ggm1, DIR + 1),
-                           mhd_cmax(PR, sR, G, A.gam, A.ggm1, DIR + 1));
-    // LLF: F = 1/2 sqrt(-g) [(F_L + ct U_L) + (F_R - ct U_R)]
-    double acc[NV];
-    flux_cons_acc<true>(PL, sL, A.gm1, DIR + 1, ct, acc);
-    const double mL = acc[RHO];  // rho_L (u^d_L + ct u^t_L): the left mass term
-    flux_cons_acc<false>(PR, sR, A.gm1, DIR + 1, -ct, acc);
-    const double hg = 0.5 * G.gdet;
-#pragma unroll
-    for (int v = 0; v < NV; v++) F[v * D.ntot + c] = hg * acc[v];
-    if (ELEC) {  // the electron entropies' flux weights (LLF of rho u^d K, rho u^t K)
-      A.elec_w[(2 * DIR) * D.ntot + c] = hg * mL;
-      A.elec_w[(2 * DIR + 1) * D.ntot + c] = hg * (acc[RHO] - mL);
-    }
-    bool interior = true;
-#pragma unroll
-    for (int e = 0; e < 3; e++) {
-      if (e == DIR) continue;
-      const int q = (e == 0) ? i : (e == 1) ? j : k;
-      interior = interior && (q >= NG) && (q < D.n[e] + NG);
-    }
-    if (interior) ctop = ct;
-  }
-  warp_block_max(ctop, &A.clk->ctop_bits[DIR]);
+  for (int v = 0; v < NV; v++) P[v] = __ldg(p + v * D.ntot);
+  face_flux<DIR, ELEC>(A, L, P, F);
 }
 
 // Flat X3: copy the k = NG layer of F1 and F2 to k = NG-1 and NG+1, and of
@@ -418,8 +438,8 @@ __device__ __forceinline__ void replicate_body(const StepArgs &A, double *F1, do
                                                long long t) {
   const Dims &D = A.D;
   if (t >= n_replicate(D)) return;
-  const long long v = t / D.n2d, ij = t % D.n2d;
-  const long long c = v * D.ntot + NG * D.n2d + ij;
+  const Idx3 q3 = unflatten(t, (int)D.n2d, NV);
+  const long long c = q3.j * D.ntot + NG * D.n2d + q3.i;
   const double f1 = F1[c], f2 = F2[c], f3 = F3[c];
   F1[c - D.n2d] = f1;
   F1[c + D.n2d] = f1;
@@ -523,9 +543,8 @@ __device__ __forceinline__ void emf_body(const StepArgs &A, const double *__rest
   const Dims &D = A.D;
   const int e0 = D.n[0] + 1, e1 = D.n[1] + 1;
   if (t >= n_edge(D)) return;
-  const int i = NG + (int)(t % e0);
-  const int j = NG + (int)((t / e0) % e1);
-  const int k = NG + (int)(t / ((long long)e0 * e1));
+  const Idx3 q3 = unflatten(t, e0, e1);
+  const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
   const long long c = zid(D, i, j, k), N = D.ntot;
   const long long im = c - 1, jm = c - D.s[0], km = c - D.n2d;
   emf[2 * N + c] = 0.25 * (F1[B2 * N + c] + F1[B2 * N + jm] - F2[B1 * N + c] - F2[B1 * N + im]);
@@ -539,9 +558,8 @@ __device__ __forceinline__ void ct_body(const StepArgs &A, double *F1, double *F
   const Dims &D = A.D;
   const int e0 = D.n[0] + 1, e1 = D.n[1] + 1;
   if (t >= n_edge(D)) return;
-  const int i = NG + (int)(t % e0);
-  const int j = NG + (int)((t / e0) % e1);
-  const int k = NG + (int)(t / ((long long)e0 * e1));
+  const Idx3 q3 = unflatten(t, e0, e1);
+  const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
   const long long c = zid(D, i, j, k), N = D.ntot;
   const double *E1 = emf, *E2 = emf + N, *E3 = emf + 2 * N;
   const bool in1 = i < D.n[0] + NG, in2 = j < D.n[1] + NG, in3 = k < D.n[2] + NG;
@@ -613,9 +631,8 @@ __device__ __forceinline__ void update_body(const StepArgs &A, const double *Pi,
   const bool active = t < nz;
   int pf = 0, ff = 0;
   if (active) {
-    const int i = NG + (int)(t % D.n[0]);
-    const int j = NG + (int)((t / D.n[0]) % D.n[1]);
-    const int k = NG + (int)(t / ((long long)D.n[0] * D.n[1]));
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
     Geo G;
@@ -686,9 +703,8 @@ __device__ __forceinline__ void floor_drift_body(const StepArgs &A, double *P,
   const bool active = t < nz;
   int ff = 0;
   if (active) {
-    const int i = NG + (int)(t % D.n[0]);
-    const int j = NG + (int)((t / D.n[0]) % D.n[1]);
-    const int k = NG + (int)(t / ((long long)D.n[0] * D.n[1]));
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     if (pflag[c] == 0) {
       const long long ij = (long long)j * D.s[0] + i;
@@ -721,9 +737,8 @@ __device__ __forceinline__ void fixup_body(const StepArgs &A, double *P, const i
   const bool active = t < nz;
   bool hit = false, lost = false;
   if (active) {
-    const int i = NG + (int)(t % D.n[0]);
-    const int j = NG + (int)((t / D.n[0]) % D.n[1]);
-    const int k = NG + (int)(t / ((long long)D.n[0] * D.n[1]));
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     if (pflag[c] != 0) {
       double sum[5] = {0.0, 0.0, 0.0, 0.0, 0.0};

@@ -58,6 +58,13 @@ WIDE_FN double w_double(u64 b) {
   return x;
 #endif
 }
+WIDE_FN double w_fma(double a, double b, double c) {
+#ifdef __CUDA_ARCH__
+  return fma(a, b, c);
+#else
+  return __builtin_fma(a, b, c);
+#endif
+}
 WIDE_FN int w_clz32(u32 a) {
 #ifdef __CUDA_ARCH__
   return __clz((int)a);
@@ -74,8 +81,16 @@ WIDE_FN int w_clz64(u64 a) {
 }
 WIDE_FN int w_min(int a, int b) { return a < b ? a : b; }
 WIDE_FN int w_max(int a, int b) { return a > b ? a : b; }
-// a >> n for 0 <= n, 0 when n > 63
-WIDE_FN u64 w_shr(u64 a, int n) { return a >> w_min(n, 63); }
+// a >> n for 0 <= n, 0 when n > 63 (the PTX shift saturates its count)
+WIDE_FN u64 w_shr(u64 a, int n) {
+#ifdef __CUDA_ARCH__
+  u64 r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
+  return r;
+#else
+  return n > 63 ? 0 : a >> n;
+#endif
+}
 // sign mask (0 or -1), magnitude of a signed value, value of a magnitude
 WIDE_FN s64 w_sign(s64 a) { return a >> 63; }
 WIDE_FN u64 w_abs(s64 a, s64 s) { return (u64)((a ^ s) - s); }
@@ -86,6 +101,10 @@ WIDE_FN s64 w_signed(u64 m, s64 s) { return ((s64)m ^ s) - s; }
 WIDE_FN u64 w_mulhi(u64 a, u64 b) {
   const u64 t = w_mul(w_hi(a), w_lo(b)), u = w_mul(w_lo(a), w_hi(b));
   return w_mul(w_hi(a), w_hi(b)) + ((u64)w_hi(t) + w_hi(u));
+}
+// the same within 1 unit for a < 2^61 and b < 2^63 (the middle sum fits)
+WIDE_FN u64 w_mulhi61(u64 a, u64 b) {
+  return w_mul(w_hi(a), w_hi(b)) + w_hi(w_mul(w_lo(a), w_hi(b)) + w_mul(w_hi(a), w_lo(b)));
 }
 WIDE_FN u64 w_sqrhi(u64 a) {
   return w_mul(w_hi(a), w_hi(a)) + (w_mul(w_hi(a), w_lo(a)) >> 31);
@@ -187,7 +206,7 @@ WIDE_FN WideNum wide_q_high(const WidePair &p, u64 D13) { return wide_weight(D13
 WIDE_FN double wide_quot(s64 N, u64 H, int x, bool bad) {
   const s64 sn = w_sign(N);
   const u64 a = w_abs(N, sn);
-  const int kh = w_clz64(H), kn = w_clz64(a | 1u);
+  const int kh = w_clz32(w_hi(H)), kn = w_clz64(a | 1u);
   const u64 h = H << kh, n = (a << kn) >> 1;
   const u32 r = w_rcp32(w_hi(h)) - 2u;  // 2: h's low word
   const u32 q0 = w_hi(w_mul(w_hi(n), r));
@@ -223,26 +242,21 @@ WIDE_FN void weno5_wide(double c, const WidePair &p0, const WidePair &p1, const 
   // the numerators, on exponent z + 3
   const int z0 = y0 + p0.x, z1 = y1 + p1.x, z2 = y2 + p2.x;
   const int z = w_max(z0, w_max(z1, z2));
-  const int k0 = w_min(z - z0 + 3, 63), k1 = w_min(z - z1 + 3, 63), k2 = w_min(z - z2 + 3, 63);
-#define WIDE_TERM(w, v, k) w_signed(w_mulhi(w, w_abs(v, w_sign(v))) >> k, w_sign(v))
+  const u64 u0 = w_shr(w0, z - z0 + 3), u1 = w_shr(w1, z - z1 + 3), u2 = w_shr(w2, z - z2 + 3);
+#define WIDE_TERM(w, v) w_signed(w_mulhi61(w, w_abs(v, w_sign(v))), w_sign(v))
   const s64 A = p0.b + (p0.b << 2) - (p0.a << 1), Cl = (p0.b << 2) - p0.a;
   const s64 B = p1.a + (p1.b << 1), Bl = (p1.a << 1) + p1.b;
   const s64 C = (p2.a << 2) - p2.b, Al = (p2.b << 1) - p2.a - (p2.a << 2);
-  const s64 nA = WIDE_TERM(w0, A, k0), nB = WIDE_TERM(w1, B, k1), nC = WIDE_TERM(w2, C, k2);
-  const s64 nCl = WIDE_TERM(w0, Cl, k0), nBl = WIDE_TERM(w1, Bl, k1), nAl = WIDE_TERM(w2, Al, k2);
+  const s64 nA = WIDE_TERM(u0, A), nB = WIDE_TERM(u1, B), nC = WIDE_TERM(u2, C);
+  const s64 nCl = WIDE_TERM(u0, Cl), nBl = WIDE_TERM(u1, Bl), nAl = WIDE_TERM(u2, Al);
 #undef WIDE_TERM
   const s64 b = nB << 1, bl = nBl << 1;
-  const s64 u = b + nC, ul = bl + nCl;
-  const s64 Nh = nA + u + (u << 1), Nl = nAl - ul - (ul << 1);
+  const s64 s = b + nC, sl = bl + nCl;
+  const s64 Nh = nA + s + (s << 1), Nl = nAl - sl - (sl << 1);
   const bool bad = w_max(p0.x, w_max(p1.x, p2.x)) >= WIDE_X_BAD;
   const int x = z - y + 63;
-#ifdef __CUDA_ARCH__
-  hi = fma(wide_quot(Nh, H, x, bad), 1.0 / 6.0, c);
-  lo = fma(wide_quot(Nl, L, x, bad), 1.0 / 6.0, c);
-#else
-  hi = __builtin_fma(wide_quot(Nh, H, x, bad), 1.0 / 6.0, c);
-  lo = __builtin_fma(wide_quot(Nl, L, x, bad), 1.0 / 6.0, c);
-#endif
+  hi = w_fma(wide_quot(Nh, H, x, bad), 1.0 / 6.0, c);
+  lo = w_fma(wide_quot(Nl, L, x, bad), 1.0 / 6.0, c);
 }
 
 // Both face values of the middle zone of a..e.
