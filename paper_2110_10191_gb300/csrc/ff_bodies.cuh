@@ -664,8 +664,7 @@ __device__ __forceinline__ void update_ff_body(const StepArgs &A, const double *
         load_geo(A.geom, D.n2d, ij, Gd);
         fl = apply_floors(pd, Gd, rho_fl, u_fl, A.gk);
       } else {
-        Geo Gd;  // not read on this path
-        fl = apply_floors_known(pd, Gd, rho_fl, u_fl, A.gk, ff_to(bsq_n) * sc.s, lor);
+        fl = apply_floors_known(pd, rho_fl, u_fl, A.gk, ff_to(bsq_n) * sc.s);
       }
     }
 #pragma unroll

@@ -111,6 +111,14 @@ __device__ __forceinline__ double div_rn(double x, double c, double rc) {
   return fma(r, rc, q0);
 }
 
+// a < b for numbers that are not NaN (false for NaN, as the comparison), off
+// the FP64 unit: equal signs compare as integers
+__device__ __forceinline__ bool less(double a, double b) {
+  const s64 x = (s64)w_bits(a), y = (s64)w_bits(b), mag = ~(1ll << 63), inf = 0x7ffll << 52;
+  const bool nan = (x & mag) > inf || (y & mag) > inf, zero = ((x | y) & mag) == 0;
+  return !nan && !zero && ((x < 0 && y < 0) ? x > y : x < y);
+}
+
 struct Dims {
   int n[3];   // interior zones
   int s[3];   // with ghosts
@@ -470,25 +478,20 @@ __device__ __forceinline__ int invert_1dw(const double U[NV], const Geo &G, cons
 // Bounds: Lorentz-factor cap first (it changes b^2), then rho and u raised in
 // the fluid frame in the order of the paper's list; every bound holds on exit.
 // ---------------------------------------------------------------------------
-// The bounds with b^2 and the Lorentz factor already known (from the
-// inversion); zones that need the Lorentz-factor cap take the general path.
-// The quotients b^2/sigma, beta b^2 / (2 (gamma - 1)) and u/T are the IEEE
+// rho and u of a zone with b^2, whose Lorentz factor is within the cap.  The
+// quotients b^2/sigma, beta b^2 / (2 (gamma - 1)) and u/T are the IEEE
 // divisions' values bit for bit (div_rn).
-__device__ __forceinline__ int apply_floors(double P[NV], const Geo &G, double rho_fl,
-                                            double u_fl, const GasK &K);
-__device__ __forceinline__ int apply_floors_known(double P[NV], const Geo &G, double rho_fl,
-                                                  double u_fl, const GasK &K, double bsq,
-                                                  double lorentz) {
-  if (lorentz > FL_GAMMA) return apply_floors(P, G, rho_fl, u_fl, K);
+__device__ __forceinline__ int apply_floors_known(double P[NV], double rho_fl, double u_fl,
+                                                  const GasK &K, double bsq) {
   int fl = 0;
-  if (P[RHO] < rho_fl) { P[RHO] = rho_fl; fl |= FF_RHO_GEOM; }
-  if (P[UU] < u_fl) { P[UU] = u_fl; fl |= FF_U_GEOM; }
+  if (less(P[RHO], rho_fl)) { P[RHO] = rho_fl; fl |= FF_RHO_GEOM; }
+  if (less(P[UU], u_fl)) { P[UU] = u_fl; fl |= FF_U_GEOM; }
   const double rs = div_rn(bsq, FL_SIGMA, FL_SIGMA_RCP);
-  if (P[RHO] < rs) { P[RHO] = rs; fl |= FF_SIGMA; }
+  if (less(P[RHO], rs)) { P[RHO] = rs; fl |= FF_SIGMA; }
   const double ub = div_rn(FL_BETA * bsq, K.ubd, K.ubd_rcp);
-  if (P[UU] < ub) { P[UU] = ub; fl |= FF_BETA; }
+  if (less(P[UU], ub)) { P[UU] = ub; fl |= FF_BETA; }
   const double rt = div_rn(P[UU], FL_TEMP, FL_TEMP_RCP);
-  if (P[RHO] < rt) { P[RHO] = rt; fl |= FF_TEMP; }
+  if (less(P[RHO], rt)) { P[RHO] = rt; fl |= FF_TEMP; }
   return fl;
 }
 
@@ -508,14 +511,7 @@ __device__ __forceinline__ int apply_floors(double P[NV], const Geo &G, double r
   }
   FState s;
   fluid_state(P, G, s);
-  if (P[RHO] < rho_fl) { P[RHO] = rho_fl; fl |= FF_RHO_GEOM; }
-  if (P[UU] < u_fl) { P[UU] = u_fl; fl |= FF_U_GEOM; }
-  const double rs = div_rn(s.bsq, FL_SIGMA, FL_SIGMA_RCP);
-  if (P[RHO] < rs) { P[RHO] = rs; fl |= FF_SIGMA; }
-  const double ub = div_rn(FL_BETA * s.bsq, K.ubd, K.ubd_rcp);
-  if (P[UU] < ub) { P[UU] = ub; fl |= FF_BETA; }
-  const double rt = div_rn(P[UU], FL_TEMP, FL_TEMP_RCP);
-  if (P[RHO] < rt) { P[RHO] = rt; fl |= FF_TEMP; }
+  fl |= apply_floors_known(P, rho_fl, u_fl, K, s.bsq);
   return fl;
 }
 

@@ -162,12 +162,16 @@ __global__ void kp_ct(BView V) {
   ct_body(it.A, it.F[0], it.F[1], it.F[2], it.emf, block_tid(V, g));
 }
 
-// at most 168 registers: 3 blocks of 128 threads per SM (172 would allow 2)
-__global__ void __maxnreg__(168) kp_update(BView V, int in, double dtfac, int ucache_mode) {
+// at most 168 registers: 3 blocks of 128 threads per SM (per cycle of a 128^3
+// grid 2.06 ms, at 128 registers 2.10, at 96 2.59 with the spills).
+// PRED: the predictor (in = 0), whose ucache_mode 1 keeps U(P^n) for the corrector
+template <bool PRED>
+__global__ void __maxnreg__(168) kp_update(BView V, double dtfac, int ucache_mode) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  update_body(it.A, it.P, arr(it, in), arr(it, 1 - in), it.F[0], it.F[1], it.F[2], it.pflag,
-              it.fflag, dtfac, it.Uc, ucache_mode, block_tid(V, g));
+  const int in = PRED ? 0 : 1;
+  update_body<PRED>(it.A, it.P, arr(it, in), arr(it, 1 - in), it.F[0], it.F[1], it.F[2], it.pflag,
+                    it.fflag, dtfac, it.Uc, ucache_mode == 1, block_tid(V, g));
 }
 
 // at most 128 registers: 4 blocks of 128 threads per SM; the spill it costs
@@ -524,7 +528,10 @@ int plan_fix_ct(const Plan &p, cudaStream_t st, PlanHook *h) {
 int plan_update_only(const Plan &p, int in, double dtfac, int ucache_mode, cudaStream_t st,
                      PlanHook *h) {
   int nl = launch(p, PC_UPD64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
-    kp_update<<<nb, bs, 0, st>>>(V, in, dtfac, ucache_mode);
+    if (in == 0)
+      kp_update<true><<<nb, bs, 0, st>>>(V, dtfac, ucache_mode);
+    else  // the predictor before it kept U(P^n)
+      kp_update<false><<<nb, bs, 0, st>>>(V, dtfac, ucache_mode);
   });
   nl += launch(p, PC_UPDX, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
     kp_update_ff<<<nb, bs, 0, st>>>(V, in, dtfac, ucache_mode);
@@ -650,7 +657,7 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
         L(PC_FACE2, [&](unsigned nb, unsigned bs, BView V) { kp_face<2><<<nb, bs, 0, st>>>(V, 0); });
         break;
       case 5:  // predictor-like update without keeping U(P^n)
-        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_update<<<nb, bs, 0, st>>>(V, 0, 0.5, 0); });
+        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_update<true><<<nb, bs, 0, st>>>(V, 0.5, 0); });
         break;
       case 16:
         L(PC_UPDX, [&](unsigned nb, unsigned bs, BView V) { kp_update_ff<<<nb, bs, 0, st>>>(V, 0, 0.5, 0); });

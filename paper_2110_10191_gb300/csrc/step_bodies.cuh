@@ -27,6 +27,7 @@
 #include "grmhd_dev.cuh"
 #include "grmhd_impl.h"
 #include "wide_face.cuh"
+#include "wide_update.cuh"
 
 namespace grmhd {
 
@@ -613,16 +614,63 @@ __device__ __forceinline__ void geo_source(const double P[NV], const FState &s, 
   }
 }
 
-// Ucache: the predictor stores U(P^n) there and the corrector, whose P_i is
-// the same P^n, reads it back instead of recomputing it (null: neither).
+// sqrt(-g)-weighted sum of a variable's flux differences over the zone c
+__device__ __forceinline__ double flux_div(const StepArgs &A, const double *__restrict__ F1,
+                                           const double *__restrict__ F2,
+                                           const double *__restrict__ F3, long long o) {
+  return (F1[o + 1] - F1[o]) * A.idx[0] + (F2[o + A.D.s[0]] - F2[o]) * A.idx[1] +
+         (F3[o + A.D.n2d] - F3[o]) * A.idx[2];
+}
+
+// U(P) and the source of a state in FP64: metrics that couple X2.
+static __device__ __noinline__ void source_fp64(const StepArgs &A, const double *__restrict__ Ps,
+                                                long long c, long long ij, double U[NV],
+                                                double S[4], double &guess) {
+  Geo G;
+  load_geo(A.geom, A.D.n2d, ij, G);
+  double p[NV];
+  for (int v = 0; v < NV; v++) p[v] = Ps[v * A.D.ntot + c];
+  FState s;
+  fluid_state(p, G, s);
+  prim_flux(p, s, G, A.gam, 0, U);
+  geo_source(p, s, G, A.conn, A.D.n2d, ij, A.gam, S);
+  const double g = s.ucon[0] * G.alpha;
+  guess = (p[RHO] + A.gam * p[UU]) * g * g;
+}
+
+// The bounds of a zone that needs the Lorentz-factor cap.
+static __device__ __noinline__ int floors_capped(const StepArgs &A, long long ij, double rho_fl,
+                                                 double u_fl, double P[NV]) {
+  Geo G;
+  load_geo(A.geom, A.D.n2d, ij, G);
+  return apply_floors(P, G, rho_fl, u_fl, A.gk);
+}
+
+// The inversion in FP64 from the guess P_i: zones for which wide_invert gives
+// no answer.
+static __device__ __noinline__ int invert_fp64(const StepArgs &A, const double U[NV],
+                                               const double *Pi, long long c, long long ij,
+                                               double P[NV], double &bsq, double &lorentz) {
+  Geo G;
+  load_geo(A.geom, A.D.n2d, ij, G);
+  double p[NV];
+  for (int v = 0; v < NV; v++) p[v] = Pi[v * A.D.ntot + c];
+  return invert_1dw(U, G, A.gk, p, P, bsq, lorentz);
+}
+
+// The predictor (PRED: P_s = P_i = P^n) keeps U(P^n) in Ucache if keep is set;
+// the corrector, whose P_i is the same P^n, reads it there.  U(P), the source and
+// the inversion run in Wide numbers (wide_update.cuh) beside the flux divergence
+// and the bounds on the FP64 unit, whose 577 instructions a zone bound the
+// former all-FP64 form (2.26 ms per launch on a 128^3 grid; 1.03 ms so).
 // Every thread of the block must call it (warp counters).
+template <bool PRED>
 __device__ __forceinline__ void update_body(const StepArgs &A, const double *Pi,
                                             const double *__restrict__ Ps, double *Pout,
                                             const double *__restrict__ F1,
                                             const double *__restrict__ F2,
                                             const double *__restrict__ F3, int *pflag, int *fflag,
-                                            double dtfac, double *Ucache, int ucache_mode,
-                                            long long t) {
+                                            double dtfac, double *Ucache, bool keep, long long t) {
   const Dims &D = A.D;
   const double dt = A.clk->dt;
   if (!(dt > 0.0)) return;  // uniform across the grid: no warp divergence
@@ -635,51 +683,70 @@ __device__ __forceinline__ void update_body(const StepArgs &A, const double *Pi,
     const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
-    Geo G;
-    load_geo(A.geom, D.n2d, ij, G);
-    double pi[NV], ps[NV], Ui[NV];
+    const double *g = A.geom + ij, *cn = A.conn + ij;
+    const auto geo = [g, &D](int comp) { return __ldg(g + comp * D.n2d); };
+    const auto conn = [cn, &D](int comp) { return __ldg(cn + comp * D.n2d); };
+    double Un[NV], S[4], guess;
+    {
+      double U[NV];
+      if (A.clk->coupled) {
+        double Uc[NV], Sc[4], gc;
+        source_fp64(A, Ps, c, ij, Uc, Sc, gc);
 #pragma unroll
-    for (int v = 0; v < NV; v++) pi[v] = Pi[v * N + c];
-    double S[4];
-    if (Ps == Pi) {
-      FState si;
-      fluid_state(pi, G, si);
-      prim_flux(pi, si, G, A.gam, 0, Ui);
-      if (ucache_mode == 1) {
+        for (int v = 0; v < NV; v++) U[v] = Uc[v];
 #pragma unroll
-        for (int v = 0; v < NV; v++) Ucache[v * N + c] = Ui[v];
-      }
-      geo_source(pi, si, G, A.conn, D.n2d, ij, A.gam, S);
-    } else {
-      if (ucache_mode == 2) {
-#pragma unroll
-        for (int v = 0; v < NV; v++) Ui[v] = Ucache[v * N + c];
+        for (int n = 0; n < 4; n++) S[n] = Sc[n];
+        guess = gc;
       } else {
-        FState si;
-        fluid_state(pi, G, si);
-        prim_flux(pi, si, G, A.gam, 0, Ui);
+        double p[NV], g2;
+#pragma unroll
+        for (int v = 0; v < NV; v++) p[v] = __ldg(Ps + v * N + c);
+        wide_source<true, PRED>(p, geo, conn, A.gm1, U, S, g2);
+        if (PRED) {  // U^t has no field part: b^i u^t - b^t u^i = B^i
+          const double gd = geo(G_GDET);
+#pragma unroll
+          for (int v = B1; v < NV; v++) U[v] = gd * p[v];
+        }
+        guess = fma(A.gam, p[UU], p[RHO]) * g2;
       }
 #pragma unroll
-      for (int v = 0; v < NV; v++) ps[v] = Ps[v * N + c];
-      FState ss;
-      fluid_state(ps, G, ss);
-      geo_source(ps, ss, G, A.conn, D.n2d, ij, A.gam, S);
-    }
-    const double idx1 = A.idx[0], idx2 = A.idx[1], idx3 = A.idx[2];
-    double Un[NV];
-#pragma unroll
-    for (int v = 0; v < NV; v++) {
-      const long long o = v * N + c;
-      const double div = (F1[o + 1] - F1[o]) * idx1 + (F2[o + D.s[0]] - F2[o]) * idx2 +
-                         (F3[o + D.n2d] - F3[o]) * idx3;
-      // the source enters the energy and momentum rows only
-      Un[v] = (v >= UU && v <= U3) ? fma(dtp, S[v - UU] - div, Ui[v]) : fma(-dtp, div, Ui[v]);
+      for (int v = 0; v < NV; v++) {
+        const long long o = v * N + c;
+        if (PRED) {
+          if (keep) Ucache[o] = U[v];
+        } else {
+          U[v] = Ucache[o];
+        }
+        const double div = flux_div(A, F1, F2, F3, o);
+        // the source enters the energy and momentum rows only
+        Un[v] = (v >= UU && v <= U3) ? fma(dtp, S[v - UU] - div, U[v]) : fma(-dtp, div, U[v]);
+      }
     }
     double pn[NV], bsq_n = 0.0, lor_n = 1.0;
-    pf = invert_1dw(Un, G, A.gk, pi, pn, bsq_n, lor_n);
-    if (pf == PF_OK && A.floors_on && !A.floor_drift && !A.elec)
-      ff = apply_floors_known(pn, G, __ldg(A.floors + ij), __ldg(A.floors + D.n2d + ij), A.gk,
-                              bsq_n, lor_n);
+    if (A.clk->coupled || !wide_invert<true>(Un, geo, A.gk, guess, pn, bsq_n, lor_n)) {
+      double u[NV], p[NV], b, l = 1.0;
+#pragma unroll
+      for (int v = 0; v < NV; v++) u[v] = Un[v];
+      b = 0.0;
+      pf = invert_fp64(A, u, Pi, c, ij, p, b, l);
+#pragma unroll
+      for (int v = 0; v < NV; v++) pn[v] = p[v];
+      bsq_n = b;
+      lor_n = l;
+    }
+    if (pf == PF_OK && A.floors_on && !A.floor_drift && !A.elec) {
+      const double rho_fl = __ldg(A.floors + ij), u_fl = __ldg(A.floors + D.n2d + ij);
+      if (lor_n > FL_GAMMA) {
+        double p[NV];
+#pragma unroll
+        for (int v = 0; v < NV; v++) p[v] = pn[v];
+        ff = floors_capped(A, ij, rho_fl, u_fl, p);
+#pragma unroll
+        for (int v = 0; v < NV; v++) pn[v] = p[v];
+      } else {
+        ff = apply_floors_known(pn, rho_fl, u_fl, A.gk, bsq_n);
+      }
+    }
 #pragma unroll
     for (int v = 0; v < NV; v++) Pout[v * N + c] = pn[v];
     pflag[c] = pf;

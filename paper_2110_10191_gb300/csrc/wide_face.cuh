@@ -20,6 +20,7 @@ struct WideState {
   Wide ucon[4], ucov[4];  // u^mu, u_mu
   Wide Bcov[4];           // B_mu
   Wide bt, bsq, iut;      // b^t, b^2, 1/u^t
+  Wide g2;                // Lorentz factor squared
 };
 
 // geo(c): component c of the location's geometry (G_*), as a double
@@ -51,6 +52,7 @@ WIDE_FN void wide_state(const double P[NV], const GeoFn &geo, WideState &s) {
   }
   const Wide one = {1ull << 61, 0, -61};
   const Wide g2 = norm(w_sum<1>(one, s.ucov[1] * v1, s.ucov[2] * v2, s.ucov[3] * v3));
+  s.g2 = g2;
   const Wide rg = w_rsqrt(g2);
   const Wide gam = norm(g2 * rg);
   const Wide al = wide_pos(geo(G_ALPHA));

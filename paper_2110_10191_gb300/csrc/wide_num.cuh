@@ -78,7 +78,8 @@ WIDE_FN Wide norm(const Wide &a) {
 
 // Signed sums on the largest exponent, the magnitudes shifted right by H more
 // bits so that the sum stays below 2^63: H = 0 for two products (each below
-// 2^62), 1 for four products or two numbers, 2 for four numbers.  A term is
+// 2^62), 1 for four products or two numbers, 2 for four numbers or one and four
+// products.  A term is
 // (m ^ s) - s; the s are gathered in one word.
 WIDE_FN u64 w_term(const Wide &a, int x) { return w_shr(a.m, x - a.x) ^ (u64)(s64)a.s; }
 WIDE_FN Wide w_sum_of(u64 terms, int s, int x) {
@@ -105,6 +106,13 @@ WIDE_FN Wide w_sum(const Wide &a, const Wide &b, const Wide &c, const Wide &d) {
   const int x = w_max(w_max(a.x, b.x), w_max(c.x, d.x)) + H;
   return w_sum_of(w_term(a, x) + w_term(b, x) + w_term(c, x) + w_term(d, x),
                   a.s + b.s + c.s + d.s, x);
+}
+
+template <int H>
+WIDE_FN Wide w_sum(const Wide &a, const Wide &b, const Wide &c, const Wide &d, const Wide &e) {
+  const int x = w_max(w_max(w_max(a.x, b.x), w_max(c.x, d.x)), e.x) + H;
+  return w_sum_of(w_term(a, x) + w_term(b, x) + w_term(c, x) + w_term(d, x) + w_term(e, x),
+                  a.s + b.s + c.s + d.s + e.s, x);
 }
 
 // the nearest double (the tail beyond 64 bits counted as zero)
@@ -154,6 +162,44 @@ WIDE_FN Wide w_rsqrt(const Wide &a) {
   r.m = (u64)(((s64)y << 39) + (c >> 20));  // (2^61, 2^62]
   r.s = 0;
   r.x = -e - 61;
+  return r;
+}
+
+// 1 / a for a normalised a, at most 2^-57 low: 2^95 / h in 32 bits (w_rcp32) and
+// one Newton step
+WIDE_FN Wide w_rcp(const Wide &a) {
+  const u64 h = a.m << 1;                // [2^63, 2^64)
+  const u32 r = w_rcp32(w_hi(h)) - 2u;   // <= 2^95 / h, within 2^-28
+  const u64 e = (1ull << 63) - (w_mul(r, w_hi(h)) + w_hi(w_mul(r, w_lo(h))));  // below 2^35
+  Wide q;
+  q.m = ((u64)r << 31) + (w_mul(r, (u32)(e >> 3)) >> 29);
+  q.s = a.s;
+  q.x = -125 - a.x;
+  return q;
+}
+
+// a 2^k as a float (24 bits of the upper word), saturating to 0 and infinity
+WIDE_FN float w_to_float(const Wide &a, int k) {
+  const int e = w_min(w_max(a.x + 32 + k, -126), 127);
+#ifdef __CUDA_ARCH__
+  const float f = __uint2float_rz(w_hi(a.m)) * __int_as_float((e + 127) << 23);
+#else
+  const float f = (float)(w_hi(a.m) & 0xffffff80u) * __builtin_ldexpf(1.0f, e);
+#endif
+  return a.s ? -f : f;
+}
+// a positive normal float
+WIDE_FN Wide wide_posf(float f) {
+#ifdef __CUDA_ARCH__
+  const u32 b = __float_as_uint(f);
+#else
+  u32 b;
+  memcpy(&b, &f, 4);
+#endif
+  Wide r;
+  r.m = (u64)((b & 0x7fffffu) | 0x800000u) << 39;  // [2^62, 2^63)
+  r.s = 0;
+  r.x = (int)(b >> 23) - (127 + 62);
   return r;
 }
 

@@ -1,0 +1,238 @@
+// wide_update.cuh -- the conserved densities, the geometric source and the 1D_W
+// inversion of one zone in Wide numbers (wide_num.cuh): the formulas of
+// prim_flux (direction 0), geo_source and invert_1dw.
+#pragma once
+
+#include <math.h>
+
+#include "wide_face.cuh"
+
+namespace grmhd {
+
+// U(P) (WANT_U) and the source S_nu = sqrt(-g) T^k_l Gamma^l_{nu k} of a state,
+// rounded to double; g2: its Lorentz factor squared.  conn(c): component c of the
+// connection.  T^k_l is formed row by row and its products with the
+// connection summed as they come.
+template <bool BLK, bool WANT_U, class GeoFn, class ConnFn>
+WIDE_FN void wide_source(const double P[NV], const GeoFn &geo, const ConnFn &conn, double gm1,
+                         double U[NV], double S[4], double &g2) {
+  WideState s;
+  wide_state<BLK>(P, geo, s);
+  g2 = w_to_double(s.g2);
+  const Wide rho = wide(P[RHO]), u = wide(P[UU]), pg = wide(gm1) * u;
+  const Wide w = norm(w_sum<2>(rho, u, pg, s.bsq));
+  const Wide pt = w_sum<1>(pg, w_scale(s.bsq, -1));
+  const Wide gd = wide_pos(geo(G_GDET));
+  Wide bcov[4];
+#pragma unroll
+  for (int n = 0; n < 4; n++) bcov[n] = norm(w_sum<1>(s.Bcov[n], s.bt * s.ucov[n])) * s.iut;
+  Wide acc[4];
+#pragma unroll
+  for (int k = 0; k < 4; k++) {
+    const Wide bk =
+        k ? norm(w_sum<1>(wide(P[B1 - 1 + (k ? k : 1)]), s.bt * s.ucon[k])) * s.iut : s.bt;
+    const Wide wu = norm(w * s.ucon[k]), nb = -norm(bk);
+    Wide T[4];
+#pragma unroll
+    for (int l = 0; l < 4; l++)
+      T[l] = (k == l) ? w_sum<1>(wu * s.ucov[l], nb * bcov[l], pt)
+                      : w_sum<0>(wu * s.ucov[l], nb * bcov[l]);
+    if (WANT_U && k == 0) {
+      const Wide mf = rho * s.ucon[0];
+      U[RHO] = w_to_double(mf * gd);
+      U[UU] = w_to_double(w_sum<1>(T[0], mf) * gd);
+#pragma unroll
+      for (int i = 1; i < 4; i++) U[UU + i] = w_to_double(T[i] * gd);
+    }
+#pragma unroll
+    for (int l = 0; l < 4; l++) T[l] = norm(T[l]);
+#pragma unroll
+    for (int nu = 0; nu < 4; nu++) {
+      const Wide p0 = T[0] * wide(conn(0 * 10 + SY(nu, k))), p1 = T[1] * wide(conn(1 * 10 + SY(nu, k)));
+      const Wide p2 = T[2] * wide(conn(2 * 10 + SY(nu, k))), p3 = T[3] * wide(conn(3 * 10 + SY(nu, k)));
+      acc[nu] = norm(k ? w_sum<2>(acc[nu], p0, p1, p2, p3) : w_sum<1>(p0, p1, p2, p3));
+    }
+  }
+#pragma unroll
+  for (int nu = 0; nu < 4; nu++) S[nu] = w_to_double(acc[nu] * gd);
+}
+
+// FP32 forms of the 1D_W function's derivative at W = wp + d and of a Newton step
+// (all quantities in units of a power of two near W)
+struct InvF {
+  float d, b, qt2, qb2, qpn, gf;  // D, B^2, Qt^2, (Q.B)^2, Q'.n, (gamma - 1)/gamma
+};
+WIDE_FN float inv_rcpf(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / x;
+#endif
+}
+WIDE_FN float inv_rsqrtf(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / __builtin_sqrtf(x);
+#endif
+}
+// v^2; f and df are meaningless for v^2 >= 1
+WIDE_FN float inv_f32(const InvF &q, float wp, float &f, float &df) {
+  const float w = wp + q.d, bw = q.b + w, iw = inv_rcpf(w), ib = inv_rcpf(bw);
+  const float x2 = q.qb2 * iw * iw;
+  const float vsq = (q.qt2 + x2 * (q.b + 2.0f * w)) * ib * ib;
+  const float omv = 1.0f - vsq, rs = inv_rsqrtf(omv), sq = omv * rs;
+  const float wmr = wp * omv - q.d * vsq * sq * inv_rcpf(1.0f + sq);
+  f = q.qpn + wp - q.gf * wmr + 0.5f * (1.0f + vsq) * q.b - 0.5f * x2;
+  const float wdv =
+      -2.0f * ib * ib * ib * (q.qt2 * w + x2 * (3.0f * w * bw + q.b * q.b));  // W dv^2/dW
+  df = 1.0f - q.gf * (omv + wdv * (0.5f * q.d * rs * iw - 1.0f)) + (0.5f * q.b * wdv + x2) * iw;
+  return vsq;
+}
+
+// The 1D_W inversion where nothing unusual happens: Newton steps in FP32 from the
+// guess W (doubled while it lies below the root) until they are below 1e-5 (or six), then Newton steps whose function is taken in Wide numbers and
+// whose derivative in FP32 (each gains 20 bits or doubles the digits), until a
+// step is below 2^-34 W', after which the error is below 2^-54 W'.  False, with
+// nothing written, where the iteration of invert_1dw is needed for its answer or
+// its failure code: input that is not finite, D <= 0, an iterate with W' < 0 or
+// v^2 > 1 - 1e-10, no convergence, u < 0.
+template <bool BLK, class GeoFn>
+WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, double guess,
+                         double P[NV], double &bsq_out, double &lorentz_out) {
+#define GCOV(m, n) wide(geo(G_GCOV + SY(m, n)))
+#define GDIA(m) wide_pos(geo(G_GCOV + SY(m, m)))
+#define GCON(m, n) wide(geo(G_GCON + SY(m, n)))
+  bool ok = true;
+#pragma unroll
+  for (int v = 0; v < NV; v++) ok = ok && w_finite(U[v]);
+  const double igd = geo(G_IGDET);
+  double b[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++) b[i] = U[B1 + i] * igd;
+  const Wide al = wide_pos(geo(G_ALPHA)), wigd = wide_pos(igd), aig = norm(al * wigd);
+  const Wide n1 = al * wide(b[0]), n2 = al * wide(b[1]), n3 = al * wide(b[2]);  // normal-frame field
+  const Wide urho = wide(U[RHO]);
+  const Wide D = norm(urho * aig);
+  ok = ok && D.s == 0 && D.m != 0;
+  const Wide Q1 = norm(aig * wide(U[U1])), Q2 = norm(aig * wide(U[U2])), Q3 = norm(aig * wide(U[U3]));
+  // c.Q with c_i = g^{ti}; Q'.n = (U_u - (1 - alpha) U_rho) / sqrt(-g) - alpha c.Q;
+  // Qt^i = gamma^ij Q_j = g^ij Q_j + alpha^2 c^i c.Q
+  const Wide c1 = GCON(0, 1), c3 = GCON(0, 3);
+  Wide cQ, Qt1, Qt2, Qt3, Bsq;
+  if (BLK) {
+    cQ = norm(w_sum<0>(c1 * Q1, c3 * Q3));
+  } else {
+    cQ = norm(w_sum<1>(c1 * Q1, GCON(0, 2) * Q2, c3 * Q3));
+  }
+  const Wide acQ = norm(al * cQ), a2cQ = norm(al * acQ);
+  const Wide Qpn = norm(w_sum<1>(
+      norm(w_sum<1>(wide(U[UU]), -(wide(geo(G_OMALPHA)) * urho))) * wigd, -acQ));
+  if (BLK) {
+    const Wide g13 = GCON(1, 3), h13 = GCOV(1, 3);
+    Qt1 = norm(w_sum<1>(GCON(1, 1) * Q1, g13 * Q3, c1 * a2cQ));
+    Qt2 = norm(GCON(2, 2) * Q2);
+    Qt3 = norm(w_sum<1>(g13 * Q1, GCON(3, 3) * Q3, c3 * a2cQ));
+    Bsq = norm(w_sum<1>(n1 * norm(w_sum<0>(GDIA(1) * n1, h13 * n3)), n2 * norm(GDIA(2) * n2),
+                        n3 * norm(w_sum<0>(h13 * n1, GDIA(3) * n3))));
+  } else {
+    const Wide g12 = GCON(1, 2), g13 = GCON(1, 3), g23 = GCON(2, 3);
+    const Wide h12 = GCOV(1, 2), h13 = GCOV(1, 3), h23 = GCOV(2, 3);
+    Qt1 = norm(w_sum<1>(GCON(1, 1) * Q1, g12 * Q2, g13 * Q3, c1 * a2cQ));
+    Qt2 = norm(w_sum<1>(g12 * Q1, GCON(2, 2) * Q2, g23 * Q3, GCON(0, 2) * a2cQ));
+    Qt3 = norm(w_sum<1>(g13 * Q1, g23 * Q2, GCON(3, 3) * Q3, c3 * a2cQ));
+    Bsq = norm(w_sum<1>(n1 * norm(w_sum<1>(GDIA(1) * n1, h12 * n2, h13 * n3)),
+                        n2 * norm(w_sum<1>(h12 * n1, GDIA(2) * n2, h23 * n3)),
+                        n3 * norm(w_sum<1>(h13 * n1, h23 * n2, GDIA(3) * n3))));
+  }
+  const Wide Qtsq = norm(w_sum<1>(Qt1 * Q1, Qt2 * Q2, Qt3 * Q3));
+  const Wide QdB = norm(w_sum<1>(Q1 * n1, Q2 * n2, Q3 * n3));
+  ok = ok && w_finite(guess) && (Qtsq.s == 0 || Qtsq.m == 0) && (Bsq.s == 0 || Bsq.m == 0);
+
+  // the guess, improved in FP32
+  Wide Wp = norm(w_sum<1>(wide(guess), -D));
+  const int e = -(int)((w_hi(w_bits(guess)) >> 20) & 0x7ff) + 1023;  // guess 2^e in [1, 2)
+  InvF q;
+  q.d = w_to_float(D, e);
+  q.b = w_to_float(Bsq, e);
+  q.qt2 = w_to_float(Qtsq, 2 * e);
+  q.qb2 = w_to_float(norm(QdB * QdB), 3 * e);
+  q.qpn = w_to_float(Qpn, e);
+  q.gf = (float)K.gf;
+  {
+    // (a root below 1e-6 D is left to the Wide steps)
+    float w = w_to_float(Wp, e), last = 1.0f;
+    if (!(w > 1e-6f * q.d)) w = 1e-6f * q.d;
+#pragma unroll 1
+    for (int it = 0; it < 6 && last > 1e-5f; it++) {
+      float f, df, n;
+      if (inv_f32(q, w, f, df) < 0.99999f) {
+        n = w - f * inv_rcpf(df);
+        if (!(n > 0.0f)) n = 0.5f * w;
+        last = fabsf(n - w) * inv_rcpf(w);
+      } else {  // below the root
+        n = w + (w + q.d);
+      }
+      w = n;
+    }
+    const bool fine = last < 0.5f && w < 1e6f;
+    if (fine)
+      Wp = w_scale(wide_posf(w), -e);
+    else if (Wp.s || Wp.m == 0)
+      ok = false;
+  }
+
+  const Wide gf = wide_pos(K.gf), hB = w_scale(Bsq, -1);
+  const Wide one = {1ull << 61, 0, -61};
+  bool done = false;
+  Wide W, iB, x, x2, omv, rs, wmr;
+#pragma unroll 1
+  for (int it = 0; it < 7 && ok; it++) {
+    W = norm(w_sum<1>(Wp, D));
+    const Wide BW = norm(w_sum<1>(Bsq, W));
+    const Wide ix = w_rcp(norm(BW * W));
+    iB = norm(W * ix);              // 1/(B^2 + W)
+    x = norm(QdB * norm(BW * ix));  // Q.B / W
+    x2 = x * x;
+    const Wide vsq = norm(norm(w_sum<1>(Qtsq, x2 * norm(w_sum<1>(Bsq, w_scale(W, 1))))) * norm(iB * iB));
+    omv = norm(w_sum<1>(one, -vsq));
+    ok = omv.s == 0 && omv.x >= -62 - 33;  // 1 - v^2 >= 2^-33
+    if (!ok) break;
+    rs = norm(w_rsqrt(omv));  // Lorentz factor
+    const Wide sq = norm(omv * rs);
+    // w - rho = W' (1 - v^2) - D v^2 sq / (1 + sq)
+    wmr = w_sum<0>(Wp * omv, -(norm(norm(D * vsq) * sq) * w_rcp(norm(w_sum<1>(one, sq)))));
+    if (done) break;
+    const Wide t = w_sum<2>(Qpn, Wp, hB, -(gf * norm(wmr)));
+    const Wide f = norm(w_sum<1>(t, hB * vsq, -w_scale(x2, -1)));
+    float ff, df;
+    inv_f32(q, w_to_float(Wp, e), ff, df);
+    const Wide step = norm(f * wide_posf(inv_rcpf(df)));
+    const Wide n = norm(w_sum<1>(Wp, -step));
+    ok = df > 0.0f && n.s == 0 && n.m != 0;
+    done = step.x < n.x - 34 || step.m == 0;
+    Wp = n;
+  }
+  ok = ok && done && (wmr.s == 0 || wmr.m == 0);
+  if (!ok) return false;
+  const Wide sq = norm(omv * rs), fac = norm(rs * iB);
+  P[RHO] = w_to_double(D * sq);
+  P[UU] = w_to_double(norm(wmr) * wide_pos(K.igam));
+  P[U1] = w_to_double(fac * norm(w_sum<1>(Qt1, x * n1)));
+  P[U2] = w_to_double(fac * norm(w_sum<1>(Qt2, x * n2)));
+  P[U3] = w_to_double(fac * norm(w_sum<1>(Qt3, x * n3)));
+#pragma unroll
+  for (int i = 0; i < 3; i++) P[B1 + i] = b[i];
+  bsq_out = w_to_double(w_sum<0>(Bsq * omv, x2));
+  lorentz_out = w_to_double(rs);
+  return true;
+#undef GCOV
+#undef GDIA
+#undef GCON
+}
+
+}  // namespace grmhd
