@@ -162,16 +162,22 @@ __global__ void kp_ct(BView V) {
   ct_body(it.A, it.F[0], it.F[1], it.F[2], it.emf, block_tid(V, g));
 }
 
-// at most 168 registers: 3 blocks of 128 threads per SM (per cycle of a 128^3
-// grid 2.06 ms, at 128 registers 2.10, at 96 2.59 with the spills).
-// PRED: the predictor (in = 0), whose ucache_mode 1 keeps U(P^n) for the corrector
+// The update's two passes.  PRED: the predictor (in = 0).  The source and the
+// guess W wait in the low faces' array, which the face fluxes have done with.
+// 20 and 24 warps per SM against some spills (both passes per cycle of a 128^3
+// grid: 168 and 128 registers 1.74 ms, 128 and 112 1.66, 96 and 80 1.58).
 template <bool PRED>
-__global__ void __maxnreg__(168) kp_update(BView V, double dtfac, int ucache_mode) {
+__global__ void __maxnreg__(96) kp_source(BView V) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  const int in = PRED ? 0 : 1;
-  update_body<PRED>(it.A, it.P, arr(it, in), arr(it, 1 - in), it.F[0], it.F[1], it.F[2], it.pflag,
-                    it.fflag, dtfac, it.Uc, ucache_mode == 1, block_tid(V, g));
+  source_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Uc, it.Lf, block_tid(V, g));
+}
+
+__global__ void __maxnreg__(80) kp_invert(BView V, int in, double dtfac) {
+  const int g = block_grid(V);
+  const StageItem &it = V.items[g];
+  invert_body(it.A, it.F[0], it.F[1], it.F[2], it.Uc, it.Lf, dtfac, it.P, arr(it, 1 - in), it.pflag,
+              it.fflag, block_tid(V, g));
 }
 
 // at most 128 registers: 4 blocks of 128 threads per SM; the spill it costs
@@ -327,8 +333,8 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_RECON1] = f64 ? n_recon_walk(D, 1, fl, rwalk) : 0;
   c[PC_RECON2] = (f64 && !fl) ? n_recon_walk(D, 2, 0, rwalk) : 0;
   for (int d = 0; d < 3; d++) {
-    c[PC_FACE0 + d] = (f64 && !elec) ? n_face_threads(n_face(D, d, fl)) : 0;
-    c[PC_FACE0E + d] = (f64 && elec) ? n_face_threads(n_face(D, d, fl)) : 0;
+    c[PC_FACE0 + d] = (f64 && !elec) ? n_face_threads(D, d, fl) : 0;
+    c[PC_FACE0E + d] = (f64 && elec) ? n_face_threads(D, d, fl) : 0;
     c[PC_FACE0F + d] = mx ? (d == 0 ? n_flux_f32_x1(D, fl) : n_flux_f32_walk(D, d, fl)) : 0;
     c[PC_FACE0X + d] = fx ? n_face(D, d, fl) : 0;
   }
@@ -340,7 +346,7 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_FIX] = n_fix(D);
   c[PC_EDGE] = n_edge(D);
   c[PC_ZONE] = n_zone(D);
-  c[PC_UPD64] = ux ? 0 : n_zone(D);
+  c[PC_UPD64] = ux ? 0 : n_update(D);
   c[PC_UPDX] = ux ? n_zone(D) : 0;
   c[PC_FLOORD] = (drift && !elec) ? n_zone(D) : 0;
   for (int d = 0; d < 3; d++) c[PC_EFACE0 + d] = elec ? n_face(D, d, fl) : 0;
@@ -529,10 +535,11 @@ int plan_update_only(const Plan &p, int in, double dtfac, int ucache_mode, cudaS
                      PlanHook *h) {
   int nl = launch(p, PC_UPD64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
     if (in == 0)
-      kp_update<true><<<nb, bs, 0, st>>>(V, dtfac, ucache_mode);
+      kp_source<true><<<nb, bs, 0, st>>>(V);
     else  // the predictor before it kept U(P^n)
-      kp_update<false><<<nb, bs, 0, st>>>(V, dtfac, ucache_mode);
+      kp_source<false><<<nb, bs, 0, st>>>(V);
   });
+  nl += launch(p, PC_UPD64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, in, dtfac); });
   nl += launch(p, PC_UPDX, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
     kp_update_ff<<<nb, bs, 0, st>>>(V, in, dtfac, ucache_mode);
   });
@@ -657,7 +664,8 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
         L(PC_FACE2, [&](unsigned nb, unsigned bs, BView V) { kp_face<2><<<nb, bs, 0, st>>>(V, 0); });
         break;
       case 5:  // predictor-like update without keeping U(P^n)
-        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_update<true><<<nb, bs, 0, st>>>(V, 0.5, 0); });
+        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_source<true><<<nb, bs, 0, st>>>(V); });
+        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, 0, 0.5); });
         break;
       case 16:
         L(PC_UPDX, [&](unsigned nb, unsigned bs, BView V) { kp_update_ff<<<nb, bs, 0, st>>>(V, 0, 0.5, 0); });

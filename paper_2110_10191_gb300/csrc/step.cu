@@ -45,13 +45,11 @@ __global__ void __launch_bounds__(BS) k_flux(StepArgs A, const double *__restric
 
 template <int DIR>
 static void launch_flux_dir(const StepArgs &A, const double *P, double *F, cudaStream_t st) {
-  const Dims &D = A.D;
-  long long nf = 1;
-  for (int e = 0; e < 3; e++) nf *= (e == DIR) ? D.n[e] + 1 : D.n[e] + 2;
+  const unsigned nb = nblk(n_face_threads(A.D, DIR, 0));
   if (A.recon == 1)
-    k_flux<DIR, 1><<<nblk(n_face_threads(nf)), BS, 0, st>>>(A, P, F);
+    k_flux<DIR, 1><<<nb, BS, 0, st>>>(A, P, F);
   else
-    k_flux<DIR, 0><<<nblk(n_face_threads(nf)), BS, 0, st>>>(A, P, F);
+    k_flux<DIR, 0><<<nb, BS, 0, st>>>(A, P, F);
 }
 
 void launch_fluxes(const StepArgs &A, const double *P, double *F[3], cudaStream_t st) {

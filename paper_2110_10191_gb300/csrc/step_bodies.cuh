@@ -52,6 +52,28 @@ __device__ __forceinline__ Idx3 unflatten(long long t, int n0, int n1) {
   return {(int)(u - q * n0), (int)(q - k * n1), (int)k};
 }
 
+// Warps over columns along X3: a warp takes `lanes` consecutive points of the
+// (X1, X2) plane of a range n0 x n1 x n2 at one k, the next warp the same points at
+// the next k, so that the warps of a block share the points' geometry in L1.
+__host__ __device__ inline long long n_column_threads(int lanes, int n0, int n1, int n2) {
+  return 32 * (((long long)n0 * n1 + lanes - 1) / lanes) * n2;
+}
+struct Column {
+  bool active;
+  int i, j, k;  // inactive lanes: of the plane's last point
+};
+__device__ __forceinline__ Column column_of(long long t, int lane, int lanes, int n0, int n1, int n2) {
+  const u32 w = (u32)(t >> 5), chunk = w / (u32)n2, plane = (u32)(n0 * n1);
+  u32 p = chunk * lanes + lane;
+  Column q;
+  q.k = (int)(w - chunk * n2);
+  q.active = p < plane;
+  if (!q.active) p = plane - 1;
+  q.j = (int)(p / (u32)n0);
+  q.i = (int)(p - q.j * n0);
+  return q;
+}
+
 // ---------------------------------------------------------------------------
 // Launch extents (threads per grid) of each body
 // ---------------------------------------------------------------------------
@@ -105,6 +127,10 @@ __host__ __device__ inline long long n_edge(const Dims &D) {
 }
 __host__ __device__ inline long long n_zone(const Dims &D) {
   return (long long)D.n[0] * D.n[1] * D.n[2];
+}
+// threads of the update's passes
+__host__ __device__ inline long long n_update(const Dims &D) {
+  return n_column_threads(32, D.n[0], D.n[1], D.n[2]);
 }
 
 // ---------------------------------------------------------------------------
@@ -336,24 +362,27 @@ __device__ __forceinline__ void recon_x1_body(const StepArgs &A, const double *_
 }
 
 // The two threads of a face: lanes 0..15 of a warp take the left states of 16
-// consecutive faces, lanes 16..31 their right states.
-__host__ __device__ inline long long n_face_threads(long long nface) { return 32 * ((nface + 15) / 16); }
+// faces, lanes 16..31 their right states.
+__host__ __device__ inline long long n_face_threads(const Dims &D, int dir, int flat3) {
+  int lo[3], ext[3];
+  face_box(D, dir, flat3, lo, ext);
+  return n_column_threads(16, ext[0], ext[1], ext[2]);
+}
 struct FaceLane {
   bool active, right;
   int i, j, k;
-  long long c;  // zone above the face (inactive lanes: of the last face)
+  long long c;  // zone above the face
 };
 template <int DIR>
 __device__ __forceinline__ FaceLane face_lane(const Dims &D, int flat3, long long t) {
   int lo[3], ext[3];
   face_box(D, DIR, flat3, lo, ext);
-  const long long nface = (long long)ext[0] * ext[1] * ext[2];
-  long long f = (t >> 5) * 16 + (t & 15);
+  // a block's last warps may lie past the last column
+  const long long n = n_column_threads(16, ext[0], ext[1], ext[2]);
+  const Column q = column_of((t < n) ? t : t & 31, (int)(t & 15), 16, ext[0], ext[1], ext[2]);
   FaceLane L;
-  L.active = f < nface;
+  L.active = q.active && t < n;
   L.right = (t & 16) != 0;
-  if (!L.active) f = nface - 1;
-  const Idx3 q = unflatten(f, ext[0], ext[1]);
   L.i = lo[0] + q.i;
   L.j = lo[1] + q.j;
   L.k = lo[2] + q.k;
@@ -589,20 +618,10 @@ __device__ __forceinline__ void count_warp(bool pred, unsigned long long *ctr) {
   if (m && (threadIdx.x & 31) == 0) atomicAdd(ctr, (unsigned long long)__popc(m));
 }
 
-__device__ __forceinline__ void geo_source(const double P[NV], const FState &s, const Geo &G,
+// S_nu = sqrt(-g) T^k_l Gamma^l_{nu k}
+__device__ __forceinline__ void geo_source(const double T[4][4], double gdet,
                                            const double *__restrict__ conn, long long n2d,
-                                           long long ij, double gam, double S[4]) {
-  // S_nu = sqrt(-g) T^k_l Gamma^l_{nu k}
-  const double pg = (gam - 1.0) * P[UU];
-  const double w = P[RHO] + P[UU] + pg + s.bsq;
-  const double pt = pg + 0.5 * s.bsq;
-  double T[4][4];
-#pragma unroll
-  for (int m = 0; m < 4; m++) {
-#pragma unroll
-    for (int n = 0; n < 4; n++) T[m][n] = w * s.ucon[m] * s.ucov[n] - s.bcon[m] * s.bcov[n];
-    T[m][m] += pt;
-  }
+                                           long long ij, double S[4]) {
 #pragma unroll
   for (int nu = 0; nu < 4; nu++) {
     double acc = 0.0;
@@ -610,7 +629,7 @@ __device__ __forceinline__ void geo_source(const double P[NV], const FState &s, 
     for (int k = 0; k < 4; k++)
 #pragma unroll
       for (int l = 0; l < 4; l++) acc += T[k][l] * __ldg(conn + (l * 10 + SY(nu, k)) * n2d + ij);
-    S[nu] = acc * G.gdet;
+    S[nu] = acc * gdet;
   }
 }
 
@@ -622,10 +641,11 @@ __device__ __forceinline__ double flux_div(const StepArgs &A, const double *__re
          (F3[o + A.D.n2d] - F3[o]) * A.idx[2];
 }
 
-// U(P) and the source of a state in FP64: metrics that couple X2.
-static __device__ __noinline__ void source_fp64(const StepArgs &A, const double *__restrict__ Ps,
+// U(P), the stress-energy tensor and the Lorentz factor squared of a state in
+// FP64: metrics that couple X2.
+static __device__ __noinline__ void tensor_fp64(const StepArgs &A, const double *__restrict__ Ps,
                                                 long long c, long long ij, double U[NV],
-                                                double S[4], double &guess) {
+                                                double T[4][4], double &g2) {
   Geo G;
   load_geo(A.geom, A.D.n2d, ij, G);
   double p[NV];
@@ -633,9 +653,14 @@ static __device__ __noinline__ void source_fp64(const StepArgs &A, const double 
   FState s;
   fluid_state(p, G, s);
   prim_flux(p, s, G, A.gam, 0, U);
-  geo_source(p, s, G, A.conn, A.D.n2d, ij, A.gam, S);
+  const double pg = (A.gam - 1.0) * p[UU];
+  const double w = p[RHO] + p[UU] + pg + s.bsq;
+  for (int m = 0; m < 4; m++) {
+    for (int n = 0; n < 4; n++) T[m][n] = w * s.ucon[m] * s.ucov[n] - s.bcon[m] * s.bcov[n];
+    T[m][m] += pg + 0.5 * s.bsq;
+  }
   const double g = s.ucon[0] * G.alpha;
-  guess = (p[RHO] + A.gam * p[UU]) * g * g;
+  g2 = g * g;
 }
 
 // The bounds of a zone that needs the Lorentz-factor cap.
@@ -658,76 +683,95 @@ static __device__ __noinline__ int invert_fp64(const StepArgs &A, const double U
   return invert_1dw(U, G, A.gk, p, P, bsq, lorentz);
 }
 
-// The predictor (PRED: P_s = P_i = P^n) keeps U(P^n) in Ucache if keep is set;
-// the corrector, whose P_i is the same P^n, reads it there.  U(P), the source and
-// the inversion run in Wide numbers (wide_update.cuh) beside the flux divergence
-// and the bounds on the FP64 unit, whose 577 instructions a zone bound the
-// former all-FP64 form (2.26 ms per launch on a 128^3 grid; 1.03 ms so).
-// Every thread of the block must call it (warp counters).
+// The update is two passes, so that each keeps its registers and its code in
+// the SM's instruction cache: source_body forms U(P^n), the source and the
+// inversion's guess W, invert_body the new conserved vector, its primitives and
+// their bounds.  The states' products and the inversion run in Wide numbers
+// (wide_update.cuh); the source's contraction (64 instructions) in the one pass
+// and the flux divergence (60) in the other run on the FP64 unit beside them,
+// whose 577 instructions a zone bound the former single pass of FP64 (per launch on
+// a 128^3 grid 2.26 ms; 0.79 ms for both passes, 1.03 as one pass of Wide numbers
+// with the source among them, which waited for spills and instructions).
+//
+// The predictor (PRED: P_s = P_i = P^n) keeps U(P^n) in Ucache for both stages.
+// scratch: S_0 .. S_3 and the guess, [5][ntot].
 template <bool PRED>
-__device__ __forceinline__ void update_body(const StepArgs &A, const double *Pi,
-                                            const double *__restrict__ Ps, double *Pout,
-                                            const double *__restrict__ F1,
+__device__ __forceinline__ void source_body(const StepArgs &A, const double *__restrict__ Ps,
+                                            double *__restrict__ Ucache,
+                                            double *__restrict__ scratch, long long t) {
+  const Dims &D = A.D;
+  if (!(A.clk->dt > 0.0) || t >= n_update(D)) return;
+  const Column q3 = column_of(t, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
+  if (!q3.active) return;
+  const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
+  const long long c = zid(D, i, j, k), N = D.ntot;
+  const long long ij = (long long)j * D.s[0] + i;
+  const double *g = A.geom + ij;
+  const auto geo = [g, &D](int comp) { return __ldg(g + comp * D.n2d); };
+  double p[NV], U[NV], T[4][4], S[4], g2;
+#pragma unroll
+  for (int v = 0; v < NV; v++) p[v] = __ldg(Ps + v * N + c);
+  if (A.clk->coupled) {
+    double Uc[NV], Tc[4][4], gc;
+    tensor_fp64(A, Ps, c, ij, Uc, Tc, gc);
+#pragma unroll
+    for (int v = 0; v < NV; v++) U[v] = Uc[v];
+#pragma unroll
+    for (int m = 0; m < 4; m++)
+#pragma unroll
+      for (int n = 0; n < 4; n++) T[m][n] = Tc[m][n];
+    g2 = gc;
+  } else {
+    wide_tensor<true, PRED>(p, geo, A.gm1, U, T, g2);
+  }
+  const double gd = geo(G_GDET);
+  if (PRED) {  // U^t has no field part: b^i u^t - b^t u^i = B^i
+#pragma unroll
+    for (int v = 0; v < NV; v++) Ucache[v * N + c] = (v < B1) ? U[v] : gd * p[v];
+  }
+  geo_source(T, gd, A.conn, D.n2d, ij, S);
+#pragma unroll
+  for (int n = 0; n < 4; n++) scratch[n * N + c] = S[n];
+  scratch[4 * N + c] = fma(A.gam, p[UU], p[RHO]) * g2;
+}
+
+// U(P^n) + dt' (S - div F), its inversion and the bounds; Pi: the guess of the
+// FP64 iteration.  Every thread of the block must call it (warp counters).
+__device__ __forceinline__ void invert_body(const StepArgs &A, const double *__restrict__ F1,
                                             const double *__restrict__ F2,
-                                            const double *__restrict__ F3, int *pflag, int *fflag,
-                                            double dtfac, double *Ucache, bool keep, long long t) {
+                                            const double *__restrict__ F3,
+                                            const double *__restrict__ Ucache,
+                                            const double *__restrict__ scratch, double dtfac,
+                                            const double *Pi, double *Pout, int *pflag, int *fflag,
+                                            long long t) {
   const Dims &D = A.D;
   const double dt = A.clk->dt;
   if (!(dt > 0.0)) return;  // uniform across the grid: no warp divergence
   const double dtp = dtfac * dt;
-  const long long nz = n_zone(D);
-  const bool active = t < nz;
+  const bool in = t < n_update(D);
+  const Column q3 = column_of(in ? t : t & 31, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
+  const bool active = in && q3.active;
   int pf = 0, ff = 0;
   if (active) {
-    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
     const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
-    const double *g = A.geom + ij, *cn = A.conn + ij;
+    const double *g = A.geom + ij;
     const auto geo = [g, &D](int comp) { return __ldg(g + comp * D.n2d); };
-    const auto conn = [cn, &D](int comp) { return __ldg(cn + comp * D.n2d); };
-    double Un[NV], S[4], guess;
-    {
-      double U[NV];
-      if (A.clk->coupled) {
-        double Uc[NV], Sc[4], gc;
-        source_fp64(A, Ps, c, ij, Uc, Sc, gc);
+    double Un[NV], pn[NV], bsq_n = 0.0, lor_n = 1.0;
 #pragma unroll
-        for (int v = 0; v < NV; v++) U[v] = Uc[v];
-#pragma unroll
-        for (int n = 0; n < 4; n++) S[n] = Sc[n];
-        guess = gc;
-      } else {
-        double p[NV], g2;
-#pragma unroll
-        for (int v = 0; v < NV; v++) p[v] = __ldg(Ps + v * N + c);
-        wide_source<true, PRED>(p, geo, conn, A.gm1, U, S, g2);
-        if (PRED) {  // U^t has no field part: b^i u^t - b^t u^i = B^i
-          const double gd = geo(G_GDET);
-#pragma unroll
-          for (int v = B1; v < NV; v++) U[v] = gd * p[v];
-        }
-        guess = fma(A.gam, p[UU], p[RHO]) * g2;
-      }
-#pragma unroll
-      for (int v = 0; v < NV; v++) {
-        const long long o = v * N + c;
-        if (PRED) {
-          if (keep) Ucache[o] = U[v];
-        } else {
-          U[v] = Ucache[o];
-        }
-        const double div = flux_div(A, F1, F2, F3, o);
-        // the source enters the energy and momentum rows only
-        Un[v] = (v >= UU && v <= U3) ? fma(dtp, S[v - UU] - div, U[v]) : fma(-dtp, div, U[v]);
-      }
+    for (int v = 0; v < NV; v++) {
+      const long long o = v * N + c;
+      const double div = flux_div(A, F1, F2, F3, o), u = __ldg(Ucache + o);
+      // the source enters the energy and momentum rows only
+      Un[v] = (v >= UU && v <= U3) ? fma(dtp, __ldg(scratch + (v - UU) * N + c) - div, u)
+                                   : fma(-dtp, div, u);
     }
-    double pn[NV], bsq_n = 0.0, lor_n = 1.0;
+    const double guess = __ldg(scratch + 4 * N + c);
     if (A.clk->coupled || !wide_invert<true>(Un, geo, A.gk, guess, pn, bsq_n, lor_n)) {
-      double u[NV], p[NV], b, l = 1.0;
+      double u[NV], p[NV], b = 0.0, l = 1.0;
 #pragma unroll
       for (int v = 0; v < NV; v++) u[v] = Un[v];
-      b = 0.0;
       pf = invert_fp64(A, u, Pi, c, ij, p, b, l);
 #pragma unroll
       for (int v = 0; v < NV; v++) pn[v] = p[v];
@@ -736,7 +780,7 @@ __device__ __forceinline__ void update_body(const StepArgs &A, const double *Pi,
     }
     if (pf == PF_OK && A.floors_on && !A.floor_drift && !A.elec) {
       const double rho_fl = __ldg(A.floors + ij), u_fl = __ldg(A.floors + D.n2d + ij);
-      if (lor_n > FL_GAMMA) {
+      if (less(FL_GAMMA, lor_n)) {
         double p[NV];
 #pragma unroll
         for (int v = 0; v < NV; v++) p[v] = pn[v];

@@ -1,5 +1,5 @@
-// wide_update.cuh -- the conserved densities, the geometric source and the 1D_W
-// inversion of one zone in Wide numbers (wide_num.cuh): the formulas of
+// wide_update.cuh -- the conserved densities, the stress-energy tensor and the
+// 1D_W inversion of one zone in Wide numbers (wide_num.cuh): the formulas of
 // prim_flux (direction 0), geo_source and invert_1dw.
 #pragma once
 
@@ -9,52 +9,42 @@
 
 namespace grmhd {
 
-// U(P) (WANT_U) and the source S_nu = sqrt(-g) T^k_l Gamma^l_{nu k} of a state,
-// rounded to double; g2: its Lorentz factor squared.  conn(c): component c of the
-// connection.  T^k_l is formed row by row and its products with the
-// connection summed as they come.
-template <bool BLK, bool WANT_U, class GeoFn, class ConnFn>
-WIDE_FN void wide_source(const double P[NV], const GeoFn &geo, const ConnFn &conn, double gm1,
-                         double U[NV], double S[4], double &g2) {
+// Rows of a state, rounded to double: U(P) but its field part (WANT_U) and T^k_l.
+// g2: the Lorentz factor squared.
+template <bool BLK, bool WANT_U, class GeoFn>
+WIDE_FN void wide_tensor(const double P[NV], const GeoFn &geo, double gm1, double U[NV],
+                         double T[4][4], double &g2) {
   WideState s;
   wide_state<BLK>(P, geo, s);
   g2 = w_to_double(s.g2);
   const Wide rho = wide(P[RHO]), u = wide(P[UU]), pg = wide(gm1) * u;
   const Wide w = norm(w_sum<2>(rho, u, pg, s.bsq));
   const Wide pt = w_sum<1>(pg, w_scale(s.bsq, -1));
-  const Wide gd = wide_pos(geo(G_GDET));
   Wide bcov[4];
 #pragma unroll
   for (int n = 0; n < 4; n++) bcov[n] = norm(w_sum<1>(s.Bcov[n], s.bt * s.ucov[n])) * s.iut;
-  Wide acc[4];
 #pragma unroll
   for (int k = 0; k < 4; k++) {
     const Wide bk =
         k ? norm(w_sum<1>(wide(P[B1 - 1 + (k ? k : 1)]), s.bt * s.ucon[k])) * s.iut : s.bt;
     const Wide wu = norm(w * s.ucon[k]), nb = -norm(bk);
-    Wide T[4];
+    const Wide gd = wide_pos(geo(G_GDET));
 #pragma unroll
-    for (int l = 0; l < 4; l++)
-      T[l] = (k == l) ? w_sum<1>(wu * s.ucov[l], nb * bcov[l], pt)
-                      : w_sum<0>(wu * s.ucov[l], nb * bcov[l]);
-    if (WANT_U && k == 0) {
-      const Wide mf = rho * s.ucon[0];
-      U[RHO] = w_to_double(mf * gd);
-      U[UU] = w_to_double(w_sum<1>(T[0], mf) * gd);
-#pragma unroll
-      for (int i = 1; i < 4; i++) U[UU + i] = w_to_double(T[i] * gd);
-    }
-#pragma unroll
-    for (int l = 0; l < 4; l++) T[l] = norm(T[l]);
-#pragma unroll
-    for (int nu = 0; nu < 4; nu++) {
-      const Wide p0 = T[0] * wide(conn(0 * 10 + SY(nu, k))), p1 = T[1] * wide(conn(1 * 10 + SY(nu, k)));
-      const Wide p2 = T[2] * wide(conn(2 * 10 + SY(nu, k))), p3 = T[3] * wide(conn(3 * 10 + SY(nu, k)));
-      acc[nu] = norm(k ? w_sum<2>(acc[nu], p0, p1, p2, p3) : w_sum<1>(p0, p1, p2, p3));
+    for (int l = 0; l < 4; l++) {
+      const Wide t = (k == l) ? w_sum<1>(wu * s.ucov[l], nb * bcov[l], pt)
+                              : w_sum<0>(wu * s.ucov[l], nb * bcov[l]);
+      T[k][l] = w_to_double(t);
+      if (WANT_U && k == 0) {
+        if (l == 0) {
+          const Wide mf = rho * s.ucon[0];
+          U[RHO] = w_to_double(mf * gd);
+          U[UU] = w_to_double(w_sum<1>(t, mf) * gd);
+        } else {
+          U[UU + l] = w_to_double(t * gd);
+        }
+      }
     }
   }
-#pragma unroll
-  for (int nu = 0; nu < 4; nu++) S[nu] = w_to_double(acc[nu] * gd);
 }
 
 // FP32 forms of the 1D_W function's derivative at W = wp + d and of a Newton step

@@ -1,4 +1,5 @@
-"""U(P), the geometric source and the 1D_W inversion in Wide numbers
+"""U(P), the stress-energy tensor (by the geometric source it gives) and the 1D_W
+inversion in Wide numbers
 (csrc/wide_update.cuh), built for the host, against the oracle's FP64.
 
 Tolerances.  U and S: sums of a dozen products, each rounded to 2^-53 on the
@@ -22,12 +23,11 @@ U53 = 2.0 ** -53
 SRC = r"""
 #include "wide_update.cuh"
 using namespace grmhd;
-extern "C" void source(const double *P, const double *g, const double *c, int blk, double *U,
-                       double *S, double *g2) {
+extern "C" void tensor(const double *P, const double *g, int blk, double *U, double (*T)[4],
+                       double *g2) {
   auto geo = [&](int k) { return g[k]; };
-  auto conn = [&](int k) { return c[k]; };
-  if (blk) wide_source<true, true>(P, geo, conn, GAM - 1.0, U, S, *g2);
-  else wide_source<false, true>(P, geo, conn, GAM - 1.0, U, S, *g2);
+  if (blk) wide_tensor<true, true>(P, geo, GAM - 1.0, U, T, *g2);
+  else wide_tensor<false, true>(P, geo, GAM - 1.0, U, T, *g2);
 }
 extern "C" int invert(const double *U, const double *g, double guess, int blk, double *P,
                       double *bl) {
@@ -61,8 +61,7 @@ def _point(kind, rng):
     gi, al = q["gcon"], q["alpha"]
     g = np.array([q["gcov"][m, n] for m, n in sy] + [gi[m, n] for m, n in sy] +
                  [q["gdet"], al, 1 / al, 1 / q["gdet"], (1 + 1 / gi[0, 0]) / (1 + al)])
-    c = np.array([q["conn"][l, m, n] for l in range(4) for m, n in sy])
-    return X, q["gcov"], g, c
+    return X, q["gcov"], g, q["conn"]
 
 
 def _state(g, rng, it):
@@ -82,15 +81,16 @@ def _state(g, rng, it):
 def test_source_and_inversion(wide, kind, blk):
     rng = np.random.default_rng(3 + kind)
     for it in range(400):
-        X, gcov, g, c = _point(kind, rng)
+        X, gcov, g, conn = _point(kind, rng)
         P = _state(gcov, rng, it)
-        U, S, g2, out, bl = np.zeros(8), np.zeros(4), np.zeros(1), np.zeros(8), np.zeros(2)
-        wide.source(_p(P), _p(g), _p(c), blk, _p(U), _p(S), _p(g2))
+        U, T, g2, out, bl = np.zeros(8), np.zeros((4, 4)), np.zeros(1), np.zeros(8), np.zeros(2)
+        wide.tensor(_p(P), _p(g), blk, _p(U), _p(T), _p(g2))
+        S = g[20] * np.einsum("kl,lnk->n", T, conn)
         Uo, So = oracle.prim_to_flux(kind, 0.9375, 0.3, X, GAM, P, 0), oracle.source_at(kind, 0.9375, 0.3, X, GAM, P)
         scale = np.abs(Uo[:5]).max()
         assert np.abs(U[:5] - Uo[:5]).max() <= 1e-12 * scale
         assert abs(U[0] - Uo[0]) <= 64 * U53 * abs(Uo[0])
-        assert np.abs(S - So[1:5]).max() <= 1e-12 * max(np.abs(c).max() * scale * np.abs(gcov).max(), 0.0)
+        assert np.abs(S - So[1:5]).max() <= 1e-12 * max(np.abs(conn).max() * scale * np.abs(gcov).max(), 0.0)
         gam2 = g2[0]
         guess = (P[0] + GAM * P[1]) * gam2 * rng.uniform(0.9, 1.1)
         assert wide.invert(_p(Uo), _p(g), ctypes.c_double(guess), blk, _p(out), _p(bl)) == 1
