@@ -303,11 +303,11 @@ PREC_DTYPE = {
     1: "mixed: FP32 reconstruction, fluid states, signal speeds, LLF fluxes; "
        "FP64 geometry, flux-CT, update, 1D_W inversion, bounds",
     3: "mixed + float-float update: FP32 reconstruction, fluid states, signal speeds, LLF "
-       "fluxes; float-float U(P), geometric source and 1D_W inversion; FP64 state, geometry, "
-       "flux divergence, flux-CT, bounds",
-    2: "float-float: reconstruction, fluid states, signal speeds, LLF fluxes, U(P), geometric "
-       "source and 1D_W inversion in pairs of FP32 words (~48 significant bits); FP64 state, "
-       "geometry, flux divergence, flux-CT, bounds",
+       "fluxes; float-float U(P) and geometric source; FP64 state, geometry, flux divergence, "
+       "flux-CT, 1D_W inversion, bounds",
+    2: "float-float: reconstruction, fluid states, signal speeds, LLF fluxes, U(P) and geometric "
+       "source in pairs of FP32 words (~48 significant bits); FP64 state, geometry, flux "
+       "divergence, flux-CT, 1D_W inversion, bounds",
 }
 
 

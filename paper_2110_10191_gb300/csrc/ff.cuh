@@ -22,6 +22,8 @@
 
 #include <cuda_runtime.h>
 
+#include "wide.cuh"
+
 namespace grmhd {
 
 struct ff {
@@ -48,12 +50,46 @@ __device__ __forceinline__ ff ff_make(float hi, float lo) {
 }
 
 // double -> float-float: the high word is x rounded to float, the low word
-// the rounded remainder (48 of the 53 bits are kept)
+// the rounded remainder (48 of the 53 bits are kept).  The conversion
+// instructions occupy the FP64 unit for 66 cycles each, which kernels with enough
+// FP32 work beside them hide.
 __device__ __forceinline__ ff ff_from(double x) {
   ff r;
   r.hi = __double2float_rn(x);
   r.lo = __double2float_rn(__dsub_rn(x, (double)r.hi));
   return r;
+}
+
+// The same on the integer pipes where both words are normal floats: the bits
+// taken apart, the remainder, 29 bits, converted as an integer (a tie may round
+// the other way, the sum of the words stays the same).
+__device__ __forceinline__ ff ff_from_bits(double x) {
+  const u64 b = w_bits(x);
+  const u32 sign = w_hi(b) & 0x80000000u;
+  const int e = (int)((w_hi(b) >> 20) & 0x7ff);
+  if ((u32)(e - 950) >= 200u) return ff_from(x);
+  const u64 m = (b & (~0ull >> 1)) + (1ull << 28);
+  const int rest = (int)(w_lo(b) << 3) >> 3;  // x - hi in units of x's last place
+  const float lo = __fmul_rn(__int2float_rn(rest), __int_as_float((e - 948) << 23));
+  ff r;
+  r.hi = __uint_as_float(((u32)(m >> 29) - (896u << 23)) | sign);
+  r.lo = __uint_as_float(__float_as_uint(lo) ^ sign);
+  return r;
+}
+
+// a float as a double, normal values and zeros by their bits
+__device__ __forceinline__ double f_to_double(float f) {
+  const u32 u = __float_as_uint(f), m = u & 0x7fffffffu;
+  if (m != 0u && m - 0x800000u >= 0x7f000000u) return (double)f;  // subnormal, infinite, NaN
+  const u32 hi = (m ? (m >> 3) + (896u << 20) : 0u) | (u & 0x80000000u);
+  return w_double((u64)hi << 32 | (u64)(u << 29));
+}
+
+// d 2^k for a result in the normal range
+__device__ __forceinline__ double d_scale(double d, int k) {
+  const u64 b = w_bits(d);
+  const u32 f = (w_hi(b) >> 20) & 0x7ffu;
+  return (f == 0u || f == 0x7ffu) ? d : w_double(b + ((u64)(s64)k << 52));
 }
 
 __device__ __forceinline__ ff ff_f(float x) {
@@ -63,7 +99,11 @@ __device__ __forceinline__ ff ff_f(float x) {
   return r;
 }
 
+// float-float -> double, by the conversion instructions and by the bits
 __device__ __forceinline__ double ff_to(ff a) { return __dadd_rn((double)a.hi, (double)a.lo); }
+__device__ __forceinline__ double ff_to_bits(ff a) {
+  return __dadd_rn(f_to_double(a.hi), f_to_double(a.lo));
+}
 
 __device__ __forceinline__ ff ff_neg(ff a) {
   ff r;
@@ -119,7 +159,6 @@ __device__ __forceinline__ ff ff_sqr(ff a) {
 }
 
 // a b + c
-__device__ __forceinline__ ff ff_fma(ff a, ff b, ff c) { return ff_add(ff_mul(a, b), c); }
 
 // 1/a: FP32 seed r0 (the hardware approximation, within about an ulp of
 // 1/hi; a is never near the float underflow in these bodies, which work in

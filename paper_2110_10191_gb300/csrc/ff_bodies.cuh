@@ -1,13 +1,13 @@
-// ff_bodies.cuh -- per-thread bodies of the float-float mode
-// (GRMHD_PREC_FF): the reconstruction, the fluid states, the signal speeds,
-// the local Lax-Friedrichs flux, U(P), the geometric source and the 1D_W
-// inversion in float-float arithmetic (ff.cuh, about 48 significant bits) on
-// the FP32 pipe; the state, the fluxes, the flux divergence, the flux-CT and
-// the bounds stay FP64.  Same formulas as the FP64 bodies (grmhd_dev.cuh),
-// with the energy flux and energy density formed without the rest-mass
-// cancellation as in the FP32 bodies (grmhd_f32.cuh), since the 5 bits the
-// float pair lacks would otherwise be lost 1e3-fold at rho >> u, and with
-// every zone or face computed in units scaled by its density (FFScale).
+// ff_bodies.cuh -- per-thread bodies of the float-float modes: the flux stage of
+// GRMHD_PREC_FF (reconstruction, fluid states, signal speeds, local Lax-Friedrichs
+// flux) and the source pass of the update of GRMHD_PREC_FF and
+// GRMHD_PREC_MIXED_FF (U(P), geometric source), in float-float arithmetic (ff.cuh,
+// about 48 significant bits) on the FP32 pipe; what is stored and the rest of the
+// step as in the FP64 mode.  Same formulas as the FP64 mode's, with the energy
+// flux and energy density formed without the rest-mass cancellation as in the
+// FP32 bodies (grmhd_f32.cuh), since the 5 bits the float pair lacks would
+// otherwise be lost 1e3-fold at rho >> u, and with every zone or face computed in
+// units scaled by its density (FFScale).
 //
 // Data: the stage input split once per stage into high and low float words
 // ([2][8][ntot]: all high words, then all low words), the face values in the
@@ -41,8 +41,9 @@ __device__ __forceinline__ void ff_store(float *hi, long long lo_off, long long 
 // (1e-38..3e38) cuts into floor-density atmospheres, where products such as
 // (Q.B)^2 fall below 1e-38.
 struct FFScale {
-  float is, irs;   // 1/s, 1/sqrt(s): into the scaled units
-  double s, rs;    // s, sqrt(s): back, applied in FP64
+  float is, irs;  // 1/s, 1/sqrt(s): into the scaled units
+  double s, rs;   // s, sqrt(s): back, applied in FP64
+  int m;          // sqrt(s) = 2^m: back, on a double's exponent (d_scale)
 };
 
 __device__ __forceinline__ FFScale ff_scale_for(float rho) {
@@ -56,6 +57,7 @@ __device__ __forceinline__ FFScale ff_scale_for(float rho) {
   c.irs = ldexpf(1.0f, -m);
   c.s = ldexp(1.0, 2 * m);
   c.rs = ldexp(1.0, m);
+  c.m = m;
   return c;
 }
 
@@ -80,7 +82,7 @@ __device__ __forceinline__ void to_ff_body(const double *__restrict__ src, float
     v.hi = (x > 0.0) ? 3.4028234663852886e38f : -3.4028234663852886e38f;
     v.lo = 0.0f;
   } else {
-    v = ff_from(x);
+    v = ff_from_bits(x);
   }
   dst[t] = v.hi;
   dst[n + t] = v.lo;
@@ -366,13 +368,14 @@ __device__ __forceinline__ void face_ff_body(const StepArgs &A, const float *__r
 }
 
 // ---------------------------------------------------------------------------
-// Update: U(P), the geometric source and the 1D_W inversion in float-float
+// The update's source pass in float-float
 // ---------------------------------------------------------------------------
-// sqrt(-g)-weighted conserved densities of a state (prim_flux with dir 0),
+// sqrt(-g)-weighted conserved densities of a state (prim_flux with dir 0) but
+// the field's,
 // the energy density without the rest-mass cancellation:
 // T^t_t + rho u^t = rho u^t (1 + u_t) + (w - rho) u^t u_t - b^t b_t + p_t
 __device__ __forceinline__ void prim_cons_ff(const ff P[NV], const FStateFF &s, const GeoFF &G, ff gm1,
-                                             ff U[NV]) {
+                                             ff U[B1]) {
   const ff pg = ff_mul(P[UU], gm1);
   const ff w = ff_add(ff_add(P[RHO], P[UU]), ff_add(pg, s.bsq));
   const ff pt = ff_add(pg, ff_ldexp(s.bsq, 0.5f));
@@ -385,9 +388,6 @@ __device__ __forceinline__ void prim_cons_ff(const ff P[NV], const FStateFF &s, 
   U[UU] = ff_mul(G.gdet, en);
 #pragma unroll
   for (int i = 1; i < 4; i++) U[UU + i] = ff_mul(G.gdet, ff_sub(ff_mul(wu, s.ucov[i]), ff_mul(bt, s.bcov[i])));
-#pragma unroll
-  for (int i = 1; i < 4; i++)
-    U[B1 + i - 1] = ff_mul(G.gdet, ff_sub(ff_mul(s.bcon[i], ut), ff_mul(bt, s.ucon[i])));
 }
 
 // S_nu = sqrt(-g) T^k_l Gamma^l_{nu k} (geo_source) from the split connection
@@ -417,263 +417,51 @@ __device__ __forceinline__ void geo_source_ff(const ff P[NV], const FStateFF &s,
   }
 }
 
-// 1D_W inversion (invert_1dw) in float-float: the same iteration rule, the
-// same cancellation-free Q'.n and spatial inverse metric; the decisions are
-// taken on float-float values against the same constants (split into float
-// words: 1 - 1e-10 = 0x3f800000 + 0xaedbe700, 1e-8 = 0x322bcc77 + 0x248c230e).
-__device__ __forceinline__ int invert_1dw_ff(const ff U[NV], const GeoFF &G, ff gam, ff igam, ff gf,
-                                             const ff Pg[NV], ff P[NV], ff &bsq_out, ff &lorentz_out) {
-  const ff vsq_max = {__int_as_float(0x3f800000), __int_as_float((int)0xaedbe700u)};
-  const ff tol = {__int_as_float(0x322bcc77), __int_as_float(0x248c230e)};
-  const ff z = ff_f(0.0f);
-#pragma unroll
-  for (int v = 0; v < NV; v++) P[v] = Pg[v];
-  const ff igd = G.igdet, al = G.alpha;
-  P[B1] = ff_mul(U[B1], igd);
-  P[B2] = ff_mul(U[B2], igd);
-  P[B3] = ff_mul(U[B3], igd);
-  const ff aig = ff_mul(al, igd);
-  const ff D = ff_mul(U[RHO], aig);
-  if (!(D.hi > 0.0f)) return PF_D;
-  const ff n1 = ff_mul(al, P[B1]), n2 = ff_mul(al, P[B2]), n3 = ff_mul(al, P[B3]);
-  const ff Q1 = ff_mul(aig, U[U1]), Q2 = ff_mul(aig, U[U2]), Q3 = ff_mul(aig, U[U3]);
-  const ff c1 = G.gcon[SY(0, 1)], c2 = G.gcon[SY(0, 2)], c3 = G.gcon[SY(0, 3)];
-  const ff Qpn = ff_sub(ff_mul(ff_sub(U[UU], ff_mul(G.omalpha, U[RHO])), igd),
-                        ff_mul(al, dot3(Q1, c1, Q2, c2, Q3, c3)));
-  const ff mig00 = ff_sqr(al);  // -1/g^tt
-  const ff h11 = ff_add(G.gcon[SY(1, 1)], ff_mul(ff_sqr(c1), mig00));
-  const ff h12 = ff_add(G.gcon[SY(1, 2)], ff_mul(ff_mul(c1, c2), mig00));
-  const ff h13 = ff_add(G.gcon[SY(1, 3)], ff_mul(ff_mul(c1, c3), mig00));
-  const ff h22 = ff_add(G.gcon[SY(2, 2)], ff_mul(ff_sqr(c2), mig00));
-  const ff h23 = ff_add(G.gcon[SY(2, 3)], ff_mul(ff_mul(c2, c3), mig00));
-  const ff h33 = ff_add(G.gcon[SY(3, 3)], ff_mul(ff_sqr(c3), mig00));
-  const ff Qt1 = dot3(h11, Q1, h12, Q2, h13, Q3);
-  const ff Qt2 = dot3(h12, Q1, h22, Q2, h23, Q3);
-  const ff Qt3 = dot3(h13, Q1, h23, Q2, h33, Q3);
-  const ff Qtsq = dot3(Qt1, Q1, Qt2, Q2, Qt3, Q3);
-  const ff QdB = dot3(Q1, n1, Q2, n2, Q3, n3);
-  const ff Bsq = dot3(n1, dot3(G.gcov[SY(1, 1)], n1, G.gcov[SY(1, 2)], n2, G.gcov[SY(1, 3)], n3), n2,
-                      dot3(G.gcov[SY(1, 2)], n1, G.gcov[SY(2, 2)], n2, G.gcov[SY(2, 3)], n3), n3,
-                      dot3(G.gcov[SY(1, 3)], n1, G.gcov[SY(2, 3)], n2, G.gcov[SY(3, 3)], n3));
-  // guess
-  const ff g1 = Pg[U1], g2 = Pg[U2], g3 = Pg[U3];
-  const ff qsq = dot3(g1, dot3(G.gcov[SY(1, 1)], g1, G.gcov[SY(1, 2)], g2, G.gcov[SY(1, 3)], g3), g2,
-                      dot3(G.gcov[SY(1, 2)], g1, G.gcov[SY(2, 2)], g2, G.gcov[SY(2, 3)], g3), g3,
-                      dot3(G.gcov[SY(1, 3)], g1, G.gcov[SY(2, 3)], g2, G.gcov[SY(3, 3)], g3));
-  ff Wp = ff_sub(ff_mul(ff_add(Pg[RHO], ff_mul(gam, Pg[UU])), ff_add_f(qsq, 1.0f)), D);
-  if (Wp.hi < 0.0f) Wp = z;
-  int converged = 0, extra = 0, invalid = 0, have_hi = 0;
-  ff lo = z, hi = z;
-  for (int it = 0; it < INV_MAXIT + INV_EXTRA; it++) {
-    const ff W = ff_add(Wp, D);
-    const ff W2 = ff_sqr(W);
-    const ff BW = ff_add(Bsq, W);
-    const ff ix = ff_rcp(ff_mul(BW, W));  // 1/W = BW ix, 1/(B^2+W) = W ix
-    const ff a = ff_mul(W, ix);           // 1/(B^2 + W)
-    const ff qx = ff_mul(QdB, ix);        // Q.B / (W (B^2 + W))
-    // v^2 = Qt^2/(B^2+W)^2 + (Q.B)^2 (B^2 + 2W)/(W^2 (B^2+W)^2), each factor in range
-    ff vsq = ff_add(ff_mul(Qtsq, ff_sqr(a)), ff_mul(ff_mul(qx, ff_add(Bsq, ff_ldexp(W, 2.0f))), qx));
-    invalid = 0;
-    if (ff_gt(vsq, vsq_max)) {
-      lo = ff_max(lo, Wp);
-      Wp = have_hi ? ff_ldexp(ff_add(lo, hi), 0.5f) : ff_add(Wp, W);
-      invalid = 1;
-      if (converged || it + 1 >= INV_MAXIT) break;
-      continue;
-    }
-    if (vsq.hi < 0.0f) vsq = z;
-    const ff omv = ff_add_f(ff_neg(vsq), 1.0f);
-    const ff rsq = ff_rsqrt(omv);  // 1/sqrt(1 - v^2)
-    const ff sq = ff_mul(omv, rsq);
-    const ff wmr = ff_sub(ff_mul(Wp, omv), ff_mul(ff_mul(ff_mul(D, vsq), sq), ff_rcp(ff_add_f(sq, 1.0f))));
-    const ff iW = ff_mul(BW, ix);
-    const ff qw0 = ff_mul(QdB, iW);
-    const ff f = ff_sub(ff_add(ff_add(Qpn, Wp), ff_mul(ff_ldexp(ff_add_f(vsq, 1.0f), 0.5f), Bsq)),
-                        ff_add(ff_mul(gf, wmr), ff_ldexp(ff_sqr(qw0), 0.5f)));
-    if (f.hi > 0.0f) {
-      hi = have_hi ? ff_min(hi, Wp) : Wp;
-      have_hi = 1;
-    } else {
-      lo = ff_max(lo, Wp);
-    }
-    const ff poly = ff_add(ff_mul_f(ff_add(W2, ff_mul(W, Bsq)), 3.0f), ff_sqr(Bsq));
-    // dv^2/dW = -2 (Qt^2 W^3 + (Q.B)^2 poly) / (W (B^2+W))^3, as
-    // -2 [Qt^2 a^3 + qx^2 (poly ix)]
-    const ff dv = ff_mul_f(ff_add(ff_mul(ff_mul(Qtsq, a), ff_sqr(a)),
-                                  ff_mul(ff_sqr(qx), ff_mul(poly, ix))), -2.0f);
-    const ff dpdW = ff_mul(gf, ff_add(omv, ff_mul(dv, ff_sub(ff_mul(ff_ldexp(D, 0.5f), rsq), W))));
-    const ff qw = ff_mul(QdB, iW);  // Q.B / W
-    const ff df = ff_add(ff_add(ff_add_f(ff_neg(dpdW), 1.0f), ff_mul(ff_ldexp(Bsq, 0.5f), dv)),
-                         ff_mul(ff_sqr(qw), iW));
-    ff Wn = ff_sub(Wp, ff_div(f, df));
-    if (Wn.hi < 0.0f) Wn = ff_ldexp(Wp, 0.5f);
-    if (converged) {
-      Wp = Wn;
-      if (++extra >= INV_EXTRA) break;
-      continue;
-    }
-    if (!ff_gt(ff_abs(ff_sub(Wn, Wp)), ff_mul(tol, ff_abs(W)))) converged = 1;
-    Wp = Wn;
-    if (!converged && it + 1 >= INV_MAXIT) break;
-  }
-  const ff W = ff_add(Wp, D);
-  if (!converged) return PF_NOCONV;
-  if (!(W.hi > 0.0f) || !isfinite(W.hi)) return PF_W;
-  const ff BW = ff_add(Bsq, W);
-  const ff ix = ff_rcp(ff_mul(BW, W));
-  const ff a = ff_mul(W, ix), qx = ff_mul(QdB, ix);
-  ff vsq = ff_add(ff_mul(Qtsq, ff_sqr(a)), ff_mul(ff_mul(qx, ff_add(Bsq, ff_ldexp(W, 2.0f))), qx));
-  if (!(vsq.hi < 1.0f || (vsq.hi == 1.0f && vsq.lo < 0.0f)) || invalid) return PF_VSQ;
-  if (vsq.hi < 0.0f) vsq = z;
-  const ff omv = ff_add_f(ff_neg(vsq), 1.0f);
-  const ff rsq = ff_rsqrt(omv);  // Lorentz factor
-  const ff sq = ff_mul(omv, rsq);
-  const ff rho = ff_mul(D, sq);
-  const ff uu = ff_mul(ff_sub(ff_mul(Wp, omv), ff_mul(ff_mul(ff_mul(D, vsq), sq), ff_rcp(ff_add_f(sq, 1.0f)))),
-                       igam);
-  if (!(rho.hi > 0.0f)) return PF_RHO;
-  if (uu.hi < 0.0f) return PF_U;
-  const ff fac = ff_mul(rsq, ff_mul(W, ix));  // gamma / (W + B^2)
-  const ff qbw = ff_mul(QdB, ff_mul(BW, ix));  // Q.B / W
-  bsq_out = ff_add(ff_mul(Bsq, omv), ff_sqr(qbw));
-  lorentz_out = rsq;
-  P[RHO] = rho;
-  P[UU] = uu;
-  P[U1] = ff_mul(fac, ff_add(Qt1, ff_mul(qbw, n1)));
-  P[U2] = ff_mul(fac, ff_add(Qt2, ff_mul(qbw, n2)));
-  P[U3] = ff_mul(fac, ff_add(Qt3, ff_mul(qbw, n3)));
-  return PF_OK;
-}
-
-// One thread per interior zone (update_body): U(P^n) (or its cache), the
-// source of P_s, the inversion in float-float; the flux divergence, the
-// conserved sum, the bounds and all stored arrays in FP64.  Every thread
-// of the block must call it (warp counters).
-// Pff (may be null): the split stage input of the flux stage, which is P_s:
-// the update reads P_s's words there instead of splitting P_s again (in the
-// predictor P_s = P_i = P^n).  Ucache holds U(P^n) as split words in P^n's scaled
-// units ([2][8][ntot] floats in the space of [8][ntot] doubles): the
-// corrector, which scales by the same P^n density, reads it back as is.
-__device__ __forceinline__ void update_ff_body(const StepArgs &A, const double *Pi,
-                                               const double *__restrict__ Ps, double *Pout,
-                                               const double *__restrict__ F1,
-                                               const double *__restrict__ F2,
-                                               const double *__restrict__ F3, int *pflag, int *fflag,
-                                               double dtfac, double *Ucache, int ucache_mode,
-                                               const float *__restrict__ Pff, long long t) {
+// source_body with U(P) and the source in float-float (one thread per zone, in
+// units scaled by the zone's density); the field's part and what is stored are
+// FP64.  Pff (may be null): the split stage input of the flux stage, which is P_s.
+// (As one pass with a float-float inversion the update took 1.06 to 1.16 ms per
+// launch on a 128^3 grid, bound by latency at 16 warps per SM; with the Wide
+// inversion as a pass of its own, 0.79 ms for both.)
+template <bool PRED>
+__device__ __forceinline__ void source_ff_body(const StepArgs &A, const double *__restrict__ Ps,
+                                               const float *__restrict__ Pff,
+                                               double *__restrict__ Ucache,
+                                               double *__restrict__ scratch, long long t) {
   const Dims &D = A.D;
-  const double dt = A.clk->dt;
-  if (!(dt > 0.0)) return;  // uniform across the grid
-  const double dtp = dtfac * dt;
-  const long long nz = n_zone(D);
-  const bool active = t < nz;
-  int pf = 0, fl = 0;
-  if (active) {
-    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
-    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
-    const long long c = zid(D, i, j, k), N = D.ntot;
-    const long long ij = (long long)j * D.s[0] + i;
-    GeoFF G;
-    load_geo_ff(A.geomff, (long long)NLOC * G_NCOMP * D.n2d, D.n2d, ij, G);
-    const ff gam = {A.gam_ff[0], A.gam_ff[1]}, gm1 = {A.gm1_ff[0], A.gm1_ff[1]};
-    const ff igam = {A.igam_ff[0], A.igam_ff[1]}, gf = {A.gf_ff[0], A.gf_ff[1]};
-    const long long clo = (long long)C_NCOMP * D.n2d;
-    ff pi[NV], Ui[NV], S[4];
-    if (Ps == Pi && Pff) {
+  if (!(A.clk->dt > 0.0) || t >= n_update(D)) return;
+  const Column q3 = column_of(t, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
+  if (!q3.active) return;
+  const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
+  const long long c = zid(D, i, j, k), N = D.ntot;
+  const long long ij = (long long)j * D.s[0] + i;
+  GeoFF G;
+  load_geo_ff(A.geomff, (long long)NLOC * G_NCOMP * D.n2d, D.n2d, ij, G);
+  const ff gm1 = {A.gm1_ff[0], A.gm1_ff[1]};
+  ff p[NV], S[4];
 #pragma unroll
-      for (int v = 0; v < NV; v++) pi[v] = ff_load(Pff, (long long)NV * N, v * N + c);
-    } else {
+  for (int v = 0; v < NV; v++)
+    p[v] = Pff ? ff_load(Pff, (long long)NV * N, v * N + c) : ff_from(__ldg(Ps + v * N + c));
+  const FFScale sc = ff_scale_for(p[RHO].hi);
+  ff_scale_prims(p, sc);
+  FStateFF s;
+  fluid_state_ff(p, G, s);
+  if (PRED) {
+    ff U[B1];
+    prim_cons_ff(p, s, G, gm1, U);
+    const double gd = __ldg(A.geom + (long long)G_GDET * D.n2d + ij);
 #pragma unroll
-      for (int v = 0; v < NV; v++) pi[v] = ff_from(Pi[v * N + c]);
-    }
-    float *Ucf = reinterpret_cast<float *>(Ucache);
-    const long long uhalf = (long long)NV * N;
-    // scaled units from P^n's density (the same in both stages, so that
-    // U(P^n) kept by the predictor is read back in the corrector's units)
-    const FFScale sc = ff_scale_for(pi[RHO].hi);
-    ff_scale_prims(pi, sc);
-    if (Ps == Pi) {
-      FStateFF si;
-      fluid_state_ff(pi, G, si);
-      prim_cons_ff(pi, si, G, gm1, Ui);
-      if (ucache_mode == 1) {
+    for (int v = 0; v < B1; v++) Ucache[v * N + c] = d_scale(ff_to_bits(U[v]), 2 * sc.m);
 #pragma unroll
-        for (int v = 0; v < NV; v++) ff_store(Ucf, uhalf, v * N + c, Ui[v]);
-      }
-      geo_source_ff(pi, si, G, A.connff, clo, D.n2d, ij, gm1, S);
-    } else {
-      if (ucache_mode == 2) {
-#pragma unroll
-        for (int v = 0; v < NV; v++) Ui[v] = ff_load(Ucf, uhalf, v * N + c);
-      } else {
-        FStateFF si;
-        fluid_state_ff(pi, G, si);
-        prim_cons_ff(pi, si, G, gm1, Ui);
-      }
-      ff ps[NV];
-      if (Pff) {  // the corrector's flux stage split P_s
-#pragma unroll
-        for (int v = 0; v < NV; v++) ps[v] = ff_load(Pff, (long long)NV * N, v * N + c);
-      } else {
-#pragma unroll
-        for (int v = 0; v < NV; v++) ps[v] = ff_from(Ps[v * N + c]);
-      }
-      ff_scale_prims(ps, sc);
-      FStateFF ss;
-      fluid_state_ff(ps, G, ss);
-      geo_source_ff(ps, ss, G, A.connff, clo, D.n2d, ij, gm1, S);
-    }
-    const double idx1 = A.idx[0], idx2 = A.idx[1], idx3 = A.idx[2];
-    const ff dtpf = ff_from(dtp);
-    // The field is updated in FP64, sqrt(-g) B (P^n) - dt' div F_B, as the
-    // FP64 update does: flux-CT's divergence-free increments then keep div B
-    // at FP64 round-off; the inversion reads the result's words.
-    const double gdd = __ldg(A.geom + (long long)G_GDET * D.n2d + ij);
-    const double igdd = __ldg(A.geom + (long long)G_IGDET * D.n2d + ij);
-    double UB[3];
-    ff Un[NV];
-#pragma unroll
-    for (int v = 0; v < NV; v++) {
-      const long long o = v * N + c;
-      const double div = (F1[o + 1] - F1[o]) * idx1 + (F2[o + D.s[0]] - F2[o]) * idx2 +
-                         (F3[o + D.n2d] - F3[o]) * idx3;
-      if (v >= B1) {
-        UB[v - B1] = gdd * Pi[o] + dtp * (0.0 - div);
-        Un[v] = ff_from(UB[v - B1] * (double)sc.irs);
-        continue;
-      }
-      ff rhs = ff_neg(ff_from(div * (double)sc.is));
-      if (v >= UU && v <= U3) rhs = ff_add(rhs, S[v - UU]);
-      Un[v] = ff_add(Ui[v], ff_mul(dtpf, rhs));
-    }
-    ff pn[NV], bsq_n = ff_f(0.0f), lor_n = ff_f(1.0f);
-    pf = invert_1dw_ff(Un, G, gam, igam, gf, pi, pn, bsq_n, lor_n);
-    double pd[NV];
-#pragma unroll
-    for (int v = 0; v < B1; v++) {
-      pd[v] = ff_to(pn[v]);
-      if (v == RHO || v == UU) pd[v] *= sc.s;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; q++) pd[B1 + q] = UB[q] * igdd;
-    if (pf == PF_OK && A.floors_on && !A.floor_drift && !A.elec) {
-      const double rho_fl = __ldg(A.floors + ij), u_fl = __ldg(A.floors + D.n2d + ij);
-      const double lor = ff_to(lor_n);
-      if (lor > FL_GAMMA) {  // the Lorentz-factor cap needs the FP64 fluid state
-        Geo Gd;
-        load_geo(A.geom, D.n2d, ij, Gd);
-        fl = apply_floors(pd, Gd, rho_fl, u_fl, A.gk);
-      } else {
-        fl = apply_floors_known(pd, rho_fl, u_fl, A.gk, ff_to(bsq_n) * sc.s);
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < NV; v++) Pout[v * N + c] = pd[v];
-    pflag[c] = pf;
-    fflag[c] = fl;
+    for (int v = B1; v < NV; v++) Ucache[v * N + c] = gd * __ldg(Ps + v * N + c);
   }
-  count_warp(active && pf != 0, &A.clk->counters[0]);
-  count_warp(active && fl != 0, &A.clk->counters[1]);
+  geo_source_ff(p, s, G, A.connff, (long long)C_NCOMP * D.n2d, D.n2d, ij, gm1, S);
+#pragma unroll
+  for (int n = 0; n < 4; n++) scratch[n * N + c] = d_scale(ff_to_bits(S[n]), 2 * sc.m);
+  // the inversion's guess W = (rho + gamma u) gamma_L^2, to FP32
+  const float lor = s.ucon[0].hi * G.alpha.hi;
+  scratch[4 * N + c] =
+      d_scale(f_to_double(fmaf(A.gam_ff[0], p[UU].hi, p[RHO].hi) * (lor * lor)), 2 * sc.m);
 }
 
 }  // namespace grmhd

@@ -61,8 +61,8 @@ struct StepArgs {
   int xlo[3], xhi[3];
   // gamma, gamma - 1 and gamma (gamma - 1) split into float words (high, low)
   // for the float-float flux stage
-  float gam_ff[2], gm1_ff[2], ggm1_ff[2], igam_ff[2], gf_ff[2];  // gf = (gamma - 1)/gamma
-  const float *geomff, *connff;  // float-float mode: split geometry and connection
+  float gam_ff[2], gm1_ff[2], ggm1_ff[2];
+  const float *geomff, *connff;  // float-float modes: split geometry and connection
   int bc[3][2];
   const double *geom;
   const double *conn;
@@ -82,9 +82,9 @@ inline void set_gas_constants(StepArgs &A) {
 
 // the float-float words of the adiabatic-index constants
 inline void set_ff_constants(StepArgs &A) {
-  const double v[5] = {A.gam, A.gam - 1.0, A.gam * (A.gam - 1.0), A.igam, (A.gam - 1.0) / A.gam};
-  float *o[5] = {A.gam_ff, A.gm1_ff, A.ggm1_ff, A.igam_ff, A.gf_ff};
-  for (int q = 0; q < 5; q++) {
+  const double v[3] = {A.gam, A.gam - 1.0, A.gam * (A.gam - 1.0)};
+  float *o[3] = {A.gam_ff, A.gm1_ff, A.ggm1_ff};
+  for (int q = 0; q < 3; q++) {
     o[q][0] = (float)v[q];
     o[q][1] = (float)(v[q] - (double)o[q][0]);
   }

@@ -173,20 +173,19 @@ __global__ void __maxnreg__(96) kp_source(BView V) {
   source_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Uc, it.Lf, block_tid(V, g));
 }
 
+// the source pass of the float-float modes
+template <bool PRED>
+__global__ void __maxnreg__(96) kp_source_ff(BView V) {
+  const int g = block_grid(V);
+  const StageItem &it = V.items[g];
+  source_ff_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Pff, it.Uc, it.Lf, block_tid(V, g));
+}
+
 __global__ void __maxnreg__(80) kp_invert(BView V, int in, double dtfac) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   invert_body(it.A, it.F[0], it.F[1], it.F[2], it.Uc, it.Lf, dtfac, it.P, arr(it, 1 - in), it.pflag,
               it.fflag, block_tid(V, g));
-}
-
-// at most 128 registers: 4 blocks of 128 threads per SM; the spill it costs
-// is cheaper than the occupancy it buys for this latency-bound FP32 code
-__global__ void __maxnreg__(128) kp_update_ff(BView V, int in, double dtfac, int ucache_mode) {
-  const int g = block_grid(V);
-  const StageItem &it = V.items[g];
-  update_ff_body(it.A, it.P, arr(it, in), arr(it, 1 - in), it.F[0], it.F[1], it.F[2], it.pflag,
-                 it.fflag, dtfac, it.Uc, ucache_mode, it.Pff, block_tid(V, g));
 }
 
 template <int DIR>
@@ -321,11 +320,9 @@ int upload_tables(Plan &p) {
 void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rwalk,
                  long long c[PC_N]) {
   const int fl = flat3;
-  // the flux stage: FP64, FP32 (mixed, and mixed with the float-float
-  // update) or float-float; the update: FP64 or float-float
+  // the flux stage: FP64, FP32 or float-float
   const bool f64 = prec == GRMHD_PREC_FP64, fx = prec == GRMHD_PREC_FF;
   const bool mx = prec == GRMHD_PREC_MIXED || prec == GRMHD_PREC_MIXED_FF;
-  const bool ux = prec == GRMHD_PREC_FF || prec == GRMHD_PREC_MIXED_FF;
   c[PC_BX1] = n_bounds_x1(D);
   c[PC_BX2] = n_bounds_x2(D);
   c[PC_BX3] = n_bounds_x3(D);
@@ -346,8 +343,10 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_FIX] = n_fix(D);
   c[PC_EDGE] = n_edge(D);
   c[PC_ZONE] = n_zone(D);
-  c[PC_UPD64] = ux ? 0 : n_update(D);
-  c[PC_UPDX] = ux ? n_zone(D) : 0;
+  const bool ux = fx || prec == GRMHD_PREC_MIXED_FF;  // the source pass in float-float
+  c[PC_SRC64] = ux ? 0 : n_update(D);
+  c[PC_SRCX] = ux ? n_update(D) : 0;
+  c[PC_UPD] = n_update(D);
   c[PC_FLOORD] = (drift && !elec) ? n_zone(D) : 0;
   for (int d = 0; d < 3; d++) c[PC_EFACE0 + d] = elec ? n_face(D, d, fl) : 0;
   c[PC_EREC01] = elec ? n_recon(D, fl) : 0;
@@ -533,16 +532,19 @@ int plan_fix_ct(const Plan &p, cudaStream_t st, PlanHook *h) {
 
 int plan_update_only(const Plan &p, int in, double dtfac, int ucache_mode, cudaStream_t st,
                      PlanHook *h) {
-  int nl = launch(p, PC_UPD64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
+  int nl = launch(p, PC_SRCX, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
+    if (in == 0)
+      kp_source_ff<true><<<nb, bs, 0, st>>>(V);
+    else
+      kp_source_ff<false><<<nb, bs, 0, st>>>(V);
+  });
+  nl += launch(p, PC_SRC64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
     if (in == 0)
       kp_source<true><<<nb, bs, 0, st>>>(V);
     else  // the predictor before it kept U(P^n)
       kp_source<false><<<nb, bs, 0, st>>>(V);
   });
-  nl += launch(p, PC_UPD64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, in, dtfac); });
-  nl += launch(p, PC_UPDX, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
-    kp_update_ff<<<nb, bs, 0, st>>>(V, in, dtfac, ucache_mode);
-  });
+  nl += launch(p, PC_UPD, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, in, dtfac); });
   nl += launch(p, PC_FLOORD, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
     kp_floor_drift<<<nb, bs, 0, st>>>(V, 1 - in);
   });
@@ -638,10 +640,10 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
     int which;  // what one pass launches
   };
   const Group groups[] = {{PC_RECON0, 0},   {PC_RECON1, 6},  {PC_RECON2, 1},   {PC_FACE0, 2},
-                          {PC_FACE1, 3},    {PC_FACE2, 4},   {PC_UPD64, 5},
+                          {PC_FACE1, 3},    {PC_FACE2, 4},   {PC_UPD, 5},
                           {PC_FACE0F, 8},   {PC_FACE1F, 9},  {PC_FACE2F, 10},  {PC_RECON01X, 11},
                           {PC_RECON2X, 12}, {PC_FACE0X, 13}, {PC_FACE1X, 14},  {PC_FACE2X, 15},
-                          {PC_UPDX, 16}};
+                          {PC_SRC64, 16},   {PC_SRCX, 17}};
   auto pass = [&](int which) {
     auto L = [&](int cls, auto &&body) { launch(p, cls, 0, nullptr, body); };
     switch (which) {
@@ -663,12 +665,10 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
       case 4:
         L(PC_FACE2, [&](unsigned nb, unsigned bs, BView V) { kp_face<2><<<nb, bs, 0, st>>>(V, 0); });
         break;
-      case 5:  // predictor-like update without keeping U(P^n)
-        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_source<true><<<nb, bs, 0, st>>>(V); });
-        L(PC_UPD64, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, 0, 0.5); });
-        break;
-      case 16:
-        L(PC_UPDX, [&](unsigned nb, unsigned bs, BView V) { kp_update_ff<<<nb, bs, 0, st>>>(V, 0, 0.5, 0); });
+      case 5:  // the inversion, of what the source pass before it leaves
+        L(PC_SRC64, [&](unsigned nb, unsigned bs, BView V) { kp_source<true><<<nb, bs, 0, st>>>(V); });
+        L(PC_SRCX, [&](unsigned nb, unsigned bs, BView V) { kp_source_ff<true><<<nb, bs, 0, st>>>(V); });
+        L(PC_UPD, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, 0, 0.5); });
         break;
       case 8:
         L(PC_FACE0F, [&](unsigned nb, unsigned bs, BView V) { kp_flux_f32<0><<<nb, bs, 0, st>>>(V); });
@@ -694,6 +694,12 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
         break;
       case 15:
         L(PC_FACE2X, [&](unsigned nb, unsigned bs, BView V) { kp_face_ff<2><<<nb, bs, 0, st>>>(V); });
+        break;
+      case 16:
+        L(PC_SRC64, [&](unsigned nb, unsigned bs, BView V) { kp_source<true><<<nb, bs, 0, st>>>(V); });
+        break;
+      case 17:
+        L(PC_SRCX, [&](unsigned nb, unsigned bs, BView V) { kp_source_ff<true><<<nb, bs, 0, st>>>(V); });
         break;
     }
   };

@@ -60,8 +60,9 @@ enum {
   PC_FIX,
   PC_EDGE,   // EMFs and CT
   PC_ZONE,   // fixup (every grid)
-  PC_UPD64,  // FP64 update (FP64 and mixed-precision grids)
-  PC_UPDX,   // float-float update (float-float and mixed + float-float grids)
+  PC_SRC64,  // the update's source pass (FP64 and mixed-precision grids)
+  PC_SRCX,   // in float-float (float-float and mixed + float-float grids)
+  PC_UPD,    // its inversion pass (every grid)
   PC_FLOORD, // drift-frame bounds (grids with bounds in the drift frame, no electrons)
   PC_EREC01, // electron entropy reconstruction along X1, X2 (grids with electrons)
   PC_EREC2,  // along X3

@@ -18,7 +18,7 @@ struct grmhd_sim {
   double *P, *Ph, *F[3], *emf, *Lf, *Rf, *Uc;
   double *geom, *conn, *floors;
   float *Pf, *geomf;    // FP32 copies (mixed precision only)
-  float *Pff, *geomff, *connff;  // split float-float copies (float-float mode only)
+  float *Pff, *geomff, *connff;  // split float-float copies (float-float modes only)
   // electrons only: entropies of the stage arrays, their fluxes, U_rho(P^n),
   // the faces' signal speeds
   double *K, *Kh, *FK[3], *Uek, *elec_w, *KLf, *KRf;
