@@ -94,7 +94,7 @@ static void free_all(grmhd_sim *s) {
   plan_free(s->plan);
   double *d[] = {s->P,      s->Ph,    s->F[0], s->F[1], s->F[2],  s->emf,
                  s->Lf,     s->Rf,    s->Uc,   s->geom, s->conn,  s->floors,
-                 s->K,      s->Kh,    s->FK[0], s->FK[1], s->FK[2], s->Uek,
+                 s->K,      s->Kh,    s->FK[0], s->FK[1], s->FK[2],
                  s->elec_w, s->KLf, s->KRf};
   for (double *p : d)
     if (p) cudaFree(p);
@@ -182,8 +182,8 @@ extern "C" int grmhd_footprint(const grmhd_grid *grid, const grmhd_metric *metri
     b += 2 * sizeof(float) * NV * tot;
   if (pr == GRMHD_PREC_FF || pr == GRMHD_PREC_MIXED_FF)  // split geometry and connection
     b += 2 * sizeof(float) * (NLOC * G_NCOMP + C_NCOMP) * n2d;
-  if (params->electrons.model)  // K, Kh, FK[3], KLf, KRf (2 each), Uek, elec_w (6)
-    b += sizeof(double) * 21 * tot;
+  if (params->electrons.model)  // K, Kh, FK[3], KLf, KRf (2 each), elec_w (6)
+    b += sizeof(double) * 20 * tot;
   b += (size_t)plan_bytes(D, flat3_of(D, params), params->precision,
                          params->floors_on && params->floor_frame == GRMHD_FLOOR_DRIFT,
                          params->electrons.model != GRMHD_ELEC_OFF);
@@ -257,7 +257,6 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
          cudaMalloc(&s->FK[0], kb) == cudaSuccess && cudaMalloc(&s->FK[1], kb) == cudaSuccess &&
          cudaMalloc(&s->FK[2], kb) == cudaSuccess && cudaMalloc(&s->KLf, kb) == cudaSuccess &&
          cudaMalloc(&s->KRf, kb) == cudaSuccess &&
-         cudaMalloc(&s->Uek, sizeof(double) * (size_t)tot) == cudaSuccess &&
          cudaMalloc(&s->elec_w, sizeof(double) * 6 * (size_t)tot) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -366,7 +365,6 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
   it.K = s->K;
   it.Kh = s->Kh;
   for (int d = 0; d < 3; d++) it.FK[d] = s->FK[d];
-  it.Uek = s->Uek;
   it.KLf = s->KLf;
   it.KRf = s->KRf;
   rc = plan_build(s->plan, &it, 1);

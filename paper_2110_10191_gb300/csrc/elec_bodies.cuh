@@ -165,9 +165,9 @@ __device__ __forceinline__ void elec_flux_body(const StepArgs &A, const double *
 // unbounded state), the heating kappa_e = kappa_e,adv + f_e (gamma_e - 1) /
 // (gamma - 1) rho_s^(gamma - gamma_e) ((gamma - 1) u/rho^gamma -
 // kappa_tot,adv) with f_e from the source state P_s, the fluid's bounds and
-// the closing steps.  U_rho(P_i) is formed in the predictor (P_i = P^n is
-// intact there) and kept in Uek for the corrector, whose output overwrote
-// P^n.  Every thread of the block must call it (warp counters).
+// the closing steps.  U_rho(P_i) is what the update keeps of U(P^n); scratch holds
+// b^2 of P_s, and b^2 and the Lorentz factor of the unbounded state.  Every thread
+// of the block must call it (warp counters).
 __device__ __forceinline__ void elec_post_body(const StepArgs &A, const double *Ps, double *Pout,
                                                const double *__restrict__ F1,
                                                const double *__restrict__ F2,
@@ -175,34 +175,24 @@ __device__ __forceinline__ void elec_post_body(const StepArgs &A, const double *
                                                const double *__restrict__ FK1,
                                                const double *__restrict__ FK2,
                                                const double *__restrict__ FK3, const double *Ki,
-                                               const double *Ks, double *Kout, double *Uek,
+                                               const double *Ks, double *Kout,
+                                               const double *__restrict__ Ucache,
+                                               const double *__restrict__ scratch,
                                                const int *__restrict__ pflag, int *fflag,
-                                               double dtfac, int stage, long long t) {
+                                               double dtfac, long long t) {
   const Dims &D = A.D;
   const double dt = A.clk->dt;
   if (!(dt > 0.0)) return;
   const double dtp = dtfac * dt;
-  const bool active = t < n_zone(D);
+  const bool in = t < n_update(D);
+  const Column q3 = column_of(in ? t : t & 31, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
+  const bool active = in && q3.active;
   int ff = 0;
   if (active) {
-    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
     const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
-    Geo G;
-    load_geo(A.geom, D.n2d, ij, G);
-    double ps[NV];
-#pragma unroll
-    for (int v = 0; v < NV; v++) ps[v] = Ps[v * N + c];
-    FState ss;
-    fluid_state(ps, G, ss);
-    double Uri;
-    if (stage == 0) {  // P_s = P_i = P^n
-      Uri = G.gdet * (ps[RHO] * ss.ucon[0]);
-      Uek[c] = Uri;
-    } else {
-      Uri = Uek[c];
-    }
+    const double rho_s = Ps[RHO * N + c], u_s = Ps[UU * N + c], Uri = Ucache[RHO * N + c];
     const double idx1 = A.idx[0], idx2 = A.idx[1], idx3 = A.idx[2];
     const long long o = RHO * N + c;
     const double divr = (F1[o + 1] - F1[o]) * idx1 + (F2[o + D.s[0]] - F2[o]) * idx2 +
@@ -220,16 +210,15 @@ __device__ __forceinline__ void elec_post_body(const StepArgs &A, const double *
       double pn[NV];
 #pragma unroll
       for (int v = 0; v < NV; v++) pn[v] = Pout[v * N + c];
-      const double ls = log(ps[RHO]), ln = log(pn[RHO]);
-      const double fel = elec_fraction(A, ps[RHO], ls, ps[UU], Ks[N + c], ss.bsq);
+      const double ls = log(rho_s), ln = log(pn[RHO]);
+      const double fel = elec_fraction(A, rho_s, ls, u_s, Ks[N + c], scratch[SCR_BSQ_S * N + c]);
       const double ktot_new = (A.gam - 1.0) * pn[UU] / exp(A.gam * ln);
       kn[1] = kn[1] + fel * (A.game - 1.0) / (A.gam - 1.0) * exp((A.gam - A.game) * ls) *
                           (ktot_new - kn[0]);
       const double rho_n = pn[RHO];
       if (A.floors_on) {
-        const double rho_fl = __ldg(A.floors + ij), u_fl = __ldg(A.floors + D.n2d + ij);
-        ff = A.floor_drift ? apply_floors_drift(pn, G, rho_fl, u_fl, A.gk)
-                           : apply_floors(pn, G, rho_fl, u_fl, A.gk);
+        const double bsq = scratch[SCR_BSQ * N + c], lor = scratch[SCR_LORENTZ * N + c];
+        ff = A.floor_drift ? floors_drift(A, ij, pn, bsq, lor) : floors_fluid(A, ij, pn, bsq, lor);
       }
       ff |= elec_close(A, pn, kn, (pn[RHO] == rho_n) ? ln : log(pn[RHO]));
 #pragma unroll

@@ -460,8 +460,9 @@ __device__ __forceinline__ void source_ff_body(const StepArgs &A, const double *
   for (int n = 0; n < 4; n++) scratch[n * N + c] = d_scale(ff_to_bits(S[n]), 2 * sc.m);
   // the inversion's guess W = (rho + gamma u) gamma_L^2, to FP32
   const float lor = s.ucon[0].hi * G.alpha.hi;
-  scratch[4 * N + c] =
+  scratch[SCR_GUESS * N + c] =
       d_scale(f_to_double(fmaf(A.gam_ff[0], p[UU].hi, p[RHO].hi) * (lor * lor)), 2 * sc.m);
+  if (A.elec) scratch[SCR_BSQ_S * N + c] = d_scale(ff_to_bits(s.bsq), 2 * sc.m);
 }
 
 }  // namespace grmhd

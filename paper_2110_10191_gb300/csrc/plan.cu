@@ -203,12 +203,12 @@ __global__ void kp_elec_flux(BView V) {
 }
 
 // stage in: P_s = arr(in), output arr(1 - in); kappa_i is always K (of P^n)
-__global__ void kp_elec_post(BView V, int in, double dtfac) {
+__global__ void __maxnreg__(96) kp_elec_post(BView V, int in, double dtfac) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   elec_post_body(it.A, arr(it, in), arr(it, 1 - in), it.F[0], it.F[1], it.F[2], it.FK[0],
-                 it.FK[1], it.FK[2], it.K, karr(it, in), karr(it, 1 - in), it.Uek, it.pflag,
-                 it.fflag, dtfac, in, block_tid(V, g));
+                 it.FK[1], it.FK[2], it.K, karr(it, in), karr(it, 1 - in), it.Uc, it.Lf, it.pflag,
+                 it.fflag, dtfac, block_tid(V, g));
 }
 
 __global__ void kp_elec_fix(BView V, int out) {
@@ -217,10 +217,10 @@ __global__ void kp_elec_fix(BView V, int out) {
   elec_fix_body(it.A, arr(it, out), karr(it, out), it.pflag, it.fflag, block_tid(V, g));
 }
 
-__global__ void kp_floor_drift(BView V, int out) {
+__global__ void __maxnreg__(128) kp_floor_drift(BView V, int out) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  floor_drift_body(it.A, arr(it, out), it.pflag, it.fflag, block_tid(V, g));
+  floor_drift_body(it.A, arr(it, out), it.Lf, it.pflag, it.fflag, block_tid(V, g));
 }
 
 __global__ void kp_fixup(BView V, int out) {
@@ -347,11 +347,11 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_SRC64] = ux ? 0 : n_update(D);
   c[PC_SRCX] = ux ? n_update(D) : 0;
   c[PC_UPD] = n_update(D);
-  c[PC_FLOORD] = (drift && !elec) ? n_zone(D) : 0;
+  c[PC_FLOORD] = (drift && !elec) ? n_update(D) : 0;
   for (int d = 0; d < 3; d++) c[PC_EFACE0 + d] = elec ? n_face(D, d, fl) : 0;
   c[PC_EREC01] = elec ? n_recon(D, fl) : 0;
   c[PC_EREC2] = (elec && !fl) ? n_recon(D, 0) : 0;
-  c[PC_EZONE] = elec ? n_zone(D) : 0;
+  c[PC_EZONE] = elec ? n_update(D) : 0;
 }
 
 long long plan_bytes(const Dims &D, int flat3, int prec, int drift, int elec) {

@@ -28,7 +28,7 @@ struct StageItem {
   int prec;            // GRMHD_PREC_*: the flux stage's arithmetic
   // electrons (A.elec): (kappa_tot, kappa_e) of the stage arrays ([2][ntot]
   // each, with P and Ph), their fluxes, and U_rho(P^n) kept by the predictor
-  double *K, *Kh, *FK[3], *Uek;
+  double *K, *Kh, *FK[3];
   double *KLf, *KRf;  // their face values along the current direction
 };
 

@@ -641,11 +641,11 @@ __device__ __forceinline__ double flux_div(const StepArgs &A, const double *__re
          (F3[o + A.D.n2d] - F3[o]) * A.idx[2];
 }
 
-// U(P), the stress-energy tensor and the Lorentz factor squared of a state in
-// FP64: metrics that couple X2.
+// U(P), the stress-energy tensor, the Lorentz factor squared and b^2 of a state
+// in FP64: metrics that couple X2.
 static __device__ __noinline__ void tensor_fp64(const StepArgs &A, const double *__restrict__ Ps,
                                                 long long c, long long ij, double U[NV],
-                                                double T[4][4], double &g2) {
+                                                double T[4][4], double &g2, double &bsq) {
   Geo G;
   load_geo(A.geom, A.D.n2d, ij, G);
   double p[NV];
@@ -661,14 +661,66 @@ static __device__ __noinline__ void tensor_fp64(const StepArgs &A, const double 
   }
   const double g = s.ucon[0] * G.alpha;
   g2 = g * g;
+  bsq = s.bsq;
 }
 
 // The bounds of a zone that needs the Lorentz-factor cap.
-static __device__ __noinline__ int floors_capped(const StepArgs &A, long long ij, double rho_fl,
-                                                 double u_fl, double P[NV]) {
+static __device__ __noinline__ int floors_capped(const StepArgs &A, long long ij, double P[NV]) {
   Geo G;
   load_geo(A.geom, A.D.n2d, ij, G);
-  return apply_floors(P, G, rho_fl, u_fl, A.gk);
+  return apply_floors(P, G, __ldg(A.floors + ij), __ldg(A.floors + A.D.n2d + ij), A.gk);
+}
+// The fluid-frame bounds of a zone whose b^2 and Lorentz factor are known.
+__device__ __forceinline__ int floors_fluid(const StepArgs &A, long long ij, double P[NV],
+                                            double bsq, double lorentz) {
+  if (!less(FL_GAMMA, lorentz))
+    return apply_floors_known(P, __ldg(A.floors + ij), __ldg(A.floors + A.D.n2d + ij), A.gk, bsq);
+  double p[NV];
+#pragma unroll
+  for (int v = 0; v < NV; v++) p[v] = P[v];
+  const int ff = floors_capped(A, ij, p);
+#pragma unroll
+  for (int v = 0; v < NV; v++) P[v] = p[v];
+  return ff;
+}
+
+// The drift-frame bounds in FP64: zones that need the Lorentz-factor cap, metrics
+// that couple X2, sums that wide_invert gives no answer for.
+static __device__ __noinline__ int floors_drift_fp64(const StepArgs &A, long long ij, double P[NV]) {
+  Geo G;
+  load_geo(A.geom, A.D.n2d, ij, G);
+  return apply_floors_drift(P, G, __ldg(A.floors + ij), __ldg(A.floors + A.D.n2d + ij), A.gk);
+}
+// The drift-frame bounds (apply_floors_drift) of a zone whose b^2 and Lorentz
+// factor are known, the sum with the parcel and its inversion in Wide numbers.
+__device__ __forceinline__ int floors_drift(const StepArgs &A, long long ij, double P[NV],
+                                            double bsq, double lorentz) {
+  int ff = 0;
+  if (!A.clk->coupled && !less(FL_GAMMA, lorentz)) {
+    double Pf[NV];
+#pragma unroll
+    for (int v = 0; v < NV; v++) Pf[v] = P[v];
+    ff = apply_floors_known(Pf, __ldg(A.floors + ij), __ldg(A.floors + A.D.n2d + ij), A.gk, bsq);
+    if (!ff) return 0;
+    const double *g = A.geom + ij;
+    const long long n2d = A.D.n2d;
+    const auto geo = [g, n2d](int comp) { return __ldg(g + comp * n2d); };
+    double U[NV], pn[NV], guess, b, l;
+    wide_drift_sum(P, geo, A.gam, Pf[RHO] - P[RHO], Pf[UU] - P[UU], FL_DRIFT_BSQ * Pf[RHO], Pf[RHO],
+                   Pf[UU], U, guess);
+    if (wide_invert<true>(U, geo, A.gk, guess, pn, b, l)) {
+#pragma unroll
+      for (int v = 0; v < NV; v++) P[v] = pn[v];
+      return ff | FF_DRIFT | floors_fluid(A, ij, P, b, l);
+    }
+  }
+  double p[NV];
+#pragma unroll
+  for (int v = 0; v < NV; v++) p[v] = P[v];
+  ff = floors_drift_fp64(A, ij, p);
+#pragma unroll
+  for (int v = 0; v < NV; v++) P[v] = p[v];
+  return ff;
 }
 
 // The inversion in FP64 from the guess P_i: zones for which wide_invert gives
@@ -694,7 +746,10 @@ static __device__ __noinline__ int invert_fp64(const StepArgs &A, const double U
 // with the source among them, which waited for spills and instructions).
 //
 // The predictor (PRED: P_s = P_i = P^n) keeps U(P^n) in Ucache for both stages.
-// scratch: S_0 .. S_3 and the guess, [5][ntot].
+// scratch ([8][ntot]): S_0 .. S_3 and the guess; b^2 of P_s (for electron grids);
+// then, from invert_body, b^2 and the Lorentz factor of the result, where a later
+// pass takes the bounds.
+enum { SCR_GUESS = 4, SCR_BSQ_S, SCR_BSQ, SCR_LORENTZ };
 template <bool PRED>
 __device__ __forceinline__ void source_body(const StepArgs &A, const double *__restrict__ Ps,
                                             double *__restrict__ Ucache,
@@ -708,12 +763,12 @@ __device__ __forceinline__ void source_body(const StepArgs &A, const double *__r
   const long long ij = (long long)j * D.s[0] + i;
   const double *g = A.geom + ij;
   const auto geo = [g, &D](int comp) { return __ldg(g + comp * D.n2d); };
-  double p[NV], U[NV], T[4][4], S[4], g2;
+  double p[NV], U[NV], T[4][4], S[4], g2, bsq;
 #pragma unroll
   for (int v = 0; v < NV; v++) p[v] = __ldg(Ps + v * N + c);
   if (A.clk->coupled) {
-    double Uc[NV], Tc[4][4], gc;
-    tensor_fp64(A, Ps, c, ij, Uc, Tc, gc);
+    double Uc[NV], Tc[4][4], gc, bc;
+    tensor_fp64(A, Ps, c, ij, Uc, Tc, gc, bc);
 #pragma unroll
     for (int v = 0; v < NV; v++) U[v] = Uc[v];
 #pragma unroll
@@ -721,8 +776,9 @@ __device__ __forceinline__ void source_body(const StepArgs &A, const double *__r
 #pragma unroll
       for (int n = 0; n < 4; n++) T[m][n] = Tc[m][n];
     g2 = gc;
+    bsq = bc;
   } else {
-    wide_tensor<true, PRED>(p, geo, A.gm1, U, T, g2);
+    wide_tensor<true, PRED>(p, geo, A.gm1, U, T, g2, bsq);
   }
   const double gd = geo(G_GDET);
   if (PRED) {  // U^t has no field part: b^i u^t - b^t u^i = B^i
@@ -732,7 +788,8 @@ __device__ __forceinline__ void source_body(const StepArgs &A, const double *__r
   geo_source(T, gd, A.conn, D.n2d, ij, S);
 #pragma unroll
   for (int n = 0; n < 4; n++) scratch[n * N + c] = S[n];
-  scratch[4 * N + c] = fma(A.gam, p[UU], p[RHO]) * g2;
+  scratch[SCR_GUESS * N + c] = fma(A.gam, p[UU], p[RHO]) * g2;
+  if (A.elec) scratch[SCR_BSQ_S * N + c] = bsq;
 }
 
 // U(P^n) + dt' (S - div F), its inversion and the bounds; Pi: the guess of the
@@ -740,9 +797,8 @@ __device__ __forceinline__ void source_body(const StepArgs &A, const double *__r
 __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__restrict__ F1,
                                             const double *__restrict__ F2,
                                             const double *__restrict__ F3,
-                                            const double *__restrict__ Ucache,
-                                            const double *__restrict__ scratch, double dtfac,
-                                            const double *Pi, double *Pout, int *pflag, int *fflag,
+                                            const double *__restrict__ Ucache, double *scratch,
+                                            double dtfac, const double *Pi, double *Pout, int *pflag, int *fflag,
                                             long long t) {
   const Dims &D = A.D;
   const double dt = A.clk->dt;
@@ -764,10 +820,10 @@ __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__r
       const long long o = v * N + c;
       const double div = flux_div(A, F1, F2, F3, o), u = __ldg(Ucache + o);
       // the source enters the energy and momentum rows only
-      Un[v] = (v >= UU && v <= U3) ? fma(dtp, __ldg(scratch + (v - UU) * N + c) - div, u)
+      Un[v] = (v >= UU && v <= U3) ? fma(dtp, scratch[(v - UU) * N + c] - div, u)
                                    : fma(-dtp, div, u);
     }
-    const double guess = __ldg(scratch + 4 * N + c);
+    const double guess = scratch[SCR_GUESS * N + c];
     if (A.clk->coupled || !wide_invert<true>(Un, geo, A.gk, guess, pn, bsq_n, lor_n)) {
       double u[NV], p[NV], b = 0.0, l = 1.0;
 #pragma unroll
@@ -778,18 +834,11 @@ __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__r
       bsq_n = b;
       lor_n = l;
     }
-    if (pf == PF_OK && A.floors_on && !A.floor_drift && !A.elec) {
-      const double rho_fl = __ldg(A.floors + ij), u_fl = __ldg(A.floors + D.n2d + ij);
-      if (less(FL_GAMMA, lor_n)) {
-        double p[NV];
-#pragma unroll
-        for (int v = 0; v < NV; v++) p[v] = pn[v];
-        ff = floors_capped(A, ij, rho_fl, u_fl, p);
-#pragma unroll
-        for (int v = 0; v < NV; v++) pn[v] = p[v];
-      } else {
-        ff = apply_floors_known(pn, rho_fl, u_fl, A.gk, bsq_n);
-      }
+    if (A.floor_drift || A.elec) {  // the bounds are a later pass's
+      scratch[SCR_BSQ * N + c] = bsq_n;
+      scratch[SCR_LORENTZ * N + c] = lor_n;
+    } else if (pf == PF_OK && A.floors_on) {
+      ff = floors_fluid(A, ij, pn, bsq_n, lor_n);
     }
 #pragma unroll
     for (int v = 0; v < NV; v++) Pout[v * N + c] = pn[v];
@@ -806,25 +855,24 @@ __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__r
 // of the block must call it (warp counters).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void floor_drift_body(const StepArgs &A, double *P,
+                                                 const double *__restrict__ scratch,
                                                  const int *__restrict__ pflag, int *fflag,
                                                  long long t) {
   const Dims &D = A.D;
   if (!(A.clk->dt > 0.0)) return;
-  const long long nz = n_zone(D);
-  const bool active = t < nz;
+  const bool in = t < n_update(D);
+  const Column q3 = column_of(in ? t : t & 31, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
+  const bool active = in && q3.active;
   int ff = 0;
   if (active) {
-    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
     const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
     const long long c = zid(D, i, j, k), N = D.ntot;
     if (pflag[c] == 0) {
-      const long long ij = (long long)j * D.s[0] + i;
-      Geo G;
-      load_geo(A.geom, D.n2d, ij, G);
       double p[NV];
 #pragma unroll
       for (int v = 0; v < NV; v++) p[v] = P[v * N + c];
-      ff = apply_floors_drift(p, G, __ldg(A.floors + ij), __ldg(A.floors + D.n2d + ij), A.gk);
+      ff = floors_drift(A, (long long)j * D.s[0] + i, p, scratch[SCR_BSQ * N + c],
+                        scratch[SCR_LORENTZ * N + c]);
       if (ff) {
 #pragma unroll
         for (int v = 0; v < NV; v++) P[v * N + c] = p[v];

@@ -20,7 +20,7 @@ struct WideState {
   Wide ucon[4], ucov[4];  // u^mu, u_mu
   Wide Bcov[4];           // B_mu
   Wide bt, bsq, iut;      // b^t, b^2, 1/u^t
-  Wide g2;                // Lorentz factor squared
+  Wide g2, B2;            // Lorentz factor squared, B_i B^i
 };
 
 // geo(c): component c of the location's geometry (G_*), as a double
@@ -59,8 +59,8 @@ WIDE_FN void wide_state(const double P[NV], const GeoFn &geo, WideState &s) {
   const Wide ga = norm(gam * al);
   s.iut = norm(al * rg);
   s.bt = norm(w_sum<1>(b1 * s.ucov[1], b2 * s.ucov[2], b3 * s.ucov[3]));
-  const Wide B2w = w_sum<1>(b1 * s.Bcov[1], b2 * s.Bcov[2], b3 * s.Bcov[3]);
-  s.bsq = norm(norm(w_sum<1>(B2w, s.bt * s.bt)) * (s.iut * s.iut));
+  s.B2 = w_sum<1>(b1 * s.Bcov[1], b2 * s.Bcov[2], b3 * s.Bcov[3]);
+  s.bsq = norm(norm(w_sum<1>(s.B2, s.bt * s.bt)) * (s.iut * s.iut));
   s.ucon[0] = gam * wide_pos(geo(G_IALPHA));
   s.ucon[1] = w_sum<1>(v1, -(ga * GCON(0, 1)));
   s.ucon[2] = BLK ? v2 : w_sum<1>(v2, -(ga * GCON(0, 2)));

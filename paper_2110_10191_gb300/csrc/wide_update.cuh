@@ -10,13 +10,14 @@
 namespace grmhd {
 
 // Rows of a state, rounded to double: U(P) but its field part (WANT_U) and T^k_l.
-// g2: the Lorentz factor squared.
+// g2, bsq: the Lorentz factor squared and b^2.
 template <bool BLK, bool WANT_U, class GeoFn>
 WIDE_FN void wide_tensor(const double P[NV], const GeoFn &geo, double gm1, double U[NV],
-                         double T[4][4], double &g2) {
+                         double T[4][4], double &g2, double &bsq) {
   WideState s;
   wide_state<BLK>(P, geo, s);
   g2 = w_to_double(s.g2);
+  bsq = w_to_double(s.bsq);
   const Wide rho = wide(P[RHO]), u = wide(P[UU]), pg = wide(gm1) * u;
   const Wide w = norm(w_sum<2>(rho, u, pg, s.bsq));
   const Wide pt = w_sum<1>(pg, w_scale(s.bsq, -1));
@@ -223,6 +224,55 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
 #undef GCOV
 #undef GDIA
 #undef GCON
+}
+
+// U of a state P plus that of the drift-frame bounds' parcel (apply_floors_drift):
+// density and internal energy dr, du, no field, the drift velocity utilde_d = f
+// (utilde - q B) with q = (utilde.B)/B^2, f = 1/sqrt(1 + (utilde.B)^2/B^2), or the
+// fluid's where B^2 <= bsq_min.  guess: W of a state with P's velocity and
+// density and internal energy rho_f, u_f.
+template <class GeoFn>
+WIDE_FN void wide_drift_sum(const double P[NV], const GeoFn &geo, double gam, double dr, double du,
+                            double bsq_min, double rho_f, double u_f, double U[NV], double &guess) {
+  WideState s;
+  wide_state<true>(P, geo, s);
+  guess = w_fma(gam, u_f, rho_f) * w_to_double(s.g2);
+  const double B2 = w_to_double(s.B2);
+  Wide q = {0, 0, -2000}, f = {1ull << 62, 0, -62};
+  const Wide one = {1ull << 61, 0, -61};
+  if (B2 > bsq_min) {
+    q = norm(s.bt * w_rcp(norm(s.B2)));
+    f = norm(w_rsqrt(norm(w_sum<1>(one, s.bt * q))));
+  }
+  // the parcel's utilde, u_mu, u^t
+  Wide vd[3], ud[4];
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    vd[i] = norm(f * norm(w_sum<1>(wide(P[U1 + i]), -(q * wide(P[B1 + i])))));
+    ud[i + 1] = norm(f * norm(w_sum<1>(s.ucov[i + 1], -(q * s.Bcov[i + 1]))));
+  }
+  const Wide g2 = norm(w_sum<1>(one, ud[1] * vd[0], ud[2] * vd[1], ud[3] * vd[2]));
+  const Wide gd = norm(g2 * w_rsqrt(g2));
+  ud[0] = norm(w_sum<1>(wide(geo(G_GCOV + SY(0, 1))) * vd[0], wide(geo(G_GCOV + SY(0, 3))) * vd[2],
+                        -(gd * wide_pos(geo(G_ALPHA)))));
+  const Wide utd = norm(gd * wide_pos(geo(G_IALPHA)));
+  // T^t_nu of both: (w u^t - k b^t) u_nu - k B_nu + w_d u^t_d u_d,nu, k = b^t / u^t
+  const double gm1 = gam - 1.0;
+  const Wide rho = wide(P[RHO]), pg = wide(gm1) * wide(P[UU]);
+  const Wide w = norm(w_sum<2>(rho, wide(P[UU]), pg, s.bsq));
+  const Wide k = norm(s.bt * s.iut);
+  const Wide k1 = norm(w_sum<1>(w * s.ucon[0], -(k * s.bt))), nk = -k;
+  const Wide kd = norm(wide(w_fma(gam, du, dr)) * utd);
+  const Wide pt = w_sum<2>(pg, w_scale(s.bsq, -1), wide(gm1 * du));
+  const Wide mass = w_sum<1>(rho * s.ucon[0], wide(dr) * utd), sg = wide_pos(geo(G_GDET));
+  U[RHO] = w_to_double(norm(mass) * sg);
+#pragma unroll
+  for (int n = 0; n < 4; n++) {
+    const Wide t = w_sum<1>(k1 * s.ucov[n], nk * s.Bcov[n], kd * ud[n]);
+    U[UU + n] = w_to_double(norm(n ? t : w_sum<2>(t, pt, mass)) * sg);
+  }
+#pragma unroll
+  for (int i = 0; i < 3; i++) U[B1 + i] = geo(G_GDET) * P[B1 + i];
 }
 
 }  // namespace grmhd

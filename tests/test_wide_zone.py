@@ -26,8 +26,9 @@ using namespace grmhd;
 extern "C" void tensor(const double *P, const double *g, int blk, double *U, double (*T)[4],
                        double *g2) {
   auto geo = [&](int k) { return g[k]; };
-  if (blk) wide_tensor<true, true>(P, geo, GAM - 1.0, U, T, *g2);
-  else wide_tensor<false, true>(P, geo, GAM - 1.0, U, T, *g2);
+  double b2;
+  if (blk) wide_tensor<true, true>(P, geo, GAM - 1.0, U, T, *g2, b2);
+  else wide_tensor<false, true>(P, geo, GAM - 1.0, U, T, *g2, b2);
 }
 extern "C" int invert(const double *U, const double *g, double guess, int blk, double *P,
                       double *bl) {
