@@ -37,6 +37,7 @@ struct SimHook : PlanHook {
       cudaEventRecord(e0, s->st);
     }
   }
+  bool serial() const override { return s->prof_on != 0; }
   void end(int cls) override {
     if (s->prof_on) {
       cudaEvent_t e1 = take_event();
@@ -92,8 +93,8 @@ static void free_all(grmhd_sim *s) {
   s->gev = nullptr;
   s->gst = nullptr;
   plan_free(s->plan);
-  double *d[] = {s->P,      s->Ph,    s->F[0], s->F[1], s->F[2],  s->emf,
-                 s->Lf,     s->Rf,    s->Uc,   s->geom, s->conn,  s->floors,
+  double *d[] = {s->P,  // and Ph, F, Lf, Rf, Uc, split with it
+                 s->emf,    s->geom,  s->conn, s->floors,
                  s->K,      s->Kh,    s->FK[0], s->FK[1], s->FK[2],
                  s->elec_w, s->KLf, s->KRf};
   for (double *p : d)
@@ -187,6 +188,7 @@ extern "C" int grmhd_footprint(const grmhd_grid *grid, const grmhd_metric *metri
   b += (size_t)plan_bytes(D, flat3_of(D, params), params->precision,
                          params->floors_on && params->floor_frame == GRMHD_FLOOR_DRIFT,
                          params->electrons.model != GRMHD_ELEC_OFF);
+  if (splits(D, pr)) b += sizeof(double) * NV * tot * SPLIT_SETS;
   *bytes = b;
   return GRMHD_OK;
 }
@@ -230,10 +232,10 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
   D.ntot = tot;
   D.n2d = (long long)D.s[0] * D.s[1];
   const size_t fb = sizeof(double) * NV * (size_t)tot;
-  bool ok = cudaMalloc(&s->P, fb) == cudaSuccess && cudaMalloc(&s->Ph, fb) == cudaSuccess &&
-            cudaMalloc(&s->F[0], fb) == cudaSuccess && cudaMalloc(&s->F[1], fb) == cudaSuccess &&
-            cudaMalloc(&s->F[2], fb) == cudaSuccess && cudaMalloc(&s->Lf, fb) == cudaSuccess &&
-            cudaMalloc(&s->Rf, fb) == cudaSuccess && cudaMalloc(&s->Uc, fb) == cudaSuccess &&
+  // P, Ph, F[3], Lf, Rf, Uc and what a split grid adds share one allocation
+  const int prec = params->precision;
+  const int nset = 8 + (splits(D, prec) ? SPLIT_SETS : 0);
+  bool ok = cudaMalloc(&s->P, fb * nset) == cudaSuccess &&
             cudaMalloc(&s->emf, sizeof(double) * 3 * (size_t)tot) == cudaSuccess &&
             cudaMalloc(&s->geom, sizeof(double) * NLOC * G_NCOMP * (size_t)D.n2d) == cudaSuccess &&
             cudaMalloc(&s->conn, sizeof(double) * C_NCOMP * (size_t)D.n2d) == cudaSuccess &&
@@ -241,7 +243,10 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
             cudaMalloc(&s->pflag, sizeof(int) * (size_t)tot) == cudaSuccess &&
             cudaMalloc(&s->fflag, sizeof(int) * (size_t)tot) == cudaSuccess &&
             cudaMalloc(&s->clk, sizeof(Clock)) == cudaSuccess;
-  const int prec = params->precision;
+  if (ok) {
+    double **set[] = {&s->Ph, &s->F[0], &s->F[1], &s->F[2], &s->Lf, &s->Rf, &s->Uc, &s->split};
+    for (int q = 0; q < 8 && q + 1 < nset; q++) *set[q] = s->P + (q + 1) * NV * D.ntot;
+  }
   if (ok && (prec == GRMHD_PREC_MIXED || prec == GRMHD_PREC_MIXED_FF))
     ok = cudaMalloc(&s->Pf, sizeof(float) * NV * (size_t)tot) == cudaSuccess &&
          cudaMalloc(&s->geomf, sizeof(float) * NLOC * G_NCOMP * (size_t)D.n2d) == cudaSuccess;
@@ -270,9 +275,7 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
     for (double *q : {s->K, s->Kh, s->FK[0], s->FK[1], s->FK[2], s->KLf, s->KRf})
       if (cudaMemsetAsync(q, 0, kb, st) != cudaSuccess) rc = GRMHD_ERR_CUDA;
   // zero every field so that entries outside the computed ranges read as 0
-  if (cudaMemsetAsync(s->P, 0, fb, st) != cudaSuccess || cudaMemsetAsync(s->Ph, 0, fb, st) != cudaSuccess ||
-      cudaMemsetAsync(s->F[0], 0, fb, st) != cudaSuccess || cudaMemsetAsync(s->F[1], 0, fb, st) != cudaSuccess ||
-      cudaMemsetAsync(s->F[2], 0, fb, st) != cudaSuccess ||
+  if (cudaMemsetAsync(s->P, 0, 5 * fb, st) != cudaSuccess ||  // P, Ph, F[3]
       cudaMemsetAsync(s->emf, 0, sizeof(double) * 3 * (size_t)tot, st) != cudaSuccess ||
       cudaMemsetAsync(s->pflag, 0, sizeof(int) * (size_t)tot, st) != cudaSuccess ||
       cudaMemsetAsync(s->fflag, 0, sizeof(int) * (size_t)tot, st) != cudaSuccess)
@@ -352,8 +355,13 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
   it.Ph = s->Ph;
   for (int d = 0; d < 3; d++) it.F[d] = s->F[d];
   it.emf = s->emf;
-  it.Lf = s->Lf;
-  it.Rf = s->Rf;
+  for (int d = 0; d < 3; d++) {
+    double *own = (s->split && d) ? s->split + (2 * d - 2) * NV * D.ntot : nullptr;
+    it.Lf[d] = own ? own : s->Lf;
+    it.Rf[d] = own ? own + NV * D.ntot : s->Rf;
+  }
+  it.scr = s->split ? s->split + 4 * NV * D.ntot : s->Lf;
+  it.split = s->split || prec == GRMHD_PREC_MIXED || prec == GRMHD_PREC_MIXED_FF;
   it.Uc = s->Uc;
   it.pflag = s->pflag;
   it.fflag = s->fflag;
@@ -553,6 +561,7 @@ static int step_graph(grmhd_sim *s, int nsteps) {
 
 extern "C" int grmhd_step(grmhd_sim *s, int nsteps, grmhd_stats *stats) {
   if (!s || nsteps < 0) return GRMHD_ERR_INVALID;
+  plan_side_streams(s->plan);
   if (nsteps >= 2 && !s->prof_on) {  // many cycles, no per-class timing: replay a graph
     const int rc = step_graph(s, nsteps);
     if (rc != GRMHD_OK) return rc;
@@ -589,7 +598,7 @@ extern "C" int grmhd_predictor(grmhd_sim *s) {
   if (!s) return GRMHD_ERR_INVALID;
   {
     SimHook h(s);
-    plan_stage(s->plan, 0, 0, s->st, &h);
+    plan_stage(s->plan, 0, s->st, &h);
   }
   int rc = launched();
   if (rc != GRMHD_OK) return rc;
@@ -606,7 +615,7 @@ extern "C" int grmhd_get_fluxes(grmhd_sim *s, double *F, double *ctop) {
   if (!s || !F) return GRMHD_ERR_INVALID;
   {
     SimHook h(s);
-    plan_fluxes(s->plan, 0, s->st, &h);
+    plan_fluxes(s->plan, 0, false, s->st, &h);
     plan_fix_ct(s->plan, s->st, &h);
   }
   int rc = launched();
@@ -633,7 +642,7 @@ extern "C" int grmhd_next_dt(grmhd_sim *s, double *dt) {
   CK(cudaMemcpyAsync(&c0, s->clk, sizeof(c0), cudaMemcpyDeviceToHost, s->st));
   {
     SimHook h(s);
-    plan_fluxes(s->plan, 0, s->st, &h);
+    plan_fluxes(s->plan, 0, false, s->st, &h);
     plan_clock(s->plan, 1, s->st, &h);
   }
   int rc = launched();

@@ -90,6 +90,7 @@ extern "C" int grmhd_batch_destroy(grmhd_batch *b) {
 extern "C" int grmhd_batch_step(grmhd_batch *b, int nsteps, int use_graph) {
   if (!b || nsteps < 0) return GRMHD_ERR_INVALID;
   if (nsteps == 0) return GRMHD_OK;
+  plan_side_streams(b->plan);
   // the batch's work follows everything already enqueued for its grids
   for (cudaStream_t q : b->member_streams) {
     if (cudaEventRecord(b->ev, q) != cudaSuccess) return GRMHD_ERR_CUDA;

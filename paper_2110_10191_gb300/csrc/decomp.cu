@@ -407,16 +407,17 @@ extern "C" int grmhd_decomp_step(grmhd_decomp *dc, int nsteps, grmhd_stats *stat
   if (!dc || nsteps < 0) return GRMHD_ERR_INVALID;
   const Plan &p = dc->plan;
   cudaStream_t st = dc->st;
+  plan_side_streams(dc->plan);
   for (int n = 0; n < nsteps; n++)
     for (int stage = 0; stage < 2; stage++) {
       const int in = stage, out = 1 - stage;
-      plan_fluxes(p, in, st, nullptr);
+      plan_fluxes(p, in, true, st, nullptr);
       if (stage == 0) {
         kx_ctop_reduce<<<1, 32, 0, st>>>(p.items, p.ngrid);
         plan_clock(p, 1, st, nullptr);
       }
       plan_fix_ct(p, st, nullptr);
-      plan_update_only(p, in, stage ? 1.0 : 0.5, stage ? 2 : 1, st, nullptr);
+      plan_invert(p, in, stage ? 1.0 : 0.5, st, nullptr);
       for (int q = 0; q < 3; q++) exchange(dc, dc->layer[q], out);
       plan_fixup(p, out, st, nullptr);
       fill(dc, out);

@@ -57,14 +57,14 @@ __global__ void __launch_bounds__(BS_MAX) kp_recon(BView V, int in) {
   const double *Ps = arr(it, in);
   if (it.A.recon == 1) {
     if (DIR == 0)
-      recon_x1_body<1>(it.A, Ps, it.Lf, it.Rf, t);
+      recon_x1_body<1>(it.A, Ps, it.Lf[DIR], it.Rf[DIR], t);
     else
-      recon_body<DIR, 1>(it.A, Ps, it.Lf, it.Rf, t);
+      recon_body<DIR, 1>(it.A, Ps, it.Lf[DIR], it.Rf[DIR], t);
   } else {
     if (DIR == 0)
-      recon_x1_body<0>(it.A, Ps, it.Lf, it.Rf, t);
+      recon_x1_body<0>(it.A, Ps, it.Lf[DIR], it.Rf[DIR], t);
     else
-      recon_body<DIR, 0>(it.A, Ps, it.Lf, it.Rf, t);
+      recon_body<DIR, 0>(it.A, Ps, it.Lf[DIR], it.Rf[DIR], t);
   }
 }
 
@@ -77,7 +77,7 @@ __global__ void __maxnreg__(72) kp_face(BView V, int in) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   const long long t = block_tid(V, g);
-  const double *Lf = it.Lf, *Rf = it.Rf;
+  const double *Lf = it.Lf[DIR], *Rf = it.Rf[DIR];
   if (DIR == 2 && it.A.flat3) Lf = Rf = arr(it, in);  // flat X3: the primitives
   face_body<DIR, ELEC>(it.A, Lf, Rf, it.F[DIR], t);
 }
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(BS_MAX) kp_recon_ff(BView V) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   const long long t = block_tid(V, g);
-  float *Lf = (float *)it.Lf, *Rf = (float *)it.Rf;
+  float *Lf = (float *)it.Lf[DIR], *Rf = (float *)it.Rf[DIR];
   if (it.A.recon == 1)
     recon_ff_body<DIR, 1>(it.A, it.Pff, Lf, Rf, t);
   else
@@ -131,7 +131,7 @@ __global__ void __maxnreg__(128) kp_face_ff(BView V) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   const long long t = block_tid(V, g);
-  const float *Lf = (const float *)it.Lf, *Rf = (const float *)it.Rf;
+  const float *Lf = (const float *)it.Lf[DIR], *Rf = (const float *)it.Rf[DIR];
   if (DIR == 2 && it.A.flat3) Lf = Rf = it.Pff;
   face_ff_body<DIR>(it.A, it.geomff, Lf, Rf, it.F[DIR], t);
 }
@@ -162,15 +162,14 @@ __global__ void kp_ct(BView V) {
   ct_body(it.A, it.F[0], it.F[1], it.F[2], it.emf, block_tid(V, g));
 }
 
-// The update's two passes.  PRED: the predictor (in = 0).  The source and the
-// guess W wait in the low faces' array, which the face fluxes have done with.
+// The update's two passes.  PRED: the predictor (in = 0).
 // 20 and 24 warps per SM against some spills (both passes per cycle of a 128^3
 // grid: 168 and 128 registers 1.74 ms, 128 and 112 1.66, 96 and 80 1.58).
 template <bool PRED>
 __global__ void __maxnreg__(96) kp_source(BView V) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  source_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Uc, it.Lf, block_tid(V, g));
+  source_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Uc, it.scr, block_tid(V, g));
 }
 
 // the source pass of the float-float modes
@@ -178,13 +177,13 @@ template <bool PRED>
 __global__ void __maxnreg__(96) kp_source_ff(BView V) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  source_ff_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Pff, it.Uc, it.Lf, block_tid(V, g));
+  source_ff_body<PRED>(it.A, PRED ? it.P : it.Ph, it.Pff, it.Uc, it.scr, block_tid(V, g));
 }
 
 __global__ void __maxnreg__(80) kp_invert(BView V, int in, double dtfac) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  invert_body(it.A, it.F[0], it.F[1], it.F[2], it.Uc, it.Lf, dtfac, it.P, arr(it, 1 - in), it.pflag,
+  invert_body(it.A, it.F[0], it.F[1], it.F[2], it.Uc, it.scr, dtfac, it.P, arr(it, 1 - in), it.pflag,
               it.fflag, block_tid(V, g));
 }
 
@@ -207,7 +206,7 @@ __global__ void __maxnreg__(96) kp_elec_post(BView V, int in, double dtfac) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
   elec_post_body(it.A, arr(it, in), arr(it, 1 - in), it.F[0], it.F[1], it.F[2], it.FK[0],
-                 it.FK[1], it.FK[2], it.K, karr(it, in), karr(it, 1 - in), it.Uc, it.Lf, it.pflag,
+                 it.FK[1], it.FK[2], it.K, karr(it, in), karr(it, 1 - in), it.Uc, it.scr, it.pflag,
                  it.fflag, dtfac, block_tid(V, g));
 }
 
@@ -220,7 +219,7 @@ __global__ void kp_elec_fix(BView V, int out) {
 __global__ void __maxnreg__(128) kp_floor_drift(BView V, int out) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  floor_drift_body(it.A, arr(it, out), it.Lf, it.pflag, it.fflag, block_tid(V, g));
+  floor_drift_body(it.A, arr(it, out), it.scr, it.pflag, it.fflag, block_tid(V, g));
 }
 
 __global__ void kp_fixup(BView V, int out) {
@@ -412,6 +411,8 @@ int plan_build(Plan &p, const StageItem *items, int n) {
   }
   p.zones = zones;
   p.tab_cap = cap;
+  p.may_split = zones <= SPLIT_ZONES;
+  for (int g = 0; g < n; g++) p.may_split = p.may_split && items[g].split;
   if (cudaMalloc(&p.items, sizeof(StageItem) * n) != cudaSuccess ||
       cudaMalloc(&p.tab, sizeof(int) * (size_t)(cap > 0 ? cap : 1)) != cudaSuccess) {
     cudaGetLastError();
@@ -430,6 +431,15 @@ int plan_build(Plan &p, const StageItem *items, int n) {
 void plan_free(Plan &p) {
   if (p.items) cudaFree(p.items);
   if (p.tab) cudaFree(p.tab);
+  for (int q = 0; q < 3; q++) {
+    if (p.side[q]) cudaStreamDestroy(p.side[q]);
+    if (p.join[q]) cudaEventDestroy(p.join[q]);
+    p.side[q] = nullptr;
+    p.join[q] = nullptr;
+  }
+  if (p.fork) cudaEventDestroy(p.fork);
+  p.fork = nullptr;
+  p.concurrent = 0;
   delete[] p.count;
   delete[] p.host_items;
   p.items = nullptr;
@@ -482,34 +492,80 @@ int plan_clock(const Plan &p, int op, cudaStream_t st, PlanHook *h) {
   return 1;
 }
 
-int plan_fluxes(const Plan &p, int in, cudaStream_t st, PlanHook *h) {
-  int nl = plan_clock(p, 0, st, h);
+void plan_side_streams(Plan &p) {
+  if (!p.may_split || p.concurrent) return;
+  bool ok = p.fork || cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int q = 0; q < 3 && ok; q++)
+    ok = (p.side[q] || cudaStreamCreateWithFlags(&p.side[q], cudaStreamNonBlocking) == cudaSuccess) &&
+         (p.join[q] || cudaEventCreateWithFlags(&p.join[q], cudaEventDisableTiming) == cudaSuccess);
+  if (!ok) cudaGetLastError();  // one after the other, then
+  p.concurrent = ok;
+}
+
+namespace {
+
+// reconstruction and face fluxes along one direction, in every precision
+template <int DIR>
+int flux_dir(const Plan &p, int in, cudaStream_t st, PlanHook *h) {
   const int R = GRMHD_K_RECON, F = GRMHD_K_FLUX;
-  // FP64 grids
-  nl += launch(p, PC_RECON0, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<0><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE0, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<0><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE0E, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<0, true><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_RECON1, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<1><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE1, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<1><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE1E, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<1, true><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_RECON2, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<2><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE2, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<2><<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE2E, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<2, true><<<nb, bs, 0, st>>>(V, in); });
-  // mixed-precision grids
+  int nl = launch(p, PC_RECON0 + DIR, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon<DIR><<<nb, bs, 0, st>>>(V, in); });
+  nl += launch(p, PC_FACE0 + DIR, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<DIR><<<nb, bs, 0, st>>>(V, in); });
+  nl += launch(p, PC_FACE0E + DIR, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face<DIR, true><<<nb, bs, 0, st>>>(V, in); });
+  nl += launch(p, PC_FACE0F + DIR, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_flux_f32<DIR><<<nb, bs, 0, st>>>(V); });
+  nl += launch(p, (DIR == 2) ? PC_RECON2X : PC_RECON01X, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon_ff<DIR><<<nb, bs, 0, st>>>(V); });
+  nl += launch(p, PC_FACE0X + DIR, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face_ff<DIR><<<nb, bs, 0, st>>>(V); });
+  return nl;
+}
+
+// the update's source pass
+int source_pass(const Plan &p, int in, cudaStream_t st, PlanHook *h) {
+  int nl = launch(p, PC_SRCX, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
+    if (in == 0)
+      kp_source_ff<true><<<nb, bs, 0, st>>>(V);
+    else
+      kp_source_ff<false><<<nb, bs, 0, st>>>(V);
+  });
+  nl += launch(p, PC_SRC64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
+    if (in == 0)
+      kp_source<true><<<nb, bs, 0, st>>>(V);
+    else  // the predictor before it kept U(P^n)
+      kp_source<false><<<nb, bs, 0, st>>>(V);
+  });
+  return nl;
+}
+
+}  // namespace
+
+int plan_fluxes(const Plan &p, int in, bool with_source, cudaStream_t st, PlanHook *h) {
+  // (the corrector's signal speeds are not used)
+  int nl = in == 0 ? plan_clock(p, 0, st, h) : 0;
+  const int R = GRMHD_K_RECON;
+  // the FP32 and the split copies of the stage input
   nl += launch(p, PC_TOF32, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_to_f32<<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_FACE0F, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_flux_f32<0><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_FACE1F, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_flux_f32<1><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_FACE2F, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_flux_f32<2><<<nb, bs, 0, st>>>(V); });
-  // float-float grids
   nl += launch(p, PC_TOFF, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_to_ff<<<nb, bs, 0, st>>>(V, in); });
-  nl += launch(p, PC_RECON01X, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon_ff<0><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_FACE0X, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face_ff<0><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_RECON01X, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon_ff<1><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_FACE1X, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face_ff<1><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_RECON2X, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_recon_ff<2><<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_FACE2X, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_face_ff<2><<<nb, bs, 0, st>>>(V); });
+  if (p.concurrent && !(h && h->serial())) {
+    // nothing below reads what another of the four writes
+    cudaEventRecord(p.fork, st);
+    for (int q = 0; q < 3; q++)
+      if (q < 2 || with_source) cudaStreamWaitEvent(p.side[q], p.fork, 0);
+    nl += flux_dir<0>(p, in, p.side[0], h);
+    nl += flux_dir<1>(p, in, p.side[1], h);
+    if (with_source) nl += source_pass(p, in, p.side[2], h);
+    nl += flux_dir<2>(p, in, st, h);
+    for (int q = 0; q < 3; q++) {
+      if (q == 2 && !with_source) continue;
+      cudaEventRecord(p.join[q], p.side[q]);
+      cudaStreamWaitEvent(st, p.join[q], 0);
+    }
+  } else {
+    nl += flux_dir<0>(p, in, st, h);
+    nl += flux_dir<1>(p, in, st, h);
+    nl += flux_dir<2>(p, in, st, h);
+    if (with_source) nl += source_pass(p, in, st, h);  // its scratch may be face values' space
+  }
   // electron entropies (grids with electrons, any precision): per direction,
   // reconstruction and the fluxes from the face kernels' weights
+  const int F = GRMHD_K_FLUX;
   nl += launch(p, PC_EREC01, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_elec_recon<0><<<nb, bs, 0, st>>>(V, in); });
   nl += launch(p, PC_EFACE0, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_elec_flux<0><<<nb, bs, 0, st>>>(V); });
   nl += launch(p, PC_EREC01, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_elec_recon<1><<<nb, bs, 0, st>>>(V, in); });
@@ -530,21 +586,8 @@ int plan_fix_ct(const Plan &p, cudaStream_t st, PlanHook *h) {
   return nl;
 }
 
-int plan_update_only(const Plan &p, int in, double dtfac, int ucache_mode, cudaStream_t st,
-                     PlanHook *h) {
-  int nl = launch(p, PC_SRCX, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
-    if (in == 0)
-      kp_source_ff<true><<<nb, bs, 0, st>>>(V);
-    else
-      kp_source_ff<false><<<nb, bs, 0, st>>>(V);
-  });
-  nl += launch(p, PC_SRC64, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
-    if (in == 0)
-      kp_source<true><<<nb, bs, 0, st>>>(V);
-    else  // the predictor before it kept U(P^n)
-      kp_source<false><<<nb, bs, 0, st>>>(V);
-  });
-  nl += launch(p, PC_UPD, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, in, dtfac); });
+int plan_invert(const Plan &p, int in, double dtfac, cudaStream_t st, PlanHook *h) {
+  int nl = launch(p, PC_UPD, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, in, dtfac); });
   nl += launch(p, PC_FLOORD, GRMHD_K_UPDATE, h, [&](unsigned nb, unsigned bs, BView V) {
     kp_floor_drift<<<nb, bs, 0, st>>>(V, 1 - in);
   });
@@ -562,10 +605,6 @@ int plan_fixup(const Plan &p, int out, cudaStream_t st, PlanHook *h) {
   return nl;
 }
 
-int plan_update(const Plan &p, int in, double dtfac, int ucache_mode, cudaStream_t st, PlanHook *h) {
-  return plan_update_only(p, in, dtfac, ucache_mode, st, h) + plan_fixup(p, 1 - in, st, h);
-}
-
 int plan_bounds_pass(const Plan &p, int which, int pass, cudaStream_t st, PlanHook *h) {
   const int B = GRMHD_K_BOUNDS;
   if (pass == 0)
@@ -581,11 +620,12 @@ int plan_bounds(const Plan &p, int which, cudaStream_t st, PlanHook *h) {
   return nl;
 }
 
-int plan_stage(const Plan &p, int stage, int ucache_mode, cudaStream_t st, PlanHook *h) {
-  int nl = plan_fluxes(p, stage, st, h);
+int plan_stage(const Plan &p, int stage, cudaStream_t st, PlanHook *h) {
+  int nl = plan_fluxes(p, stage, true, st, h);
   if (stage == 0) nl += plan_clock(p, 1, st, h);
   nl += plan_fix_ct(p, st, h);
-  nl += plan_update(p, stage, stage ? 1.0 : 0.5, ucache_mode, st, h);
+  nl += plan_invert(p, stage, stage ? 1.0 : 0.5, st, h);
+  nl += plan_fixup(p, 1 - stage, st, h);
   nl += plan_bounds(p, 1 - stage, st, h);
   return nl;
 }
@@ -593,8 +633,8 @@ int plan_stage(const Plan &p, int stage, int ucache_mode, cudaStream_t st, PlanH
 int plan_steps(const Plan &p, int nsteps, cudaStream_t st, PlanHook *h) {
   int nl = 0;
   for (int n = 0; n < nsteps; n++) {
-    nl += plan_stage(p, 0, 1, st, h);  // predictor keeps U(P^n)
-    nl += plan_stage(p, 1, 2, st, h);  // corrector reads it back
+    nl += plan_stage(p, 0, st, h);  // predictor: keeps U(P^n)
+    nl += plan_stage(p, 1, st, h);  // corrector: reads it back
     nl += plan_clock(p, 2, st, h);
   }
   return nl;
@@ -632,7 +672,7 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
         cudaSuccess)
       return GRMHD_ERR_CUDA;
   // representative scratch: face values, CT fluxes and a CFL dt of the current state
-  plan_fluxes(p, 0, st, nullptr);
+  plan_fluxes(p, 0, false, st, nullptr);
   plan_clock(p, 1, st, nullptr);
   plan_fix_ct(p, st, nullptr);
   struct Group {

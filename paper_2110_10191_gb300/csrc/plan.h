@@ -11,6 +11,7 @@
 
 #include <cuda_runtime.h>
 
+#include "../../include/grmhd.h"
 #include "grmhd_impl.h"
 
 namespace grmhd {
@@ -19,7 +20,12 @@ namespace grmhd {
 struct StageItem {
   StepArgs A;
   double *P, *Ph;  // stage arrays: P^n / P^{n+1} and P^{n+1/2}
-  double *F[3], *emf, *Lf, *Rf, *Uc;
+  double *F[3], *emf, *Uc;
+  // face values along each direction, and the update's scratch (SCR_*, [8][ntot]):
+  // arrays of their own where split is set, else one pair, which the directions
+  // use in turn and whose low half is the scratch when they have done
+  double *Lf[3], *Rf[3], *scr;
+  int split;
   int *pflag, *fflag;
   float *Pf;           // mixed precision: FP32 primitives (8 x ntot)
   const float *geomf;  // mixed precision: FP32 geometry
@@ -92,6 +98,12 @@ struct Plan {
   int sched[PC_N];   // block order of each class (SCHED_*)
   int map_base[PC_N], loc_base[PC_N], nblocks[PC_N];
   long long zones;  // interior zones over all grids
+  // every grid split, and few enough zones: the directions' flux kernels and the
+  // source pass may run on streams of their own, forked from and joined to the
+  // plan's; concurrent once those exist (plan_side_streams)
+  int may_split, concurrent;
+  cudaStream_t side[3];
+  cudaEvent_t fork, join[3];
   int tuned;        // 1 after plan_autotune
 };
 
@@ -99,6 +111,7 @@ struct Plan {
 struct PlanHook {
   virtual void begin(int kclass, int nlaunch) = 0;
   virtual void end(int kclass) = 0;
+  virtual bool serial() const { return false; }  // times every launch: one after the other
   virtual ~PlanHook() {}
 };
 
@@ -116,6 +129,19 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
 // those launches RWALK_MIN_THREADS threads, 20 warps per SM, else 1 (one thread
 // per zone, which forms each pair of differences three times and costs 6% more
 // where both fill the GPU: 301 against 283 us over 128x128x64 zones).
+// Largest number of interior zones, of a grid and of a plan, whose directions get
+// face arrays of their own and run side by side.  A small grid's kernels leave
+// most of the GPU idle, each waiting for its threads' chains of work; side by side
+// a cycle of a 64x64 mode takes 114 us against 167, of 217x217 zones 281 against
+// 324, of 64^3 1162 against 1285, of 128^3 7.03 against 7.26 ms (where the kernels'
+// tails overlap); beyond, the gain no longer pays for the memory.
+constexpr long long SPLIT_ZONES = 1 << 21;
+constexpr int SPLIT_SETS = 5;  // arrays of [8][ntot] they take
+// (FP32 fluxes need no face arrays: their space is the update's scratch at once)
+inline bool splits(const Dims &D, int prec) {
+  return prec != GRMHD_PREC_MIXED && prec != GRMHD_PREC_MIXED_FF &&
+         (long long)D.n[0] * D.n[1] * D.n[2] <= SPLIT_ZONES;
+}
 constexpr long long RWALK_MIN_THREADS = 152 * 640;
 int plan_rwalk(const StageItem *items, int n);
 // Set the plan's reconstruction walk length (1, 2, 4, 8 or 16 zones per
@@ -125,6 +151,9 @@ int plan_set_rwalk(Plan &p, int rw);
 // device bytes a one-grid plan of such a grid holds (item + block tables)
 long long plan_bytes(const Dims &D, int flat3, int prec, int drift, int elec);
 void plan_free(Plan &p);
+// Create the streams of a plan that may split, before its first step (and outside
+// a capture); without them it runs in sequence.
+void plan_side_streams(Plan &p);
 // Re-lay the block tables of class cls for bs threads per block and block
 // order sched (the results of every grid do not depend on either).
 int plan_set_class(Plan &p, int cls, int bs, int sched);
@@ -141,27 +170,26 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
 // The functions below enqueue on st and return the number of kernels
 // launched; launch errors are left for cudaGetLastError().
 // stage input: 0 = P, 1 = Ph.  Signal-speed reset, reconstruction + face
-// fluxes (FP64, FP32 or float-float per grid), flat-X3 copies.
-int plan_fluxes(const Plan &p, int in, cudaStream_t st, PlanHook *h);
+// fluxes (FP64, FP32 or float-float per grid), flat-X3 copies; with_source: and
+// the update's source pass.
+int plan_fluxes(const Plan &p, int in, bool with_source, cudaStream_t st, PlanHook *h);
 // per-grid clock: 0 reset the signal-speed maxima, 1 CFL time step, 2 advance
 int plan_clock(const Plan &p, int op, cudaStream_t st, PlanHook *h);
 // boundary flux fixes + flux-CT
 int plan_fix_ct(const Plan &p, cudaStream_t st, PlanHook *h);
-// U(P) + dtfac dt (S(in) - div F) -> inversion -> bounds into the other array
-// (in 0: P -> Ph, in 1: Ph -> P), then the fixup; ucache_mode as launch_update
-int plan_update(const Plan &p, int in, double dtfac, int ucache_mode, cudaStream_t st, PlanHook *h);
+// U(P^n) + dtfac dt (S - div F) of the source pass's scratch -> inversion -> bounds
+// into the other array (in 0: Ph, in 1: P), and the passes that close the state
+// (drift-frame bounds, electrons)
+int plan_invert(const Plan &p, int in, double dtfac, cudaStream_t st, PlanHook *h);
+int plan_fixup(const Plan &p, int out, cudaStream_t st, PlanHook *h);
 // ghost fill of P (which 0) or Ph (which 1)
 int plan_bounds(const Plan &p, int which, cudaStream_t st, PlanHook *h);
-// the pieces of plan_update and plan_bounds, for a decomposed grid that
-// exchanges block edges between them: the update alone (into 1 - in), the
-// fixup of array out, one ghost-fill pass (0: X1, 1: X2, 2: X3)
-int plan_update_only(const Plan &p, int in, double dtfac, int ucache_mode, cudaStream_t st,
-                     PlanHook *h);
-int plan_fixup(const Plan &p, int out, cudaStream_t st, PlanHook *h);
+// one ghost-fill pass (0: X1, 1: X2, 2: X3), for a decomposed grid that exchanges
+// block edges between them
 int plan_bounds_pass(const Plan &p, int which, int pass, cudaStream_t st, PlanHook *h);
 // one stage: stage 0 predictor (P -> Ph, dt/2, with the CFL step),
 // stage 1 corrector (Ph -> P, dt)
-int plan_stage(const Plan &p, int stage, int ucache_mode, cudaStream_t st, PlanHook *h);
+int plan_stage(const Plan &p, int stage, cudaStream_t st, PlanHook *h);
 // full predictor-corrector steps (U(P^n) kept between the stages)
 int plan_steps(const Plan &p, int nsteps, cudaStream_t st, PlanHook *h);
 

@@ -16,6 +16,7 @@ struct grmhd_sim {
   grmhd_params params;
   cudaStream_t st;
   double *P, *Ph, *F[3], *emf, *Lf, *Rf, *Uc;
+  double *split;  // small grids: face values of X2 and X3, the update's scratch (SPLIT_SETS x 8 x ntot)
   double *geom, *conn, *floors;
   float *Pf, *geomf;    // FP32 copies (mixed precision only)
   float *Pff, *geomff, *connff;  // split float-float copies (float-float modes only)

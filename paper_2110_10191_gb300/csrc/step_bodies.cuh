@@ -755,7 +755,7 @@ __device__ __forceinline__ void source_body(const StepArgs &A, const double *__r
                                             double *__restrict__ Ucache,
                                             double *__restrict__ scratch, long long t) {
   const Dims &D = A.D;
-  if (!(A.clk->dt > 0.0) || t >= n_update(D)) return;
+  if (t >= n_update(D)) return;
   const Column q3 = column_of(t, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
   if (!q3.active) return;
   const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
