@@ -412,7 +412,7 @@ static int set_common(grmhd_sim *s, const double *P, int on_device, int ghost) {
   }
   {
     SimHook h(s);
-    plan_bounds(s->plan, 0, s->st, &h);
+    plan_bounds(s->plan, 0, 0, s->st, &h);
   }
   // the ghosts of a fixed side keep their set values in both stage arrays
   CK(cudaMemcpyAsync(s->Ph, s->P, sizeof(double) * NV * (size_t)D.ntot, cudaMemcpyDeviceToDevice,
@@ -447,7 +447,7 @@ extern "C" int grmhd_set_electrons(grmhd_sim *s, const double *K, int with_ghost
   }
   {
     SimHook h(s);
-    plan_bounds(s->plan, 0, s->st, &h);  // refills the primitives' ghosts too (unchanged)
+    plan_bounds(s->plan, 0, 0, s->st, &h);  // refills the primitives' ghosts too (unchanged)
   }
   CK(cudaMemcpyAsync(s->Kh, s->K, sizeof(double) * 2 * (size_t)D.ntot, cudaMemcpyDeviceToDevice,
                      s->st));
@@ -599,6 +599,7 @@ extern "C" int grmhd_predictor(grmhd_sim *s) {
   {
     SimHook h(s);
     plan_stage(s->plan, 0, s->st, &h);
+    plan_clock(s->plan, 0, s->st, &h);
   }
   int rc = launched();
   if (rc != GRMHD_OK) return rc;
@@ -613,18 +614,20 @@ extern "C" int grmhd_predictor(grmhd_sim *s) {
 
 extern "C" int grmhd_get_fluxes(grmhd_sim *s, double *F, double *ctop) {
   if (!s || !F) return GRMHD_ERR_INVALID;
+  Clock c;
   {
     SimHook h(s);
-    plan_fluxes(s->plan, 0, false, s->st, &h);
-    plan_fix_ct(s->plan, s->st, &h);
+    plan_whole_fluxes(s->plan, 0, s->st, &h);
+    const cudaError_t e =
+        cudaMemcpyAsync(&c, s->clk, sizeof(c), cudaMemcpyDeviceToHost, s->st);
+    plan_clock(s->plan, 0, s->st, &h);
+    CK(e);
   }
   int rc = launched();
   if (rc != GRMHD_OK) return rc;
   const size_t per = sizeof(double) * NV * (size_t)s->D.ntot;
   for (int d = 0; d < 3; d++)
     CK(cudaMemcpyAsync((char *)F + d * per, s->F[d], per, cudaMemcpyDeviceToHost, s->st));
-  Clock c;
-  CK(cudaMemcpyAsync(&c, s->clk, sizeof(c), cudaMemcpyDeviceToHost, s->st));
   CK(cudaStreamSynchronize(s->st));
   if (ctop) {
     for (int d = 0; d < 3; d++) {
@@ -651,6 +654,7 @@ extern "C" int grmhd_next_dt(grmhd_sim *s, double *dt) {
   CK(cudaStreamSynchronize(s->st));
   *dt = c1.dt;
   c1.dt = c0.dt;  // leave the reported last-step dt unchanged
+  memset(c1.ctop_bits, 0, sizeof(c1.ctop_bits));
   CK(cudaMemcpyAsync(s->clk, &c1, sizeof(c1), cudaMemcpyHostToDevice, s->st));
   CK(cudaStreamSynchronize(s->st));
   return GRMHD_OK;

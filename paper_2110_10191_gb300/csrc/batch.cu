@@ -158,7 +158,7 @@ extern "C" int grmhd_batch_set_launch(grmhd_batch *b, int kclass, int threads, i
     ncls = 12;
   } else if (kclass == GRMHD_K_UPDATE) {
     cls = zone;
-    ncls = 3;
+    ncls = 4;
   } else {
     return GRMHD_ERR_INVALID;
   }

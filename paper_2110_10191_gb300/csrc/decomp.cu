@@ -411,12 +411,13 @@ extern "C" int grmhd_decomp_step(grmhd_decomp *dc, int nsteps, grmhd_stats *stat
   for (int n = 0; n < nsteps; n++)
     for (int stage = 0; stage < 2; stage++) {
       const int in = stage, out = 1 - stage;
+      if (stage == 0) plan_clock(p, 0, st, nullptr);
       plan_fluxes(p, in, true, st, nullptr);
       if (stage == 0) {
         kx_ctop_reduce<<<1, 32, 0, st>>>(p.items, p.ngrid);
         plan_clock(p, 1, st, nullptr);
       }
-      plan_fix_ct(p, st, nullptr);
+      plan_emf(p, 0, st, nullptr);
       plan_invert(p, in, stage ? 1.0 : 0.5, st, nullptr);
       for (int q = 0; q < 3; q++) exchange(dc, dc->layer[q], out);
       plan_fixup(p, out, st, nullptr);

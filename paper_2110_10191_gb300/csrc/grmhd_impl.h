@@ -95,11 +95,11 @@ void launch_geometry(const GeomArgs &A, cudaStream_t st);
 // Single-grid kernels of the allocation-free flux entry point:
 // zero clk->ctop_bits before a flux pass
 void launch_ctop_reset(const StepArgs &A, cudaStream_t st);
-// fluxes of P (fused reconstruction + LLF), with the interior ctop maxima
+// fluxes of P (fused reconstruction + LLF, with their boundary fixes), with the interior ctop maxima
 // into clk->ctop_bits
 void launch_fluxes(const StepArgs &A, const double *P, double *F[3], cudaStream_t st);
-// boundary flux fixes + flux-CT (emf scratch: 3 x ntot)
-void launch_fix_ct(const StepArgs &A, double *F[3], double *emf, cudaStream_t st);
+// flux-CT (emf scratch: 3 x ntot)
+void launch_ct(const StepArgs &A, double *F[3], double *emf, cudaStream_t st);
 
 // FP32 copy of n doubles (clamped to the float range)
 void launch_to_f32(long long n, const double *src, float *dst, cudaStream_t st);

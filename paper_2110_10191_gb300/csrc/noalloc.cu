@@ -151,7 +151,7 @@ extern "C" int grmhd_fluxes_noalloc(const grmhd_grid *grid, const grmhd_metric *
   launch_ctop_reset(A, st);
   double *Fd[3] = {F, F + NV * D.ntot, F + 2 * NV * D.ntot};
   launch_fluxes(A, P, Fd, st);
-  launch_fix_ct(A, Fd, (double *)(base + off_emf), st);
+  launch_ct(A, Fd, (double *)(base + off_emf), st);
   if (cudaGetLastError() != cudaSuccess) {
     forget_scratch(dev);
     return GRMHD_ERR_CUDA;

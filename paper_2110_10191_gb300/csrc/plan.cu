@@ -49,6 +49,19 @@ __global__ void kp_bounds(BView V, int which) {
   if (X == 2) bounds_x3_body(it.A, P, K, t);
 }
 
+// all ghosts; end: and the clock's advance and the signal speeds' reset, which close
+// a cycle, in one thread per grid
+__global__ void kp_bounds_all(BView V, int which, int end) {
+  const int g = block_grid(V);
+  const StageItem &it = V.items[g];
+  const long long t = block_tid(V, g);
+  bounds_all_body(it.A, arr(it, which), karr(it, which), t);
+  if (end && t == 0) {
+    advance_body(it.A);
+    reset_ctop_body(it.A.clk);
+  }
+}
+
 template <int DIR>
 __global__ void __launch_bounds__(BS_MAX) kp_recon(BView V, int in) {
   const int g = block_grid(V);
@@ -150,10 +163,14 @@ __global__ void kp_fix(BView V) {
                 block_tid(V, g));
 }
 
-__global__ void kp_emf(BView V) {
+// step: within a step (a flat X3 on its one layer); take_dt: and the CFL step, in one
+// thread per grid (the update after this reads it)
+__global__ void kp_emf(BView V, int step, int take_dt) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  emf_body(it.A, it.F[0], it.F[1], it.F[2], it.emf, block_tid(V, g));
+  const long long t = block_tid(V, g);
+  emf_body(it.A, it.F[0], it.F[1], it.F[2], it.emf, step && it.A.flat3, t);
+  if (take_dt && t == 0) dt_body(it.A);
 }
 
 __global__ void kp_ct(BView V) {
@@ -183,7 +200,7 @@ __global__ void __maxnreg__(96) kp_source_ff(BView V) {
 __global__ void __maxnreg__(80) kp_invert(BView V, int in, double dtfac) {
   const int g = block_grid(V);
   const StageItem &it = V.items[g];
-  invert_body(it.A, it.F[0], it.F[1], it.F[2], it.Uc, it.scr, dtfac, it.P, arr(it, 1 - in), it.pflag,
+  invert_body(it.A, it.F[0], it.F[1], it.F[2], it.emf, it.Uc, it.scr, dtfac, it.P, arr(it, 1 - in), it.pflag,
               it.fflag, block_tid(V, g));
 }
 
@@ -325,6 +342,7 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_BX1] = n_bounds_x1(D);
   c[PC_BX2] = n_bounds_x2(D);
   c[PC_BX3] = n_bounds_x3(D);
+  c[PC_BALL] = n_bounds_all(D);
   c[PC_RECON0] = f64 ? n_recon_walk(D, 0, fl, rwalk) : 0;
   c[PC_RECON1] = f64 ? n_recon_walk(D, 1, fl, rwalk) : 0;
   c[PC_RECON2] = (f64 && !fl) ? n_recon_walk(D, 2, 0, rwalk) : 0;
@@ -339,8 +357,9 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_RECON01X] = fx ? n_recon(D, fl) : 0;
   c[PC_RECON2X] = (fx && !fl) ? n_recon(D, 0) : 0;
   c[PC_REPL] = fl ? n_replicate(D) : 0;
-  c[PC_FIX] = n_fix(D);
-  c[PC_EDGE] = n_edge(D);
+  c[PC_FIX] = f64 ? 0 : n_fix(D);  // (the FP64 face fluxes fix their own)
+  c[PC_EDGE] = n_edge(D, 0);
+  c[PC_EDGES] = n_edge(D, fl);
   c[PC_ZONE] = n_zone(D);
   const bool ux = fx || prec == GRMHD_PREC_MIXED_FF;  // the source pass in float-float
   c[PC_SRC64] = ux ? 0 : n_update(D);
@@ -537,11 +556,9 @@ int source_pass(const Plan &p, int in, cudaStream_t st, PlanHook *h) {
 }  // namespace
 
 int plan_fluxes(const Plan &p, int in, bool with_source, cudaStream_t st, PlanHook *h) {
-  // (the corrector's signal speeds are not used)
-  int nl = in == 0 ? plan_clock(p, 0, st, h) : 0;
   const int R = GRMHD_K_RECON;
   // the FP32 and the split copies of the stage input
-  nl += launch(p, PC_TOF32, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_to_f32<<<nb, bs, 0, st>>>(V, in); });
+  int nl = launch(p, PC_TOF32, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_to_f32<<<nb, bs, 0, st>>>(V, in); });
   nl += launch(p, PC_TOFF, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_to_ff<<<nb, bs, 0, st>>>(V, in); });
   if (p.concurrent && !(h && h->serial())) {
     // nothing below reads what another of the four writes
@@ -572,16 +589,21 @@ int plan_fluxes(const Plan &p, int in, bool with_source, cudaStream_t st, PlanHo
   nl += launch(p, PC_EFACE1, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_elec_flux<1><<<nb, bs, 0, st>>>(V); });
   nl += launch(p, PC_EREC2, R, h, [&](unsigned nb, unsigned bs, BView V) { kp_elec_recon<2><<<nb, bs, 0, st>>>(V, in); });
   nl += launch(p, PC_EFACE2, F, h, [&](unsigned nb, unsigned bs, BView V) { kp_elec_flux<2><<<nb, bs, 0, st>>>(V); });
-  // flat-X3 grids
-  nl += launch(p, PC_REPL, GRMHD_K_OTHER, h,
-               [&](unsigned nb, unsigned bs, BView V) { kp_replicate<<<nb, bs, 0, st>>>(V); });
+  // boundary flux fixes
+  nl += launch(p, PC_FIX, GRMHD_K_CT, h, [&](unsigned nb, unsigned bs, BView V) { kp_fix<<<nb, bs, 0, st>>>(V); });
   return nl;
 }
 
-int plan_fix_ct(const Plan &p, cudaStream_t st, PlanHook *h) {
+int plan_emf(const Plan &p, int take_dt, cudaStream_t st, PlanHook *h) {
+  return launch(p, PC_EDGES, GRMHD_K_CT, h, [&](unsigned nb, unsigned bs, BView V) { kp_emf<<<nb, bs, 0, st>>>(V, 1, take_dt); });
+}
+
+int plan_whole_fluxes(const Plan &p, int in, cudaStream_t st, PlanHook *h) {
   const int C = GRMHD_K_CT;
-  int nl = launch(p, PC_FIX, C, h, [&](unsigned nb, unsigned bs, BView V) { kp_fix<<<nb, bs, 0, st>>>(V); });
-  nl += launch(p, PC_EDGE, C, h, [&](unsigned nb, unsigned bs, BView V) { kp_emf<<<nb, bs, 0, st>>>(V); });
+  int nl = plan_fluxes(p, in, false, st, h);
+  nl += launch(p, PC_REPL, GRMHD_K_OTHER, h,
+               [&](unsigned nb, unsigned bs, BView V) { kp_replicate<<<nb, bs, 0, st>>>(V); });
+  nl += launch(p, PC_EDGE, C, h, [&](unsigned nb, unsigned bs, BView V) { kp_emf<<<nb, bs, 0, st>>>(V, 0, 0); });
   nl += launch(p, PC_EDGE, C, h, [&](unsigned nb, unsigned bs, BView V) { kp_ct<<<nb, bs, 0, st>>>(V); });
   return nl;
 }
@@ -614,19 +636,22 @@ int plan_bounds_pass(const Plan &p, int which, int pass, cudaStream_t st, PlanHo
   return launch(p, PC_BX3, B, h, [&](unsigned nb, unsigned bs, BView V) { kp_bounds<2><<<nb, bs, 0, st>>>(V, which); });
 }
 
-int plan_bounds(const Plan &p, int which, cudaStream_t st, PlanHook *h) {
-  int nl = 0;
-  for (int pass = 0; pass < 3; pass++) nl += plan_bounds_pass(p, which, pass, st, h);
-  return nl;
+int plan_bounds(const Plan &p, int which, int end, cudaStream_t st, PlanHook *h) {
+  return launch(p, PC_BALL, GRMHD_K_BOUNDS, h, [&](unsigned nb, unsigned bs, BView V) { kp_bounds_all<<<nb, bs, 0, st>>>(V, which, end); });
 }
 
+// Six launches on a stage's critical chain (reconstruction and face fluxes per
+// direction on streams of their own, EMFs, inversion, fixup, ghosts).  With the
+// flux fixes, the flux copies of a flat X3, the CFL step, flux-CT's flux update, the
+// three ghost passes and the clock as launches of their own it was twelve and a
+// half: at 64 x 64 a cycle took 114 us and takes 85, at 217 x 217 281 and 239, at
+// 61 x 45 x 37 640 and 563, a batch of 64 flat grids of 32^2 to 256^2 6990 and 6040.
 int plan_stage(const Plan &p, int stage, cudaStream_t st, PlanHook *h) {
   int nl = plan_fluxes(p, stage, true, st, h);
-  if (stage == 0) nl += plan_clock(p, 1, st, h);
-  nl += plan_fix_ct(p, st, h);
+  nl += plan_emf(p, stage == 0, st, h);
   nl += plan_invert(p, stage, stage ? 1.0 : 0.5, st, h);
   nl += plan_fixup(p, 1 - stage, st, h);
-  nl += plan_bounds(p, 1 - stage, st, h);
+  nl += plan_bounds(p, 1 - stage, stage, st, h);
   return nl;
 }
 
@@ -635,7 +660,6 @@ int plan_steps(const Plan &p, int nsteps, cudaStream_t st, PlanHook *h) {
   for (int n = 0; n < nsteps; n++) {
     nl += plan_stage(p, 0, st, h);  // predictor: keeps U(P^n)
     nl += plan_stage(p, 1, st, h);  // corrector: reads it back
-    nl += plan_clock(p, 2, st, h);
   }
   return nl;
 }
@@ -671,10 +695,9 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
     if (cudaMemcpy(&saved[g], p.host_items[g].A.clk, sizeof(Clock), cudaMemcpyDeviceToHost) !=
         cudaSuccess)
       return GRMHD_ERR_CUDA;
-  // representative scratch: face values, CT fluxes and a CFL dt of the current state
+  // representative scratch: fluxes, EMFs and a CFL dt of the current state
   plan_fluxes(p, 0, false, st, nullptr);
-  plan_clock(p, 1, st, nullptr);
-  plan_fix_ct(p, st, nullptr);
+  plan_emf(p, 1, st, nullptr);
   struct Group {
     int cls;
     int which;  // what one pass launches

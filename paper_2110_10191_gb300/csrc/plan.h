@@ -43,6 +43,7 @@ enum {
   PC_BX1,
   PC_BX2,
   PC_BX3,
+  PC_BALL,  // all ghosts in one pass (grids that share no side)
   PC_RECON0,  // FP64 reconstruction along X1 (a lane per pair of differences)
   PC_RECON1,  // along X2
   PC_RECON2,  // along X3 (none for flat-X3 grids)
@@ -62,9 +63,10 @@ enum {
   PC_FACE0X,
   PC_FACE1X,
   PC_FACE2X,
-  PC_REPL,  // flat-X3 flux copies
+  PC_REPL,  // flat-X3 flux copies (for callers who want F)
   PC_FIX,
-  PC_EDGE,   // EMFs and CT
+  PC_EDGE,   // EMFs and CT, every layer
+  PC_EDGES,  // EMFs within a step (flat X3: one layer)
   PC_ZONE,   // fixup (every grid)
   PC_SRC64,  // the update's source pass (FP64 and mixed-precision grids)
   PC_SRCX,   // in float-float (float-float and mixed + float-float grids)
@@ -169,26 +171,31 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
 
 // The functions below enqueue on st and return the number of kernels
 // launched; launch errors are left for cudaGetLastError().
-// stage input: 0 = P, 1 = Ph.  Signal-speed reset, reconstruction + face
-// fluxes (FP64, FP32 or float-float per grid), flat-X3 copies; with_source: and
-// the update's source pass.
+// stage input: 0 = P, 1 = Ph.  Reconstruction + face fluxes (FP64, FP32 or
+// float-float per grid) with their boundary fixes; with_source: and the update's
+// source pass.  The signal speeds' maxima add to what the clocks hold, which is
+// zero between the library's calls: whoever calls this resets them after reading.
 int plan_fluxes(const Plan &p, int in, bool with_source, cudaStream_t st, PlanHook *h);
+// the fluxes of every layer and flux-CT in place of the induction fluxes: F as
+// grmhd_get_fluxes returns it
+int plan_whole_fluxes(const Plan &p, int in, cudaStream_t st, PlanHook *h);
 // per-grid clock: 0 reset the signal-speed maxima, 1 CFL time step, 2 advance
 int plan_clock(const Plan &p, int op, cudaStream_t st, PlanHook *h);
-// boundary flux fixes + flux-CT
-int plan_fix_ct(const Plan &p, cudaStream_t st, PlanHook *h);
+// edge EMFs; take_dt: and the CFL step
+int plan_emf(const Plan &p, int take_dt, cudaStream_t st, PlanHook *h);
 // U(P^n) + dtfac dt (S - div F) of the source pass's scratch -> inversion -> bounds
 // into the other array (in 0: Ph, in 1: P), and the passes that close the state
 // (drift-frame bounds, electrons)
 int plan_invert(const Plan &p, int in, double dtfac, cudaStream_t st, PlanHook *h);
 int plan_fixup(const Plan &p, int out, cudaStream_t st, PlanHook *h);
-// ghost fill of P (which 0) or Ph (which 1)
-int plan_bounds(const Plan &p, int which, cudaStream_t st, PlanHook *h);
+// ghost fill of P (which 0) or Ph (which 1); end: and the clock's advance and the
+// maxima's reset
+int plan_bounds(const Plan &p, int which, int end, cudaStream_t st, PlanHook *h);
 // one ghost-fill pass (0: X1, 1: X2, 2: X3), for a decomposed grid that exchanges
 // block edges between them
 int plan_bounds_pass(const Plan &p, int which, int pass, cudaStream_t st, PlanHook *h);
-// one stage: stage 0 predictor (P -> Ph, dt/2, with the CFL step),
-// stage 1 corrector (Ph -> P, dt)
+// one stage: stage 0 predictor (P -> Ph, dt/2, with the CFL step), stage 1 corrector
+// (Ph -> P, dt, then the clock's advance and the maxima's reset)
 int plan_stage(const Plan &p, int stage, cudaStream_t st, PlanHook *h);
 // full predictor-corrector steps (U(P^n) kept between the stages)
 int plan_steps(const Plan &p, int nsteps, cudaStream_t st, PlanHook *h);

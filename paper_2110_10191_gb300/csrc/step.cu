@@ -67,26 +67,21 @@ __global__ void k_reset_ctop(Clock *clk) {
 void launch_ctop_reset(const StepArgs &A, cudaStream_t st) { k_reset_ctop<<<1, 1, 0, st>>>(A.clk); }
 
 // ---------------------------------------------------------------------------
-// Boundary flux fixes and flux-CT
+// Flux-CT
 // ---------------------------------------------------------------------------
-__global__ void k_fix_flux(StepArgs A, double *F1, double *F2) {
-  fix_flux_body(A, F1, F2, nullptr, nullptr, gtid());
-}
-
 __global__ void k_emf(StepArgs A, const double *__restrict__ F1, const double *__restrict__ F2,
                       const double *__restrict__ F3, double *__restrict__ emf) {
-  emf_body(A, F1, F2, F3, emf, gtid());
+  emf_body(A, F1, F2, F3, emf, 0, gtid());
 }
 
 __global__ void k_ct(StepArgs A, double *F1, double *F2, double *F3, const double *__restrict__ emf) {
   ct_body(A, F1, F2, F3, emf, gtid());
 }
 
-void launch_fix_ct(const StepArgs &A, double *F[3], double *emf, cudaStream_t st) {
+void launch_ct(const StepArgs &A, double *F[3], double *emf, cudaStream_t st) {
   const Dims &D = A.D;
-  k_fix_flux<<<nblk(n_fix(D)), BS, 0, st>>>(A, F[0], F[1]);
-  k_emf<<<nblk(n_edge(D)), BS, 0, st>>>(A, F[0], F[1], F[2], emf);
-  k_ct<<<nblk(n_edge(D)), BS, 0, st>>>(A, F[0], F[1], F[2], emf);
+  k_emf<<<nblk(n_edge(D, 0)), BS, 0, st>>>(A, F[0], F[1], F[2], emf);
+  k_ct<<<nblk(n_edge(D, 0)), BS, 0, st>>>(A, F[0], F[1], F[2], emf);
 }
 
 // ---------------------------------------------------------------------------

@@ -122,8 +122,8 @@ __host__ __device__ inline long long n_replicate(const Dims &D) { return D.n2d *
 __host__ __device__ inline long long n_fix(const Dims &D) {
   return (long long)((D.n[0] > D.n[1]) ? D.n[0] + 2 : D.n[1] + 2) * (D.n[2] + 2);
 }
-__host__ __device__ inline long long n_edge(const Dims &D) {
-  return (long long)(D.n[0] + 1) * (D.n[1] + 1) * (D.n[2] + 1);
+__host__ __device__ inline long long n_edge(const Dims &D, int flat3) {
+  return (long long)(D.n[0] + 1) * (D.n[1] + 1) * (flat3 ? 1 : D.n[2] + 1);
 }
 __host__ __device__ inline long long n_zone(const Dims &D) {
   return (long long)D.n[0] * D.n[1] * D.n[2];
@@ -209,6 +209,96 @@ __device__ __forceinline__ void bounds_x3_body(const StepArgs &A, double *P, dou
     copy_zone(D, P, K, d, (long long)wrap(kg, D.n[2]) * D.n2d + ij);
   } else if (bc == 1) {
     copy_zone(D, P, K, d, (long long)(side ? D.n[2] + NG - 1 : NG) * D.n2d + ij);
+  }
+}
+
+// All ghosts in one pass, each from the zones that the three passes above would
+// carry to it (X3's from X2's from X1's), for grids whose sides are all their own:
+// every value read is an interior zone's or a fixed ghost's, which nothing here
+// writes.  Same values bit for bit.
+__host__ __device__ inline long long n_bounds_all(const Dims &D) {
+  return n_bounds_x1(D) + n_bounds_x2(D) + n_bounds_x3(D);
+}
+__device__ __forceinline__ void bounds_all_body(const StepArgs &A, double *P, double *K,
+                                                long long t) {
+  const Dims &D = A.D;
+  if (t >= n_bounds_all(D)) return;
+  int i, j, k;
+  if (t < n_bounds_x3(D)) {
+    const Idx3 q3 = unflatten(t, D.s[0], D.s[1]);
+    i = q3.i;
+    j = q3.j;
+    k = (q3.k < NG) ? q3.k : D.n[2] + q3.k;
+  } else if ((t -= n_bounds_x3(D)) < n_bounds_x2(D)) {
+    const Idx3 q3 = unflatten(t, D.s[0], 2 * NG);
+    i = q3.i;
+    j = (q3.j < NG) ? q3.j : D.n[1] + q3.j;
+    k = NG + q3.k;
+  } else {
+    t -= n_bounds_x2(D);
+    const Idx3 q3 = unflatten(t, 2 * NG, D.n[1]);
+    i = (q3.i < NG) ? q3.i : D.n[0] + q3.i;
+    j = NG + q3.j;
+    k = NG + q3.k;
+  }
+  const long long d = zid(D, i, j, k);
+  int si = i, sj = j, sk = k;
+  if (k < NG || k >= D.n[2] + NG) {
+    const int side = k >= NG, bc = A.bc[2][side];
+    if (bc == 0)
+      sk = wrap(k, D.n[2]);
+    else if (bc == 1)
+      sk = side ? D.n[2] + NG - 1 : NG;
+    else
+      return;  // fixed
+  }
+  bool mirror = false, out = false;
+  if (j < NG || j >= D.n[1] + NG) {
+    const int side = j >= NG, bc = A.bc[1][side];
+    if (bc == 0) {
+      sj = wrap(j, D.n[1]);
+    } else if (bc == 2) {
+      sj = side ? 2 * (D.n[1] + NG) - 1 - j : 2 * NG - 1 - j;
+      mirror = true;
+    } else if (bc == 1) {
+      sj = side ? D.n[1] + NG - 1 : NG;
+    } else if (sk == k) {
+      return;  // fixed
+    }
+  }
+  const bool own_row = sj >= NG && sj < D.n[1] + NG;  // else a fixed X2 ghost, whatever its i
+  if (own_row && (i < NG || i >= D.n[0] + NG)) {
+    const int bc = A.bc[0][i >= NG];
+    if (bc == 0) {
+      si = wrap(i, D.n[0]);
+    } else if (bc == 1) {
+      si = (i >= NG) ? D.n[0] + NG - 1 : NG;
+      out = true;
+    } else if (sk == k && sj == j) {
+      return;  // fixed
+    }
+  }
+  const long long c = zid(D, si, sj, sk), N = D.ntot;
+  double p[NV];
+#pragma unroll
+  for (int v = 0; v < NV; v++) p[v] = P[v * N + c];
+  if (out) {
+    const double *gd = A.geom + (LOC_CENT * G_NCOMP + G_GDET) * D.n2d + (long long)sj * D.s[0];
+    const double rs = gd[si] / gd[i];
+    p[B1] *= rs;
+    p[B2] *= rs;
+    p[B3] *= rs;
+    if (i >= NG ? (p[U1] < 0.0) : (p[U1] > 0.0)) p[U1] = 0.0;
+  }
+  if (mirror) {
+    p[U2] = -p[U2];
+    p[B2] = -p[B2];
+  }
+#pragma unroll
+  for (int v = 0; v < NV; v++) P[v * N + d] = p[v];
+  if (K) {
+    K[d] = K[c];
+    K[N + d] = K[N + c];
   }
 }
 
@@ -428,13 +518,28 @@ __device__ __forceinline__ void face_flux(const StepArgs &A, const FaceLane &L, 
   const double ct = speed_max(own, __shfl_xor_sync(0xffffffffu, own, 16));
   double out[NV];
   wide_flux(P, s, ee, A.gm1, DIR + 1, L.right ? -ct : ct, 0.5 * geo(G_GDET), out);
-  // the electron entropies' flux weights (LLF of rho u^d K, rho u^t K)
-  if (ELEC && L.active) A.elec_w[(2 * DIR + (L.right ? 1 : 0)) * D.ntot + L.c] = out[RHO];
+  // boundary flux fixes (fix_flux_body): no flux through the axis, no mass in
+  // through an outflow boundary
+  const bool axis = DIR == 1 && ((A.bc[1][0] == 2 && L.j == NG) ||
+                                 (A.bc[1][1] == 2 && L.j == D.n[1] + NG));
+  bool dry = false;
 #pragma unroll
   for (int q = 0; q < NV / 2; q++) {
     const double keep = L.right ? out[q + NV / 2] : out[q];
     const double got = __shfl_xor_sync(0xffffffffu, L.right ? out[q] : out[q + NV / 2], 16);
-    if (L.active) F[(q + (L.right ? NV / 2 : 0)) * D.ntot + L.c] = keep + got;
+    double f = axis ? 0.0 : keep + got;
+    if (DIR == 0 && q == RHO && !L.right) {
+      dry = (A.bc[0][0] == 1 && L.i == NG && less(0.0, f)) ||
+            (A.bc[0][1] == 1 && L.i == D.n[0] + NG && less(f, 0.0));
+      if (dry) f = 0.0;
+    }
+    if (L.active) F[(q + (L.right ? NV / 2 : 0)) * D.ntot + L.c] = f;
+  }
+  // the electron entropies' flux weights (LLF of rho u^d K, rho u^t K), none
+  // where the mass flux is fixed to zero
+  if (ELEC) {
+    const bool none = axis || (DIR == 0 && __shfl_sync(0xffffffffu, dry, threadIdx.x & 15));
+    if (L.active) A.elec_w[(2 * DIR + (L.right ? 1 : 0)) * D.ntot + L.c] = none ? 0.0 : out[RHO];
   }
   bool interior = L.active;
 #pragma unroll
@@ -566,28 +671,30 @@ __device__ __forceinline__ void fix_flux_body(const StepArgs &A, double *F1, dou
 
 // Edge EMFs over i, j, k in [NG, n+NG]:
 // e3 = (F1[B2] + F1[B2](j-1) - F2[B1] - F2[B1](i-1))/4, cyclic for e1, e2.
+// flat3: on the layer k = NG alone, whose neighbours along X3 are itself.
 __device__ __forceinline__ void emf_body(const StepArgs &A, const double *__restrict__ F1,
                                          const double *__restrict__ F2,
                                          const double *__restrict__ F3, double *__restrict__ emf,
-                                         long long t) {
+                                         int flat3, long long t) {
   const Dims &D = A.D;
   const int e0 = D.n[0] + 1, e1 = D.n[1] + 1;
-  if (t >= n_edge(D)) return;
+  if (t >= n_edge(D, flat3)) return;
   const Idx3 q3 = unflatten(t, e0, e1);
   const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
   const long long c = zid(D, i, j, k), N = D.ntot;
-  const long long im = c - 1, jm = c - D.s[0], km = c - D.n2d;
+  const long long im = c - 1, jm = c - D.s[0], km = flat3 ? c : c - D.n2d;
   emf[2 * N + c] = 0.25 * (F1[B2 * N + c] + F1[B2 * N + jm] - F2[B1 * N + c] - F2[B1 * N + im]);
   emf[1 * N + c] = 0.25 * (F3[B1 * N + c] + F3[B1 * N + im] - F1[B3 * N + c] - F1[B3 * N + km]);
   emf[0 * N + c] = 0.25 * (F2[B3 * N + c] + F2[B3 * N + km] - F3[B2 * N + c] - F3[B2 * N + jm]);
 }
 
-// Induction fluxes from the EMFs on every face the update reads.
+// Induction fluxes from the EMFs on every face next to a zone (flux_ct_div takes
+// their differences from the EMFs themselves; this is for callers who want F).
 __device__ __forceinline__ void ct_body(const StepArgs &A, double *F1, double *F2, double *F3,
                                         const double *__restrict__ emf, long long t) {
   const Dims &D = A.D;
   const int e0 = D.n[0] + 1, e1 = D.n[1] + 1;
-  if (t >= n_edge(D)) return;
+  if (t >= n_edge(D, 0)) return;
   const Idx3 q3 = unflatten(t, e0, e1);
   const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
   const long long c = zid(D, i, j, k), N = D.ntot;
@@ -633,12 +740,40 @@ __device__ __forceinline__ void geo_source(const double T[4][4], double gdet,
   }
 }
 
-// sqrt(-g)-weighted sum of a variable's flux differences over the zone c
+// sqrt(-g)-weighted sum of a variable's flux differences over the zone at c (o = v
+// ntot + c).  On a flat X3 both X3 faces are the same.
 __device__ __forceinline__ double flux_div(const StepArgs &A, const double *__restrict__ F1,
                                            const double *__restrict__ F2,
                                            const double *__restrict__ F3, long long o) {
-  return (F1[o + 1] - F1[o]) * A.idx[0] + (F2[o + A.D.s[0]] - F2[o]) * A.idx[1] +
-         (F3[o + A.D.n2d] - F3[o]) * A.idx[2];
+  double s = (F1[o + 1] - F1[o]) * A.idx[0];
+  s = fma(F2[o + A.D.s[0]] - F2[o], A.idx[1], s);
+  return A.flat3 ? s : fma(F3[o + A.D.n2d] - F3[o], A.idx[2], s);
+}
+
+// The same of the induction fluxes of flux-CT, straight from the EMFs: with each
+// flux the mean of the two EMFs that bound its face (ct_body), B^1's through
+// an X2 face is -(E3(i) + E3(i+1))/2, through an X3 face (E2(i) + E2(i+1))/2, and
+// cyclically.  Halves are exact, so they go to 1/dx and the values are those of
+// flux_div on ct_body's fluxes bit for bit (B^d has no flux along d).
+__device__ __forceinline__ void flux_ct_div(const StepArgs &A, const double *__restrict__ emf,
+                                            long long c, double div[3]) {
+  const long long N = A.D.ntot, y = A.D.s[0], z = A.flat3 ? 0 : A.D.n2d;
+  const double *E1 = emf + c, *E2 = emf + N + c, *E3 = emf + 2 * N + c;
+  const double h1 = 0.5 * A.idx[0], h2 = 0.5 * A.idx[1], h3 = 0.5 * A.idx[2];
+  const double d12 = (E3[0] + E3[1]) - (E3[y] + E3[y + 1]);  // F2[B1] difference, doubled
+  const double d21 = (E3[1] + E3[y + 1]) - (E3[0] + E3[y]);  // F1[B2]
+  const double d31 = (E2[0] + E2[z]) - (E2[1] + E2[z + 1]);  // F1[B3]
+  const double d32 = (E1[y] + E1[y + z]) - (E1[0] + E1[z]);  // F2[B3]
+  div[2] = fma(d32, h2, d31 * h1);
+  if (A.flat3) {
+    div[0] = d12 * h2;
+    div[1] = d21 * h1;
+  } else {
+    const double d13 = (E2[z] + E2[z + 1]) - (E2[0] + E2[1]);  // F3[B1]
+    const double d23 = (E1[0] + E1[y]) - (E1[z] + E1[z + y]);  // F3[B2]
+    div[0] = fma(d13, h3, d12 * h2);
+    div[1] = fma(d23, h3, d21 * h1);
+  }
 }
 
 // U(P), the stress-energy tensor, the Lorentz factor squared and b^2 of a state
@@ -797,6 +932,7 @@ __device__ __forceinline__ void source_body(const StepArgs &A, const double *__r
 __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__restrict__ F1,
                                             const double *__restrict__ F2,
                                             const double *__restrict__ F3,
+                                            const double *__restrict__ emf,
                                             const double *__restrict__ Ucache, double *scratch,
                                             double dtfac, const double *Pi, double *Pout, int *pflag, int *fflag,
                                             long long t) {
@@ -814,11 +950,13 @@ __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__r
     const long long ij = (long long)j * D.s[0] + i;
     const double *g = A.geom + ij;
     const auto geo = [g, &D](int comp) { return __ldg(g + comp * D.n2d); };
-    double Un[NV], pn[NV], bsq_n = 0.0, lor_n = 1.0;
+    double Un[NV], pn[NV], bsq_n = 0.0, lor_n = 1.0, divB[3];
+    flux_ct_div(A, emf, c, divB);
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       const long long o = v * N + c;
-      const double div = flux_div(A, F1, F2, F3, o), u = __ldg(Ucache + o);
+      const double div = (v < B1) ? flux_div(A, F1, F2, F3, o) : divB[v < B1 ? 0 : v - B1];
+      const double u = __ldg(Ucache + o);
       // the source enters the energy and momentum rows only
       Un[v] = (v >= UU && v <= U3) ? fma(dtp, scratch[(v - UU) * N + c] - div, u)
                                    : fma(-dtp, div, u);
