@@ -21,6 +21,7 @@
 #pragma once
 
 #include "step_bodies.cuh"
+#include "wide_pow.cuh"
 
 namespace grmhd {
 
@@ -76,6 +77,17 @@ static __device__ __noinline__ double elec_fraction(const StepArgs &A, double rh
   return 0.0;
 }
 
+// kappa_e after the heating (elec_post_body) of a zone in FP64
+static __device__ __noinline__ double elec_heat(const StepArgs &A, double rho_s, double u_s,
+                                                double kel_s, double bsq_s, double rho_n,
+                                                double u_n, const double kn[2]) {
+  const double ls = log(rho_s);
+  const double fel = elec_fraction(A, rho_s, ls, u_s, kel_s, bsq_s);
+  const double ktot = (A.gam - 1.0) * u_n / exp(A.gam * log(rho_n));
+  return kn[1] + fel * (A.game - 1.0) / (A.gam - 1.0) * exp((A.gam - A.game) * ls) *
+                     (ktot - kn[0]);
+}
+
 // The closing steps of a zone once the fluid's bounds are done: u lowered
 // to P_gas/rho^gamma = 3 where it exceeds that (with the bounds on),
 // kappa_tot reset to (gamma - 1) u / rho^gamma, kappa_e held to
@@ -83,7 +95,8 @@ static __device__ __noinline__ double elec_fraction(const StepArgs &A, double rh
 // gamma_e) / ((gamma - 1)/(gamma_e - 1) + R (gamma - 1)/(gamma_p - 1)) at
 // R = tpte_max .. tpte_min (a kappa_e that is not a number takes the lower).
 // lr = ln P[RHO].
-__device__ __forceinline__ int elec_close(const StepArgs &A, double P[NV], double K[2], double lr) {
+static __device__ __noinline__ int elec_close(const StepArgs &A, double P[NV], double K[2],
+                                              double lr) {
   int fl = 0;
   const double g1 = A.gam - 1.0;
   const double rg = exp(A.gam * lr);
@@ -103,6 +116,75 @@ __device__ __forceinline__ int elec_close(const StepArgs &A, double P[NV], doubl
   if (!(kel == kel)) kel = kmin;
   K[1] = fmin(fmax(kel, kmin), kmax);
   return fl;
+}
+
+// ---------------------------------------------------------------------------
+// The same in Wide numbers (wide_num.cuh, wide_pow.cuh).  With log, exp, pow and
+// the divisions in FP64 the pass after the update was bound by that unit's 460
+// instructions a zone: 0.84 ms per launch on a 96^3 grid with Kawazura's model, 0.15
+// now.  Zones whose state leaves the range the powers are taken in (densities within
+// 2^+-52, energies and entropies within 2^+-100) take the FP64 form above; b^2 may be
+// anything finite, since beta is held within 1e+-20 (rounding leaves b^2 of 1e-40 and
+// less around a magnetised region).
+// ---------------------------------------------------------------------------
+constexpr int ELEC_RHO_RANGE = 52, ELEC_RANGE = 100;
+
+// elec_fraction's heating of kn[1]: the advected entropies kn, the source state s,
+// the new state n; ln: log2 rho_n, kt: kappa_tot of the new state.  False: take the
+// FP64 form.
+__device__ __forceinline__ bool elec_heat_wide(const StepArgs &A, double rho_s, double u_s,
+                                               double kel_s, double bsq_s, double rho_n,
+                                               double u_n, Wide kn[2], s64 &ln, Wide &kt) {
+  if (!w_within(rho_s, ELEC_RHO_RANGE) || !w_within(rho_n, ELEC_RHO_RANGE) ||
+      !w_within(u_s, ELEC_RANGE) || !w_within(u_n, ELEC_RANGE) || !w_within(kel_s, ELEC_RANGE) ||
+      !w_finite(bsq_s))
+    return false;
+  const s64 l = w_log2(wide_pos(rho_s));
+  const Wide ls = w_log_num(l);
+  Wide fel;
+  if (A.elec == GRMHD_ELEC_KAWAZURA) {
+    fel = wide_kawazura(A.game, A.gamp, A.ek.ige, rho_s, ls, u_s, kel_s, bsq_s);
+  } else {
+    const double f = elec_fraction(A, rho_s, (double)l * (0.6931471805599453 * 0x1p-55), u_s,
+                                   kel_s, bsq_s);
+    if (!w_finite(f)) return false;
+    fel = wide(f);
+  }
+  ln = w_log2(wide_pos(rho_n));
+  kt = wide_pos(A.gm1) * wide_pos(u_n) * w_exp2(-(w_log_num(ln) * wide_pos(A.gam)));
+  const Wide heat = fel * wide_pos(A.ek.c) * w_exp2(ls * wide(A.ek.dgam)) *
+                    norm(w_sum<0>(kt, -kn[0]));
+  kn[1] = w_sum<0>(kn[1], heat);
+  return true;
+}
+
+// elec_close from Wide entropies: moved: the bounds changed P (rho0: its density
+// before), else ln and kt hold.  False: take the FP64 form (P unchanged).
+__device__ __forceinline__ bool elec_close_wide(const StepArgs &A, double P[NV], bool moved,
+                                                double rho0, s64 ln, Wide kt, const Wide &kel,
+                                                double K[2], int &fl) {
+  if (!w_within(P[RHO], ELEC_RHO_RANGE) || !w_within(P[UU], ELEC_RANGE)) return false;
+  fl = 0;
+  if (moved && P[RHO] != rho0) ln = w_log2(wide_pos(P[RHO]));
+  const Wide l = w_log_num(ln);
+  const Wide rg = w_exp2(-(l * wide_pos(A.gam)));
+  if (moved) kt = wide_pos(A.gm1) * wide_pos(P[UU]) * rg;
+  K[0] = w_to_double(kt);
+  if (A.floors_on && less(KTOT_MAX, K[0])) {
+    P[UU] = w_to_double(wide_pos(KTOT_MAX) * wide_pos(A.ek.ig) * w_rcp(norm(rg)));
+    fl = FF_KTOT;
+    kt = wide_pos(A.gm1) * wide(P[UU]) * rg;
+    K[0] = w_to_double(kt);
+  }
+  const Wide kk = norm(kt * w_exp2(l * wide(A.ek.dgam)));
+  const Wide dmin = wide_pos(A.ek.dmin), dmax = wide_pos(A.ek.dmax), k = norm(kel);
+  if (w_sum<1>(k * dmin, -kk).s)
+    K[1] = w_to_double(kk * w_rcp(dmin));
+  else if (w_sum<1>(kk, -(k * dmax)).s)
+    K[1] = w_to_double(kk * w_rcp(dmax));
+  else
+    K[1] = w_to_double(k);
+  return true;
 }
 
 // Zone-centric reconstruction of both entropies along DIR (the zones of
@@ -193,34 +275,53 @@ __device__ __forceinline__ void elec_post_body(const StepArgs &A, const double *
     const long long c = zid(D, i, j, k), N = D.ntot;
     const long long ij = (long long)j * D.s[0] + i;
     const double rho_s = Ps[RHO * N + c], u_s = Ps[UU * N + c], Uri = Ucache[RHO * N + c];
-    const double idx1 = A.idx[0], idx2 = A.idx[1], idx3 = A.idx[2];
-    const long long o = RHO * N + c;
-    const double divr = (F1[o + 1] - F1[o]) * idx1 + (F2[o + D.s[0]] - F2[o]) * idx2 +
-                        (F3[o + D.n2d] - F3[o]) * idx3;
-    const double Urn = Uri + dtp * (0.0 - divr);
-    double kn[2];
+    const double Urn = fma(-dtp, flux_div(A, F1, F2, F3, RHO * N + c), Uri);
+    double num[2], kn[2];
 #pragma unroll
     for (int q = 0; q < 2; q++) {
       const long long oq = q * N + c;
-      const double divk = (FK1[oq + 1] - FK1[oq]) * idx1 + (FK2[oq + D.s[0]] - FK2[oq]) * idx2 +
-                          (FK3[oq + D.n2d] - FK3[oq]) * idx3;
-      kn[q] = (Uri * Ki[oq] + dtp * (0.0 - divk)) / Urn;
+      num[q] = fma(-dtp, flux_div(A, FK1, FK2, FK3, oq), Uri * Ki[oq]);
+    }
+    const bool in_range = A.ek.wide && w_within(Urn, ELEC_RANGE) &&
+                          w_within(fabs(num[0]), 2 * ELEC_RANGE) &&
+                          w_within(fabs(num[1]), 2 * ELEC_RANGE);
+    Wide kw[2];
+    if (in_range) {
+      const Wide r = w_rcp(wide_pos(Urn));
+#pragma unroll
+      for (int q = 0; q < 2; q++) {
+        kw[q] = wide(num[q]) * r;
+        kn[q] = w_to_double(kw[q]);
+      }
+    } else {
+      kn[0] = num[0] / Urn;
+      kn[1] = num[1] / Urn;
     }
     if (pflag[c] == 0) {
       double pn[NV];
 #pragma unroll
       for (int v = 0; v < NV; v++) pn[v] = Pout[v * N + c];
-      const double ls = log(rho_s), ln = log(pn[RHO]);
-      const double fel = elec_fraction(A, rho_s, ls, u_s, Ks[N + c], scratch[SCR_BSQ_S * N + c]);
-      const double ktot_new = (A.gam - 1.0) * pn[UU] / exp(A.gam * ln);
-      kn[1] = kn[1] + fel * (A.game - 1.0) / (A.gam - 1.0) * exp((A.gam - A.game) * ls) *
-                          (ktot_new - kn[0]);
-      const double rho_n = pn[RHO];
+      const double rho_n = pn[RHO], u_n = pn[UU], kel_s = Ks[N + c];
+      const double bsq_s = scratch[SCR_BSQ_S * N + c];
+      s64 ln = 0;
+      Wide kt;
+      const bool wide_zone =
+          in_range && elec_heat_wide(A, rho_s, u_s, kel_s, bsq_s, rho_n, u_n, kw, ln, kt);
+      if (!wide_zone) kn[1] = elec_heat(A, rho_s, u_s, kel_s, bsq_s, rho_n, u_n, kn);
       if (A.floors_on) {
         const double bsq = scratch[SCR_BSQ * N + c], lor = scratch[SCR_LORENTZ * N + c];
         ff = A.floor_drift ? floors_drift(A, ij, pn, bsq, lor) : floors_fluid(A, ij, pn, bsq, lor);
       }
-      ff |= elec_close(A, pn, kn, (pn[RHO] == rho_n) ? ln : log(pn[RHO]));
+      int fk;
+      if (!wide_zone || !elec_close_wide(A, pn, ff != 0, rho_n, ln, kt, kw[1], kn, fk)) {
+        if (wide_zone) kn[1] = w_to_double(kw[1]);
+        double p[NV];
+        p[RHO] = pn[RHO];
+        p[UU] = pn[UU];
+        fk = elec_close(A, p, kn, log(p[RHO]));
+        pn[UU] = p[UU];
+      }
+      ff |= fk;
 #pragma unroll
       for (int v = 0; v < NV; v++) Pout[v * N + c] = pn[v];
       fflag[c] = ff;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "grmhd_dev.cuh"
 
 namespace grmhd {
@@ -32,6 +34,14 @@ struct Clock {
   int coupled;
 };
 
+// Constants of the electron entropies' pass: (gamma_e - 1)/(gamma - 1), 1/(gamma_e -
+// 1), 1/(gamma - 1), gamma - gamma_e, and P_gas/rho^gamma over the kappa_e bound at T_p/T_e
+// = tpte_max and tpte_min.  wide: all within the range of its Wide numbers.
+struct ElecK {
+  double c, ige, ig, dgam, dmin, dmax;
+  int wide;
+};
+
 // boundary code of a side shared with another block of a decomposed grid:
 // the bounds leave its ghosts to the exchange between blocks
 constexpr int BC_EXCHANGE = 4;
@@ -51,6 +61,7 @@ struct StepArgs {
   // electrons and protons, the constant share, the bounds on T_p/T_e
   int elec;
   double game, gamp, fel_const, tpte_min, tpte_max;
+  ElecK ek;  // (set_elec_constants)
   // electrons: per face, the weights of the left and right entropies in
   // their LLF flux, [3][2][ntot] (direction, side)
   double *elec_w;
@@ -78,6 +89,19 @@ inline void set_gas_constants(StepArgs &A) {
   A.gk.gf = (A.gam - 1.0) / A.gam;
   A.gk.ubd = 2.0 * (A.gam - 1.0);
   A.gk.ubd_rcp = 1.0 / A.gk.ubd;
+}
+
+inline void set_elec_constants(StepArgs &A) {
+  const double g1 = A.gam - 1.0, a = g1 / (A.game - 1.0), b = g1 / (A.gamp - 1.0);
+  A.ek.c = (A.game - 1.0) / g1;
+  A.ek.ige = 1.0 / (A.game - 1.0);
+  A.ek.ig = 1.0 / g1;
+  A.ek.dgam = A.gam - A.game;
+  A.ek.dmin = std::fma(A.tpte_max, b, a);
+  A.ek.dmax = std::fma(A.tpte_min, b, a);
+  // powers of densities within 2^+-52 then stay below 2^127
+  A.ek.wide = A.gam <= 2.4 && A.game <= 2.4 && A.gamp <= 1e9 && g1 >= 1e-9 &&
+              A.game - 1.0 >= 1e-9 && A.gamp - 1.0 >= 1e-9 && A.ek.dmin <= 1e20;
 }
 
 // the float-float words of the adiabatic-index constants
