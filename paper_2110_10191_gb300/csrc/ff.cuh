@@ -60,17 +60,20 @@ __device__ __forceinline__ ff ff_from(double x) {
   return r;
 }
 
-// The same on the integer pipes where both words are normal floats: the bits
-// taken apart, the remainder, 29 bits, converted as an integer (a tie may round
-// the other way, the sum of the words stays the same).
+// The same on the integer pipes where the high word is a normal float or zero: the
+// bits taken apart, the remainder, 29 bits, converted as an integer and scaled in two
+// steps of which only the last may round, to a subnormal (a tie of the high word may
+// round the other way, the sum of the words stays the same).
 __device__ __forceinline__ ff ff_from_bits(double x) {
   const u64 b = w_bits(x);
   const u32 sign = w_hi(b) & 0x80000000u;
   const int e = (int)((w_hi(b) >> 20) & 0x7ff);
-  if ((u32)(e - 950) >= 200u) return ff_from(x);
+  if (e < 873) return ff{__uint_as_float(sign), __uint_as_float(sign)};  // below float's last place
+  if ((u32)(e - 897) >= 240u) return ff_from(x);
   const u64 m = (b & (~0ull >> 1)) + (1ull << 28);
   const int rest = (int)(w_lo(b) << 3) >> 3;  // x - hi in units of x's last place
-  const float lo = __fmul_rn(__int2float_rn(rest), __int_as_float((e - 948) << 23));
+  const float lo = __fmul_rn(__fmul_rn(__int2float_rn(rest), 0x1p-64f),
+                             __int_as_float((e - 884) << 23));
   ff r;
   r.hi = __uint_as_float(((u32)(m >> 29) - (896u << 23)) | sign);
   r.lo = __uint_as_float(__float_as_uint(lo) ^ sign);

@@ -78,7 +78,7 @@ __device__ __forceinline__ void to_ff_body(const double *__restrict__ src, float
   if (t >= n) return;
   const double x = src[t];
   ff v;
-  if (fabs(x) > 3.4028234663852886e38) {
+  if ((w_hi(w_bits(x)) & 0x7fffffffu) >= (1151u << 20) && fabs(x) > 3.4028234663852886e38) {
     v.hi = (x > 0.0) ? 3.4028234663852886e38f : -3.4028234663852886e38f;
     v.lo = 0.0f;
   } else {

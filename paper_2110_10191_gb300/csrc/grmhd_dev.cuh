@@ -481,11 +481,35 @@ __device__ __forceinline__ int invert_1dw(const double U[NV], const Geo &G, cons
 // rho and u of a zone with b^2, whose Lorentz factor is within the cap.  The
 // quotients b^2/sigma, beta b^2 / (2 (gamma - 1)) and u/T are the IEEE
 // divisions' values bit for bit (div_rn).
+// |d| truncated to a float; false where that is no normal float
+__device__ __forceinline__ bool trunc_f(double d, float &f) {
+  const u64 b = w_bits(d) & (~0ull >> 1);
+  f = __uint_as_float((u32)(b >> 29) - (896u << 23));
+  return (w_hi(b) >> 20) - 897u < 253u;
+}
+// That the three bounds below which depend on rho, u and b^2 alone leave P as it
+// is, decided in FP32 with 2^-20 to spare (their quotients take ten FP64 instructions,
+// the bounds raise few zones): false where that is not certain.
+__device__ __forceinline__ bool bounds_clear(double rho, double u, double bsq, const GasK &K) {
+  constexpr float M = 1.0f - 0x1p-20f;
+  float r, w, b, ubd;
+  const bool plain = trunc_f(rho, r) && trunc_f(u, w) && trunc_f(K.ubd, ubd) &&
+                     (s64)w_bits(rho) > 0 && (s64)w_bits(u) > 0;
+  if (!trunc_f(bsq, b)) {
+    if ((w_hi(w_bits(bsq)) & 0x7fffffffu) >= (897u << 20)) return false;
+    b = 0x1p-126f;
+  }
+  const float x = M * r, y = M * w * ubd;
+  return plain && x * (float)FL_SIGMA > b && x * (float)FL_TEMP > w &&
+         y > (float)FL_BETA * b && y > 0x1p-100f;
+}
+
 __device__ __forceinline__ int apply_floors_known(double P[NV], double rho_fl, double u_fl,
                                                   const GasK &K, double bsq) {
   int fl = 0;
   if (less(P[RHO], rho_fl)) { P[RHO] = rho_fl; fl |= FF_RHO_GEOM; }
   if (less(P[UU], u_fl)) { P[UU] = u_fl; fl |= FF_U_GEOM; }
+  if (bounds_clear(P[RHO], P[UU], bsq, K)) return fl;
   const double rs = div_rn(bsq, FL_SIGMA, FL_SIGMA_RCP);
   if (less(P[RHO], rs)) { P[RHO] = rs; fl |= FF_SIGMA; }
   const double ub = div_rn(FL_BETA * bsq, K.ubd, K.ubd_rcp);

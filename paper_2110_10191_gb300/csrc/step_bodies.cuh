@@ -669,8 +669,9 @@ __device__ __forceinline__ void fix_flux_body(const StepArgs &A, double *F1, dou
   }
 }
 
-// Edge EMFs over i, j, k in [NG, n+NG]:
-// e3 = (F1[B2] + F1[B2](j-1) - F2[B1] - F2[B1](i-1))/4, cyclic for e1, e2.
+// Edge EMFs, four times over (the factor goes to 1/dx in flux_ct_div and to the
+// half in ct_body, exactly), over i, j, k in [NG, n+NG]:
+// 4 e3 = F1[B2] + F1[B2](j-1) - F2[B1] - F2[B1](i-1), cyclic for e1, e2.
 // flat3: on the layer k = NG alone, whose neighbours along X3 are itself.
 __device__ __forceinline__ void emf_body(const StepArgs &A, const double *__restrict__ F1,
                                          const double *__restrict__ F2,
@@ -683,9 +684,9 @@ __device__ __forceinline__ void emf_body(const StepArgs &A, const double *__rest
   const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
   const long long c = zid(D, i, j, k), N = D.ntot;
   const long long im = c - 1, jm = c - D.s[0], km = flat3 ? c : c - D.n2d;
-  emf[2 * N + c] = 0.25 * (F1[B2 * N + c] + F1[B2 * N + jm] - F2[B1 * N + c] - F2[B1 * N + im]);
-  emf[1 * N + c] = 0.25 * (F3[B1 * N + c] + F3[B1 * N + im] - F1[B3 * N + c] - F1[B3 * N + km]);
-  emf[0 * N + c] = 0.25 * (F2[B3 * N + c] + F2[B3 * N + km] - F3[B2 * N + c] - F3[B2 * N + jm]);
+  emf[2 * N + c] = F1[B2 * N + c] + F1[B2 * N + jm] - F2[B1 * N + c] - F2[B1 * N + im];
+  emf[1 * N + c] = F3[B1 * N + c] + F3[B1 * N + im] - F1[B3 * N + c] - F1[B3 * N + km];
+  emf[0 * N + c] = F2[B3 * N + c] + F2[B3 * N + km] - F3[B2 * N + c] - F3[B2 * N + jm];
 }
 
 // Induction fluxes from the EMFs on every face next to a zone (flux_ct_div takes
@@ -702,17 +703,17 @@ __device__ __forceinline__ void ct_body(const StepArgs &A, double *F1, double *F
   const bool in1 = i < D.n[0] + NG, in2 = j < D.n[1] + NG, in3 = k < D.n[2] + NG;
   if (in2 && in3) {  // X1 face
     F1[B1 * N + c] = 0.0;
-    F1[B2 * N + c] = 0.5 * (E3[c] + E3[c + D.s[0]]);
-    F1[B3 * N + c] = -0.5 * (E2[c] + E2[c + D.n2d]);
+    F1[B2 * N + c] = 0.125 * (E3[c] + E3[c + D.s[0]]);
+    F1[B3 * N + c] = -0.125 * (E2[c] + E2[c + D.n2d]);
   }
   if (in1 && in3) {  // X2 face
-    F2[B1 * N + c] = -0.5 * (E3[c] + E3[c + 1]);
+    F2[B1 * N + c] = -0.125 * (E3[c] + E3[c + 1]);
     F2[B2 * N + c] = 0.0;
-    F2[B3 * N + c] = 0.5 * (E1[c] + E1[c + D.n2d]);
+    F2[B3 * N + c] = 0.125 * (E1[c] + E1[c + D.n2d]);
   }
   if (in1 && in2) {  // X3 face
-    F3[B1 * N + c] = 0.5 * (E2[c] + E2[c + 1]);
-    F3[B2 * N + c] = -0.5 * (E1[c] + E1[c + D.s[0]]);
+    F3[B1 * N + c] = 0.125 * (E2[c] + E2[c + 1]);
+    F3[B2 * N + c] = -0.125 * (E1[c] + E1[c + D.s[0]]);
     F3[B3 * N + c] = 0.0;
   }
 }
@@ -753,24 +754,26 @@ __device__ __forceinline__ double flux_div(const StepArgs &A, const double *__re
 // The same of the induction fluxes of flux-CT, straight from the EMFs: with each
 // flux the mean of the two EMFs that bound its face (ct_body), B^1's through
 // an X2 face is -(E3(i) + E3(i+1))/2, through an X3 face (E2(i) + E2(i+1))/2, and
-// cyclically.  Halves are exact, so they go to 1/dx and the values are those of
-// flux_div on ct_body's fluxes bit for bit (B^d has no flux along d).
+// cyclically (B^d has no flux along d).  The four EMFs of one kind around the
+// zone enter two such differences each, as p + q and p - q of their differences over
+// the diagonals p = E(0,0) - E(1,1), q = E(1,0) - E(0,1).
 __device__ __forceinline__ void flux_ct_div(const StepArgs &A, const double *__restrict__ emf,
                                             long long c, double div[3]) {
   const long long N = A.D.ntot, y = A.D.s[0], z = A.flat3 ? 0 : A.D.n2d;
   const double *E1 = emf + c, *E2 = emf + N + c, *E3 = emf + 2 * N + c;
-  const double h1 = 0.5 * A.idx[0], h2 = 0.5 * A.idx[1], h3 = 0.5 * A.idx[2];
-  const double d12 = (E3[0] + E3[1]) - (E3[y] + E3[y + 1]);  // F2[B1] difference, doubled
-  const double d21 = (E3[1] + E3[y + 1]) - (E3[0] + E3[y]);  // F1[B2]
-  const double d31 = (E2[0] + E2[z]) - (E2[1] + E2[z + 1]);  // F1[B3]
-  const double d32 = (E1[y] + E1[y + z]) - (E1[0] + E1[z]);  // F2[B3]
+  const double h1 = 0.125 * A.idx[0], h2 = 0.125 * A.idx[1], h3 = 0.125 * A.idx[2];
+  const double p3 = E3[0] - E3[y + 1], q3 = E3[1] - E3[y];
+  const double p2 = E2[0] - E2[z + 1], q2 = E2[z] - E2[1];
+  const double p1 = E1[0] - E1[y + z], q1 = E1[y] - E1[z];
+  // B^2 through X1 faces: E3(1,.) - E3(0,.); B^1 through X2 faces: E3(.,0) - E3(.,1)
+  const double d21 = q3 - p3, d12 = q3 + p3;
+  const double d31 = q2 + p2, d32 = q1 - p1;
   div[2] = fma(d32, h2, d31 * h1);
   if (A.flat3) {
     div[0] = d12 * h2;
     div[1] = d21 * h1;
   } else {
-    const double d13 = (E2[z] + E2[z + 1]) - (E2[0] + E2[1]);  // F3[B1]
-    const double d23 = (E1[0] + E1[y]) - (E1[z] + E1[z + y]);  // F3[B2]
+    const double d13 = q2 - p2, d23 = q1 + p1;  // through X3 faces
     div[0] = fma(d13, h3, d12 * h2);
     div[1] = fma(d23, h3, d21 * h1);
   }
