@@ -324,9 +324,9 @@ int grmhd_autotune(grmhd_sim *sim, int trials, double *ms_before, double *ms_aft
  * that many consecutive zones of a column along the direction, and
  * consecutive zones share their stencil differences. With 1, one thread
  * takes one zone.  0 restores the automatic choice: the longest walk that
- * still gives every reconstruction launch 152 x 640 threads, else 1.  The
- * values do not depend on the setting; only the launch shape and the FP64
- * instruction count do.  Synchronises the device.  *chosen (may be NULL)
+ * still gives every reconstruction launch 152 x 384 threads (one per
+ * primitive), and 1 below 152 x 256 zones.  The values do not depend on the
+ * setting; only the launch shape and the instruction count do.  Synchronises the device.  *chosen (may be NULL)
  * receives the length in use.  GRMHD_ERR_INVALID for other values. */
 int grmhd_set_recon_walk(grmhd_sim *sim, int zones_per_thread, int *chosen);
 
@@ -410,7 +410,7 @@ int grmhd_fluxes_noalloc(const grmhd_grid *grid, const grmhd_metric *metric,
  * the units: one launch of each kernel of the stage covers every grid of a
  * batch, so small grids (2D problems, many served requests) do not leave
  * most SMs idle, and a step costs the same launches whatever the number of
- * grids (32 when every grid is FP64; mixed-precision grids add the FP32
+ * grids (22 when every grid is FP64; mixed-precision grids add the FP32
  * flux kernels).  Each grid keeps its own buffers, geometry, boundary
  * conditions, reconstruction, precision, CFL time step and clock (t_final
  * included).  A simulation stepped alone runs the same kernels as a batch

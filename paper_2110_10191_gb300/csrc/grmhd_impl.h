@@ -56,6 +56,7 @@ struct StepArgs {
   // zones per thread of the FP64 reconstruction along a column (2..16), or 1:
   // one thread per zone; set by the plan from its grids' sizes
   int rwalk;
+  int x1_split;  // its X1 pass takes a thread per primitive (set by the plan likewise)
   int floor_drift;  // bounds in the drift frame: a separate pass after the update
   // electron entropies (GRMHD_ELEC_* model, 0: off): adiabatic indices of
   // electrons and protons, the constant share, the bounds on T_p/T_e

@@ -334,7 +334,7 @@ int upload_tables(Plan &p) {
 }  // namespace
 
 void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rwalk,
-                 long long c[PC_N]) {
+                 int x1_split, long long c[PC_N]) {
   const int fl = flat3;
   // the flux stage: FP64, FP32 or float-float
   const bool f64 = prec == GRMHD_PREC_FP64, fx = prec == GRMHD_PREC_FF;
@@ -343,9 +343,9 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_BX2] = n_bounds_x2(D);
   c[PC_BX3] = n_bounds_x3(D);
   c[PC_BALL] = n_bounds_all(D);
-  c[PC_RECON0] = f64 ? n_recon_walk(D, 0, fl, rwalk) : 0;
-  c[PC_RECON1] = f64 ? n_recon_walk(D, 1, fl, rwalk) : 0;
-  c[PC_RECON2] = (f64 && !fl) ? n_recon_walk(D, 2, 0, rwalk) : 0;
+  c[PC_RECON0] = f64 ? (x1_split ? NV : 1) * n_recon_walk(D, 0, fl, rwalk) : 0;
+  c[PC_RECON1] = f64 ? NV * n_recon_walk(D, 1, fl, rwalk) : 0;
+  c[PC_RECON2] = (f64 && !fl) ? NV * n_recon_walk(D, 2, 0, rwalk) : 0;
   for (int d = 0; d < 3; d++) {
     c[PC_FACE0 + d] = (f64 && !elec) ? n_face_threads(D, d, fl) : 0;
     c[PC_FACE0E + d] = (f64 && elec) ? n_face_threads(D, d, fl) : 0;
@@ -374,28 +374,39 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
 
 long long plan_bytes(const Dims &D, int flat3, int prec, int drift, int elec) {
   long long c[PC_N], ints = 0;
-  plan_counts(D, flat3, prec, drift, elec, 1, c);  // one thread per zone: the most blocks
+  plan_counts(D, flat3, prec, drift, elec, 1, 1, c);  // one thread per zone: the most blocks
   for (int q = 0; q < PC_N; q++) ints += 2 * nblk(c[q], 64);
   return (long long)sizeof(StageItem) + 4 * ints;
 }
 
 int plan_rwalk(const StageItem *items, int n) {
   for (int rw = RWALK; rw >= 2; rw /= 2) {
-    long long least = -1;  // the FP64 walk launch (X2 or X3) with the fewest threads
+    long long least = -1, zones = 0;  // of the FP64 walk launch (X2 or X3) with the fewest threads
     bool any = false;
     for (int d = 1; d < 3; d++) {
-      long long tot = 0;
+      long long tot = 0, one = 0;
       for (int g = 0; g < n; g++) {
         const StepArgs &A = items[g].A;
         if (items[g].prec != GRMHD_PREC_FP64 || (d == 2 && A.flat3)) continue;
-        tot += n_recon_walk(A.D, d, A.flat3, rw);
+        tot += NV * n_recon_walk(A.D, d, A.flat3, rw);
+        one += n_recon_walk(A.D, d, A.flat3, 1);
         any = true;
       }
-      if (tot > 0 && (least < 0 || tot < least)) least = tot;
+      if (tot > 0 && (least < 0 || tot < least)) {
+        least = tot;
+        zones = one;
+      }
     }
-    if (!any || least >= RWALK_MIN_THREADS) return rw;
+    if (!any || (least >= RWALK_MIN_THREADS && zones >= RWALK_MIN_ZONES)) return rw;
   }
   return 1;
+}
+
+int plan_x1_split(const StageItem *items, int n) {
+  long long tot = 0;
+  for (int g = 0; g < n; g++)
+    if (items[g].prec == GRMHD_PREC_FP64) tot += n_recon_walk(items[g].A.D, 0, items[g].A.flat3, 1);
+  return tot < X1_MIN_THREADS;
 }
 
 int plan_build(Plan &p, const StageItem *items, int n) {
@@ -410,13 +421,17 @@ int plan_build(Plan &p, const StageItem *items, int n) {
   }
   memcpy(p.host_items, items, sizeof(StageItem) * n);
   const int rw = plan_rwalk(items, n);
-  for (int g = 0; g < n; g++) p.host_items[g].A.rwalk = rw;
+  const int xs = plan_x1_split(items, n);
+  for (int g = 0; g < n; g++) {
+    p.host_items[g].A.rwalk = rw;
+    p.host_items[g].A.x1_split = xs;
+  }
   long long zones = 0, cap = 0;
   for (int g = 0; g < n; g++) {
     long long c[PC_N], c1[PC_N];
     const StepArgs &A = items[g].A;
-    plan_counts(A.D, A.flat3, items[g].prec, A.floor_drift, A.elec, rw, c);
-    plan_counts(A.D, A.flat3, items[g].prec, A.floor_drift, A.elec, 1, c1);
+    plan_counts(A.D, A.flat3, items[g].prec, A.floor_drift, A.elec, rw, xs, c);
+    plan_counts(A.D, A.flat3, items[g].prec, A.floor_drift, A.elec, 1, 1, c1);
     for (int q = 0; q < PC_N; q++) {
       p.count[(size_t)q * n + g] = c[q];
       // room for the smallest block the tuner tries and any walk length
@@ -478,7 +493,7 @@ int plan_set_rwalk(Plan &p, int rw) {
     StageItem &it = p.host_items[g];
     it.A.rwalk = rw;
     long long c[PC_N];
-    plan_counts(it.A.D, it.A.flat3, it.prec, it.A.floor_drift, it.A.elec, rw, c);
+    plan_counts(it.A.D, it.A.flat3, it.prec, it.A.floor_drift, it.A.elec, rw, it.A.x1_split, c);
     for (int q = PC_RECON0; q <= PC_RECON2; q++) p.count[(size_t)q * n + g] = c[q];
   }
   if (cudaMemcpy(p.items, p.host_items, sizeof(StageItem) * n, cudaMemcpyHostToDevice) != cudaSuccess)

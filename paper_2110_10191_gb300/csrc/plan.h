@@ -123,14 +123,9 @@ struct PlanHook {
 int plan_build(Plan &p, const StageItem *items, int n);
 // threads per launch class of one grid (dimensions, flat X3, GRMHD_PREC_*,
 // bounds in the drift frame, electrons evolved, the plan's reconstruction
-// walk length)
+// walk length and whether its X1 pass takes a thread per primitive)
 void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rwalk,
-                 long long c[PC_N]);
-// The FP64 reconstruction's walk length along X2 and X3 for a plan of these
-// grids: the longest of 16, 8, 4, 2 zones per thread that still gives each of
-// those launches RWALK_MIN_THREADS threads, 20 warps per SM, else 1 (one thread
-// per zone, which forms each pair of differences three times and costs 6% more
-// where both fill the GPU: 301 against 283 us over 128x128x64 zones).
+                 int x1_split, long long c[PC_N]);
 // Largest number of interior zones, of a grid and of a plan, whose directions get
 // face arrays of their own and run side by side.  A small grid's kernels leave
 // most of the GPU idle, each waiting for its threads' chains of work; side by side
@@ -144,8 +139,25 @@ inline bool splits(const Dims &D, int prec) {
   return prec != GRMHD_PREC_MIXED && prec != GRMHD_PREC_MIXED_FF &&
          (long long)D.n[0] * D.n[1] * D.n[2] <= SPLIT_ZONES;
 }
-constexpr long long RWALK_MIN_THREADS = 152 * 640;
+// The FP64 reconstruction's walk length along X2 and X3 for a plan of these grids: the
+// longest of 16, 8, 4, 2 zones per thread that still gives each of those launches
+// RWALK_MIN_THREADS threads, 12 warps per SM; 1 (one thread per zone and primitive,
+// which forms each pair of differences three times) where a primitive has fewer
+// than RWALK_MIN_ZONES zones, which walks gain 3% at most.  A cycle with 1, 2, 4, 8
+// and 16 zones per thread: 217x217 zones 236, 238, 229, 233, 236 us; 61x45x37 534, 542,
+// 514, 499, 491; 400x400 611, 606, 605, 587, 592; 32^3 247, 248, 241, 239, 249; 128^3 7.26,
+// 7.43, 7.06, 6.88, 6.77 ms.  (A thread that walked all 8 primitives left the last
+// wave nearly empty: a 128^3 launch took 0.45 ms, 0.40 so; a 61x45x37 cycle 550 and 508
+// us.)
+constexpr long long RWALK_MIN_THREADS = 152 * 384;
+constexpr long long RWALK_MIN_ZONES = 152 * 256;
 int plan_rwalk(const StageItem *items, int n);
+// Whether a plan's X1 reconstruction takes a thread per primitive: where threads for all 8
+// would be fewer than X1_MIN_THREADS, 8 warps per SM (a cycle of 64x64 zones 83 against
+// 89 us, of 128x128 110 against 117, of 217x217 238 against 239, of 61x45x37 519
+// against 501: each primitive repeats the index arithmetic).
+constexpr long long X1_MIN_THREADS = 152 * 256;
+int plan_x1_split(const StageItem *items, int n);
 // Set the plan's reconstruction walk length (1, 2, 4, 8 or 16 zones per
 // thread; 0: plan_rwalk's choice) and re-lay the reconstruction's block
 // tables.  The values do not depend on it.

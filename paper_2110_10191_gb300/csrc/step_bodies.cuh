@@ -92,14 +92,25 @@ __host__ __device__ inline long long n_recon(const Dims &D, int flat3) {
 constexpr int RWALK = 16;
 // pairs that a warp of recon_x1_body finishes
 constexpr int X1_LANES = 30;
-// threads of the FP64 reconstruction along dir: along X1 a warp per X1_LANES
-// pairs (recon_x1_body); else one per column and segment of rw zones along dir
-// (rw >= 2), or one per zone (rw = 1)
+// threads of one variable of the FP64 reconstruction along dir: along X1 a warp per
+// X1_LANES pairs (recon_x1_body); else one per column and segment of rw zones along
+// dir (rw >= 2), or one per zone (rw = 1)
 __host__ __device__ inline long long n_recon_walk(const Dims &D, int dir, int flat3, int rw) {
   const long long e[3] = {D.n[0] + 2, D.n[1] + 2, flat3 ? 1 : D.n[2] + 2};
   if (dir == 0) return 32 * (((e[0] + 2) * e[1] * e[2] - 2 + X1_LANES - 1) / X1_LANES);
   if (rw <= 1) return e[0] * e[1] * e[2];
   return e[0] * e[1] * e[2] / e[dir] * ((e[dir] + rw - 1) / rw);
+}
+// thread t of NV per -> the variable, t within it (per threads a variable)
+__device__ __forceinline__ int split_var(long long &t, long long per) {
+  int v = 0;
+#pragma unroll
+  for (int b = NV / 2; b >= 1; b /= 2)
+    if (t >= b * per) {
+      t -= b * per;
+      v += b;
+    }
+  return v;
 }
 // faces along dir: dir index NG .. n+NG, transverse NG-1 .. n+NG (flux-CT
 // needs one transverse layer on each side); flat X3 keeps the k = NG layer
@@ -327,12 +338,13 @@ __device__ __forceinline__ void warp_block_max(double v, unsigned long long *dst
 
 // Zone-centric reconstruction along X2 or X3: both face values of each zone's
 // 8 primitives (zones NG-1 .. n+NG along DIR and the extended transverse range),
-// each zone's WENO smoothness indicators formed once.  With A.rwalk >= 2 one
-// thread walks a segment of A.rwalk zones of one column along DIR, so that
-// consecutive zones share their differences and indicators (WenoWalk);
-// consecutive threads take neighbouring columns along X1.  With A.rwalk = 1
-// (grids too small to fill the GPU with walks) one thread takes one zone.  Same
-// values either way.  Lf = value at the zone's low face, Rf = at its high face.
+// each zone's WENO smoothness indicators formed once.  A thread takes one primitive:
+// with A.rwalk >= 2 it walks a segment of A.rwalk zones of one column along DIR, so
+// that consecutive zones share their differences and indicators (WenoWalk); with
+// A.rwalk = 1 (grids too small to fill the GPU with walks) it takes one zone.
+// Consecutive threads take neighbouring columns along X1, the primitives follow
+// one another.  Same values either way.  Lf = value at the zone's low face, Rf = at
+// its high face.
 template <int DIR, int RECON>
 __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__restrict__ P,
                                            double *__restrict__ Lf, double *__restrict__ Rf,
@@ -342,25 +354,23 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
   const int kb = A.flat3 ? NG : NG - 1;
   const long long st = (DIR == 1) ? D.s[0] : D.n2d;
   const int rw = A.rwalk;
+  const int v = split_var(t, n_recon_walk(D, DIR, A.flat3, rw));
   if (rw <= 1) {
     if (t >= (long long)e0 * e1 * e2) return;
     const Idx3 q3 = unflatten(t, e0, e1);
-    const long long c = zid(D, NG - 1 + q3.i, NG - 1 + q3.j, kb + q3.k);
-#pragma unroll
-    for (int v = 0; v < NV; v++) {
-      const double *p = P + v * D.ntot + c;
-      double lo, hi;
-      if (RECON == 1) {
-        weno5_wide_pair(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st),
-                        __ldg(p + 2 * st), lo, hi);
-      } else {
-        const double x1 = __ldg(p), h = mc_half_slope(x1 - __ldg(p - st), __ldg(p + st) - x1);
-        lo = x1 - h;
-        hi = x1 + h;
-      }
-      Lf[v * D.ntot + c] = lo;
-      Rf[v * D.ntot + c] = hi;
+    const long long o = v * D.ntot + zid(D, NG - 1 + q3.i, NG - 1 + q3.j, kb + q3.k);
+    const double *p = P + o;
+    double lo, hi;
+    if (RECON == 1) {
+      weno5_wide_pair(__ldg(p - 2 * st), __ldg(p - st), __ldg(p), __ldg(p + st), __ldg(p + 2 * st),
+                      lo, hi);
+    } else {
+      const double x1 = __ldg(p), h = mc_half_slope(x1 - __ldg(p - st), __ldg(p + st) - x1);
+      lo = x1 - h;
+      hi = x1 + h;
     }
+    Lf[o] = lo;
+    Rf[o] = hi;
     return;
   }
   const int ed = (DIR == 1) ? e1 : e2;
@@ -372,22 +382,19 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
   const int j = NG - 1 + ((DIR == 1) ? m0 : cb);
   const int k = (DIR == 2) ? NG - 1 + m0 : kb + cb;
   const int n = min(rw, ed - m0);
-  const long long c = zid(D, i, j, k);
-#pragma unroll 1
-  for (int v = 0; v < NV; v++) {
-    const double *p = P + v * D.ntot + c;
-    double *lf = Lf + v * D.ntot + c, *rf = Rf + v * D.ntot + c;
-    if (RECON == 1) {
-      weno5_walk(p, lf, rf, st, n);
-    } else {
-      double x1 = __ldg(p), dm = x1 - __ldg(p - st);
-      for (int m = 0; m < n; m++) {
-        const double x2 = __ldg(p + (m + 1) * st), dp = x2 - x1, h = mc_half_slope(dm, dp);
-        lf[m * st] = x1 - h;
-        rf[m * st] = x1 + h;
-        x1 = x2;
-        dm = dp;
-      }
+  const long long o = v * D.ntot + zid(D, i, j, k);
+  const double *p = P + o;
+  double *lf = Lf + o, *rf = Rf + o;
+  if (RECON == 1) {
+    weno5_walk(p, lf, rf, st, n);
+  } else {
+    double x1 = __ldg(p), dm = x1 - __ldg(p - st);
+    for (int m = 0; m < n; m++) {
+      const double x2 = __ldg(p + (m + 1) * st), dp = x2 - x1, h = mc_half_slope(dm, dp);
+      lf[m * st] = x1 - h;
+      rf[m * st] = x1 + h;
+      x1 = x2;
+      dm = dp;
     }
   }
 }
@@ -401,7 +408,9 @@ __device__ __forceinline__ void recon_body(const StepArgs &A, const double *__re
 // consecutive ones, 30 of them its own (lanes 0 and 1 only serve the lanes
 // above).  Against walks of 32 rows per warp staged in shared memory, whose 152
 // registers and tile left 10 warps per SM waiting for loads, a 128x128x64 grid's
-// launch went from 446 to 220 us.  Same values as recon_body's.  Every thread of the warp must call it.
+// launch went from 446 to 220 us.  A thread takes all 8 primitives, or one of them
+// (A.x1_split: small grids).  Same values as recon_body's.  Every thread of the warp
+// must call it.
 template <int RECON>
 __device__ __forceinline__ void recon_x1_body(const StepArgs &A, const double *__restrict__ P,
                                               double *__restrict__ Lf, double *__restrict__ Rf,
@@ -410,6 +419,8 @@ __device__ __forceinline__ void recon_x1_body(const StepArgs &A, const double *_
   const int e1 = D.n[1] + 2, e2 = A.flat3 ? 1 : D.n[2] + 2, row = D.n[0] + 4;
   const int lane = (int)(t & 31);
   const long long npair = (long long)row * e1 * e2;
+  // whole warps of one variable, or of all of them
+  const int v0 = A.x1_split ? split_var(t, n_recon_walk(D, 0, A.flat3, 1)) : 0;
   const long long g = (t >> 5) * X1_LANES + lane;
   const long long h = (g < npair) ? g : npair - 1;
   const Idx3 q3 = unflatten(h, row, e1);
@@ -417,7 +428,7 @@ __device__ __forceinline__ void recon_x1_body(const StepArgs &A, const double *_
   const long long c = zid(D, NG - 3 + q, NG - 1 + q3.j, (A.flat3 ? NG : NG - 1) + q3.k);
   const bool own = g < npair && lane >= 2 && q >= 2;
 #pragma unroll 1
-  for (int v = 0; v < NV; v++) {
+  for (int v = v0; v < (A.x1_split ? v0 + 1 : NV); v++) {
     const double *p = P + v * D.ntot + c;
     const double x0 = __ldg(p), x1 = __ldg(p + 1);
     double lo, hi;
