@@ -103,10 +103,10 @@ __device__ __forceinline__ ff mc_slope_ff(ff x0, ff x1, ff x2) {
 
 // Both WENO5 face values of the middle zone of a..e: the FP64 body's
 // first/second-difference form, with the weights d_k/(eps + beta_k)^2
-// normalised by the smallest (eps + beta): r_k = min_j e_j / e_k <= 1, so
-// no product leaves the float exponent range (eps = 1e-26 makes e_k^2 as
-// small as 1e-50); a weight that underflows is negligible next to the
-// dominant one, which is 1.
+// normalised by the power of two m below the smallest (eps + beta): r_k = m / e_k
+// in (0, 1], so no product leaves the float exponent range (eps = 1e-26 makes
+// e_k^2 as small as 1e-50); a weight that underflows is negligible next to the
+// dominant one, which is above 1/4.
 __device__ __forceinline__ void weno5_pair_ff(ff a, ff b, ff c, ff d, ff e, ff &lo, ff &hi) {
   const ff dm2 = ff_sub(b, a), dm1 = ff_sub(c, b), dp1 = ff_sub(d, c), dp2 = ff_sub(e, d);
   const ff D0 = ff_sub(dm1, dm2), D1 = ff_sub(dp1, dm1), D2 = ff_sub(dp2, dp1);
@@ -122,8 +122,8 @@ __device__ __forceinline__ void weno5_pair_ff(ff a, ff b, ff c, ff d, ff e, ff &
   const ff e0 = ff_add(ff_add(ff_mul_f(ff_sqr(D0), 13.0f), ff_mul_f(ff_sqr(s0), 3.0f)), eps12);
   const ff e1 = ff_add(ff_add(ff_mul_f(ff_sqr(D1), 13.0f), ff_mul_f(ff_sqr(s1), 3.0f)), eps12);
   const ff e2 = ff_add(ff_add(ff_mul_f(ff_sqr(D2), 13.0f), ff_mul_f(ff_sqr(s2), 3.0f)), eps12);
-  const ff emin = ff_min(ff_min(e0, e1), e2);
-  const ff r0 = ff_mul(emin, ff_rcp(e0)), r1 = ff_mul(emin, ff_rcp(e1)), r2 = ff_mul(emin, ff_rcp(e2));
+  const float m = __int_as_float(__float_as_int(fminf(fminf(e0.hi, e1.hi), e2.hi)) & 0x7f800000);
+  const ff r0 = ff_ldexp(ff_rcp(e0), m), r1 = ff_ldexp(ff_rcp(e1), m), r2 = ff_ldexp(ff_rcp(e2), m);
   const ff w0 = ff_sqr(r0), w1 = ff_mul_f(ff_sqr(r1), 6.0f), w2 = ff_sqr(r2);
   const ff w2x3 = ff_mul_f(w2, 3.0f), w0x3 = ff_mul_f(w0, 3.0f);
   const ff m3 = ff_mul_f(dm1, 3.0f), p3 = ff_mul_f(dp1, 3.0f);
