@@ -410,10 +410,10 @@ int grmhd_fluxes_noalloc(const grmhd_grid *grid, const grmhd_metric *metric,
  * the units: one launch of each kernel of the stage covers every grid of a
  * batch, so small grids (2D problems, many served requests) do not leave
  * most SMs idle, and a step costs the same launches whatever the number of
- * grids (22 when every grid is FP64; mixed-precision grids add the FP32
- * flux kernels).  Each grid keeps its own buffers, geometry, boundary
- * conditions, reconstruction, precision, CFL time step and clock (t_final
- * included).  A simulation stepped alone runs the same kernels as a batch
+ * grids (22 when every grid is FP64, 20 when they are flat in X3 too;
+ * mixed-precision grids add the FP32 flux kernels).  Each grid keeps its own
+ * buffers, geometry, boundary conditions, reconstruction, precision, CFL time
+ * step and clock (t_final included).  A simulation stepped alone runs the same kernels as a batch
  * of one, so a grid's state after n batched steps is bitwise its state
  * after grmhd_step(sim, n) alone. */
 typedef struct grmhd_batch grmhd_batch; /* opaque, library-owned */

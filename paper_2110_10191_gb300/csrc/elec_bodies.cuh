@@ -10,7 +10,8 @@
 //   elec_flux_body<d>  (after the face fluxes of every direction) forms their
 //                      local Lax-Friedrichs flux from the weights that the
 //                      face kernels (FP64, FP32 or float-float) stored;
-//   fix_flux_body      zeroes them where the mass flux is zeroed;
+//   fix_flux_body      zeroes them where the mass flux is zeroed (FP64 grids: the
+//                      face kernels zero their weights there);
 //   elec_post_body     (after the update, whose bounds wait for it) carries
 //                      the entropies to the new state, heats the electrons by
 //                      the model's share of the dissipation, applies the

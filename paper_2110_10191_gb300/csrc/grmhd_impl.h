@@ -66,7 +66,7 @@ struct StepArgs {
   // electrons: per face, the weights of the left and right entropies in
   // their LLF flux, [3][2][ntot] (direction, side)
   double *elec_w;
-  int flat3;  // n3 = 1 with periodic X3: fluxes on the single k layer, copied
+  int flat3;  // n3 = 1 with periodic X3: fluxes and EMFs on the single k layer
   // sides that continue into a neighbouring block of a decomposed grid (1)
   // rather than ending at a physical boundary (0): the fixup may average
   // over the first ghost layer there, which holds the neighbour's zones

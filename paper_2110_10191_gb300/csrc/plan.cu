@@ -659,8 +659,9 @@ int plan_bounds(const Plan &p, int which, int end, cudaStream_t st, PlanHook *h)
 // direction on streams of their own, EMFs, inversion, fixup, ghosts).  With the
 // flux fixes, the flux copies of a flat X3, the CFL step, flux-CT's flux update, the
 // three ghost passes and the clock as launches of their own it was twelve and a
-// half: at 64 x 64 a cycle took 114 us and takes 85, at 217 x 217 281 and 239, at
-// 61 x 45 x 37 640 and 563, a batch of 64 flat grids of 32^2 to 256^2 6990 and 6040.
+// half: by that alone a cycle went from 114 to 85 us at 64 x 64, 281 to 239 at 217 x 217,
+// 640 to 563 at 61 x 45 x 37, 6990 to 6040 for a batch of 64 flat grids of 32^2
+// to 256^2.
 int plan_stage(const Plan &p, int stage, cudaStream_t st, PlanHook *h) {
   int nl = plan_fluxes(p, stage, true, st, h);
   nl += plan_emf(p, stage == 0, st, h);

@@ -33,7 +33,7 @@ struct StageItem {
   const float *geomff; // float-float: split geometry ([2][NLOC][G_NCOMP][n2d])
   int prec;            // GRMHD_PREC_*: the flux stage's arithmetic
   // electrons (A.elec): (kappa_tot, kappa_e) of the stage arrays ([2][ntot]
-  // each, with P and Ph), their fluxes, and U_rho(P^n) kept by the predictor
+  // each, with P and Ph) and their fluxes
   double *K, *Kh, *FK[3];
   double *KLf, *KRf;  // their face values along the current direction
 };

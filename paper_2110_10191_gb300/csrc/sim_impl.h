@@ -20,8 +20,8 @@ struct grmhd_sim {
   double *geom, *conn, *floors;
   float *Pf, *geomf;    // FP32 copies (mixed precision only)
   float *Pff, *geomff, *connff;  // split float-float copies (float-float modes only)
-  // electrons only: entropies of the stage arrays, their fluxes, U_rho(P^n),
-  // the faces' signal speeds
+  // electrons only: entropies of the stage arrays, their fluxes, the faces' flux
+  // weights, face values
   double *K, *Kh, *FK[3], *elec_w, *KLf, *KRf;
   int *pflag, *fflag;
   grmhd::Clock *clk;

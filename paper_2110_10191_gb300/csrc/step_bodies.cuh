@@ -1,10 +1,10 @@
 // step_bodies.cuh -- the per-thread bodies of the kernels of one
 // predictor-corrector stage of the HARM scheme (iharm3D, arXiv:2110.10191):
-//   bounds (ghost fill) -> zone-centric reconstruction -> face fluxes (LLF,
-//   with a warp/block max of the signal speed for the CFL step) -> dt ->
-//   boundary flux fixes -> flux-CT EMFs (Toth 2000; paper, "Implementation
-//   Notes", first paragraph) -> update + 1D_W inversion + bounds (same
-//   section) -> fixup of failed zones.
+//   zone-centric reconstruction -> face fluxes (LLF, with their boundary fixes and
+//   a warp/block max of the signal speed for the CFL step) -> flux-CT EMFs (Toth
+//   2000; paper, "Implementation Notes", first paragraph), dt -> update (its source
+//   pass may run beside the fluxes) + 1D_W inversion + bounds (same section) ->
+//   fixup of failed zones -> ghost fill.
 //
 // Each body takes the step arguments of one grid and the linear index t of
 // its thread within that grid's launch range.  The plan kernels (plan.cu)
@@ -13,15 +13,15 @@
 // never spans two grids: the block reductions (signal speed maxima, warp
 // counts) see the threads of one grid only.
 //
-// Every thread owns one face, edge or zone; fields are SoA float64 in HBM
-// with i fastest, so warps read and write 256-byte contiguous runs.
+// A thread owns an edge, a zone, half a face or a stretch of one primitive's column;
+// fields are SoA float64 in HBM with i fastest, so warps read and write contiguous runs.
 //
 // Flat X3 (A.flat3: n3 = 1 with periodic X3): every k layer of the
 // primitives is an exact copy of the single interior layer, so the fluxes
-// along X1 and X2 are computed on that layer only and copied to the layers
-// above and below it (replicate_body), and the X3 faces read the primitives
-// themselves as their face states (reconstruction of constant data returns
-// the data exactly).  The results are bitwise those of the full extent.
+// along X1 and X2 are computed on that layer only, the update takes the layer's X3
+// differences as zero, and the X3 faces read the primitives themselves as their
+// face states (reconstruction of constant data returns the data exactly).  Callers
+// who want the fluxes get them copied to the layers above and below (replicate_body).
 #pragma once
 
 #include "grmhd_dev.cuh"
