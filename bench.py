@@ -50,19 +50,20 @@ WORKLOADS = {
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# each FP64-bound kernel class on the 128^3 torus: the mean over the class's
-# launches (the three directions of kp_recon and kp_face, both stages of
-# kp_update) in the one-pass ncu launch list of the 2-cycle bench command.
+# each hot kernel class of the FP64 step on the 128^3 torus: the mean over the
+# class's launches (the three directions of kp_recon and kp_face, both stages and
+# both passes, kp_source and kp_invert, of the update) in the one-pass ncu launch
+# list of the 2-cycle bench command.
 # The figures hold while the kernel sources hash to src_hash; otherwise the
 # bench reports the traffic as unknown (null).
-NCU_TRAFFIC = {"src_hash": "5e804b7ef44b62a1",
-               "torus128": {"recon": 187957174 + 238592572, "flux": 295317248 + 110696210,
-                            "update": 727520073 + 204079488}}
-# sm__inst_executed_pipe_fp64.avg.pct_of_peak_sustained_active of full ncu
-# captures of single launches (kp_recon<0> and <1>, the X3 walk taken as X2's;
-# kp_face<0,0>; kp_update): the hardware's view of the same kernels, as a
-# fraction of the nominal 2 FP64 instructions per SM per clock
-NCU_FP64_PIPE = {"torus128": {"recon": 0.858, "flux": 0.905, "update": 0.888}}
+NCU_TRAFFIC = {"src_hash": "f4ba0e7ccb5b17a1",
+               "torus128": {"recon": 155200000 + 226110000, "flux": 295320000 + 224430000,
+                            "update": 357870000 + 271250000}}
+# sm__inst_executed_pipe_fp64.avg.pct_of_peak_sustained_active of ncu captures of
+# single launches (the mean over kp_recon<0..2>; over kp_face<0..2,0>; over kp_source<1>
+# and kp_invert): the hardware's view of the same kernels, as a fraction of the
+# nominal 2 FP64 instructions per SM per clock
+NCU_FP64_PIPE = {"torus128": {"recon": 0.251, "flux": 0.673, "update": 0.676}}
 
 
 def kernel_source_hash():
@@ -770,18 +771,21 @@ def build_roofline(prof, cpu, pr, zones, fp64, config, variant="none"):
                 hbm = float(json.load(f)["hbm_gbs"]) * 1e9
         except (OSError, KeyError, ValueError):
             pass
-        # algorithmic work and bytes per launch of each FP64-bound kernel class:
+        # algorithmic work and bytes per launch of each hot kernel class:
         # face: two states in, one flux out (24 doubles per face); recon: the
         # primitives in, two face values out (24 doubles per zone of the
-        # extended range); update: predictor 48, corrector 56 doubles per zone
+        # extended range); update: predictor 48, corrector 56 doubles per zone and
+        # stage, shared among the launches of a stage's update
+        passes = max(prof["update"][1] / max(prof["flux"][1] / 3.0, 1.0), 1.0)
         work = {
             "flux": ("kp_face (LLF face fluxes from reconstructed states)",
                      cpu["_face_flops_per_face"] * sum(faces) / 3.0, 24 * 8 * sum(faces) / 3.0),
             "recon": ("kp_recon (WENO5 face states, both faces of every zone)",
                       cpu["_recon_flops_per_face"] * sum(faces) / 3.0,
                       24 * 8 * (pr.n[0] + 2) * (pr.n[1] + 2) * (pr.n[2] + 2)),
-            "update": ("kp_update (conserved update + 1D_W inversion + bounds)",
-                       cpu["_update_flops_per_zone_stage"] * zones, 52 * 8 * zones),
+            "update": ("kp_source, kp_invert (conserved update + 1D_W inversion + bounds)",
+                       cpu["_update_flops_per_zone_stage"] * zones / passes,
+                       52 * 8 * zones / passes),
         }
         same_src = kernel_source_hash() == NCU_TRAFFIC["src_hash"]
         traffic = NCU_TRAFFIC.get(config) if same_src else None
@@ -818,12 +822,10 @@ def build_roofline(prof, cpu, pr, zones, fp64, config, variant="none"):
                         "algorithmic_bytes": kd["algorithmic_bytes"], "traffic": kd["traffic"],
                         "fp64_pipe_ncu": kd["fp64_pipe_ncu"],
                         "note": "algorithmic flops are the counting oracle's (adds, multiplies, "
-                                "divisions and square roots counted as one each); the kernel spends "
-                                "several FP64 instructions on each division and square root and a "
-                                "lone add or multiply takes an issue slot worth two flops, while an "
-                                "FMA does two counted flops in one slot and the kernels form fewer "
-                                "terms than the oracle's plain order (shared differences of the "
-                                "reconstruction walk), so a saturated kernel can read above 1",
+                                "divisions and square roots counted as one each) against the FP64 "
+                                "unit's peak; the kernels do most of that work on the integer pipes, "
+                                "in numbers of 55 to 63 bits, beside the FP64 unit, so they read "
+                                "above 1",
                         "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per "
                                           "launch of %s, mean over its launches in the ncu launch "
                                           "list of this workload" % kd["kernel"].split()[0]}

@@ -122,7 +122,7 @@ static __device__ __noinline__ int elec_close(const StepArgs &A, double P[NV], d
 // ---------------------------------------------------------------------------
 // The same in Wide numbers (wide_num.cuh, wide_pow.cuh).  With log, exp, pow and
 // the divisions in FP64 the pass after the update was bound by that unit's 460
-// instructions a zone: 0.84 ms per launch on a 96^3 grid with Kawazura's model, 0.15
+// instructions a zone: 0.84 ms per launch on a 96^3 grid with Kawazura's model, 0.13
 // now.  Zones whose state leaves the range the powers are taken in (densities within
 // 2^+-52, energies and entropies within 2^+-100) take the FP64 form above; b^2 may be
 // anything finite, since beta is held within 1e+-20 (rounding leaves b^2 of 1e-40 and

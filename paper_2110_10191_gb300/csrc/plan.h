@@ -129,8 +129,8 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
 // Largest number of interior zones, of a grid and of a plan, whose directions get
 // face arrays of their own and run side by side.  A small grid's kernels leave
 // most of the GPU idle, each waiting for its threads' chains of work; side by side
-// a cycle of a 64x64 mode takes 114 us against 167, of 217x217 zones 281 against
-// 324, of 64^3 1162 against 1285, of 128^3 7.03 against 7.26 ms (where the kernels'
+// a cycle of a 64x64 mode takes 82 us against 119, of 217x217 zones 227 against
+// 264, of 64^3 1042 against 1148, of 100^3 3.37 against 3.47 ms (where the kernels'
 // tails overlap); beyond, the gain no longer pays for the memory.
 constexpr long long SPLIT_ZONES = 1 << 21;
 constexpr int SPLIT_SETS = 5;  // arrays of [8][ntot] they take
