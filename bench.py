@@ -56,7 +56,7 @@ WORKLOADS = {
 # list of the 2-cycle bench command.
 # The figures hold while the kernel sources hash to src_hash; otherwise the
 # bench reports the traffic as unknown (null).
-NCU_TRAFFIC = {"src_hash": "f4ba0e7ccb5b17a1",
+NCU_TRAFFIC = {"src_hash": "d2cbd87004ae6e76",
                "torus128": {"recon": 155200000 + 226110000, "flux": 295320000 + 224430000,
                             "update": 357870000 + 271250000}}
 # sm__inst_executed_pipe_fp64.avg.pct_of_peak_sustained_active of ncu captures of

@@ -265,7 +265,7 @@ __device__ __forceinline__ void elec_post_body(const StepArgs &A, const double *
                                                double dtfac, long long t) {
   const Dims &D = A.D;
   const double dt = A.clk->dt;
-  if (!(dt > 0.0)) return;
+  if (!less(0.0, dt)) return;
   const double dtp = dtfac * dt;
   const bool in = t < n_update(D);
   const Column q3 = column_of(in ? t : t & 31, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
@@ -340,45 +340,36 @@ __device__ __forceinline__ void elec_fix_body(const StepArgs &A, double *P, doub
                                               const int *__restrict__ pflag, int *fflag,
                                               long long t) {
   const Dims &D = A.D;
-  if (!(A.clk->dt > 0.0)) return;
-  const bool active = t < n_zone(D);
-  bool hit = false;
-  if (active) {
-    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
-    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
+  if (!less(0.0, A.clk->dt)) return;
+  for_failed_zones(A, pflag, t, [&](int i, int j, int k) {
     const long long c = zid(D, i, j, k), N = D.ntot;
-    if (pflag[c] != 0) {
-      double sum = 0.0;
-      int cnt = 0;
-      for (int dk = -1; dk <= 1; dk++)
-        for (int dj = -1; dj <= 1; dj++)
-          for (int di = -1; di <= 1; di++) {
-            if (di == 0 && dj == 0 && dk == 0) continue;
-            const int ii = i + di, jj = j + dj, kk = k + dk;
-            if (ii < NG - A.xlo[0] || ii >= D.n[0] + NG + A.xhi[0] || jj < NG - A.xlo[1] ||
-                jj >= D.n[1] + NG + A.xhi[1] || kk < NG - A.xlo[2] || kk >= D.n[2] + NG + A.xhi[2])
-              continue;
-            const long long nb = zid(D, ii, jj, kk);
-            if (pflag[nb] != 0) continue;
-            sum += K[N + nb];
-            cnt++;
-          }
-      if (cnt > 0) {
-        double p[NV], kn[2] = {0.0, sum / (double)cnt};
-#pragma unroll
-        for (int v = 0; v < NV; v++) p[v] = P[v * N + c];
-        const int f = elec_close(A, p, kn, log(p[RHO]));
-        P[UU * N + c] = p[UU];
-        K[c] = kn[0];
-        K[N + c] = kn[1];
-        if (f) {
-          hit = fflag[c] == 0;
-          fflag[c] |= f;
+    double sum = 0.0;
+    int cnt = 0;
+    for (int dk = -1; dk <= 1; dk++)
+      for (int dj = -1; dj <= 1; dj++)
+        for (int di = -1; di <= 1; di++) {
+          if (di == 0 && dj == 0 && dk == 0) continue;
+          const int ii = i + di, jj = j + dj, kk = k + dk;
+          if (ii < NG - A.xlo[0] || ii >= D.n[0] + NG + A.xhi[0] || jj < NG - A.xlo[1] ||
+              jj >= D.n[1] + NG + A.xhi[1] || kk < NG - A.xlo[2] || kk >= D.n[2] + NG + A.xhi[2])
+            continue;
+          const long long nb = zid(D, ii, jj, kk);
+          if (pflag[nb] != 0) continue;
+          sum += K[N + nb];
+          cnt++;
         }
-      }
-    }
-  }
-  count_warp(hit, &A.clk->counters[1]);
+    if (cnt == 0) return 0;
+    double p[NV], kn[2] = {0.0, sum / (double)cnt};
+#pragma unroll
+    for (int v = 0; v < NV; v++) p[v] = P[v * N + c];
+    const int f = elec_close(A, p, kn, log(p[RHO]));
+    P[UU * N + c] = p[UU];
+    K[c] = kn[0];
+    K[N + c] = kn[1];
+    const int hit = f && fflag[c] == 0;
+    if (f) fflag[c] |= f;
+    return hit;
+  });
 }
 
 }  // namespace grmhd

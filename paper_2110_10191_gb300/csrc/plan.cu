@@ -360,7 +360,7 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_FIX] = f64 ? 0 : n_fix(D);  // (the FP64 face fluxes fix their own)
   c[PC_EDGE] = n_edge(D, 0);
   c[PC_EDGES] = n_edge(D, fl);
-  c[PC_ZONE] = n_zone(D);
+  c[PC_ZONE] = n_fixup(D);
   const bool ux = fx || prec == GRMHD_PREC_MIXED_FF;  // the source pass in float-float
   c[PC_SRC64] = ux ? 0 : n_update(D);
   c[PC_SRCX] = ux ? n_update(D) : 0;
@@ -370,6 +370,7 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
   c[PC_EREC01] = elec ? n_recon(D, fl) : 0;
   c[PC_EREC2] = (elec && !fl) ? n_recon(D, 0) : 0;
   c[PC_EZONE] = elec ? n_update(D) : 0;
+  c[PC_EFIX] = elec ? n_fixup(D) : 0;
 }
 
 long long plan_bytes(const Dims &D, int flat3, int prec, int drift, int elec) {
@@ -637,7 +638,7 @@ int plan_invert(const Plan &p, int in, double dtfac, cudaStream_t st, PlanHook *
 int plan_fixup(const Plan &p, int out, cudaStream_t st, PlanHook *h) {
   int nl = launch(p, PC_ZONE, GRMHD_K_FIXUP, h,
                   [&](unsigned nb, unsigned bs, BView V) { kp_fixup<<<nb, bs, 0, st>>>(V, out); });
-  nl += launch(p, PC_EZONE, GRMHD_K_FIXUP, h,
+  nl += launch(p, PC_EFIX, GRMHD_K_FIXUP, h,
                [&](unsigned nb, unsigned bs, BView V) { kp_elec_fix<<<nb, bs, 0, st>>>(V, out); });
   return nl;
 }

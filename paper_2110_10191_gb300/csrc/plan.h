@@ -77,7 +77,8 @@ enum {
   PC_EFACE0, // electron entropy fluxes per direction
   PC_EFACE1,
   PC_EFACE2,
-  PC_EZONE,  // electron heating + bounds, and their fixup (grids with electrons)
+  PC_EZONE,  // electron heating + bounds (grids with electrons)
+  PC_EFIX,   // and their fixup
   PC_N
 };
 

@@ -952,7 +952,7 @@ __device__ __forceinline__ void invert_body(const StepArgs &A, const double *__r
                                             long long t) {
   const Dims &D = A.D;
   const double dt = A.clk->dt;
-  if (!(dt > 0.0)) return;  // uniform across the grid: no warp divergence
+  if (!less(0.0, dt)) return;  // uniform across the grid: no warp divergence
   const double dtp = dtfac * dt;
   const bool in = t < n_update(D);
   const Column q3 = column_of(in ? t : t & 31, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
@@ -1011,7 +1011,7 @@ __device__ __forceinline__ void floor_drift_body(const StepArgs &A, double *P,
                                                  const int *__restrict__ pflag, int *fflag,
                                                  long long t) {
   const Dims &D = A.D;
-  if (!(A.clk->dt > 0.0)) return;
+  if (!less(0.0, A.clk->dt)) return;
   const bool in = t < n_update(D);
   const Column q3 = column_of(in ? t : t & 31, (int)(t & 31), 32, D.n[0], D.n[1], D.n[2]);
   const bool active = in && q3.active;
@@ -1038,61 +1038,95 @@ __device__ __forceinline__ void floor_drift_body(const StepArgs &A, double *P,
 // ---------------------------------------------------------------------------
 // Fixup: a failed zone takes the mean of rho, u, utilde over the non-failed
 // interior zones of its 3x3x3 neighbourhood (B is kept), then the bounds.
-// Every thread of the block must call it (warp counters).
 // ---------------------------------------------------------------------------
+// 1: a bound acted, 2: no valid neighbour
+__device__ __forceinline__ int fixup_zone(const StepArgs &A, double *P, const int *__restrict__ pflag,
+                                          int *fflag, int i, int j, int k) {
+  const Dims &D = A.D;
+  const long long c = zid(D, i, j, k), N = D.ntot;
+  double sum[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  int cnt = 0;
+  for (int dk = -1; dk <= 1; dk++)
+    for (int dj = -1; dj <= 1; dj++)
+      for (int di = -1; di <= 1; di++) {
+        if (di == 0 && dj == 0 && dk == 0) continue;
+        const int ii = i + di, jj = j + dj, kk = k + dk;
+        if (ii < NG - A.xlo[0] || ii >= D.n[0] + NG + A.xhi[0] || jj < NG - A.xlo[1] ||
+            jj >= D.n[1] + NG + A.xhi[1] || kk < NG - A.xlo[2] || kk >= D.n[2] + NG + A.xhi[2])
+          continue;
+        const long long nb = zid(D, ii, jj, kk);
+        if (pflag[nb] != 0) continue;
+#pragma unroll
+        for (int v = 0; v < 5; v++) sum[v] += P[v * N + nb];
+        cnt++;
+      }
+  if (cnt == 0) return 2;
+  double p[NV];
+#pragma unroll
+  for (int v = 0; v < NV; v++) p[v] = P[v * N + c];
+#pragma unroll
+  for (int v = 0; v < 5; v++) p[v] = sum[v] / (double)cnt;
+  int f = 0;
+  if (A.floors_on) {
+    const long long ij = (long long)j * D.s[0] + i;
+    Geo G;
+    load_geo(A.geom, D.n2d, ij, G);
+    f = apply_floors(p, G, __ldg(A.floors + ij), __ldg(A.floors + D.n2d + ij), A.gk);
+    if (f) fflag[c] |= f;
+  }
+#pragma unroll
+  for (int v = 0; v < NV; v++) P[v * N + c] = p[v];
+  return f != 0;
+}
+
+// A thread looks at the failure flags of FIXUP_ZONES zones along X3, loaded together:
+// next to no zone fails, and with a zone a thread the passes over the flags waited
+// for them one wave after another (35 us a launch on a 128^3 grid, 14 so).  The
+// failed ones, which come in clusters (an axisymmetric state fails along all of X3), are
+// listed in shared memory and dealt out to the block's threads.
+constexpr int FIXUP_ZONES = 8;
+__host__ __device__ inline long long n_fixup(const Dims &D) {
+  return (long long)D.n[0] * D.n[1] * ((D.n[2] + FIXUP_ZONES - 1) / FIXUP_ZONES);
+}
+// Calls zone(i, j, k), whose result's bits 0 and 1 are counted, for each failed zone of
+// the block's threads.  Every thread of the block must call it.
+template <class ZoneFn>
+__device__ __forceinline__ void for_failed_zones(const StepArgs &A, const int *__restrict__ pflag,
+                                                 long long t, const ZoneFn &zone) {
+  __shared__ unsigned short list[BS_MAX * FIXUP_ZONES];
+  __shared__ unsigned count;
+  const Dims &D = A.D;
+  if (threadIdx.x == 0) count = 0;
+  u32 bad = 0;
+  if (t < n_fixup(D)) {
+    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
+    const int k = NG + FIXUP_ZONES * q3.k;
+    const long long c = zid(D, NG + q3.i, NG + q3.j, k);
+#pragma unroll
+    for (int m = 0; m < FIXUP_ZONES; m++)
+      if (k + m < D.n[2] + NG) bad |= (pflag[c + m * D.n2d] != 0 ? 1u : 0u) << m;
+  }
+  if (!__syncthreads_or(bad != 0)) return;
+  if (bad) {
+    unsigned at = atomicAdd(&count, (unsigned)__popc(bad));
+    for (; bad; bad &= bad - 1)
+      list[at++] = (unsigned short)(threadIdx.x * FIXUP_ZONES + __ffs((int)bad) - 1);
+  }
+  __syncthreads();
+  const unsigned n = count;
+  for (unsigned e = threadIdx.x; e < n; e += blockDim.x) {
+    const Idx3 q3 = unflatten(t - threadIdx.x + list[e] / FIXUP_ZONES, D.n[0], D.n[1]);
+    const int f = zone(NG + q3.i, NG + q3.j, NG + FIXUP_ZONES * q3.k + list[e] % FIXUP_ZONES);
+    if (f & 1) atomicAdd(&A.clk->counters[1], 1ull);
+    if (f & 2) atomicAdd(&A.clk->counters[2], 1ull);
+  }
+}
 __device__ __forceinline__ void fixup_body(const StepArgs &A, double *P, const int *__restrict__ pflag,
                                            int *fflag, long long t) {
-  const Dims &D = A.D;
-  if (!(A.clk->dt > 0.0)) return;
-  const long long nz = n_zone(D);
-  const bool active = t < nz;
-  bool hit = false, lost = false;
-  if (active) {
-    const Idx3 q3 = unflatten(t, D.n[0], D.n[1]);
-    const int i = NG + q3.i, j = NG + q3.j, k = NG + q3.k;
-    const long long c = zid(D, i, j, k), N = D.ntot;
-    if (pflag[c] != 0) {
-      double sum[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-      int cnt = 0;
-      for (int dk = -1; dk <= 1; dk++)
-        for (int dj = -1; dj <= 1; dj++)
-          for (int di = -1; di <= 1; di++) {
-            if (di == 0 && dj == 0 && dk == 0) continue;
-            const int ii = i + di, jj = j + dj, kk = k + dk;
-            if (ii < NG - A.xlo[0] || ii >= D.n[0] + NG + A.xhi[0] || jj < NG - A.xlo[1] ||
-                jj >= D.n[1] + NG + A.xhi[1] || kk < NG - A.xlo[2] || kk >= D.n[2] + NG + A.xhi[2])
-              continue;
-            const long long nb = zid(D, ii, jj, kk);
-            if (pflag[nb] != 0) continue;
-#pragma unroll
-            for (int v = 0; v < 5; v++) sum[v] += P[v * N + nb];
-            cnt++;
-          }
-      if (cnt == 0) {
-        lost = true;
-      } else {
-        double p[NV];
-#pragma unroll
-        for (int v = 0; v < NV; v++) p[v] = P[v * N + c];
-#pragma unroll
-        for (int v = 0; v < 5; v++) p[v] = sum[v] / (double)cnt;
-        if (A.floors_on) {
-          const long long ij = (long long)j * D.s[0] + i;
-          Geo G;
-          load_geo(A.geom, D.n2d, ij, G);
-          const int f = apply_floors(p, G, __ldg(A.floors + ij), __ldg(A.floors + D.n2d + ij), A.gk);
-          if (f) {
-            fflag[c] |= f;
-            hit = true;
-          }
-        }
-#pragma unroll
-        for (int v = 0; v < NV; v++) P[v * N + c] = p[v];
-      }
-    }
-  }
-  count_warp(hit, &A.clk->counters[1]);
-  count_warp(lost, &A.clk->counters[2]);
+  if (!less(0.0, A.clk->dt)) return;
+  for_failed_zones(A, pflag, t, [&](int i, int j, int k) {
+    return fixup_zone(A, P, pflag, fflag, i, j, k);
+  });
 }
 
 }  // namespace grmhd
