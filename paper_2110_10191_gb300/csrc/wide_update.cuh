@@ -182,7 +182,7 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
   bool done = false;
   Wide W, iB, x, x2, omv, rs, wmr;
 #pragma unroll 1
-  for (int it = 0; it < 7 && ok; it++) {
+  for (int it = 0; it < 8 && ok; it++) {  // seven steps; the last pass evaluates only
     W = norm(w_sum<1>(Wp, D));
     const Wide BW = norm(w_sum<1>(Bsq, W));
     const Wide ix = w_rcp(norm(BW * W));
@@ -197,7 +197,7 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
     const Wide sq = norm(omv * rs);
     // w - rho = W' (1 - v^2) - D v^2 sq / (1 + sq)
     wmr = w_sum<0>(Wp * omv, -(norm(norm(D * vsq) * sq) * w_rcp(norm(w_sum<1>(one, sq)))));
-    if (done) break;
+    if (done || it == 7) break;
     const Wide t = w_sum<2>(Qpn, Wp, hB, -(gf * norm(wmr)));
     const Wide f = norm(w_sum<1>(t, hB * vsq, -w_scale(x2, -1)));
     float ff, df;
