@@ -161,3 +161,53 @@ def test_the_state_is_the_last_iterates(wide, gam, kind):
     worst, _ = _check(wide, np.random.default_rng(11), gam, (8.0, 20.0), (-2, 0), None, None,
                       0.3, 1500, kind)
     assert worst.max() <= 1.0
+
+
+@pytest.mark.parametrize("lorentz", [(1.0, 8.0), (20.0, 50.0), (50.0, 1000.0)])
+@pytest.mark.parametrize("sigma,along", [(None, None), ((-4, 2.6), None), ((0, 4), 0.1)])
+@pytest.mark.parametrize("gam", [4.0 / 3.0, 5.0 / 3.0])
+def test_an_answer_is_the_root(wide, gam, sigma, along, lorentz):
+    """Any Lorentz factor and magnetisation, a guess off by up to e: no answer, or
+    the root's."""
+    seed = int(lorentz[1]) + 7 * (sigma is None) + 3 * (along is None)
+    worst, _ = _check(wide, np.random.default_rng(seed), gam, lorentz, (-6, 0.5), sigma, along, 1.0,
+                      400, seed % 2)
+    assert worst.max() <= 1.0
+
+
+def test_no_answer_from_a_derivative_that_overflows(wide):
+    """Lorentz factor 1000: 1 - v^2 rounds to zero in FP32."""
+    g = np.array([-1.0, 0, 0, 0, 1, 0, 0, 1, 0, 1] * 2 + [1.0, 1.0, 1.0, 1.0, 0.0])
+    P = np.array([1.0, 2.004076452014, 927.43315163681, 368.26909591672, -65.15076572658,
+                  733.51245163870, -657.53838453502, 172.05451506445])
+    X, gam = (0.0, 0.0, 0.0, 0.0), 4.0 / 3.0
+    U = oracle.prim_to_flux(0, 0.0, 0.3, X, gam, P, 0)
+    ok, out, bl = wide(U, g, gam, 3671075.19870)
+    if ok:
+        r = Root(U, g, gam, (P[0] + gam * P[1]) * (1 + P[2:5] @ P[2:5]) - U[0])
+        assert abs(out[0] / r.rho - 1) <= r.tol_rho and abs(out[1] / r.u - 1) <= r.tol_u
+
+
+@pytest.mark.parametrize("sigma", [None, (-4, 2.6)])
+@pytest.mark.parametrize("gam", [4.0 / 3.0, 13.0 / 9.0, 5.0 / 3.0])
+def test_no_further_off_than_fp64(wide, gam, sigma):
+    """Over Lorentz factors up to the bound of 50, the worst errors of rho and u are no
+    larger than those of the FP64 iteration on the same conserved vectors."""
+    rng = np.random.default_rng(5)
+    worst = np.zeros((2, 2))
+    for _ in range(600):
+        X, gcov, g = _point(0, rng)
+        lf = 50.0 ** rng.uniform()
+        P = _state(gcov, rng, X, 0, lf, 10.0 ** rng.uniform(-4, 0),
+                   10.0 ** rng.uniform(*sigma) if sigma else 0.0, None)
+        U = oracle.prim_to_flux(0, 0.9375, 0.3, X, gam, P, 0)
+        off = np.exp(rng.uniform(-0.3, 0.3))
+        W = (P[0] + gam * P[1]) * lf * lf
+        ok, out, _ = wide(U, g, gam, W * off)
+        rc, P64 = oracle.cons_to_prim(0, 0.9375, 0.3, X, gam, U, P * np.array([off] * 2 + [1] * 6))
+        if not ok or rc:
+            continue
+        r = Root(U, g, gam, W - U[0] * g[21] * g[23])
+        for q, p in enumerate((out, P64)):
+            worst[q] = np.maximum(worst[q], [abs(p[0] / r.rho - 1), abs(p[1] / r.u - 1)])
+    assert (worst[0] <= worst[1]).all(), worst
