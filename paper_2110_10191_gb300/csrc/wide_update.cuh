@@ -95,7 +95,10 @@ WIDE_FN float inv_f32(const InvF &q, float wp, float &f, float &df) {
 }
 
 // The 1D_W inversion where nothing unusual happens: Newton steps in FP32 from the
-// guess W (doubled while it lies below the root) until they are below 1e-5 (or six), then
+// guess W until they are below 1e-5 (or twelve; an iterate beyond v^2 = 1 lies below the
+// root and is replaced by the middle between it and the least W' above the root, or doubled
+// while none is known: without the bracket Newton and doubling alternated for good
+// at Lorentz factors above 8, and up to 88% of such states were left to FP64), then
 // Newton steps whose function is taken in Wide numbers and whose derivative in FP32 of
 // Wide values (each gains 20 bits or doubles the digits), until what f leaves is below
 // 2^-56 of its largest term, the noise of its own operations (2^-57 of 1/(W (B^2 + W))):
@@ -109,7 +112,7 @@ WIDE_FN float inv_f32(const InvF &q, float wp, float &f, float &df) {
 // u = 1e-6 to 1 rho, adiabatic indices 4/3 and 5/3, against the root in 113 bits, here and
 // of the FP64 iteration: Lorentz factors 1 to 3, rho 5e-15 and 1e-13, u 2e-9 and 9e-8; 20 to
 // 50, rho 1e-12 and 7e-11, u 5e-7 and 1e-5.  Three passes, 3.3 at 20 to 50.
-constexpr int INV_WIDE_MAXIT = 8;
+constexpr int INV_F32_MAXIT = 12, INV_WIDE_MAXIT = 8;
 constexpr u64 INV_RESIDUAL = 8;  // in units of 2^-59 of the largest term
 
 template <bool BLK, class GeoFn>
@@ -176,18 +179,19 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
   q.gf = (float)K.gf;
   {
     // (a root below 1e-6 D is left to the Wide steps)
-    float w = w_to_float(Wp, e), last = 1.0f;
+    float w = w_to_float(Wp, e), last = 1.0f, hi = INFINITY;
     if (!(w > 1e-6f * q.d)) w = 1e-6f * q.d;
 #pragma unroll 1
-    for (int it = 0; it < 6 && last > 1e-5f; it++) {
+    for (int it = 0; it < INV_F32_MAXIT && last > 1e-5f; it++) {
       float f, df, n;
       if (inv_f32(q, w, f, df) < 0.99999f) {
+        if (f > 0.0f) hi = w;
         n = w - f * inv_rcpf(df);
         if (!(n > 0.0f)) n = 0.5f * w;
-        last = fabsf(n - w) * inv_rcpf(w);
       } else {  // below the root
-        n = w + (w + q.d);
+        n = (hi < INFINITY) ? 0.5f * (w + hi) : w + (w + q.d);
       }
+      last = fabsf(n - w) * inv_rcpf(w);
       w = n;
     }
     const bool fine = last < 0.5f && w < 1e6f;

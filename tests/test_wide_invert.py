@@ -211,3 +211,20 @@ def test_no_further_off_than_fp64(wide, gam, sigma):
         for q, p in enumerate((out, P64)):
             worst[q] = np.maximum(worst[q], [abs(p[0] / r.rho - 1), abs(p[1] / r.u - 1)])
     assert (worst[0] <= worst[1]).all(), worst
+
+
+@pytest.mark.parametrize("lorentz", [(1.0, 8.0), (8.0, 20.0), (20.0, 50.0)])
+@pytest.mark.parametrize("sigma", [None, (-4, 2.6)])
+@pytest.mark.parametrize("gam", [4.0 / 3.0, 13.0 / 9.0, 5.0 / 3.0])
+def test_relativistic_states_are_answered(wide, gam, sigma, lorentz):
+    """From guesses off by up to e, at most 1% are left to the FP64 iteration."""
+    rng = np.random.default_rng(17)
+    count, answered = 500, 0
+    for _ in range(count):
+        X, gcov, g = _point(0, rng)
+        lf = lorentz[0] * (lorentz[1] / lorentz[0]) ** rng.uniform()
+        P = _state(gcov, rng, X, 0, lf, 10.0 ** rng.uniform(-6, 0),
+                   10.0 ** rng.uniform(*sigma) if sigma else 0.0, None)
+        U = oracle.prim_to_flux(0, 0.9375, 0.3, X, gam, P, 0)
+        answered += wide(U, g, gam, (P[0] + gam * P[1]) * lf * lf * np.exp(rng.uniform(-1, 1)))[0]
+    assert answered >= 0.99 * count
