@@ -468,10 +468,11 @@ extern "C" int grmhd_get_electrons(grmhd_sim *s, double *K, int with_ghosts, int
   if (with_ghosts) {
     CK(cudaMemcpyAsync(K, s->K, sizeof(double) * 2 * (size_t)D.ntot, kind, s->st));
   } else {
-    launch_pack(D, s->K, s->Kh, 0, s->st, 2);
+    // (Kh keeps the ghosts of fixed sides between calls; the face values do not)
+    launch_pack(D, s->K, s->KLf, 0, s->st, 2);
     int rc = launched();
     if (rc != GRMHD_OK) return rc;
-    CK(cudaMemcpyAsync(K, s->Kh, sizeof(double) * 2 * (size_t)nz, kind, s->st));
+    CK(cudaMemcpyAsync(K, s->KLf, sizeof(double) * 2 * (size_t)nz, kind, s->st));
   }
   if (!on_device) CK(cudaStreamSynchronize(s->st));
   return GRMHD_OK;
@@ -485,10 +486,11 @@ extern "C" int grmhd_get_prims(grmhd_sim *s, double *P, int with_ghosts, int on_
   if (with_ghosts) {
     CK(cudaMemcpyAsync(P, s->P, sizeof(double) * NV * (size_t)D.ntot, kind, s->st));
   } else {
-    launch_pack(D, s->P, s->Ph, 0, s->st);
+    // (Ph keeps the ghosts of fixed sides between calls; every predictor forms Uc anew)
+    launch_pack(D, s->P, s->Uc, 0, s->st);
     int rc = launched();
     if (rc != GRMHD_OK) return rc;
-    CK(cudaMemcpyAsync(P, s->Ph, sizeof(double) * NV * (size_t)nz, kind, s->st));
+    CK(cudaMemcpyAsync(P, s->Uc, sizeof(double) * NV * (size_t)nz, kind, s->st));
   }
   if (!on_device) CK(cudaStreamSynchronize(s->st));
   return GRMHD_OK;
