@@ -51,7 +51,7 @@ WIDE_FN void wide_tensor(const double P[NV], const GeoFn &geo, double gm1, doubl
 // The 1D_W function f(W') and its derivative in FP32 (all quantities in units of a
 // power of two near W)
 struct InvF {
-  float d, b, qt2, qb2, qpn, gf;  // D, B^2, Qt^2, (Q.B)^2, Q'.n, (gamma - 1)/gamma
+  float d, b, qt2, qb2, c, gf;  // D, B^2, Qt^2, (Q.B)^2, Q'.n + B^2, (gamma - 1)/gamma
 };
 WIDE_FN float inv_rcpf(float x) {
 #ifdef __CUDA_ARCH__
@@ -71,26 +71,25 @@ WIDE_FN float inv_rsqrtf(float x) {
   return 1.0f / __builtin_sqrtf(x);
 #endif
 }
-// df/dW' from W, 1 - v^2, the Lorentz factor rs and x2 = (Q.B/W)^2.  With dv^2/dW =
-// -2 (v^2 W + x2) / (W (B^2 + W)) the derivative of the formula below is
+// df/dW' from W, 1 - v^2, the Lorentz factor rs and b^2 = B^2 (1 - v^2) + (Q.B/W)^2.  With
+// dv^2/dW = -2 (v^2 W + (Q.B/W)^2) / (W (B^2 + W)) the derivative of the formula below is
 //   df = A (1 - 2 gf + gf r) + gf (1 - v^2) (1 - r),
-// A = (W + b^2)/(W + B^2), b^2 = B^2 (1 - v^2) + x2, r = D rs / W = rho / (rho + gamma u):
-// no difference of large terms at any Lorentz factor or magnetisation (gamma <= 2), so
-// that it has the relative accuracy of 1 - v^2 and rs.
-WIDE_FN float inv_df(const InvF &q, float w, float omv, float rs, float x2) {
-  const float r = q.d * rs * inv_rcpf(w);
-  const float A = (w + (q.b * omv + x2)) * inv_rcpf(w + q.b);
+// A = (W + b^2)/(W + B^2), r = D rs / W = rho / (rho + gamma u): no difference of large
+// terms at any Lorentz factor or magnetisation (gamma <= 2), so that it has the relative
+// accuracy of 1 - v^2.
+WIDE_FN float inv_df(const InvF &q, float w, float omv, float rs, float b2) {
+  const float r = q.d * rs * inv_rcpf(w), A = (w + b2) * inv_rcpf(w + q.b);
   return A * ((1.0f - 2.0f * q.gf) + q.gf * r) + q.gf * omv * (1.0f - r);
 }
 // v^2; f and df are meaningless for v^2 >= 1
 WIDE_FN float inv_f32(const InvF &q, float wp, float &f, float &df) {
-  const float w = wp + q.d, bw = q.b + w, iw = inv_rcpf(w), ib = inv_rcpf(bw);
+  const float w = wp + q.d, iw = inv_rcpf(w), ib = inv_rcpf(q.b + w);
   const float x2 = q.qb2 * iw * iw;
   const float vsq = (q.qt2 + x2 * (q.b + 2.0f * w)) * ib * ib;
-  const float omv = 1.0f - vsq, rs = inv_rsqrtf(omv), sq = omv * rs;
+  const float omv = 1.0f - vsq, rs = inv_rsqrtf(omv), sq = omv * rs, b2 = q.b * omv + x2;
   const float wmr = wp * omv - q.d * vsq * sq * inv_rcpf(1.0f + sq);
-  f = q.qpn + wp - q.gf * wmr + 0.5f * (1.0f + vsq) * q.b - 0.5f * x2;
-  df = inv_df(q, w, omv, rs, x2);
+  f = q.c + wp - q.gf * wmr - 0.5f * b2;
+  df = inv_df(q, w, omv, rs, b2);
   return vsq;
 }
 
@@ -101,10 +100,9 @@ WIDE_FN float inv_f32(const InvF &q, float wp, float &f, float &df) {
 // at Lorentz factors above 8, and up to 88% of such states were left to FP64), then
 // Newton steps whose function is taken in Wide numbers and whose derivative in FP32 of
 // Wide values (each gains 20 bits or doubles the digits), until what f leaves is below
-// 2^-56 of its largest term, the noise of its own operations (2^-57 of 1/(W (B^2 + W))):
-// a step's size says nothing where the derivative may be off.  The state comes from
-// the pass that finds f so.  False, with
-// nothing written, where the iteration of invert_1dw is needed for its answer or
+// 2^-INV_RESIDUAL of B^2 or of its largest term, about the noise of its own operations
+// (1/(W (B^2 + W)) is good to 2^-57): a step's size says nothing where the derivative
+// may be off.  The state comes from the pass that finds f so.  False, with nothing written, where the iteration of invert_1dw is needed for its answer or
 // its failure code: input that is not finite, D <= 0, an iterate with
 // v^2 > 1 - 1e-10, no convergence, u < 0.
 //
@@ -113,7 +111,7 @@ WIDE_FN float inv_f32(const InvF &q, float wp, float &f, float &df) {
 // of the FP64 iteration: Lorentz factors 1 to 3, rho 5e-15 and 1e-13, u 2e-9 and 9e-8; 20 to
 // 50, rho 1e-12 and 7e-11, u 5e-7 and 1e-5.  Three passes, 3.3 at 20 to 50.
 constexpr int INV_F32_MAXIT = 12, INV_WIDE_MAXIT = 8;
-constexpr u64 INV_RESIDUAL = 8;  // in units of 2^-59 of the largest term
+constexpr int INV_RESIDUAL = 56;
 
 template <bool BLK, class GeoFn>
 WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, double guess,
@@ -167,6 +165,9 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
   const Wide QdB = norm(w_sum<1>(Q1 * n1, Q2 * n2, Q3 * n3));
   ok = ok && w_finite(guess) && (Qtsq.s == 0 || Qtsq.m == 0) && (Bsq.s == 0 || Bsq.m == 0);
 
+  // f = Q'.n + W' - gf (w - rho) + (1 + v^2) B^2/2 - (Q.B/W)^2/2 = C + W' - gf (w - rho) - b^2/2
+  const Wide C = norm(w_sum<1>(Qpn, Bsq));
+
   // the guess, improved in FP32
   Wide Wp = norm(w_sum<1>(wide(guess), -D));
   const int e = -(int)((w_hi(w_bits(guess)) >> 20) & 0x7ff) + 1023;  // guess 2^e in [1, 2)
@@ -175,7 +176,7 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
   q.b = w_to_float(Bsq, e);
   q.qt2 = w_to_float(Qtsq, 2 * e);
   q.qb2 = w_to_float(norm(QdB * QdB), 3 * e);
-  q.qpn = w_to_float(Qpn, e);
+  q.c = w_to_float(C, e);
   q.gf = (float)K.gf;
   {
     // (a root below 1e-6 D is left to the Wide steps)
@@ -201,18 +202,18 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
       ok = false;
   }
 
-  const Wide gf = wide_pos(K.gf), hB = w_scale(Bsq, -1);
+  const Wide gf = wide_pos(K.gf);
   const Wide one = {1ull << 61, 0, -61};
   bool done = false;
-  Wide W, iB, x, x2, omv, rs, wmr;
+  Wide iB, x, bsq, omv, rs, wmr;
 #pragma unroll 1
   for (int it = 0; it < INV_WIDE_MAXIT && ok; it++) {
-    W = norm(w_sum<1>(Wp, D));
+    const Wide W = norm(w_sum<1>(Wp, D));
     const Wide BW = norm(w_sum<1>(Bsq, W));
     const Wide ix = w_rcp(norm(BW * W));
     iB = norm(W * ix);              // 1/(B^2 + W)
     x = norm(QdB * norm(BW * ix));  // Q.B / W
-    x2 = x * x;
+    const Wide x2 = x * x;
     const Wide vsq = norm(norm(w_sum<1>(Qtsq, x2 * norm(w_sum<1>(Bsq, w_scale(W, 1))))) * norm(iB * iB));
     omv = norm(w_sum<1>(one, -vsq));
     ok = omv.s == 0 && omv.x >= -62 - 33;  // 1 - v^2 >= 2^-33
@@ -221,14 +222,14 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
     const Wide sq = norm(omv * rs);
     // w - rho = W' (1 - v^2) - D v^2 sq / (1 + sq)
     wmr = w_sum<0>(Wp * omv, -(norm(norm(D * vsq) * sq) * w_rcp(norm(w_sum<1>(one, sq)))));
-    const Wide t = w_sum<2>(Qpn, Wp, hB, -(gf * norm(wmr)));
-    const Wide f = w_sum<1>(t, hB * vsq, -w_scale(x2, -1));
-    // (the two sums shift their largest term right by two bits and one)
-    done = f.m < INV_RESIDUAL;
+    bsq = w_sum<0>(Bsq * omv, x2);
+    const Wide f = w_sum<2>(C, Wp, -(gf * norm(wmr)), -w_scale(bsq, -1));
+    // (the sum shifts its largest term right by two bits)
+    done = f.m < 1ull << w_min(w_max(f.x - 2, Bsq.x) - f.x + (62 - INV_RESIDUAL), 62);
     if (done) break;
-    const float df = inv_df(q, w_to_float(W, e), w_to_float(omv, 0), w_to_float(rs, 0),
-                            w_to_float(norm(x2), e));
-    const Wide step = norm(norm(f) * wide_posf(inv_rcpf(df)));
+    const float vf = w_to_float(omv, 0);
+    const float df = inv_df(q, w_to_float(W, e), vf, inv_rsqrtf(vf), w_to_float(bsq, e));
+    const Wide step = norm(f) * wide_posf(inv_rcpf(df));
     const Wide n = norm(w_sum<1>(Wp, -step));
     ok = df > 0.0f;
     // below zero by the derivative's error: the root is nearer to it than that
@@ -244,7 +245,7 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
   P[U3] = w_to_double(fac * norm(w_sum<1>(Qt3, x * n3)));
 #pragma unroll
   for (int i = 0; i < 3; i++) P[B1 + i] = b[i];
-  bsq_out = w_to_double(w_sum<0>(Bsq * omv, x2));
+  bsq_out = w_to_double(bsq);
   lorentz_out = w_to_double(rs);
   return true;
 #undef GCOV
