@@ -745,9 +745,7 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
       case 4:
         L(PC_FACE2, [&](unsigned nb, unsigned bs, BView V) { kp_face<2><<<nb, bs, 0, st>>>(V, 0); });
         break;
-      case 5:  // the inversion, of what the source pass before it leaves
-        L(PC_SRC64, [&](unsigned nb, unsigned bs, BView V) { kp_source<true><<<nb, bs, 0, st>>>(V); });
-        L(PC_SRCX, [&](unsigned nb, unsigned bs, BView V) { kp_source_ff<true><<<nb, bs, 0, st>>>(V); });
+      case 5:
         L(PC_UPD, [&](unsigned nb, unsigned bs, BView V) { kp_invert<<<nb, bs, 0, st>>>(V, 0, 0.5); });
         break;
       case 8:
@@ -789,6 +787,8 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
   for (const Group &gr : groups) {
     if (p.nblocks[gr.cls] <= 0) continue;
     const int bs0 = p.bs[gr.cls], sc0 = p.sched[gr.cls];
+    // the inversion's scratch, which the reconstructions before it may share
+    if (gr.cls == PC_UPD) source_pass(p, 0, st, nullptr);
     double best = time_passes(st, trials, [&] { pass(gr.which); });
     before += best;
     int best_bs = bs0, best_sc = sc0;
