@@ -475,7 +475,11 @@ int grmhd_batch_sync(grmhd_batch *batch);
 
 /* Device bytes grmhd_create would allocate for this grid (state, stage
  * scratch, fluxes, geometry, flags, clock, the FP32 copies of the mixed
- * mode and the launch plan); GRMHD_ERR_INVALID as grmhd_create. */
+ * mode and the launch plan); GRMHD_ERR_INVALID as grmhd_create.  FP64 and
+ * float-float grids of at most 2^21 zones count five arrays of [8][zones
+ * with ghosts] doubles that let their directions run side by side;
+ * grmhd_create leaves them out, and steps the grid slower to the same
+ * result, where that much memory is not free. */
 int grmhd_footprint(const grmhd_grid *grid, const grmhd_metric *metric,
                     const grmhd_params *params, size_t *bytes);
 

@@ -165,8 +165,8 @@ static int flat3_of(const Dims &D, const grmhd_params *params) {
   return (D.n[2] == 1 && params->bc[2][0] == GRMHD_BC_PERIODIC && !params->electrons.model) ? 1 : 0;
 }
 
-extern "C" int grmhd_footprint(const grmhd_grid *grid, const grmhd_metric *metric,
-                               const grmhd_params *params, size_t *bytes) {
+int sim_footprint(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
+                  bool lean, size_t *bytes) {
   Dims D;
   if (!bytes) return GRMHD_ERR_INVALID;
   const int rc = validate_problem(grid, metric, params, &D);
@@ -188,15 +188,18 @@ extern "C" int grmhd_footprint(const grmhd_grid *grid, const grmhd_metric *metri
   b += (size_t)plan_bytes(D, flat3_of(D, params), params->precision,
                          params->floors_on && params->floor_frame == GRMHD_FLOOR_DRIFT,
                          params->electrons.model != GRMHD_ELEC_OFF);
-  if (splits(D, pr)) b += sizeof(double) * NV * tot * SPLIT_SETS;
+  if (!lean && splits(D, pr)) b += sizeof(double) * NV * tot * SPLIT_SETS;
   *bytes = b;
   return GRMHD_OK;
 }
 
-int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
-               void *stream, const BlockSpec *blk, grmhd_sim **out) {
-  if (!out) return GRMHD_ERR_INVALID;
-  *out = nullptr;
+extern "C" int grmhd_footprint(const grmhd_grid *grid, const grmhd_metric *metric,
+                               const grmhd_params *params, size_t *bytes) {
+  return sim_footprint(grid, metric, params, false, bytes);
+}
+
+static int build_sim(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
+                     void *stream, const BlockSpec *blk, bool lean, grmhd_sim **out) {
   if (!blk) {
     const int rc = validate_problem(grid, metric, params, nullptr);
     if (rc != GRMHD_OK) return rc;
@@ -234,7 +237,7 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
   const size_t fb = sizeof(double) * NV * (size_t)tot;
   // P, Ph, F[3], Lf, Rf, Uc and what a split grid adds share one allocation
   const int prec = params->precision;
-  const int nset = 8 + (splits(D, prec) ? SPLIT_SETS : 0);
+  const int nset = 8 + (!lean && splits(D, prec) ? SPLIT_SETS : 0);
   bool ok = cudaMalloc(&s->P, fb * nset) == cudaSuccess &&
             cudaMalloc(&s->emf, sizeof(double) * 3 * (size_t)tot) == cudaSuccess &&
             cudaMalloc(&s->geom, sizeof(double) * NLOC * G_NCOMP * (size_t)D.n2d) == cudaSuccess &&
@@ -386,9 +389,19 @@ int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_p
   return GRMHD_OK;
 }
 
+int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
+               void *stream, const BlockSpec *blk, bool lean, grmhd_sim **out) {
+  if (!out) return GRMHD_ERR_INVALID;
+  *out = nullptr;
+  const int rc = build_sim(grid, metric, params, stream, blk, lean, out);
+  // what runs the directions side by side is left out where memory is short
+  return (rc == GRMHD_ERR_NOMEM && !lean) ? build_sim(grid, metric, params, stream, blk, true, out)
+                                          : rc;
+}
+
 extern "C" int grmhd_create(const grmhd_grid *grid, const grmhd_metric *metric,
                             const grmhd_params *params, void *stream, grmhd_sim **out) {
-  return sim_create(grid, metric, params, stream, nullptr, out);
+  return sim_create(grid, metric, params, stream, nullptr, false, out);
 }
 
 extern "C" int grmhd_destroy(grmhd_sim *s) {

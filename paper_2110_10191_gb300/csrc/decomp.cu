@@ -215,7 +215,7 @@ extern "C" int grmhd_decomp_create(const grmhd_grid *grid, const grmhd_metric *m
           if (xl) bp.bc[d][0] = BC_EXCHANGE;
           if (xh) bp.bc[d][1] = BC_EXCHANGE;
         }
-        rc = sim_create(grid, metric, &bp, stream, &sp, &dc->blocks[b]);
+        rc = sim_create(grid, metric, &bp, stream, &sp, false, &dc->blocks[b]);
         if (rc != GRMHD_OK) {
           decomp_free(dc);
           delete dc;

@@ -56,9 +56,13 @@ struct BlockSpec {
 // grmhd_create for a whole grid (blk == NULL) or for one block of a
 // decomposed grid (grid: the global grid; params->bc with GRMHD_BC_EXCHANGE
 // on the sides shared with other blocks; no validation: the caller
-// validated the global problem).
+// validated the global problem).  lean: without the arrays of a split grid (plan.h),
+// which are also left out where they do not fit; the same results, slower.
 int sim_create(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
-               void *stream, const BlockSpec *blk, grmhd_sim **out);
+               void *stream, const BlockSpec *blk, bool lean, grmhd_sim **out);
+// grmhd_footprint, or (lean) that of a simulation created so
+int sim_footprint(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
+                  bool lean, size_t *bytes);
 // the argument checks of grmhd_create
 int validate_problem(const grmhd_grid *grid, const grmhd_metric *metric, const grmhd_params *params,
                      grmhd::Dims *Dout);
