@@ -546,8 +546,9 @@ int grmhd_server_create(const grmhd_server_config *cfg, grmhd_server **out);
  * buffers alive and untouched until the request's result has been polled.
  * t_arrival: the request's arrival on the server clock (a negative value:
  * now); time-to-result is counted from it.  Returns at once; a request
- * whose footprint exceeds the whole budget is refused (GRMHD_ERR_NOMEM),
- * invalid arguments give GRMHD_ERR_INVALID. */
+ * whose footprint, without the arrays that grmhd_create may leave out,
+ * exceeds the whole budget is refused (GRMHD_ERR_NOMEM), invalid arguments
+ * give GRMHD_ERR_INVALID. */
 int grmhd_server_submit(grmhd_server *srv, long long id, const grmhd_grid *grid,
                         const grmhd_metric *metric, const grmhd_params *params,
                         const double *P_in, int in_ghosts, double *P_out, int out_ghosts,

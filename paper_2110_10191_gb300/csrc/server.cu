@@ -19,7 +19,7 @@
 #include <thread>
 #include <vector>
 
-#include "../../include/grmhd.h"
+#include "sim_impl.h"
 
 namespace {
 
@@ -35,6 +35,7 @@ struct Request {
   int in_ghosts, out_ghosts;
   long long nsteps, remaining;
   size_t bytes;
+  bool lean;  // created without a split grid's arrays, which alone exceed the budget
   long long zones;
   double t_arrival, t_admit, t_done;
   int status;
@@ -129,7 +130,8 @@ static void admit(grmhd_server *s) {
     int rc = (cudaStreamCreateWithFlags(&r->st, cudaStreamNonBlocking) == cudaSuccess)
                  ? GRMHD_OK
                  : GRMHD_ERR_CUDA;
-    if (rc == GRMHD_OK) rc = grmhd_create(&r->grid, &r->metric, &r->params, r->st, &r->sim);
+    if (rc == GRMHD_OK)
+      rc = sim_create(&r->grid, &r->metric, &r->params, r->st, nullptr, r->lean, &r->sim);
     {
       std::lock_guard<std::mutex> lk(s->mu);
       if (rc == GRMHD_OK) {
@@ -304,7 +306,10 @@ static int submit(grmhd_server *s, long long id, const grmhd_grid *grid,
   const bool elec = params->electrons.model != GRMHD_ELEC_OFF;
   if (elec != (K_in != nullptr) || elec != (K_out != nullptr)) return GRMHD_ERR_INVALID;
   size_t bytes = 0;
-  const int rc = grmhd_footprint(grid, metric, params, &bytes);
+  int rc = sim_footprint(grid, metric, params, false, &bytes);
+  if (rc != GRMHD_OK) return rc;
+  const bool lean = bytes > s->cfg.hbm_budget;
+  if (lean) rc = sim_footprint(grid, metric, params, true, &bytes);
   if (rc != GRMHD_OK) return rc;
   if (bytes > s->cfg.hbm_budget) return GRMHD_ERR_NOMEM;
   Request *r = new (std::nothrow) Request();
@@ -322,6 +327,7 @@ static int submit(grmhd_server *s, long long id, const grmhd_grid *grid,
   r->out_ghosts = out_ghosts ? 1 : 0;
   r->nsteps = r->remaining = nsteps;
   r->bytes = bytes;
+  r->lean = lean;
   r->zones = (long long)grid->n1 * grid->n2 * grid->n3;
   r->t_arrival = t_arrival < 0.0 ? now_s(s) : t_arrival;
   r->t_admit = -1.0;

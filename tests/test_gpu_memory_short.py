@@ -44,3 +44,21 @@ def test_create_with_little_memory_free(grmhd):
         del hold
         torch.cuda.empty_cache()
     assert np.array_equal(got, ref)
+
+
+def test_server_budget_below_the_full_footprint(grmhd):
+    pr = pb.fm_torus(24, 20, 8)
+    ref = _alone(grmhd, pr, 3)
+    srv = grmhd.Server(hbm_budget=grmhd.footprint(pr) - 1)
+    try:
+        srv.submit(0, pr, 3)
+        srv.drain(timeout_ms=60000)
+        res, st = srv.poll(4), srv.stats()
+        assert len(res) == 1 and res[0]["status"] == 0 and np.array_equal(res[0]["P"], ref)
+        assert st["peak_bytes"] == grmhd.footprint(pr) - _split_bytes(pr)
+    finally:
+        srv.close()
+    srv = grmhd.Server(hbm_budget=grmhd.footprint(pr) - _split_bytes(pr) - 1)
+    with pytest.raises(grmhd.GrmhdError):
+        srv.submit(0, pr, 3)
+    srv.close()
