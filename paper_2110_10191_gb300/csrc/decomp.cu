@@ -159,14 +159,11 @@ static int bidx(const grmhd_decomp *dc, int bx, int by, int bz) {
   return bx + dc->nb[0] * (by + dc->nb[1] * bz);
 }
 
-extern "C" int grmhd_decomp_create(const grmhd_grid *grid, const grmhd_metric *metric,
-                                   const grmhd_params *params, const int nblocks[3], void *stream,
-                                   grmhd_decomp **out) {
-  if (!out || !nblocks) return GRMHD_ERR_INVALID;
-  *out = nullptr;
-  Dims G;
-  int rc = validate_problem(grid, metric, params, &G);
-  if (rc != GRMHD_OK) return rc;
+// grmhd_decomp_create of a valid problem of dimensions G; lean: of lean blocks
+static int build_decomp(const grmhd_grid *grid, const grmhd_metric *metric,
+                        const grmhd_params *params, const Dims &G, const int nblocks[3],
+                        void *stream, bool lean, grmhd_decomp **out) {
+  int rc = GRMHD_OK;
   for (int d = 0; d < 3; d++) {
     if (nblocks[d] < 1 || nblocks[d] > G.n[d]) return GRMHD_ERR_INVALID;
     if (nblocks[d] > 1 && G.n[d] / nblocks[d] < NG) return GRMHD_ERR_INVALID;  // blocks >= NG zones
@@ -215,7 +212,7 @@ extern "C" int grmhd_decomp_create(const grmhd_grid *grid, const grmhd_metric *m
           if (xl) bp.bc[d][0] = BC_EXCHANGE;
           if (xh) bp.bc[d][1] = BC_EXCHANGE;
         }
-        rc = sim_create(grid, metric, &bp, stream, &sp, false, &dc->blocks[b]);
+        rc = sim_create(grid, metric, &bp, stream, &sp, lean, &dc->blocks[b]);
         if (rc != GRMHD_OK) {
           decomp_free(dc);
           delete dc;
@@ -283,6 +280,22 @@ extern "C" int grmhd_decomp_create(const grmhd_grid *grid, const grmhd_metric *m
   }
   *out = dc;
   return GRMHD_OK;
+}
+
+extern "C" int grmhd_decomp_create(const grmhd_grid *grid, const grmhd_metric *metric,
+                                   const grmhd_params *params, const int nblocks[3], void *stream,
+                                   grmhd_decomp **out) {
+  if (!out || !nblocks) return GRMHD_ERR_INVALID;
+  *out = nullptr;
+  Dims G;
+  int rc = validate_problem(grid, metric, params, &G);
+  if (rc != GRMHD_OK) return rc;
+  // the blocks step as one plan, which splits by the zones of all of them
+  const bool lean = n_zone(G) > SPLIT_ZONES;
+  rc = build_decomp(grid, metric, params, G, nblocks, stream, lean, out);
+  return (rc == GRMHD_ERR_NOMEM && !lean)
+             ? build_decomp(grid, metric, params, G, nblocks, stream, true, out)
+             : rc;
 }
 
 extern "C" int grmhd_decomp_destroy(grmhd_decomp *dc) {

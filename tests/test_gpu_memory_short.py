@@ -62,3 +62,17 @@ def test_server_budget_below_the_full_footprint(grmhd):
     with pytest.raises(grmhd.GrmhdError):
         srv.submit(0, pr, 3)
     srv.close()
+
+
+def test_blocks_of_a_large_grid_take_no_more_than_it(grmhd):
+    """A decomposed grid of more than 2^21 zones does not run its directions side by
+    side, whatever the size of its blocks."""
+    import torch
+    pr = pb.fm_torus(160, 128, 128)
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    d = grmhd.Decomp(pr, (2, 1, 1))
+    used = free - torch.cuda.mem_get_info()[0]
+    d.close()
+    # ghosts of two blocks against one: 6 of 166 layers, and the exchange's tables
+    assert used <= 1.1 * grmhd.footprint(pr)
