@@ -131,8 +131,11 @@ void plan_counts(const Dims &D, int flat3, int prec, int drift, int elec, int rw
 // face arrays of their own and run side by side.  A small grid's kernels leave
 // most of the GPU idle, each waiting for its threads' chains of work; side by side
 // a cycle of a 64x64 mode takes 82 us against 119, of 217x217 zones 227 against
-// 264, of 64^3 1042 against 1148, of 100^3 3.37 against 3.47 ms (where the kernels'
-// tails overlap); beyond, the gain no longer pays for the memory.
+// 264, of 64^3 1.02 against 1.13 ms for 0.11 GB more memory; of larger grids, where only
+// the kernels' tails overlap, 100^3 3.36 against 3.46 ms (0.38 GB), 128^3 6.79 against
+// 6.89 (0.77), 136^3 8.07 against 8.16 (0.92), 160^3 12.95 against 13.05 (1.46), 192^3
+// 22.15 against 22.23 (2.48).  The line lies where the gain, 1.4% there, has come down to
+// 1%; the arrays are left out where they do not fit (sim_create).
 constexpr long long SPLIT_ZONES = 1 << 21;
 constexpr int SPLIT_SETS = 5;  // arrays of [8][ntot] they take
 // (FP32 fluxes need no face arrays: their space is the update's scratch at once)
@@ -187,7 +190,8 @@ int plan_autotune(Plan &p, int trials, cudaStream_t st, double *ms_before, doubl
 // stage input: 0 = P, 1 = Ph.  Reconstruction + face fluxes (FP64, FP32 or
 // float-float per grid) with their boundary fixes; with_source: and the update's
 // source pass.  The signal speeds' maxima add to what the clocks hold, which is
-// zero between the library's calls: whoever calls this resets them after reading.
+// zero between the library's calls: whoever calls this resets them after reading (a
+// decomposed grid, whose blocks nothing else steps, before its next step).
 int plan_fluxes(const Plan &p, int in, bool with_source, cudaStream_t st, PlanHook *h);
 // the fluxes of every layer and flux-CT in place of the induction fluxes: F as
 // grmhd_get_fluxes returns it

@@ -199,7 +199,7 @@ WIDE_FN WideNum wide_q_low(const WidePair &p, u64 D13) { return wide_weight(D13,
 WIDE_FN WideNum wide_q_mid(const WidePair &p, u64 D13) { return wide_weight(D13, p.a + p.b, p.x); }
 WIDE_FN WideNum wide_q_high(const WidePair &p, u64 D13) { return wide_weight(D13, 3 * p.a - p.b, p.x); }
 
-// N / H 2^x as a double (rounded to nearest but for 2^-4 ulp), for H >= 2^54
+// N / H 2^x as a double (rounded to nearest but for 2^-4 ulp; 0 below 2^-1022), for H >= 2^54
 // and bad: NaN.  Both are normalised, h in [2^63, 2^64) and n in [2^62, 2^63),
 // and n / h = (q0 + f) / 2^31 comes in two digits from r <= 2^95 / h: q0 = n r
 // (at most 4.5 low) and f from the remainder n 2^31 - q0 h.

@@ -115,7 +115,8 @@ WIDE_FN Wide w_sum(const Wide &a, const Wide &b, const Wide &c, const Wide &d, c
                   a.s + b.s + c.s + d.s + e.s, x);
 }
 
-// the nearest double (the tail beyond 64 bits counted as zero)
+// the nearest double (the tail beyond 64 bits counted as zero); 0 below 2^-1022, infinite or
+// not a number beyond the largest
 WIDE_FN double w_to_double(const Wide &a) {
   const int k = w_clz64(a.m);
   const u64 m = a.m << (k & 63);
@@ -178,7 +179,8 @@ WIDE_FN Wide w_rcp(const Wide &a) {
   return q;
 }
 
-// a 2^k as a float (24 bits of the upper word), saturating to 0 and infinity
+// a 2^k as a float (24 bits of the upper word); infinite beyond the largest, and no less
+// than 2^-96 for a normalised a (what is smaller comes out larger)
 WIDE_FN float w_to_float(const Wide &a, int k) {
   const int e = w_min(w_max(a.x + 32 + k, -126), 127);
 #ifdef __CUDA_ARCH__
