@@ -190,7 +190,10 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
       if (inv_f32(q, w, f, df) < 0.99999f) {
         if (f > 0.0f) hi = w;
         n = w - f * inv_rcpf(df);
-        if (!(n > 0.0f)) n = 0.5f * w;
+        if (!(n > 0.0f)) {
+          if (it > 4) break;  // (no positive root, or one below FP32's noise)
+          n = 0.5f * w;
+        }
       } else {  // below the root
         n = (hi < INFINITY) ? 0.5f * (w + hi) : w + (w + q.d);
       }
@@ -233,9 +236,11 @@ WIDE_FN bool wide_invert(const double U[NV], const GeoFn &geo, const GasK &K, do
     const float df = inv_df(q, w_to_float(W, e), vf, inv_rsqrtf(vf), w_to_float(bsq, e));
     const Wide step = norm(f) * wide_posf(inv_rcpf(df));
     const Wide n = norm(w_sum<1>(Wp, -step));
-    ok = df > 0.0f;
-    // below zero by the derivative's error: the root is nearer to it than that
-    Wp = (n.s == 0 && n.m != 0) ? n : w_scale(Wp, -16);
+    // below zero by no more than the derivative's error, the root is nearer to it than
+    // that; by more there is none (u < 0)
+    const bool above = n.s == 0 && n.m != 0;
+    ok = df > 0.0f && (above || n.x < Wp.x - 12);
+    Wp = above ? n : w_scale(Wp, -16);
   }
   ok = ok && done && (wmr.s == 0 || wmr.m == 0);
   if (!ok) return false;
