@@ -56,14 +56,14 @@ WORKLOADS = {
 # list of the 2-cycle bench command.
 # The figures hold while the kernel sources hash to src_hash; otherwise the
 # bench reports the traffic as unknown (null).
-NCU_TRAFFIC = {"src_hash": "d2cbd87004ae6e76",
-               "torus128": {"recon": 155200000 + 226110000, "flux": 295320000 + 224430000,
-                            "update": 357870000 + 271250000}}
+NCU_TRAFFIC = {"src_hash": "ad1854cee720f4c6",
+               "torus128": {"recon": 155170000 + 226110000, "flux": 295310000 + 224470000,
+                            "update": 357460000 + 255070000}}
 # sm__inst_executed_pipe_fp64.avg.pct_of_peak_sustained_active of ncu captures of
 # single launches (the mean over kp_recon<0..2>; over kp_face<0..2,0>; over kp_source<1>
 # and kp_invert): the hardware's view of the same kernels, as a fraction of the
 # nominal 2 FP64 instructions per SM per clock
-NCU_FP64_PIPE = {"torus128": {"recon": 0.251, "flux": 0.673, "update": 0.676}}
+NCU_FP64_PIPE = {"torus128": {"recon": 0.251, "flux": 0.673, "update": 0.678}}
 
 
 def kernel_source_hash():
